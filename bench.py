@@ -36,8 +36,8 @@ METRIC = ("node-updates/s (GLUPS) of the FP32 step with double-float temperature
           "double Mach reflection 4096x1024")
 BYTES_PER_NODE = {"fp64": 144, "fp32": 72, "fp32_t64": 72, "fp32_tdf": 72, "fp32_cons": 72}
 # FP64 arithmetic of one node update as written (moments, equilibrium,
-# update): 56 adds / multiplies / reciprocals and 71 FMAs = 198 flops.
-FP64_FLOPS_PER_NODE = 198
+# update): 28 adds and multiplies and 71 FMAs = 170 flops.
+FP64_FLOPS_PER_NODE = 170
 PRECISION_NOTES = {
     "fp32_tdf": ("f stored and updated in FP32; T recovered from the internal energy "
                  "sum_i f_i (|v_i - u|^2 + eta_i^2), its nine products formed exactly and summed in "

@@ -49,6 +49,7 @@ KERNEL_SOURCES = {
     "k_step_tile": ("lbm_step.cu", "lbm_device.cuh", "lbm_ptx.cuh"),
     "k_step_vec": ("lbm_step.cu", "lbm_device.cuh", "lbm_ptx.cuh"),
     "k_step_simple": ("lbm_step.cu", "lbm_device.cuh", "lbm_ptx.cuh"),
+    "k_step_fp64": ("lbm_step.cu", "lbm_fp64.cuh", "lbm_device.cuh", "lbm_ptx.cuh"),
     "k_step_ring": ("lbm_step.cu", "lbm_device.cuh", "lbm_ptx.cuh"),
 }
 

@@ -1,0 +1,133 @@
+// lbm_fp64.cuh -- the node update of the FP64 step (Eqs. e4-e7, e16-e18,
+// SEC-VON-11), written for the fewest FP64 instructions.
+//
+// GB300 issues one FP64 warp instruction per SM in 16 cycles (1/64 of the
+// FP32 rate), so the FP64 step takes as long as its FP64 instruction count.
+// This form needs 99 of them a node: 54 for moments and equilibrium, 45 for
+// the five-point update.  The shared templates of lbm_device.cuh, whose
+// operation order the FP32 modes are tied to, take 124.  What is saved:
+//  * sums and differences of opposite pairs serve density and momentum;
+//  * the equilibrium is formed from density-weighted moments -- rho,
+//    p = rho T, g = rho u / c1 and g.u / c1 -- so that most products with
+//    rho fall away, and B v.u needs no product with u either;
+//  * omega and the speeds are folded into the constants (Fp64Step);
+//  * the factor (b + 2) T + u^2 of both velocity sets' B is formed once;
+//  * (v.u)^2 of the diagonals comes from u^2 and 2 ux uy;
+//  * the reciprocal of the density is one cubic Newton step from the
+//    hardware's approximation.
+#pragma once
+
+#include "lbm_device.cuh"
+
+namespace lbm {
+
+// Constants of the FP64 step; w[i][s] as in Model.  With U = u / c1,
+// g = rho U, p = rho T, and q = g.U = rho u^2 / c1^2:
+struct Fp64Step {
+    double w[9][5];
+    double kap;              // d / c1
+    double te, t1, t2;       // eta0^2 / b, c1^2 / b, c2^2 / b:  p = te f_0 + t1 (s14 - q) + t2 s58
+    double k0;               // omega A_0 / T
+    double vp;               // (b + 2) / c1^2:  V = (vp p + q) / rho
+    double a1r, a1p, a1q;    // omega rho A_1..4 = a1r rho + a1p p + a1q q
+    double a5r, a5p, a5q;    // omega rho A_5..8 + the u^2 part of its D (v.u)^2
+    double h1;               // omega D_1..4 c1^4 = omega / 2
+    double b1c, b1v;         // omega c1^2 B_1..4 = b1c + b1v V
+    double b5c, b5v;         // omega c1 d B_5..8
+    double k5;               // 2 omega D_5 c1^2 d^2
+};
+
+inline Fp64Step fp64_step(const Model<double>& M) {
+    Fp64Step C;
+    for (int i = 0; i < 9; ++i)
+        for (int s = 0; s < 5; ++s) C.w[i][s] = M.w[i][s];
+    const double b = M.b, cd = M.c1 * M.d, om = M.omega;
+    C.kap = M.d / M.c1;
+    C.te = M.eta2 * M.inv_b;
+    C.t1 = M.c1s * M.inv_b;
+    C.t2 = M.c2s * M.inv_b;
+    C.k0 = om * M.k0;
+    C.vp = (b + 2.0) / M.c1s;
+    C.a1r = om * M.a1c;
+    C.a1p = om * M.a1T;
+    C.a1q = om * M.a1u * M.c1s;
+    C.a5r = om * M.a5c;
+    C.a5p = om * M.a5T;
+    C.a5q = om * (M.a5u + M.D5 * M.d * M.d) * M.c1s;
+    C.h1 = om * M.D1 * M.c1s * M.c1s;
+    // B = bc + bT T + bu u^2 with bT = (b + 2) bu (Eq. e18)
+    C.b1c = om * M.c1s * M.b1c;
+    C.b1v = om * M.c1s * M.b1u * M.c1s;
+    C.b5c = om * cd * M.b5c;
+    C.b5v = om * cd * M.b5u * M.c1s;
+    C.k5 = 2.0 * om * M.D5 * cd * cd;
+    return C;
+}
+
+// 1 / a: the hardware approximation x (its error e = 1 - a x is about 2^-20)
+// and one step of Newton's iteration carried to third order,
+// x (1 + e + e^2), whose error is e^3.
+__device__ __forceinline__ double fp64_rcp(double a) {
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(a));
+    const double e = __fma_rn(-a, x, 1.0);
+    return __fma_rn(x, __fma_rn(e, e, e), x);
+}
+
+// The bits of health() without FP64 comparisons (they would take the FP64
+// pipe): rho > 0 and p > 0 from the sign, and V = ((b + 2) T + u^2) / c1^2 is
+// finite only if T, u and 1 / rho are.
+__device__ __forceinline__ unsigned fp64_health(double rho, double p, double V) {
+    const bool finite = (__double2hiint(V) & 0x7ff00000) != 0x7ff00000;
+    if (__double_as_longlong(rho) <= 0 || !finite) return ST_NONPHYSICAL;
+    return __double_as_longlong(p) > 0 ? 0u : ST_T_NONPOS;
+}
+
+// Relaxation terms omega f^eq_i of a node; returns its health bits.
+__device__ __forceinline__ unsigned fp64_relaxation(const Fp64Step& C, const double (&f)[9], double (&r)[9]) {
+    // differences along +x, +y and the two diagonals, sums of the pairs
+    const double ax = f[3] - f[1], ay = f[4] - f[2], ar = f[7] - f[5], am = f[6] - f[8];
+    const double s14 = (f[1] + f[3]) + (f[2] + f[4]);
+    const double s58 = (f[5] + f[7]) + (f[6] + f[8]);
+    const double rho = (f[0] + s14) + s58;
+    const double inv = fp64_rcp(rho);
+    const double gx = __fma_rn(C.kap, ar + am, ax), gy = __fma_rn(C.kap, ar - am, ay);
+    const double Ux = gx * inv, Uy = gy * inv;
+    const double xx = gx * Ux, yy = gy * Uy, xy = gx * Uy;
+    const double q = xx + yy;
+    const double p = __fma_rn(C.te, f[0], __fma_rn(C.t1, s14 - q, C.t2 * s58));
+    const double V = __fma_rn(C.vp, p, q) * inv;
+    r[0] = C.k0 * p;
+    {
+        const double A = __fma_rn(C.a1p, p, __fma_rn(C.a1q, q, C.a1r * rho));
+        const double B = __fma_rn(C.b1v, V, C.b1c);
+        const double sx = __fma_rn(C.h1, xx, A), sy = __fma_rn(C.h1, yy, A);
+        r[1] = __fma_rn(-B, gx, sx);
+        r[3] = __fma_rn(B, gx, sx);
+        r[2] = __fma_rn(-B, gy, sy);
+        r[4] = __fma_rn(B, gy, sy);
+    }
+    {
+        const double A = __fma_rn(C.a5p, p, __fma_rn(C.a5q, q, C.a5r * rho));
+        const double B = __fma_rn(C.b5v, V, C.b5c);
+        const double sr = __fma_rn(C.k5, xy, A), sm = __fma_rn(-C.k5, xy, A);
+        const double gr = gx + gy, gm = gx - gy;
+        r[5] = __fma_rn(-B, gr, sr);
+        r[7] = __fma_rn(B, gr, sr);
+        r[6] = __fma_rn(B, gm, sm);
+        r[8] = __fma_rn(-B, gm, sm);
+    }
+    return fp64_health(rho, p, V);
+}
+
+// f' = w0 c + w1 e + w2 w + w3 n + w4 s + r (Eq. SEC-VON-11, folded weights).
+__device__ __forceinline__ double fp64_update(const Fp64Step& C, int i, double r, double c, double e, double w,
+                                              double n, double s) {
+    double acc = __fma_rn(C.w[i][0], c, r);
+    acc = __fma_rn(C.w[i][1], e, acc);
+    acc = __fma_rn(C.w[i][2], w, acc);
+    acc = __fma_rn(C.w[i][3], n, acc);
+    return __fma_rn(C.w[i][4], s, acc);
+}
+
+}  // namespace lbm

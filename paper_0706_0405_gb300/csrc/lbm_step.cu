@@ -4,8 +4,10 @@
 // -> beta-upwind first and central second differences (Eqs. SEC-VON-2a/2b)
 // -> BGK relaxation and forward-Euler update, one pass over the grid, with the
 // next level's ghost layer written by the edge nodes in the same pass.
+#include "lbm_fp64.cuh"
 #include "lbm_launch.h"
 #include "lbm_ptx.cuh"
+
 
 namespace lbm {
 
@@ -17,14 +19,76 @@ constexpr uint32_t kWaitLimit = 1u << 22;
 // neighbours of all nine populations (the neighbours come from L1/L2: the
 // same line serves the adjacent threads), computes the update in registers and
 // writes nine values.
-template <typename S, int TM>
-__global__ void __launch_bounds__(256) k_step_simple(const S* __restrict__ fin, S* __restrict__ fout,
-                                                     const Model<S> M, const Grid<S> G,
+template <int TM>
+__global__ void __launch_bounds__(256) k_step_simple(const float* __restrict__ fin, float* __restrict__ fout,
+                                                     const Model<float> M, const Grid<float> G,
                                                      long long level, unsigned* status) {
     const int ix = blockIdx.x * blockDim.x + threadIdx.x;
     const int iy = blockIdx.y * blockDim.y + threadIdx.y;
     if (ix >= G.nx || iy >= G.ny) return;
-    report(status, node_step<S, TM, false>(fin, fout, M, G, ix, iy, level));
+    report(status, node_step<float, TM, false>(fin, fout, M, G, ix, iy, level));
+}
+
+// ------------------------------------------------------------ FP64 kernel
+// One thread per node with the FP64 node update of lbm_fp64.cuh, 32 nodes of
+// the flattened grid per CTA.  Bound by the FP64 pipe, whose rate is one warp
+// instruction in about 19 cycles per SM (lbm_probe_rates), so what counts is
+// the number of instructions per node and that every SM has the same share of
+// the warps: one-warp CTAs of consecutive nodes spread the smallest grids
+// over all SMs (CTAs of 64 x 4 nodes put a 400 x 4 grid on seven) and leave
+// neither idle lanes at a row's end nor a ragged last wave.  Each step is a
+// programmatic dependent of the one before.  Measured, us a step, against
+// CTAs of 64 x 4 nodes with the templates' update (124 instructions a node
+// instead of 99): 400 x 4 12.3 -> 6.1, 400 x 100 16.8 -> 11.2, 1024 x 256
+// 65.6 -> 52.9, 2048 x 512 239 -> 198 (99 instructions a node at the probe's
+// FMA rate are 196).  CTAs of 2, 4 and 8 warps: 400 x 100 up to 6 us slower,
+// large grids equal.
+__global__ void __launch_bounds__(32) k_step_fp64(const double* __restrict__ fin, double* __restrict__ fout,
+                                                  const Fp64Step M, const Grid<double> G, long long level,
+                                                  unsigned* status) {
+    // a programmatic dependent of the previous step: no level is touched
+    // before that grid has completed
+    grid_dependency_wait();
+    grid_dependents_launch();
+    const long long n = (long long)G.nx * G.ny;
+    const long long q = (long long)blockIdx.x * 32 + threadIdx.x;
+    if (q >= n) return;
+    int ix, iy;
+    if (n <= 0xffffffffLL) {
+        iy = (int)((unsigned)q / (unsigned)G.nx);
+        ix = (int)((unsigned)q % (unsigned)G.nx);
+    } else {
+        iy = (int)(q / G.nx);
+        ix = (int)(q % G.nx);
+    }
+    const size_t pl = (size_t)G.plane;
+    const double* in = fin + cell(G, ix, iy);
+    double f[9], r[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = __ldg(in + i * pl);
+    report(status, fp64_relaxation(M, f, r));
+    double* out = fout + cell(G, ix, iy);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const double* p = in + i * pl;
+        r[i] = fp64_update(M, i, r[i], f[i], __ldg(p + 1), __ldg(p - 1), __ldg(p + G.row), __ldg(p - G.row));
+        out[i * pl] = r[i];
+    }
+    if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) write_ghosts(G, fout, ix, iy, r, level + 1);
+}
+
+cudaError_t launch_fp64(const double* fin, double* fout, const Model<double>& M, const Grid<double>& G,
+                        long long level, unsigned* status, cudaStream_t st) {
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)(((long long)G.nx * G.ny + 31) / 32));
+    lc.blockDim = dim3(32);
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, k_step_fp64, fin, fout, fp64_step(M), G, level, status);
 }
 
 // ------------------------------------------------- FP32 vectorised kernel
@@ -589,11 +653,13 @@ cudaError_t launch_step(const S* fin, S* fout, const Model<S>& M, const Grid<S>&
             if (cfg.ring == 6) return launch_ring<256, 6, TM>(fin, fout, M, G, level, status, cfg.grid, st);
             return launch_ring<256, 4, TM>(fin, fout, M, G, level, status, cfg.grid, st);
         }
+        dim3 block(64, 4);
+        dim3 grid((G.nx + block.x - 1) / block.x, (G.ny + block.y - 1) / block.y);
+        k_step_simple<TM><<<grid, block, 0, st>>>(fin, fout, M, G, level, status);
+        return cudaGetLastError();
+    } else {
+        return launch_fp64(fin, fout, M, G, level, status, st);
     }
-    dim3 block(64, 4);
-    dim3 grid((G.nx + block.x - 1) / block.x, (G.ny + block.y - 1) / block.y);
-    k_step_simple<S, TM><<<grid, block, 0, st>>>(fin, fout, M, G, level, status);
-    return cudaGetLastError();
 }
 
 #define LBM_STEP_INST(S, TM)                                                                     \
