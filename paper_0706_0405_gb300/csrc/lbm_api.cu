@@ -514,6 +514,7 @@ lbm_status lbm_create(int nx, int ny, double b, double tau, double dt, double dx
     if (prec == LBM_FP64) c->cfg = StepConfig{STEP_SIMPLE, 0, 0, 0};
     c->md = build_model(*c);
     c->mf = cast_model<float>(c->md);
+    c->f64 = fp64_step(c->md, b, tau, dt, dvm->c1, dvm->c2, dvm->eta0);
     c->gd = build_grid<double>(*c, c->md);
     c->gf = build_grid<float>(*c, c->md);
     const size_t fbytes = level_bytes(c);
@@ -621,6 +622,7 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
     if (!c->ready) return fail(c, LBM_E_STATE, "lbm_step before lbm_init / lbm_set_f / lbm_load");
     for (int k = 0; k < n; ++k) {
         c->cfg.tmap = c->tmap_ok ? &c->tmap[c->cur] : nullptr;
+        c->cfg.fp64 = &c->f64;
         cudaError_t e = dispatch(c, [&](auto tag, auto tm) {
             using S = decltype(tag);
             constexpr int TM = decltype(tm)::value;
@@ -872,6 +874,7 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step: unpacking abar");
     StepConfig rcfg = c->cfg;  // recomputation reads segment buffers through their own tensor maps
     if (rcfg.variant == STEP_TILE && !tile) rcfg = StepConfig{STEP_SIMPLE, 0, 0, 0};
+    rcfg.fp64 = &c->f64;
     int ac = 0;
     long long L = c->step;
     const long long target = c->step - n;

@@ -46,6 +46,7 @@ struct lbm_ctx {
     size_t stage_bytes = 0;
     Model<double> md{};
     Model<float> mf{};
+    Fp64Step f64{};  // constants of the FP64 step
     Grid<double> gd{};
     Grid<float> gf{};
     StepConfig cfg{};

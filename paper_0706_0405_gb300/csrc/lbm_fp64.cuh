@@ -17,6 +17,8 @@
 //    hardware's approximation.
 #pragma once
 
+#include <cmath>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -37,30 +39,68 @@ struct Fp64Step {
     double k5;               // 2 omega D_5 c1^2 d^2
 };
 
-inline Fp64Step fp64_step(const Model<double>& M) {
+// Unevaluated sum of two doubles, about 106 bits (Dekker / Knuth error-free
+// sums and products), for the constants above on the host.
+struct Wide {
+    double hi, lo;
+    Wide(double h = 0.0, double l = 0.0) : hi(h), lo(l) {}
+    static Wide sum(double a, double b) {
+        const double s = a + b, t = s - a;
+        return Wide(s, (a - (s - t)) + (b - t));
+    }
+    friend Wide operator+(Wide a, Wide b) {
+        Wide s = sum(a.hi, b.hi);
+        return sum(s.hi, s.lo + (a.lo + b.lo));
+    }
+    friend Wide operator*(Wide a, Wide b) {
+        const double p = a.hi * b.hi;
+        return sum(p, std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi));
+    }
+    friend Wide operator-(Wide a) { return Wide(-a.hi, -a.lo); }
+    friend Wide operator-(Wide a, Wide b) { return a + (-b); }
+    friend Wide operator/(Wide a, Wide b) {
+        const double q = a.hi / b.hi;
+        const Wide r = a - b * Wide(q);
+        return sum(q, (r.hi + r.lo) / b.hi);
+    }
+};
+
+// Each constant is formed in Wide arithmetic from the parameters and rounded
+// once: rounded step by step, their mutual errors act as a small source of
+// mass and energy at every node and step (on the 256 x 64 double Mach
+// reflection to t = 0.2, 2560 steps, the error in rho against extended
+// precision is 1.2e-13 rms this way and 4.2e-13 with constants formed in
+// plain double; the templates' update has 2.2e-13).
+inline Fp64Step fp64_step(const Model<double>& M, double b_, double tau, double dt, double c1_, double c2_,
+                          double eta0) {
     Fp64Step C;
     for (int i = 0; i < 9; ++i)
         for (int s = 0; s < 5; ++s) C.w[i][s] = M.w[i][s];
-    const double b = M.b, cd = M.c1 * M.d, om = M.omega;
-    C.kap = M.d / M.c1;
-    C.te = M.eta2 * M.inv_b;
-    C.t1 = M.c1s * M.inv_b;
-    C.t2 = M.c2s * M.inv_b;
-    C.k0 = om * M.k0;
-    C.vp = (b + 2.0) / M.c1s;
-    C.a1r = om * M.a1c;
-    C.a1p = om * M.a1T;
-    C.a1q = om * M.a1u * M.c1s;
-    C.a5r = om * M.a5c;
-    C.a5p = om * M.a5T;
-    C.a5q = om * (M.a5u + M.D5 * M.d * M.d) * M.c1s;
-    C.h1 = om * M.D1 * M.c1s * M.c1s;
-    // B = bc + bT T + bu u^2 with bT = (b + 2) bu (Eq. e18)
-    C.b1c = om * M.c1s * M.b1c;
-    C.b1v = om * M.c1s * M.b1u * M.c1s;
-    C.b5c = om * cd * M.b5c;
-    C.b5v = om * cd * M.b5u * M.c1s;
-    C.k5 = 2.0 * om * M.D5 * cd * cd;
+    const Wide b(b_), c1(c1_), c2(c2_), om = Wide(dt) / Wide(tau);
+    const Wide d = c2 / Wide(1.4142135623730951, -9.667293313452913e-17);  // c2 / sqrt(2)
+    const Wide c1s = c1 * c1, c2s = c2 * c2, es = Wide(eta0) * Wide(eta0), cd = c1 * d, two(2.0);
+    const Wide gap = c1s - c2s;
+    const Wide q1 = Wide(4.0) * gap, q5 = -q1;                     // denominators of A (Eq. e17)
+    const Wide d1 = two * c1s * gap, d5 = -(two * c2s * gap);      // and of B (Eq. e18)
+    const Wide D5 = Wide(1.0) / (two * c2s * c2s), bm = (b - two) / es;
+    C.kap = (d / c1).hi;
+    C.te = (es / b).hi;
+    C.t1 = (c1s / b).hi;
+    C.t2 = (c2s / b).hi;
+    C.k0 = (om * bm).hi;
+    C.vp = ((b + two) / c1s).hi;
+    C.a1r = (-(om * c2s / q1)).hi;
+    C.a1p = (om * (bm * c2s + two) / q1).hi;
+    C.a1q = (om * c2s / q1).hi;                                    // A's u^2 term (c2^2 / c1^2) / q1, times c1^2
+    C.a5r = (-(om * c1s / q5)).hi;
+    C.a5p = (om * (bm * c1s + two) / q5).hi;
+    C.a5q = (om * ((c1s / c2s) / q5 + D5 * d * d) * c1s).hi;
+    C.h1 = (om / two).hi;
+    C.b1c = (-(om * c1s * c2s / d1)).hi;
+    C.b1v = (om * c1s * c1s / d1).hi;                              // B = (-c^2 + c1^2 V) / d
+    C.b5c = (-(om * cd * c1s / d5)).hi;
+    C.b5v = (om * cd * c1s / d5).hi;
+    C.k5 = (two * om * D5 * cd * cd).hi;
     return C;
 }
 

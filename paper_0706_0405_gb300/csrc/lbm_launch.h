@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "lbm_device.cuh"
+#include "lbm_fp64.cuh"
 
 namespace lbm {
 
@@ -57,6 +58,7 @@ struct StepConfig {
     int ring = 0;             // ring: shared-memory row slots (4 or 6; 4 when tx = 128)
     int grid = 0;             // ring, tile: CTAs (0 = SMs x resident CTAs per SM)
     const CUtensorMap* tmap = nullptr;  // tile: tensor map of the input level
+    const Fp64Step* fp64 = nullptr;     // FP64: the step's constants
 };
 
 // Box of the tiled tensor copy of the tile kernel (x, y extent; 9 planes).

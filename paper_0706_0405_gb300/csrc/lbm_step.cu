@@ -4,7 +4,6 @@
 // -> beta-upwind first and central second differences (Eqs. SEC-VON-2a/2b)
 // -> BGK relaxation and forward-Euler update, one pass over the grid, with the
 // next level's ghost layer written by the edge nodes in the same pass.
-#include "lbm_fp64.cuh"
 #include "lbm_launch.h"
 #include "lbm_ptx.cuh"
 
@@ -77,7 +76,7 @@ __global__ void __launch_bounds__(32) k_step_fp64(const double* __restrict__ fin
     if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) write_ghosts(G, fout, ix, iy, r, level + 1);
 }
 
-cudaError_t launch_fp64(const double* fin, double* fout, const Model<double>& M, const Grid<double>& G,
+cudaError_t launch_fp64(const double* fin, double* fout, const Fp64Step& M, const Grid<double>& G,
                         long long level, unsigned* status, cudaStream_t st) {
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3((unsigned)(((long long)G.nx * G.ny + 31) / 32));
@@ -88,7 +87,7 @@ cudaError_t launch_fp64(const double* fin, double* fout, const Model<double>& M,
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, k_step_fp64, fin, fout, fp64_step(M), G, level, status);
+    return cudaLaunchKernelEx(&lc, k_step_fp64, fin, fout, M, G, level, status);
 }
 
 // ------------------------------------------------- FP32 vectorised kernel
@@ -658,7 +657,7 @@ cudaError_t launch_step(const S* fin, S* fout, const Model<S>& M, const Grid<S>&
         k_step_simple<TM><<<grid, block, 0, st>>>(fin, fout, M, G, level, status);
         return cudaGetLastError();
     } else {
-        return launch_fp64(fin, fout, M, G, level, status, st);
+        return launch_fp64(fin, fout, *cfg.fp64, G, level, status, st);
     }
 }
 
