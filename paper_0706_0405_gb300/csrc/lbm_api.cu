@@ -255,14 +255,18 @@ lbm_status ensure_stage(lbm_ctx* c, size_t bytes) {
     return LBM_OK;
 }
 
-lbm_status read_status(lbm_ctx* c) {
-    LBM_CUDA(c, cudaMemcpyAsync(c->h_status, c->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream),
-             "reading the status word");
+lbm_status check_status(lbm_ctx* c) {
     LBM_CUDA(c, cudaStreamSynchronize(c->stream), "synchronising the stream");
     if (*c->h_status & ST_TIMEOUT) return fail(c, LBM_E_TIMEOUT, "a bounded device wait gave up");
     if (*c->h_status & ST_NONPHYSICAL)
         return fail(c, LBM_E_NONPHYSICAL, "a level had rho <= 0 or a non-finite moment at some node");
     return LBM_OK;
+}
+
+lbm_status read_status(lbm_ctx* c) {
+    LBM_CUDA(c, cudaMemcpyAsync(c->h_status, c->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream),
+             "reading the status word");
+    return check_status(c);
 }
 
 lbm_status enter(lbm_ctx* c) {
@@ -543,11 +547,12 @@ lbm_status lbm_create(int nx, int ny, double b, double tau, double dt, double dx
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_status, sizeof(unsigned));
     const int np = c->prec == LBM_FP64 ? conservation_partials(c->gd) : conservation_partials(c->gf);
     if (e == cudaSuccess) e = dev_malloc((void**)&c->d_partials, sizeof(double) * 4 * np);
-    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_sums, sizeof(double) * 4);
+    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_left, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_sums, sizeof(double) * 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, fbytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, fbytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, 4 * sizeof(unsigned), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_left, 0, sizeof(unsigned), c->stream);
     if (e != cudaSuccess) {
         lbm_status r = cuda_fail(nullptr, e, "allocating context buffers");
         lbm_destroy(c);
@@ -571,7 +576,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->d_status);
     cudaFreeHost(c->h_status);
     cudaFree(c->d_partials);
-    cudaFree(c->d_sums);
+    cudaFree(c->d_left);
     cudaFreeHost(c->h_sums);
     cudaFree(c->d_stage);
     for (void* p : c->ck) cudaFree(p);
@@ -603,11 +608,8 @@ lbm_status lbm_init(lbm_ctx* c, const void* rho, const void* ux, const void* uy,
     LBM_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "clearing status");
     cudaError_t e = dispatch(c, [&](auto tag, auto) {
         using S = decltype(tag);
-        S* f = static_cast<S*>(c->f[c->cur]);
-        cudaError_t r = launch_init<S>(f, (const S*)d[0], (const S*)d[1], (const S*)d[2], (const S*)d[3],
-                                       model_of<S>(c), grid_of<S>(c), c->stream);
-        if (r == cudaSuccess) r = launch_fill_ghosts<S>(f, grid_of<S>(c), 0, c->stream);
-        return r;
+        return launch_init<S>(static_cast<S*>(c->f[c->cur]), (const S*)d[0], (const S*)d[1], (const S*)d[2],
+                              (const S*)d[3], model_of<S>(c), grid_of<S>(c), c->stream);
     });
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_init");
     c->ready = true;
@@ -690,12 +692,10 @@ lbm_status lbm_conservation(lbm_ctx* c, double out[4]) {
     cudaError_t e = dispatch(c, [&](auto tag, auto) {
         using S = decltype(tag);
         return launch_conservation<S>(static_cast<const S*>(c->f[c->cur]), c->md, grid_of<S>(c), c->d_partials,
-                                      c->d_sums, c->stream);
+                                      c->d_left, c->d_status, c->h_sums, c->h_status, c->stream);
     });
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_conservation");
-    LBM_CUDA(c, cudaMemcpyAsync(c->h_sums, c->d_sums, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-             "copying sums");
-    s = read_status(c);
+    s = check_status(c);
     for (int k = 0; k < 4; ++k) out[k] = c->h_sums[k];
     return s;
 }

@@ -40,7 +40,7 @@ struct lbm_ctx {
     unsigned* d_status = nullptr;
     unsigned* h_status = nullptr;
     double* d_partials = nullptr;
-    double* d_sums = nullptr;
+    unsigned* d_left = nullptr;  // the totals kernel's count of finished CTAs (zero between launches)
     double* h_sums = nullptr;
     void* d_stage = nullptr;
     size_t stage_bytes = 0;

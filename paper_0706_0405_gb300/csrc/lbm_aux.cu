@@ -1,7 +1,6 @@
 // lbm_aux.cu -- initialisation, ghost fill, moments output, FP64 conservation
 // totals and interior pack/unpack kernels of liblbm.
 #include "lbm_launch.h"
-#include "lbm_reduce.cuh"
 
 namespace lbm {
 
@@ -9,32 +8,141 @@ namespace {
 constexpr int kThreads = 256;
 
 inline unsigned blocks_for(long long n, int per) { return (unsigned)((n + per - 1) / per); }
+
+// Shape of the kernels that walk the grid row by row: CTAs of 64 x 4 threads,
+// each thread V consecutive columns of a row and every gridDim.y * 4-th row
+// from its own, so that no index is divided (a 64-bit division per element
+// had cost more than the copy: see launch_pack).
+constexpr int kRowX = 64, kRowY = 4;
+inline dim3 row_grid(long long columns, long long rows, int V) {
+    const long long gy = (rows + kRowY - 1) / kRowY;
+    return dim3(blocks_for(columns, kRowX * V), (unsigned)(gy < 32768 ? gy : 32768));
+}
+
+inline bool aligned(const void* p, size_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
+
+// V = 2 or 4 consecutive FP32 values as packed pairs.
+template <int V>
+struct Run {
+    F2 h[V / 2];
+    __device__ __forceinline__ float at(int j) const { return j & 1 ? lane1(h[j / 2]) : lane0(h[j / 2]); }
+};
+template <int V>
+struct alignas(4 * V) RunVec {
+    float v[V];
+};
+// From / to an array: one access (wide), or n <= V single ones (values past
+// n repeat the first).
+template <int V>
+__device__ __forceinline__ Run<V> load_run(const float* p, bool wide, int n) {
+    RunVec<V> r;
+    if (wide) {
+        r = *reinterpret_cast<const RunVec<V>*>(p);
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; ++j) r.v[j] = j < n ? p[j] : p[0];
+    }
+    Run<V> o;
+#pragma unroll
+    for (int k = 0; k < V / 2; ++k) o.h[k] = pair(r.v[2 * k], r.v[2 * k + 1]);
+    return o;
+}
+template <int V>
+__device__ __forceinline__ void store_run(float* p, const Run<V>& o, bool wide, int n) {
+    RunVec<V> r;
+#pragma unroll
+    for (int j = 0; j < V; ++j) r.v[j] = o.at(j);
+    if (wide) {
+        *reinterpret_cast<RunVec<V>*>(p) = r;
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (j < n) p[j] = r.v[j];
+    }
+}
 }  // namespace
 
-// f = f^eq(rho, u, T) (Eqs. e16-e18) at each interior node.
-template <typename S>
-__global__ void k_init(S* __restrict__ f, const S* __restrict__ rho, const S* __restrict__ ux,
-                       const S* __restrict__ uy, const S* __restrict__ T, const Model<S> M,
-                       const Grid<S> G) {
-    const long long n = (long long)G.nx * G.ny;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int iy = (int)(q / G.nx), ix = (int)(q % G.nx);
-        S fe[9];
+// f = f^eq(rho, u, T) (Eqs. e16-e18) at each interior node, and the ghost
+// cells of level 0 by the edge nodes (from the values just stored, read
+// back).  FP32: V x-adjacent nodes per thread in packed arithmetic, V-wide
+// accesses; wide: the fields allow them too.  HBM-bound on large grids (16 B
+// in, 36 B out a node): the stores want 16 bytes, 44 us on the 4096 x 1024
+// grid with V = 4 against 48 with one node a thread, its index divided, and
+// the ghost cells in a launch of their own.  Latency-bound on small ones,
+// where V = 2 has twice the threads: 256 tubes of 4 rows one after the other
+// 1.7-1.9 ms against 2.1 (V = 4) and 2.4 (two launches each).
+constexpr long long kInitWideNodes = 1 << 20;
+template <int V>
+__global__ void __launch_bounds__(kThreads) k_init32(float* __restrict__ f, const float* __restrict__ rho,
+                                                     const float* __restrict__ ux, const float* __restrict__ uy,
+                                                     const float* __restrict__ T, const Model<float> M,
+                                                     const Grid<float> G, bool wide) {
+    const int ix = (blockIdx.x * kRowX + threadIdx.x) * V;
+    if (ix >= G.nx) return;
+    const int n = min(V, G.nx - ix);
+    const size_t pl = (size_t)G.plane;
+    for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
+        const size_t q = (size_t)iy * G.nx + ix;
+        const Run<V> r = load_run<V>(rho + q, wide, n), u = load_run<V>(ux + q, wide, n),
+                     w = load_run<V>(uy + q, wide, n), t = load_run<V>(T + q, wide, n);
+        F2 fe[V / 2][9];
+#pragma unroll
+        for (int k = 0; k < V / 2; ++k) equilibrium_scaled<float, F2>(M, r.h[k], u.h[k], w.h[k], t.h[k], fe[k]);
+        float* out = f + cell(G, ix, iy);  // 4 V-byte aligned: ix + PADX is a multiple of V
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            Run<V> o;
+#pragma unroll
+            for (int k = 0; k < V / 2; ++k) o.h[k] = fe[k][i];
+            store_run<V>(out + i * pl, o, n == V, n);
+        }
+        if (ix == 0 || iy == 0 || ix + n == G.nx || iy == G.ny - 1) {
+            for (int j = 0; j < n; ++j) {
+                float v[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) v[i] = out[i * pl + j];
+                write_ghosts(G, f, ix + j, iy, v, 0);
+            }
+        }
+    }
+}
+
+template <int V>
+void init32(float* f, const float* rho, const float* ux, const float* uy, const float* T, const Model<float>& M,
+            const Grid<float>& G, cudaStream_t st) {
+    const bool wide = G.nx % V == 0 && aligned(rho, 4 * V) && aligned(ux, 4 * V) && aligned(uy, 4 * V) &&
+                      aligned(T, 4 * V);
+    k_init32<V><<<row_grid(G.nx, G.ny, V), dim3(kRowX, kRowY), 0, st>>>(f, rho, ux, uy, T, M, G, wide);
+}
+
+__global__ void __launch_bounds__(kThreads) k_init64(double* __restrict__ f, const double* __restrict__ rho,
+                                                     const double* __restrict__ ux, const double* __restrict__ uy,
+                                                     const double* __restrict__ T, const Model<double> M,
+                                                     const Grid<double> G) {
+    const int ix = blockIdx.x * kRowX + threadIdx.x;
+    if (ix >= G.nx) return;
+    for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
+        const size_t q = (size_t)iy * G.nx + ix;
+        double fe[9];
         equilibrium(M, rho[q], ux[q], uy[q], T[q], fe);
         const size_t c = cell(G, ix, iy);
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i * (size_t)G.plane + c] = fe[i];
+        if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) write_ghosts(G, f, ix, iy, fe, 0);
     }
 }
 
 template <typename S>
 cudaError_t launch_init(S* f, const S* rho, const S* ux, const S* uy, const S* T,
                         const Model<S>& M, const Grid<S>& G, cudaStream_t st) {
-    const long long n = (long long)G.nx * G.ny;
-    unsigned nb = blocks_for(n, kThreads);
-    if (nb > 65535u * 4u) nb = 65535u * 4u;
-    k_init<S><<<nb, kThreads, 0, st>>>(f, rho, ux, uy, T, M, G);
+    if constexpr (sizeof(S) == 4) {
+        if ((long long)G.nx * G.ny >= kInitWideNodes)
+            init32<4>(f, rho, ux, uy, T, M, G, st);
+        else
+            init32<2>(f, rho, ux, uy, T, M, G, st);
+    } else {
+        k_init64<<<row_grid(G.nx, G.ny, 1), dim3(kRowX, kRowY), 0, st>>>(f, rho, ux, uy, T, M, G);
+    }
     return cudaGetLastError();
 }
 
@@ -69,133 +177,360 @@ cudaError_t launch_fill_ghosts(S* f, const Grid<S>& G, long long level, cudaStre
     return cudaGetLastError();
 }
 
-template <typename S, int TM>
-__global__ void k_moments(const S* __restrict__ f, S* __restrict__ rho, S* __restrict__ ux,
-                          S* __restrict__ uy, S* __restrict__ T, const Model<S> M, const Grid<S> G,
-                          unsigned* status) {
-    const long long n = (long long)G.nx * G.ny;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int iy = (int)(q / G.nx), ix = (int)(q % G.nx);
-        const size_t c = cell(G, ix, iy);
-        S v[9];
+// Moments of a level.  FP32: two x-adjacent nodes per thread in packed
+// arithmetic, 8-byte accesses; wide: the outputs allow them.  Near the HBM
+// bound (36 B in, 16 B out a node) in the modes with few operations, also
+// issue-bound with the double-float sum.  4096 x 1024: 43.3 us (double-float)
+// and 35.7 (total energy), as with one node a thread; 1024 x 256 with the
+// FP64 sum 10.0, one node a thread and its index divided 16.9.  Four nodes a
+// thread: 59.9 and 47.5 (too few warps for their registers).
+template <int TM>
+__global__ void __launch_bounds__(kThreads) k_moments32(const float* __restrict__ f, float* __restrict__ rho,
+                                                        float* __restrict__ ux, float* __restrict__ uy,
+                                                        float* __restrict__ T, const Model<float> M,
+                                                        const Grid<float> G, unsigned* status, bool wide) {
+    const int ix = (blockIdx.x * kRowX + threadIdx.x) * 2;
+    unsigned bits = 0;
+    if (ix < G.nx) {
+        const int n = min(2, G.nx - ix);
+        const size_t pl = (size_t)G.plane;
+        for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
+            const float* in = f + cell(G, ix, iy);  // 8-byte aligned
+            F2 v[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) v[i] = f[i * (size_t)G.plane + c];
-        S r, u, w, t;
-        moments<S, TM>(v, M, r, u, w, t);
-        report(status, health(r, u, w, t));
-        if (rho) rho[q] = r;
-        if (ux) ux[q] = u;
-        if (uy) uy[q] = w;
-        if (T) T[q] = t;
+            for (int i = 0; i < 9; ++i) v[i] = load_run<2>(in + i * pl, n == 2, n).h[0];
+            Run<2> r, u, w, t;
+            moments<float, TM, F2>(v, M, r.h[0], u.h[0], w.h[0], t.h[0]);
+            // the second lane of a last odd node repeats the first
+            bits |= health(r.at(0), u.at(0), w.at(0), t.at(0)) | health(r.at(1), u.at(1), w.at(1), t.at(1));
+            const size_t q = (size_t)iy * G.nx + ix;
+            if (rho) store_run<2>(rho + q, r, wide, n);
+            if (ux) store_run<2>(ux + q, u, wide, n);
+            if (uy) store_run<2>(uy + q, w, wide, n);
+            if (T) store_run<2>(T + q, t, wide, n);
+        }
     }
+    report(status, bits);
+}
+
+__global__ void __launch_bounds__(kThreads) k_moments64(const double* __restrict__ f, double* __restrict__ rho,
+                                                        double* __restrict__ ux, double* __restrict__ uy,
+                                                        double* __restrict__ T, const Model<double> M,
+                                                        const Grid<double> G, unsigned* status) {
+    const int ix = blockIdx.x * kRowX + threadIdx.x;
+    unsigned bits = 0;
+    if (ix < G.nx) {
+        for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
+            const size_t c = cell(G, ix, iy);
+            double v[9], r, u, w, t;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = f[i * (size_t)G.plane + c];
+            moments<double, T_PLAIN>(v, M, r, u, w, t);
+            bits |= health(r, u, w, t);
+            const size_t q = (size_t)iy * G.nx + ix;
+            if (rho) rho[q] = r;
+            if (ux) ux[q] = u;
+            if (uy) uy[q] = w;
+            if (T) T[q] = t;
+        }
+    }
+    report(status, bits);
 }
 
 template <typename S, int TM>
 cudaError_t launch_moments(const S* f, S* rho, S* ux, S* uy, S* T, const Model<S>& M,
                            const Grid<S>& G, unsigned* status, cudaStream_t st) {
-    const long long n = (long long)G.nx * G.ny;
-    unsigned nb = blocks_for(n, kThreads);
-    if (nb > 65535u * 4u) nb = 65535u * 4u;
-    k_moments<S, TM><<<nb, kThreads, 0, st>>>(f, rho, ux, uy, T, M, G, status);
+    const dim3 block(kRowX, kRowY);
+    if constexpr (sizeof(S) == 4) {
+        const bool wide = G.nx % 2 == 0 && aligned(rho, 8) && aligned(ux, 8) && aligned(uy, 8) && aligned(T, 8);
+        k_moments32<TM><<<row_grid(G.nx, G.ny, 2), block, 0, st>>>(f, rho, ux, uy, T, M, G, status, wide);
+    } else {
+        k_moments64<<<row_grid(G.nx, G.ny, 1), block, 0, st>>>(f, rho, ux, uy, T, M, G, status);
+    }
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------ conservation totals
 // FP64 totals of rho, rho ux, rho uy and E = sum f (v^2 + eta^2) over the
-// interior.  Each block reduces a fixed, strided subset of the nodes in a
-// fixed tree order; a second single-block pass adds the block partials in a
-// fixed order, so the result does not depend on scheduling.
-constexpr int kConsBlocks = 1024;
+// interior.  Each CTA reduces a fixed, strided subset of the grid's units (a
+// unit is a run of kConsSeg columns of one row) in a fixed order; the last
+// CTA to finish adds the CTAs' partials in a fixed order, so the result does
+// not depend on scheduling, and writes it with the health word straight to
+// the caller's page-locked memory.  (With a second kernel and two
+// copies back a call took 30 us on the smallest grids, now 20.)
+constexpr int kConsSeg = 512;
+constexpr int kConsBlocks = 608;  // 4 per SM
 
 template <typename S>
 int conservation_partials(const Grid<S>& G) {
-    const long long n = (long long)G.nx * G.ny;
-    long long nb = (n + kThreads - 1) / kThreads;
-    return (int)(nb < kConsBlocks ? (nb < 1 ? 1 : nb) : kConsBlocks);
+    const long long units = (long long)G.ny * ((G.nx + kConsSeg - 1) / kConsSeg);
+    return (int)(units < kConsBlocks ? units : kConsBlocks);
 }
 
-template <typename S>
-__global__ void __launch_bounds__(kThreads) k_cons_partial(const S* __restrict__ f,
-                                                           const Model<double> M,
-                                                           const Grid<S> G,
-                                                           double* __restrict__ partials) {
-    __shared__ double sh[4][kThreads];
-    const long long n = (long long)G.nx * G.ny;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int iy = (int)(q / G.nx), ix = (int)(q % G.nx);
-        const size_t c = cell(G, ix, iy);
-        double v[9];
+namespace {
+// The nine sums of a set of populations, as totals.
+__device__ __forceinline__ void totals_of(const Model<double>& M, const double (&v)[9], double (&t)[4]) {
+    const double s14 = (v[1] + v[3]) + (v[2] + v[4]);
+    const double s58 = (v[5] + v[7]) + (v[6] + v[8]);
+    t[0] = v[0] + s14 + s58;
+    t[1] = M.c1 * (v[3] - v[1]) + M.d * ((v[6] + v[7]) - (v[5] + v[8]));
+    t[2] = M.c1 * (v[4] - v[2]) + M.d * ((v[7] + v[8]) - (v[5] + v[6]));
+    t[3] = M.eta2 * v[0] + M.c1s * s14 + M.c2s * s58;
+}
+
+// Called by one whole warp of a CTA, with the CTA's totals in lane 0: writes
+// the partials, and in the last CTA the totals and the health word.  left:
+// CTAs that have finished, zero between launches.
+__device__ __forceinline__ void finish_totals(const double (&t)[4], double* __restrict__ partials, unsigned* left,
+                                              const unsigned* status, double* out, unsigned* out_status) {
+    const int lane = threadIdx.x & 31;
+    const int nb = gridDim.x;
+    unsigned last = 0;
+    if (lane == 0) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) v[i] = (double)f[i * (size_t)G.plane + c];
-        const double s14 = (v[1] + v[3]) + (v[2] + v[4]);
-        const double s58 = (v[5] + v[7]) + (v[6] + v[8]);
-        acc[0] += v[0] + s14 + s58;
-        acc[1] += M.c1 * (v[3] - v[1]) + M.d * ((v[6] + v[7]) - (v[5] + v[8]));
-        acc[2] += M.c1 * (v[4] - v[2]) + M.d * ((v[7] + v[8]) - (v[5] + v[6]));
-        acc[3] += M.eta2 * v[0] + M.c1s * s14 + M.c2s * s58;
+        for (int q = 0; q < 4; ++q) __stcg(partials + q * nb + blockIdx.x, t[q]);
+        __threadfence();
+        last = atomicAdd(left, 1u) == (unsigned)nb - 1;
     }
-    block_sum4<kThreads>(acc, sh);
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) partials[q * gridDim.x + blockIdx.x] = acc[q];
-}
-
-__global__ void __launch_bounds__(kThreads) k_cons_final(const double* __restrict__ partials,
-                                                         int nparts, double* __restrict__ out) {
-    __shared__ double sh[4][kThreads];
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nparts; b += kThreads)
+    for (int b = lane; b < nb; b += 32)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] += partials[q * nparts + b];
-    block_sum4<kThreads>(acc, sh);
-    if (threadIdx.x == 0)
+        for (int q = 0; q < 4; ++q) acc[q] += __ldcg(partials + q * nb + b);
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] += __shfl_down_sync(0xffffffffu, acc[q], s);
+    if (lane == 0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) out[q] = acc[q];
+        *out_status = *status;
+        *left = 0;
+    }
+}
+
+// Running sum of FP32 values as h + l + c: h and l take each value by TwoSum
+// (exact), c collects what l rounds away, so the sum carries about 72 bits:
+// more than an FP64 accumulator, on the FP32 pipe.
+template <typename V>
+struct Sum3 {
+    V h{}, l{}, c{};
+    __device__ __forceinline__ void add(V x) {
+        V s, e, t, d;
+        two_sum(h, x, s, e);
+        two_sum(l, e, t, d);
+        h = s;
+        l = t;
+        c = add_(c, d);
+    }
+    __device__ __forceinline__ void add(const Sum3& o) {
+        V s, e, t, d, u, g;
+        two_sum(h, o.h, s, e);
+        two_sum(l, o.l, t, d);
+        two_sum(t, e, u, g);
+        h = s;
+        l = u;
+        c = add_(add_(c, o.c), add_(d, g));
+    }
+};
+}  // namespace
+
+// FP32 levels: 9 warps, warp i sums population i of the CTA's units with
+// 16-byte loads and packed Sum3 accumulators, and only the CTA's nine sums
+// become FP64.  HBM-bound: a call on 4096 x 1024 takes 48 us, 39 of them the kernel;
+// FP64 adds of every value (33 FP64 instructions a node, at 1/64 of the FP32
+// rate) took 330.  Sums
+// that leave the FP32 range, and levels with infinities or NaN, are taken
+// again in FP64 by the warp that saw one.
+constexpr int kConsThreads32 = 9 * 32;
+__global__ void __launch_bounds__(kConsThreads32, 4)
+    k_cons32(const float* __restrict__ f, const Model<double> M, const Grid<float> G, double* __restrict__ partials,
+             unsigned* left, const unsigned* status, double* out, unsigned* out_status) {
+    __shared__ double sums[3][9];
+    const int pop = threadIdx.x / 32, lane = threadIdx.x & 31;
+    const int segs = (G.nx + kConsSeg - 1) / kConsSeg;
+    const long long units = (long long)G.ny * segs;
+    auto run_of = [&](long long u, int& n) {
+        const int row = (int)(u / segs), x0 = (int)(u % segs) * kConsSeg;
+        n = min(kConsSeg, G.nx - x0);
+        return f + (size_t)(row + 1) * (size_t)G.row + (size_t)pop * (size_t)G.plane + (PADX + x0);  // 16-byte aligned
+    };
+    Sum3<F2> a, b;
+    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        int n;
+        const float* p = run_of(u, n);
+        float4 v[kConsSeg / 128];
+#pragma unroll
+        for (int k = 0; k < kConsSeg / 128; ++k) {
+            const int x = k * 128 + lane * 4;
+            v[k] = x + 3 < n ? __ldg(reinterpret_cast<const float4*>(p + x)) : float4{0.0f, 0.0f, 0.0f, 0.0f};
+        }
+        float tail = 0.0f;
+        if (lane < (n & 3)) tail = __ldg(p + (n & ~3) + lane);
+#pragma unroll
+        for (int k = 0; k < kConsSeg / 128; ++k) {
+            a.add(pair(v[k].x, v[k].y));
+            b.add(pair(v[k].z, v[k].w));
+        }
+        if (n & 3) a.add(pair(tail, 0.0f));
+    }
+    a.add(b);
+    Sum3<float> s, r;
+    s.h = lane0(a.h), s.l = lane0(a.l), s.c = lane0(a.c);
+    r.h = lane1(a.h), r.l = lane1(a.l), r.c = lane1(a.c);
+    s.add(r);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        r.h = __shfl_down_sync(0xffffffffu, s.h, d);
+        r.l = __shfl_down_sync(0xffffffffu, s.l, d);
+        r.c = __shfl_down_sync(0xffffffffu, s.c, d);
+        s.add(r);
+    }
+    // lane 0 holds the sum; anything not finite on the way has made it NaN or
+    // infinite, or its error terms NaN
+    const bool fine = isfinite(s.h) && isfinite(s.l) && isfinite(s.c);
+    double part[3] = {(double)s.h, (double)s.l, (double)s.c};
+    if (!__shfl_sync(0xffffffffu, (int)fine, 0)) {
+        double acc = 0.0;
+        for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+            int n;
+            const float* p = run_of(u, n);
+            for (int x = lane; x < n; x += 32) acc += (double)p[x];
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+        part[0] = acc;
+        part[1] = part[2] = 0.0;
+    }
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sums[k][pop] = part[k];
+    __syncthreads();
+    if (pop == 0) {
+        // linear in the sums: each part's totals, the small parts first
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        if (lane == 0) {
+#pragma unroll
+            for (int k = 2; k >= 0; --k) {
+                double v[9], q[4];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) v[i] = sums[k][i];
+                totals_of(M, v, q);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) t[m] += q[m];
+            }
+        }
+        finish_totals(t, partials, left, status, out, out_status);
+    }
+}
+
+// FP64 levels: one node per thread, FP64 sums of the pair differences and of
+// the three speed classes (17 FP64 instructions a node; forming the totals
+// node by node takes 27), combined once per thread.
+__global__ void __launch_bounds__(kThreads)
+    k_cons64(const double* __restrict__ f, const Model<double> M, const Grid<double> G, double* __restrict__ partials,
+             unsigned* left, const unsigned* status, double* out, unsigned* out_status) {
+    __shared__ double sh[4][kThreads / 32];
+    const int segs = (G.nx + kConsSeg - 1) / kConsSeg;
+    const long long units = (long long)G.ny * segs;
+    const size_t pl = (size_t)G.plane;
+    double s0 = 0.0, s14 = 0.0, s58 = 0.0, ax = 0.0, ay = 0.0, ar = 0.0, am = 0.0;
+    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        const int row = (int)(u / segs), x0 = (int)(u % segs) * kConsSeg;
+        const int n = min(kConsSeg, G.nx - x0);
+        const double* p = f + cell(G, x0, row);
+        for (int x = threadIdx.x; x < n; x += kThreads) {
+            double v[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = __ldg(p + i * pl + x);
+            s0 += v[0];
+            s14 += (v[1] + v[3]) + (v[2] + v[4]);
+            s58 += (v[5] + v[7]) + (v[6] + v[8]);
+            ax += v[3] - v[1];
+            ay += v[4] - v[2];
+            ar += v[7] - v[5];
+            am += v[6] - v[8];
+        }
+    }
+    double t[4] = {s0 + s14 + s58, M.c1 * ax + M.d * (ar + am), M.c1 * ay + M.d * (ar - am),
+                   M.eta2 * s0 + M.c1s * s14 + M.c2s * s58};
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) t[q] += __shfl_down_sync(0xffffffffu, t[q], d);
+    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sh[q][warp] = t[q];
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            t[q] = 0.0;
+            for (int w = 0; w < kThreads / 32; ++w) t[q] += sh[q][w];
+        }
+        finish_totals(t, partials, left, status, out, out_status);
+    }
 }
 
 template <typename S>
-cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S>& G,
-                                double* partials, double* out, cudaStream_t st) {
+cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S>& G, double* partials,
+                                unsigned* left, const unsigned* status, double* out, unsigned* out_status,
+                                cudaStream_t st) {
     const int nb = conservation_partials(G);
-    k_cons_partial<S><<<nb, kThreads, 0, st>>>(f, M, G, partials);
-    k_cons_final<<<1, kThreads, 0, st>>>(partials, nb, out);
+    if constexpr (sizeof(S) == 4)
+        k_cons32<<<nb, kConsThreads32, 0, st>>>(f, M, G, partials, left, status, out, out_status);
+    else
+        k_cons64<<<nb, kThreads, 0, st>>>(f, M, G, partials, left, status, out, out_status);
     return cudaGetLastError();
 }
 
 // ----------------------------------------------------------- pack / unpack
-template <typename S>
-__global__ void k_pack(const S* __restrict__ f, S* __restrict__ dense, const Grid<S> G, int dir) {
+// Interior of a level <-> dense 9 x ny x nx array (kUnpack: dense to level),
+// one population row at a time in the level's order ([row][population]), V
+// values per access: 16 bytes where the dense rows allow it, else one value.
+template <typename S, int V, bool kUnpack>
+__global__ void __launch_bounds__(kThreads) k_pack(S* __restrict__ f, S* __restrict__ dense, const Grid<S> G) {
+    struct alignas(V * sizeof(S)) Vec {
+        S v[V];
+    };
+    const int x = (blockIdx.x * kRowX + threadIdx.x) * V;
+    if (x >= G.nx) return;
+    const int rows = 9 * G.ny;  // ny is at most 2^24
     const long long n = (long long)G.nx * G.ny;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < 9 * n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(q / n);
-        const long long r = q - i * n;
-        const int iy = (int)(r / G.nx), ix = (int)(r % G.nx);
-        const size_t c = i * (size_t)G.plane + cell(G, ix, iy);
-        if (dir == 0)
-            dense[q] = f[c];
+    for (int r = blockIdx.y * kRowY + threadIdx.y; r < rows; r += gridDim.y * kRowY) {
+        const int iy = r / 9, i = r - iy * 9;
+        Vec* a = reinterpret_cast<Vec*>(f + (size_t)(iy + 1) * (size_t)G.row + (size_t)i * (size_t)G.plane + (PADX + x));
+        Vec* b = reinterpret_cast<Vec*>(dense + i * n + (long long)iy * G.nx + x);
+        if constexpr (kUnpack)
+            *a = *b;
         else
-            const_cast<S*>(f)[c] = dense[q];
+            *b = *a;
     }
+}
+
+// 4096 x 1024 in FP32 (302 MB moved): 50 us, against 218 with one element a
+// thread and its row and population found by 64-bit divisions.
+template <typename S, bool kUnpack>
+cudaError_t launch_copy(S* f, S* dense, const Grid<S>& G, cudaStream_t st) {
+    constexpr int V = 16 / sizeof(S);
+    const dim3 block(kRowX, kRowY);
+    if (G.nx % V == 0 && aligned(dense, 16))
+        k_pack<S, V, kUnpack><<<row_grid(G.nx, 9LL * G.ny, V), block, 0, st>>>(f, dense, G);
+    else
+        k_pack<S, 1, kUnpack><<<row_grid(G.nx, 9LL * G.ny, 1), block, 0, st>>>(f, dense, G);
+    return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t launch_pack(const S* f, S* dense, const Grid<S>& G, cudaStream_t st) {
-    unsigned nb = blocks_for(9LL * G.nx * G.ny, kThreads);
-    if (nb > 65535u * 4u) nb = 65535u * 4u;
-    k_pack<S><<<nb, kThreads, 0, st>>>(f, dense, G, 0);
-    return cudaGetLastError();
+    return launch_copy<S, false>(const_cast<S*>(f), dense, G, st);
 }
 
 template <typename S>
 cudaError_t launch_unpack(S* f, const S* dense, const Grid<S>& G, cudaStream_t st) {
-    unsigned nb = blocks_for(9LL * G.nx * G.ny, kThreads);
-    if (nb > 65535u * 4u) nb = 65535u * 4u;
-    k_pack<S><<<nb, kThreads, 0, st>>>(f, const_cast<S*>(dense), G, 1);
-    return cudaGetLastError();
+    return launch_copy<S, true>(f, const_cast<S*>(dense), G, st);
 }
 
 #define LBM_INST(S)                                                                          \
@@ -204,7 +539,8 @@ cudaError_t launch_unpack(S* f, const S* dense, const Grid<S>& G, cudaStream_t s
     template cudaError_t launch_fill_ghosts<S>(S*, const Grid<S>&, long long, cudaStream_t); \
     template int conservation_partials<S>(const Grid<S>&);                                   \
     template cudaError_t launch_conservation<S>(const S*, const Model<double>&,              \
-                                                const Grid<S>&, double*, double*,            \
+                                                const Grid<S>&, double*, unsigned*,          \
+                                                const unsigned*, double*, unsigned*,         \
                                                 cudaStream_t);                               \
     template cudaError_t launch_pack<S>(const S*, S*, const Grid<S>&, cudaStream_t);         \
     template cudaError_t launch_unpack<S>(S*, const S*, const Grid<S>&, cudaStream_t);
@@ -212,20 +548,14 @@ LBM_INST(double)
 LBM_INST(float)
 #undef LBM_INST
 
-template cudaError_t launch_moments<double, T_PLAIN>(const double*, double*, double*, double*,
-                                                     double*, const Model<double>&,
-                                                     const Grid<double>&, unsigned*, cudaStream_t);
-template cudaError_t launch_moments<float, T_INT32>(const float*, float*, float*, float*, float*,
-                                                    const Model<float>&, const Grid<float>&,
-                                                    unsigned*, cudaStream_t);
-template cudaError_t launch_moments<float, T_INT64>(const float*, float*, float*, float*, float*,
-                                                    const Model<float>&, const Grid<float>&,
-                                                    unsigned*, cudaStream_t);
-template cudaError_t launch_moments<float, T_DF>(const float*, float*, float*, float*, float*,
-                                                 const Model<float>&, const Grid<float>&,
-                                                 unsigned*, cudaStream_t);
-template cudaError_t launch_moments<float, T_CONS>(const float*, float*, float*, float*, float*,
-                                                 const Model<float>&, const Grid<float>&,
-                                                 unsigned*, cudaStream_t);
+#define LBM_MOM_INST(S, TM)                                                                                  \
+    template cudaError_t launch_moments<S, TM>(const S*, S*, S*, S*, S*, const Model<S>&, const Grid<S>&, \
+                                               unsigned*, cudaStream_t);
+LBM_MOM_INST(double, T_PLAIN)
+LBM_MOM_INST(float, T_INT32)
+LBM_MOM_INST(float, T_INT64)
+LBM_MOM_INST(float, T_DF)
+LBM_MOM_INST(float, T_CONS)
+#undef LBM_MOM_INST
 
 }  // namespace lbm

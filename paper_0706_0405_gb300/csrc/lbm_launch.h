@@ -78,7 +78,8 @@ template <typename S, int TM>
 cudaError_t launch_step(const S* fin, S* fout, const Model<S>& M, const Grid<S>& G,
                         long long level, unsigned* status, cudaStream_t st, const StepConfig& cfg);
 
-// f = f^eq(fields) on the interior (fields are ny x nx, storage type).
+// f = f^eq(fields) on the interior (fields are ny x nx, storage type), and the
+// ghost layer for time level 0.
 template <typename S>
 cudaError_t launch_init(S* f, const S* rho, const S* ux, const S* uy, const S* T,
                         const Model<S>& M, const Grid<S>& G, cudaStream_t st);
@@ -92,13 +93,16 @@ template <typename S, int TM>
 cudaError_t launch_moments(const S* f, S* rho, S* ux, S* uy, S* T, const Model<S>& M,
                            const Grid<S>& G, unsigned* status, cudaStream_t st);
 
-// FP64 totals of rho, rho u, E into out[4] (device); `partials` holds
-// conservation_partials(G) * 4 doubles.
+// FP64 totals of rho, rho u, E into out[4] and the health word `status` into
+// out_status (both page-locked host memory, valid once the stream has been
+// synchronised); `partials` holds conservation_partials(G) * 4 doubles,
+// `left` one word that is zero between launches.
 template <typename S>
 int conservation_partials(const Grid<S>& G);
 template <typename S>
-cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S>& G,
-                                double* partials, double* out, cudaStream_t st);
+cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S>& G, double* partials,
+                                unsigned* left, const unsigned* status, double* out, unsigned* out_status,
+                                cudaStream_t st);
 
 // Interior <-> dense 9 x ny x nx copies.
 template <typename S>

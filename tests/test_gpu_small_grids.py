@@ -38,3 +38,54 @@ def test_fp64_step_at_the_edges_of_its_one_warp_ctas(nx, ny, sides):
         assert lat.health() == 0
     for g, r in zip(got, oracle.fields(p, f)):
         assert np.max(np.abs(g - r)) <= 1e-10 * max(1.0, np.max(np.abs(r)))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_cons", "fp32_tdf"])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 2), (511, 3), (512, 2), (514, 3), (1027, 5)])
+def test_read_out_at_the_edges_of_its_vectors_and_units(nx, ny, prec):
+    """set_f / get_f keep every value, moments and totals match FP64 sums of
+    the stored f, for widths around the 2- and 4-value accesses and the
+    512-column units of the totals, in dense arrays of every alignment: the
+    totals to 1e-14 of the sum of their terms' magnitudes (a few FP64
+    roundings; the FP32 accumulators carry more than 53 bits)."""
+    import torch
+    p, fields = _problem(nx, ny, WALLS)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    rng = np.random.Generator(np.random.PCG64(nx + ny))
+    f = torch.tensor(rng.standard_normal((9, ny, nx)) ** 3 + 30.0, dtype=dt, device="cuda")
+    with lbm.Lattice(p, prec) as lat:
+        for shift in (0, 1):  # a dense array that starts on and off a 16-byte boundary
+            buf = torch.empty(f.numel() + shift, dtype=dt, device="cuda")[shift:].view(f.shape)
+            buf.copy_(f)
+            lbm.lbm_set_f(lat.ctx, buf, 3)
+            buf.zero_()
+            lbm.lbm_get_f(lat.ctx, buf)
+            torch.cuda.synchronize()
+            assert torch.equal(buf, f)
+        sums = lat.conservation()
+        mom = [torch.empty(ny * nx + 1, dtype=dt, device="cuda")[1:] for _ in range(4)]
+        lbm.lbm_moments(lat.ctx, *mom)
+        torch.cuda.synchronize()
+        aligned = lat.moments()
+    for a, b in zip(aligned, mom):
+        assert torch.equal(a.reshape(-1), b)
+    v = f.double().cpu().numpy().reshape(9, -1)
+    vx, vy = oracle.velocities(p.c1, p.c2)
+    e = vx ** 2 + vy ** 2
+    e[0] = p.eta0 ** 2
+    for got, w in zip(sums, (np.ones(9), vx, vy, e)):
+        terms = (w[:, None] * v).astype(np.longdouble)
+        assert abs(got - float(terms.sum())) <= 1e-14 * float(np.abs(terms).sum())
+
+
+def test_fp32_totals_of_values_whose_sum_leaves_the_fp32_range():
+    import torch
+    p, _ = _problem(600, 4, PERIODIC)
+    with lbm.Lattice(p, "fp32") as lat:
+        lat.set_f(torch.full((9, 4, 600), 3e37, dtype=torch.float32, device="cuda"))
+        big = lat.conservation()[0]
+        f = torch.ones((9, 4, 600), dtype=torch.float32, device="cuda")
+        f[2, 1, 7] = float("inf")
+        lat.set_f(f)
+        assert np.isinf(lat.conservation()[0])
+    assert big == pytest.approx(9 * 2400 * float(np.float32(3e37)), rel=1e-14)
