@@ -194,7 +194,11 @@ lbm_status lbm_init(lbm_ctx* ctx, const void* rho, const void* ux, const void* u
 
 /* Advance n >= 0 steps of Eq. (SEC-VON-11), asynchronously on the stream.
  * Each step reads level k, writes level k + 1 into the other buffer and fills
- * that level's ghost layer for t = (k + 1) dt in the same kernel. */
+ * that level's ghost layer for t = (k + 1) dt in the same kernel.  With the
+ * default launch shape, small grids (FP32 modes: about 400 000 nodes, FP64:
+ * 14 000) run n >= 3 steps in one cooperative launch that keeps the level in
+ * shared memory and writes the last two levels to the buffers; the bits are
+ * those of a launch a step. */
 lbm_status lbm_step(lbm_ctx* ctx, int n);
 
 /* Macroscopic fields of the current level (Eqs. e4, e5, e7): rho, ux, uy, T
@@ -277,7 +281,9 @@ typedef struct lbm_launch {
                     threads, two x-adjacent nodes each; each 64 x 4 tile plus
                     its halo (72 x 6 x 9 planes) arrives in shared memory by
                     one tiled tensor copy (TMA), double-buffered, and the
-                    stencil reads shared memory */
+                    stencil reads shared memory.  The default shapes (variant
+                    3, or 0 on an FP64 context, with grid = 0) let lbm_step
+                    run several steps of a small grid in one launch */
     int tx;      /* variant 1: columns per CTA, 128 or 256; variant 2: 2 or 4 */
     int ring;    /* variant 1: ring slots, 4 or 6 (4 when tx = 128) */
     int grid;    /* variants 1, 3: CTAs; 0 = one full wave (SMs x resident CTAs) */

@@ -388,6 +388,132 @@ bool make_tmap(CUtensorMap* m, void* base, const lbm_ctx& c) {
 }
 
 
+// Whether the context's grid is small enough for several steps per launch.
+bool plan_resident(lbm_ctx* c) {
+    bool ok = false;
+    dispatch(c, [&](auto tag, auto tm) {
+        using S = decltype(tag);
+        ok = resident_plan<S, decltype(tm)::value>(c->nx, c->ny, &c->res);
+        return cudaSuccess;
+    });
+    return ok;
+}
+
+// Fewest steps for which one launch of the resident kernel beats a launch a
+// step: it reads the level, exchanges n - 1 times and writes two levels.
+constexpr int kResidentMinSteps = 3;
+
+// n steps of the context in one launch (res_ok).
+cudaError_t step_resident(lbm_ctx* c, int n) {
+    return dispatch(c, [&](auto tag, auto tm) {
+        using S = decltype(tag);
+        ResRun<S> A{};
+        A.fin = static_cast<const S*>(c->f[c->cur]);
+        A.out_even = static_cast<S*>(c->f[c->cur ^ 1]);
+        A.out_odd = static_cast<S*>(c->f[c->cur]);
+        A.write_from = n - 2;
+        A.nsteps = n;
+        A.level0 = c->step;
+        A.sync = c->d_res;
+        A.xch = reinterpret_cast<unsigned long long*>(c->d_res + 64);
+        A.status = c->d_status;
+        return launch_resident<S, decltype(tm)::value>(c->res, model_of<S>(c), c->f64, grid_of<S>(c), A, c->stream);
+    });
+}
+
+lbm_status create_context(int nx, int ny, double b, double tau, double dt, double dx, const lbm_dvm* dvm,
+                          const lbm_dissipation* diss, const lbm_bc bc[4], lbm_precision prec, void* stream,
+                          void* f_buf0, void* f_buf1, bool resident, lbm_ctx** out) {
+    if (!out) return fail(nullptr, LBM_E_INVAL, "out must not be NULL");
+    *out = nullptr;
+    lbm_status s = validate(nx, ny, b, tau, dt, dx, dvm, diss, bc, prec);
+    if (s != LBM_OK) return s;
+    const bool caller_f = f_buf0 || f_buf1;
+    if (caller_f) {
+        if (!f_buf0 || !f_buf1)
+            return fail(nullptr, LBM_E_INVAL, "f_buf0 and f_buf1 must both be given or both be NULL");
+        const size_t need = lbm_level_bytes(nx, ny, prec);
+        const uintptr_t a0 = reinterpret_cast<uintptr_t>(f_buf0), a1 = reinterpret_cast<uintptr_t>(f_buf1);
+        if ((a0 | a1) % 256 != 0)
+            return fail(nullptr, LBM_E_INVAL, "f_buf0 and f_buf1 must be 256-byte aligned");
+        if ((a0 < a1 ? a1 - a0 : a0 - a1) < need)
+            return fail(nullptr, LBM_E_INVAL, "f_buf0 and f_buf1 overlap (each needs %zu bytes)", need);
+    }
+    lbm_ctx* c = new lbm_ctx();
+    if (cudaGetDevice(&c->device) != cudaSuccess) {
+        cudaGetLastError();
+        delete c;
+        return fail(nullptr, LBM_E_CUDA, "no CUDA device available");
+    }
+    c->nx = nx;
+    c->ny = ny;
+    c->pitch = ((nx + 2 * PADX) + 31) / 32 * 32;
+    c->plane = c->pitch;
+    c->row = 9LL * c->pitch;
+    c->prec = prec;
+    c->esize = prec == LBM_FP64 ? 8 : 4;
+    c->b = b;
+    c->tau = tau;
+    c->dt = dt;
+    c->dx = dx;
+    c->dvm = *dvm;
+    c->diss = *diss;
+    for (int k = 0; k < 4; ++k) c->bc[k] = bc[k];
+    c->stream = static_cast<cudaStream_t>(stream);
+    if (prec == LBM_FP64) c->cfg = StepConfig{STEP_SIMPLE, 0, 0, 0};
+    c->md = build_model(*c);
+    c->mf = cast_model<float>(c->md);
+    c->f64 = fp64_step(c->md, b, tau, dt, dvm->c1, dvm->c2, dvm->eta0);
+    c->gd = build_grid<double>(*c, c->md);
+    c->gf = build_grid<float>(*c, c->md);
+    const size_t fbytes = level_bytes(c);
+    cudaError_t e = cudaSuccess;
+    if (caller_f) {
+        // the caller's buffers: device memory of this context's device
+        void* bufs[2] = {f_buf0, f_buf1};
+        for (int k = 0; k < 2; ++k) {
+            cudaPointerAttributes at{};
+            const bool dev_ok = cudaPointerGetAttributes(&at, bufs[k]) == cudaSuccess &&
+                                (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) &&
+                                at.device == c->device;
+            cudaGetLastError();
+            if (!dev_ok) {
+                delete c;
+                return fail(nullptr, LBM_E_INVAL, "f_buf%d is not device memory of the current device", k);
+            }
+            c->f[k] = bufs[k];
+        }
+        c->f_owned = false;
+    } else {
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = dev_malloc(&c->f[k], fbytes);
+    }
+    if (resident) c->res_ok = plan_resident(c);
+    // status word, a spare, and the tile kernel's two scheduling counters; 256
+    // bytes on, the words and the exchange buffer of the resident steps
+    const size_t status_bytes = c->res_ok ? 512 + c->res.xch_bytes : 4 * sizeof(unsigned);
+    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_status, status_bytes);
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_status, sizeof(unsigned));
+    const int np = c->prec == LBM_FP64 ? conservation_partials(c->gd) : conservation_partials(c->gf);
+    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_partials, sizeof(double) * 4 * np);
+    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_left, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_sums, sizeof(double) * 4);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, fbytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, fbytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, status_bytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_left, 0, sizeof(unsigned), c->stream);
+    if (e != cudaSuccess) {
+        lbm_status r = cuda_fail(nullptr, e, "allocating context buffers");
+        lbm_destroy(c);
+        return r;
+    }
+    if (c->prec != LBM_FP64)
+        c->tmap_ok = make_tmap(&c->tmap[0], c->f[0], *c) && make_tmap(&c->tmap[1], c->f[1], *c);
+    if (c->prec != LBM_FP64 && !c->tmap_ok) c->cfg = StepConfig{STEP_VEC, 4, 0, 0};
+    if (c->res_ok) c->d_res = c->d_status + 64;
+    *out = c;
+    return LBM_OK;
+}
+
 struct CkptHeader {
     char magic[8];
     int nx, ny, prec, esize;
@@ -479,90 +605,7 @@ size_t lbm_level_bytes(int nx, int ny, lbm_precision prec) {
 lbm_status lbm_create(int nx, int ny, double b, double tau, double dt, double dx, const lbm_dvm* dvm,
                       const lbm_dissipation* diss, const lbm_bc bc[4], lbm_precision prec,
                       void* stream, void* f_buf0, void* f_buf1, lbm_ctx** out) {
-    if (!out) return fail(nullptr, LBM_E_INVAL, "out must not be NULL");
-    *out = nullptr;
-    lbm_status s = validate(nx, ny, b, tau, dt, dx, dvm, diss, bc, prec);
-    if (s != LBM_OK) return s;
-    const bool caller_f = f_buf0 || f_buf1;
-    if (caller_f) {
-        if (!f_buf0 || !f_buf1)
-            return fail(nullptr, LBM_E_INVAL, "f_buf0 and f_buf1 must both be given or both be NULL");
-        const size_t need = lbm_level_bytes(nx, ny, prec);
-        const uintptr_t a0 = reinterpret_cast<uintptr_t>(f_buf0), a1 = reinterpret_cast<uintptr_t>(f_buf1);
-        if ((a0 | a1) % 256 != 0)
-            return fail(nullptr, LBM_E_INVAL, "f_buf0 and f_buf1 must be 256-byte aligned");
-        if ((a0 < a1 ? a1 - a0 : a0 - a1) < need)
-            return fail(nullptr, LBM_E_INVAL, "f_buf0 and f_buf1 overlap (each needs %zu bytes)", need);
-    }
-    lbm_ctx* c = new lbm_ctx();
-    if (cudaGetDevice(&c->device) != cudaSuccess) {
-        cudaGetLastError();
-        delete c;
-        return fail(nullptr, LBM_E_CUDA, "no CUDA device available");
-    }
-    c->nx = nx;
-    c->ny = ny;
-    c->pitch = ((nx + 2 * PADX) + 31) / 32 * 32;
-    c->plane = c->pitch;
-    c->row = 9LL * c->pitch;
-    c->prec = prec;
-    c->esize = prec == LBM_FP64 ? 8 : 4;
-    c->b = b;
-    c->tau = tau;
-    c->dt = dt;
-    c->dx = dx;
-    c->dvm = *dvm;
-    c->diss = *diss;
-    for (int k = 0; k < 4; ++k) c->bc[k] = bc[k];
-    c->stream = static_cast<cudaStream_t>(stream);
-    if (prec == LBM_FP64) c->cfg = StepConfig{STEP_SIMPLE, 0, 0, 0};
-    c->md = build_model(*c);
-    c->mf = cast_model<float>(c->md);
-    c->f64 = fp64_step(c->md, b, tau, dt, dvm->c1, dvm->c2, dvm->eta0);
-    c->gd = build_grid<double>(*c, c->md);
-    c->gf = build_grid<float>(*c, c->md);
-    const size_t fbytes = level_bytes(c);
-    cudaError_t e = cudaSuccess;
-    if (caller_f) {
-        // the caller's buffers: device memory of this context's device
-        void* bufs[2] = {f_buf0, f_buf1};
-        for (int k = 0; k < 2; ++k) {
-            cudaPointerAttributes at{};
-            const bool dev_ok = cudaPointerGetAttributes(&at, bufs[k]) == cudaSuccess &&
-                                (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) &&
-                                at.device == c->device;
-            cudaGetLastError();
-            if (!dev_ok) {
-                delete c;
-                return fail(nullptr, LBM_E_INVAL, "f_buf%d is not device memory of the current device", k);
-            }
-            c->f[k] = bufs[k];
-        }
-        c->f_owned = false;
-    } else {
-        for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = dev_malloc(&c->f[k], fbytes);
-    }
-    // status word, a spare, and the tile kernel's two scheduling counters
-    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_status, 4 * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_status, sizeof(unsigned));
-    const int np = c->prec == LBM_FP64 ? conservation_partials(c->gd) : conservation_partials(c->gf);
-    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_partials, sizeof(double) * 4 * np);
-    if (e == cudaSuccess) e = dev_malloc((void**)&c->d_left, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_sums, sizeof(double) * 4);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, fbytes, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, fbytes, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, 4 * sizeof(unsigned), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_left, 0, sizeof(unsigned), c->stream);
-    if (e != cudaSuccess) {
-        lbm_status r = cuda_fail(nullptr, e, "allocating context buffers");
-        lbm_destroy(c);
-        return r;
-    }
-    if (c->prec != LBM_FP64)
-        c->tmap_ok = make_tmap(&c->tmap[0], c->f[0], *c) && make_tmap(&c->tmap[1], c->f[1], *c);
-    if (c->prec != LBM_FP64 && !c->tmap_ok) c->cfg = StepConfig{STEP_VEC, 4, 0, 0};
-    *out = c;
-    return LBM_OK;
+    return create_context(nx, ny, b, tau, dt, dx, dvm, diss, bc, prec, stream, f_buf0, f_buf1, true, out);
 }
 
 void lbm_destroy(lbm_ctx* c) {
@@ -622,21 +665,36 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
     if (s != LBM_OK) return s;
     if (n < 0) return fail(c, LBM_E_INVAL, "lbm_step: n must be >= 0");
     if (!c->ready) return fail(c, LBM_E_STATE, "lbm_step before lbm_init / lbm_set_f / lbm_load");
-    for (int k = 0; k < n; ++k) {
-        c->cfg.tmap = c->tmap_ok ? &c->tmap[c->cur] : nullptr;
-        c->cfg.fp64 = &c->f64;
-        cudaError_t e = dispatch(c, [&](auto tag, auto tm) {
-            using S = decltype(tag);
-            constexpr int TM = decltype(tm)::value;
-            return launch_step<S, TM>(static_cast<const S*>(c->f[c->cur]), static_cast<S*>(c->f[c->cur ^ 1]),
-                                      model_of<S>(c), grid_of<S>(c), c->step, c->d_status, c->stream, c->cfg);
-        });
+    // the default launch shape: several steps per launch on small grids
+    const bool resident =
+        c->res_ok && c->cfg.grid == 0 && c->cfg.variant == (c->prec == LBM_FP64 ? STEP_SIMPLE : STEP_TILE);
+    for (int k = 0; k < n;) {
+        int m = n - k;
+        if (c->ck_every > 0) {  // up to the next level to be recorded
+            const long long left = c->ck_every - (c->step - c->ck_base) % c->ck_every;
+            if (left < m) m = (int)left;
+        }
+        cudaError_t e;
+        if (resident && m >= kResidentMinSteps) {
+            e = step_resident(c, m);
+        } else {
+            m = 1;
+            c->cfg.tmap = c->tmap_ok ? &c->tmap[c->cur] : nullptr;
+            c->cfg.fp64 = &c->f64;
+            e = dispatch(c, [&](auto tag, auto tm) {
+                using S = decltype(tag);
+                constexpr int TM = decltype(tm)::value;
+                return launch_step<S, TM>(static_cast<const S*>(c->f[c->cur]), static_cast<S*>(c->f[c->cur ^ 1]),
+                                          model_of<S>(c), grid_of<S>(c), c->step, c->d_status, c->stream, c->cfg);
+            });
+        }
         if (e != cudaSuccess) return cuda_fail(c, e, "lbm_step");
-        c->cur ^= 1;
-        c->step += 1;
+        c->cur ^= m & 1;
+        c->step += m;
+        k += m;
         if (c->ck_every > 0 && (c->step - c->ck_base) % c->ck_every == 0) {
-            const size_t k = (size_t)((c->step - c->ck_base) / c->ck_every);
-            lbm_status r = save_checkpoint(c, k);
+            const size_t q = (size_t)((c->step - c->ck_base) / c->ck_every);
+            lbm_status r = save_checkpoint(c, q);
             if (r != LBM_OK) return r;
         }
     }

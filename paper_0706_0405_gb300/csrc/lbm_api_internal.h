@@ -50,6 +50,10 @@ struct lbm_ctx {
     Grid<double> gd{};
     Grid<float> gf{};
     StepConfig cfg{};
+    // several steps of a small grid per launch (lbm_resident.cu)
+    ResPlan res{};
+    bool res_ok = false;
+    unsigned* d_res = nullptr;  // its tag counter and leave count, then (256 bytes on) its exchange buffer
     CUtensorMap tmap[2];  // FP32: tensor maps of the two level buffers (tile kernel)
     bool tmap_ok = false;
     // adjoint: checkpoints every ck_every steps from level ck_base
@@ -105,6 +109,11 @@ Model<double> build_model(double b, double tau, double dt, double dx, const lbm_
                           const lbm_dissipation& diss);
 size_t nodes(const lbm_ctx* c);
 size_t level_bytes(const lbm_ctx* c);
+// lbm_create; resident: prepare for several steps per launch where the grid
+// is small enough (a batch steps its problems itself and does without)
+lbm_status create_context(int nx, int ny, double b, double tau, double dt, double dx, const lbm_dvm* dvm,
+                          const lbm_dissipation* diss, const lbm_bc bc[4], lbm_precision prec, void* stream,
+                          void* f_buf0, void* f_buf1, bool resident, lbm_ctx** out);
 bool make_tmap_box(CUtensorMap* m, void* base, const lbm_ctx& c, int bx, int by);
 bool make_tmap(CUtensorMap* m, void* base, const lbm_ctx& c);
 }  // namespace lbm_api

@@ -208,9 +208,8 @@ __device__ __forceinline__ double widen(float a) {
 // Internal energy sum_i f_i w_i with the nine exact FP32 products summed in
 // FP64: ten FP64 instructions (18 conversions on top of them took the
 // LBM_FP32_T64 step on the 1024 x 256 grid from 11.4 to 21.1 us, on 2048 x 512
-// from 27.9 to 56).  w[0] is a
-// sum of squares of u, so the last term is NaN when a velocity is not finite,
-// and zero otherwise.
+// from 27.9 to 56).  The last term is NaN where f[0] or w[0] (a sum of squares
+// of u) is not finite, and zero otherwise.
 __device__ __forceinline__ float int64_energy(const float (&f)[9], const float (&w)[9]) {
     double acc = __dmul_rn(widen(f[0]), widen(w[0]));
 #pragma unroll

@@ -28,7 +28,7 @@ namespace lbm {
 struct Fp64Step {
     double w[9][5];
     double kap;              // d / c1
-    double te, t1, t2;       // eta0^2 / b, c1^2 / b, c2^2 / b:  p = te f_0 + t1 (s14 - q) + t2 s58
+    double te, t1, t2;       // eta0^2 / b, c1^2 / b, c2^2 / b:  p = te f_0 + t1 s14 + t2 s58 - t1 q
     double k0;               // omega A_0 / T
     double vp;               // (b + 2) / c1^2:  V = (vp p + q) / rho
     double a1r, a1p, a1q;    // omega rho A_1..4 = a1r rho + a1p p + a1q q
@@ -123,6 +123,11 @@ __device__ __forceinline__ unsigned fp64_health(double rho, double p, double V) 
     return __double_as_longlong(p) > 0 ? 0u : ST_T_NONPOS;
 }
 
+// E / b of a node: the rest population and the sums of the two velocity sets.
+__device__ __forceinline__ double fp64_energy(const Fp64Step& C, double f0, double s14, double s58) {
+    return __fma_rn(C.te, f0, __fma_rn(C.t1, s14, C.t2 * s58));
+}
+
 // Relaxation terms omega f^eq_i of a node; returns its health bits.
 __device__ __forceinline__ unsigned fp64_relaxation(const Fp64Step& C, const double (&f)[9], double (&r)[9]) {
     // differences along +x, +y and the two diagonals, sums of the pairs
@@ -135,7 +140,7 @@ __device__ __forceinline__ unsigned fp64_relaxation(const Fp64Step& C, const dou
     const double Ux = gx * inv, Uy = gy * inv;
     const double xx = gx * Ux, yy = gy * Uy, xy = gx * Uy;
     const double q = xx + yy;
-    const double p = __fma_rn(C.te, f[0], __fma_rn(C.t1, s14 - q, C.t2 * s58));
+    const double p = __fma_rn(-C.t1, q, fp64_energy(C, f[0], s14, s58));
     const double V = __fma_rn(C.vp, p, q) * inv;
     r[0] = C.k0 * p;
     {

@@ -78,6 +78,37 @@ template <typename S, int TM>
 cudaError_t launch_step(const S* fin, S* fout, const Model<S>& M, const Grid<S>& G,
                         long long level, unsigned* status, cudaStream_t st, const StepConfig& cfg);
 
+// Several steps of a small grid in one cooperative launch (lbm_resident.cu).
+struct ResPlan {
+    int px, py;        // CTAs along x and y
+    int bw, bh;        // nodes of a tile (the last ones along x, y may be smaller)
+    int pitch;         // columns per population row of a tile in shared memory
+    int cells;         // cells a CTA publishes: 2 bw + 2 bh
+    int threads;       // per CTA
+    size_t smem;       // dynamic shared memory
+    size_t xch_bytes;  // exchange buffer, zeroed by its owner before the first launch
+};
+template <typename S>
+struct ResRun {
+    const S* fin;                // level level0, ghost cells filled
+    // step s (0-based) writes its level to (s even: out_even, odd: out_odd) +
+    // (s / 2) out_stride, if s >= write_from
+    S *out_even, *out_odd;
+    long long out_stride;
+    int write_from, nsteps;
+    long long level0;
+    unsigned long long* xch;     // exchange buffer
+    unsigned* sync;              // tag counter, count of CTAs that have left (both zero at first)
+    unsigned* status;
+};
+// False if the grid does not fit.
+template <typename S, int TM>
+bool resident_plan(int nx, int ny, ResPlan* plan);
+// M64: the constants of FP64 steps (unused otherwise).
+template <typename S, int TM>
+cudaError_t launch_resident(const ResPlan& R, const Model<S>& M, const Fp64Step& M64, const Grid<S>& G,
+                            const ResRun<S>& A, cudaStream_t st);
+
 // f = f^eq(fields) on the interior (fields are ny x nx, storage type), and the
 // ghost layer for time level 0.
 template <typename S>

@@ -89,3 +89,86 @@ def test_fp32_totals_of_values_whose_sum_leaves_the_fp32_range():
         lat.set_f(f)
         assert np.isinf(lat.conservation()[0])
     assert big == pytest.approx(9 * 2400 * float(np.float32(3e37)), rel=1e-14)
+
+
+# widths and heights around the resident kernel's tiles: one CTA, a last
+# narrower tile, a last tile of one column or row, several rounds per CTA, the
+# largest grids it takes (their shared memory nearly full) and the first it
+# leaves to the one-step kernels
+RESIDENT = [(1, 1), (33, 4), (97, 5), (153, 153), (305, 2), (700, 30), (1111, 211), (1240, 310), (1500, 320)]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_t64", "fp32_tdf", "fp32_cons"])
+@pytest.mark.parametrize("sides", [PERIODIC, WALLS, INFLOW])
+@pytest.mark.parametrize("nx,ny", RESIDENT)
+def test_steps_in_one_launch_equal_a_launch_a_step(nx, ny, sides, prec):
+    """One lbm_step(n) call (several steps per launch where the grid is small
+    enough) leaves the bits of n calls of one step, in both level buffers'
+    worth of state: after an even and an odd number of steps, after a second
+    call on the same context, and with checkpoints recorded on the way."""
+    import torch
+    p, fields = _problem(nx, ny, sides)
+    with lbm.Lattice(p, prec) as one, lbm.Lattice(p, prec) as many:
+        one.init(*fields), many.init(*fields)
+        lbm.lbm_record(many.ctx, 5)
+        for n in (3, 4, 11):
+            for _ in range(n):
+                one.step(1)
+            many.step(n)
+            assert torch.equal(one.get_f(), many.get_f()), n
+        assert one.health() == many.health()
+
+
+@pytest.mark.parametrize("sides", [PERIODIC, WALLS, INFLOW])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (33, 4), (8, 4), (97, 5), (305, 2), (120, 80), (153, 95), (160, 100)])
+def test_fp64_steps_in_one_launch_equal_a_launch_a_step(nx, ny, sides):
+    """The FP64 kernel that gives four warps to 32 nodes (one, two and three
+    groups a CTA, ragged last groups) does the one-step kernel's operations."""
+    import torch
+    p, fields = _problem(nx, ny, sides)
+    with lbm.Lattice(p, "fp64") as one, lbm.Lattice(p, "fp64") as many:
+        one.init(*fields), many.init(*fields)
+        for n in (3, 8):
+            for _ in range(n):
+                one.step(1)
+            many.step(n)
+            assert torch.equal(one.get_f(), many.get_f()), n
+
+
+def test_steps_in_one_launch_with_a_moving_split():
+    """The double Mach reflection's top boundary moves by whole cells within
+    one launch."""
+    import torch
+    p = W.dmr(40)
+    p = p.with_(sides=p.sides[:3] + (Side("dirichlet", "dirichlet", 1.0, 60.0, p.sides[3].state_lo,
+                                          p.sides[3].state_hi),))
+    assert 60.0 * p.dt * 300 > 20 * p.dx
+    with lbm.Lattice(p, "fp32_tdf") as one, lbm.Lattice(p, "fp32_tdf") as many:
+        one.init(*W.initial_fields(p)), many.init(*W.initial_fields(p))
+        for _ in range(300):
+            one.step(1)
+        many.step(300)
+        assert torch.equal(one.get_f(), many.get_f())
+
+
+def test_a_captured_call_of_several_steps_replays():
+    """lbm_step captured into a CUDA graph: each replay continues from the
+    levels the last one left (an even number of steps, so the current level's
+    buffer stays the same)."""
+    import torch
+    p, fields = _problem(200, 12, WALLS)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        lat = lbm.Lattice(p, "fp32_cons").init(*fields)
+        lat.step(4)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            lat.step(6)
+        for _ in range(3):
+            g.replay()
+        s.synchronize()
+        got = lat.get_f()
+    with lbm.Lattice(p, "fp32_cons") as ref:
+        assert torch.equal(ref.init(*fields).step(22).get_f(), got)
+    lat.close()
