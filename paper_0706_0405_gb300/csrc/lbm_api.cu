@@ -415,7 +415,7 @@ cudaError_t step_resident(lbm_ctx* c, int n) {
         A.nsteps = n;
         A.level0 = c->step;
         A.sync = c->d_res;
-        A.xch = reinterpret_cast<unsigned long long*>(c->d_res + 64);
+        A.xch = reinterpret_cast<ResWord*>(c->d_res + 64);
         A.status = c->d_status;
         return launch_resident<S, decltype(tm)::value>(c->res, model_of<S>(c), c->f64, grid_of<S>(c), A, c->stream);
     });

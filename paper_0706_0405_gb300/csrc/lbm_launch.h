@@ -88,6 +88,9 @@ struct ResPlan {
     size_t smem;       // dynamic shared memory
     size_t xch_bytes;  // exchange buffer, zeroed by its owner before the first launch
 };
+struct alignas(16) ResWord {
+    unsigned long long lo, hi;  // three 32-bit values, then the tag
+};
 template <typename S>
 struct ResRun {
     const S* fin;                // level level0, ghost cells filled
@@ -97,7 +100,7 @@ struct ResRun {
     long long out_stride;
     int write_from, nsteps;
     long long level0;
-    unsigned long long* xch;     // exchange buffer
+    ResWord* xch;                // exchange buffer
     unsigned* sync;              // tag counter, count of CTAs that have left (both zero at first)
     unsigned* status;
 };

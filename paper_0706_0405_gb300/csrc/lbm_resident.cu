@@ -8,33 +8,34 @@
 // a fixed tile, keeps its level in shared memory for all the steps and
 // exchanges only the tile's edge nodes with the CTAs next to it.  Measured, us
 // a step, launch a step -> here (FP32_TDF / FP32_CONS / FP32_T64): 400 x 4
-// 5.3 -> 1.2 / 3.6 -> 1.2 / 4.5 -> 1.5, 2000 x 4 5.4 -> 1.3 / 3.7 -> 1.2 /
-// 4.5 -> 1.6, 400 x 100 6.1 -> 2.0 / 4.7 -> 1.8 / 5.8 -> 2.5, 1024 x 256
-// 8.8 -> 5.4 / 7.3 -> 4.5 / 11.4 -> 7.0; FP64: 400 x 4 6.1 -> 2.9,
-// 2000 x 4 6.0 -> 3.9.  A small tile's step is a chain of latencies: the node
-// update 750 cycles, the exchange about 1000, barriers; a large one's is
-// issue- and shared-memory-bound (41 % of the issue slots at 1024 x 256, the
-// exchange not overlapped).
+// 5.3 -> 1.3 / 3.6 -> 1.2 / 4.5 -> 1.6, 2000 x 4 5.4 -> 1.3 / 3.7 -> 1.2 /
+// 4.5 -> 1.6, 400 x 100 6.1 -> 1.9 / 4.7 -> 1.7 / 5.8 -> 2.4, 1024 x 256
+// 8.8 -> 4.5 / 7.3 -> 3.8 / 11.4 -> 6.8; FP64: 400 x 4 6.1 -> 3.1,
+// 2000 x 4 6.0 -> 4.0.  A small tile's step is a chain of latencies: the node
+// update 950 cycles, the exchange about 1300 (of which 1000 from one CTA's
+// store to another's poll, measured between neighbours among 50 to 125 CTAs),
+// barriers 150; a large one's is issue- and shared-memory-bound.
 //  * two copies of the tile with a one-cell halo, [row][population][column]
 //    like a level; a step reads one and writes the other;
-//  * a step is: every thread updates its nodes; a CTA barrier; then different
-//    warps publish the tile's edge cells, fill its ghost cells and poll its
-//    halo cells, one cell (nine values) a thread, from tables made at the
-//    start (source and target of every cell); a second barrier.  (In the edge
-//    nodes' own threads this took up to 3600 cycles a step, where the node
-//    update takes 750; one value a thread was slower too, its polls one after
-//    the other);
-//  * an edge value travels as one 64-bit word, the value and the step it
-//    belongs to (FP64: two words, a half of the value each), written and
-//    polled with relaxed GPU-scope accesses.  The tag makes the word its own
-//    flag: no fence, no second round trip (500 cycles one way, measured
-//    between two CTAs).  Slots alternate by the step's parity: a CTA publishes
-//    step t + 2 only after it has received its neighbours' t + 1, which they
-//    publish after a barrier that follows their reads of t.  Tags come from a
-//    counter in device memory that only grows, advanced by the last CTA to
-//    leave, so replays of a captured launch work;
+//  * a step is: the threads update the tile's nodes, its edge nodes first,
+//    and publish the edge nodes' values from registers as they go; the
+//    last warps poll the halo cells, one cell (nine values) a thread, while
+//    others fill the tile's ghost cells from tables made at the start; a
+//    barrier ends the step, and one before the ghost cells where the tile has
+//    any.  (Publishing in a phase of its own after a barrier cost 0.35 us a
+//    step; ghost rules and polls in the edge nodes' own threads up to 3600
+//    cycles, where the node update takes 900);
+//  * edge values travel as 128-bit words of three 32-bit values and the step
+//    they belong to (FP64: one value), written and polled with relaxed
+//    GPU-scope accesses.  The tag makes a word its own flag: no fence, no
+//    second round trip.  Slots
+//    alternate by the step's parity: a CTA publishes step t + 2 only after it
+//    has received its neighbours' t + 1, which they publish after a barrier
+//    that follows their reads of t.  Tags come from a counter in device memory
+//    that only grows, advanced by the last CTA to leave, so replays of a
+//    captured launch work;
 //  * the place of a moving split (the double Mach reflection's top boundary)
-//    is turned into an index once a step, by the last warp;
+//    is turned into an index once a step, by a warp of its own;
 //  * the last two steps also write their levels to the context's buffers,
 //    ghosts included, so that every call leaves what the one-step kernels
 //    would have left.
@@ -48,28 +49,42 @@ namespace {
 constexpr long long kPollCycles = 4000000000LL;  // ~2 s, then a poll gives up
 constexpr int kPadL = 2;                         // columns left of the tile in shared memory (pairs stay aligned)
 
-__device__ __forceinline__ void st_word(unsigned long long* p, unsigned value, unsigned tag) {
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)tag << 32) | value) : "memory");
+__device__ __forceinline__ void st_word(ResWord* p, unsigned a, unsigned b, unsigned c, unsigned tag) {
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\t.reg .b64 l, h;\n\tmov.b64 l, {%1, %2};\n\tmov.b64 h, {%3, %4};\n\t"
+        "mov.b128 t, {l, h};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+        "r"(a), "r"(b), "r"(c), "r"(tag)
+        : "memory");
 }
-__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
+__device__ __forceinline__ ResWord ld_word(const ResWord* p) {
+    ResWord w;
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+        : "=l"(w.lo), "=l"(w.hi)
+        : "l"(p)
+        : "memory");
+    return w;
 }
+__device__ __forceinline__ unsigned word_tag(const ResWord& w) { return (unsigned)(w.hi >> 32); }
 
-// Words per value, and the value's transport.
+// Words per cell: three FP32 values each, or one FP64 value.
 template <typename S>
-constexpr int kWords = sizeof(S) / 4;
-__device__ __forceinline__ void put(unsigned long long* p, float v, unsigned tag) {
-    st_word(p, __float_as_uint(v), tag);
-}
-__device__ __forceinline__ void put(unsigned long long* p, double v, unsigned tag) {
-    st_word(p, (unsigned)__double2loint(v), tag);
-    st_word(p + 1, (unsigned)__double2hiint(v), tag);
-}
-__device__ __forceinline__ float take(const unsigned long long (&w)[1]) { return __uint_as_float((unsigned)w[0]); }
-__device__ __forceinline__ double take(const unsigned long long (&w)[2]) {
-    return __hiloint2double((int)(unsigned)w[1], (int)(unsigned)w[0]);
+constexpr int kCellWords = sizeof(S) == 4 ? 3 : 9;
+
+constexpr unsigned kNoCell = 0xffffu;
+// The exchange cell of node (lx, ly) of a tile of w x h nodes: the bottom
+// row, the top row, the left and the right column, where there are CTAs on
+// that axis.
+__host__ __device__ __forceinline__ unsigned cell_id(const ResPlan& R, int lx, int ly, int w, int h) {
+    if (R.py > 1) {
+        if (ly == 0) return lx;
+        if (ly == h - 1) return R.bw + lx;
+    }
+    if (R.px > 1) {
+        if (lx == 0) return 2 * R.bw + ly;
+        if (lx == w - 1) return 2 * R.bw + R.bh + ly;
+    }
+    return kNoCell;
 }
 
 // Values of one node after a step, FP32 modes, from the box b (populations P
@@ -101,13 +116,13 @@ __device__ __forceinline__ unsigned node_update(const Model<float>& M, const flo
 // fp64_relaxation and fp64_update, so the bits are too.
 constexpr int kQuadGroups = 3;  // 32-node groups per CTA at most
 __device__ __forceinline__ unsigned quad_update(const Fp64Step& C, const double* cur, double* nxt,
-                                                const unsigned short* item, int n_items, int P) {
+                                                const unsigned* item, int n_items, int P) {
     __shared__ double pairs[kQuadGroups][8][32];  // differences (0..3) and sums (4..7) of the warps' pairs
     __shared__ double mom[kQuadGroups][5][32];    // 1 / rho, rho, gx, gy, E / b
     const int lane = threadIdx.x & 31, role = threadIdx.x / 32 & 3, group = threadIdx.x / 128;
     const int q = group * 32 + lane;
     const bool in = q < n_items;
-    const int at = item[in ? q : 0];
+    const int at = (int)(item[in ? q : 0] & 0xffffu);
     const double* b = cur + at;
     // the pair's populations against and along its direction
     const int lo = role == 0 ? 1 : role == 1 ? 2 : role == 2 ? 5 : 8, hi = role == 0 ? 3 : role == 1 ? 4 : role == 2 ? 7 : 6;
@@ -198,24 +213,19 @@ __device__ __forceinline__ void fill_ghost(const Grid<S>& G, int side, int part,
     }
 }
 
-// Poll the nine values of one halo cell until all carry the tag, and put them
-// at dst (P apart).  False if the poll gave up.
+// Poll the words of one halo cell until all carry the tag, and put the nine
+// values at dst (P apart).  False if the poll gave up.
 template <typename S>
-__device__ __forceinline__ bool receive(const unsigned long long* src, int stride, unsigned tag, S* dst, int P,
-                                        const unsigned* status) {
-    constexpr int W = kWords<S>;
-    unsigned long long w[9][W];
+__device__ __forceinline__ bool receive(const ResWord* src, unsigned tag, S* dst, int P, const unsigned* status) {
+    constexpr int Q = kCellWords<S>;
+    ResWord w[Q];
     long long t0 = 0;
     for (unsigned spins = 0;; ++spins) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
-#pragma unroll
-            for (int k = 0; k < W; ++k) w[i][k] = ld_word(src + (size_t)(i * stride + k));
+        for (int k = 0; k < Q; ++k) w[k] = ld_word(src + k);
         unsigned miss = 0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
-#pragma unroll
-            for (int k = 0; k < W; ++k) miss |= (unsigned)(w[i][k] >> 32) ^ tag;
+        for (int k = 0; k < Q; ++k) miss |= word_tag(w[k]) ^ tag;
         if (miss == 0) break;
         if ((spins & 63) == 63) {
             const long long t = clock64();
@@ -224,7 +234,15 @@ __device__ __forceinline__ bool receive(const unsigned long long* src, int strid
         }
     }
 #pragma unroll
-    for (int i = 0; i < 9; ++i) dst[i * P] = take(w[i]);
+    for (int k = 0; k < Q; ++k) {
+        if constexpr (sizeof(S) == 4) {
+            dst[(3 * k) * P] = __uint_as_float((unsigned)w[k].lo);
+            dst[(3 * k + 1) * P] = __uint_as_float((unsigned)(w[k].lo >> 32));
+            dst[(3 * k + 2) * P] = __uint_as_float((unsigned)w[k].hi);
+        } else {
+            dst[k * P] = __longlong_as_double((long long)w[k].lo);
+        }
+    }
     return true;
 }
 }  // namespace
@@ -249,13 +267,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     S* cur = reinterpret_cast<S*>(smem);
     S* nxt = cur + buf;
     // tables: per ghost cell its place, its source's, its side and along-side
-    // index; per halo cell its source's word; per published cell its place and
-    // its cell index; per halo cell its place; per node its place
+    // index; per halo cell its source's cell; per node its place and the cell
+    // it is published as; per halo cell its place
     uint2* ghost = reinterpret_cast<uint2*>(nxt + buf);
     unsigned* halo_src = reinterpret_cast<unsigned*>(ghost + R.cells);
-    unsigned* send = halo_src + R.cells;
-    unsigned short* halo_dst = reinterpret_cast<unsigned short*>(send + R.cells);
-    unsigned short* item = halo_dst + R.cells;
+    unsigned* item = halo_src + R.cells;
+    unsigned short* halo_dst = reinterpret_cast<unsigned short*>(item + R.bw * R.bh);
     __shared__ int split_now[2][4];  // by the step's parity
     const int origin = RS + kPadL;  // node (0, 0), population 0, in a buffer
     const unsigned epoch = *(volatile unsigned*)A.sync;
@@ -268,33 +285,52 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int south = by > 0 ? cta - R.px : (pery && R.py > 1 ? cta + (R.py - 1) * R.px : -1);
     const int north = by < R.py - 1 ? cta + R.px : (pery && R.py > 1 ? cta - (R.py - 1) * R.px : -1);
 
-    const int n_items = w * h;  // the tile's nodes, row by row
-    for (int q = tid; q < n_items; q += T) item[q] = (unsigned short)(origin + q / w * RS + q % w);
+    // the tile's nodes in the order of their update: those that are published
+    // first (bottom and top row, left and right column, on the axes with other
+    // CTAs), so that few warps publish, then the rest row by row
+    const int n_items = w * h;
+    const int ey = R.py > 1, ex = R.px > 1;
+    const int n_rows = ey ? w * min(h, 2) : 0, rest_h = ey ? max(h - 2, 0) : h;
+    const int n_cols = ex ? rest_h * min(w, 2) : 0, rest_w = ex ? w - 2 : w;
+    const int n_edge = n_rows + n_cols;
+    for (int q = tid; q < n_items; q += T) {
+        int r, c, k = q;
+        if (k < n_rows) {
+            r = k < w ? 0 : h - 1;
+            c = k < w ? k : k - w;
+        } else if ((k -= n_rows) < n_cols) {
+            r = ey + k % rest_h;
+            c = k < rest_h ? 0 : w - 1;
+        } else {
+            k -= n_cols;
+            r = ey + k / rest_w;
+            c = ex + k % rest_w;
+        }
+        item[q] = (unsigned)(origin + r * RS + c) | cell_id(R, c, r, w, h) << 16;
+    }
     // halo cells that come from other CTAs: west and east columns, south and
-    // north rows.  A CTA's published cells: bottom row, top row (bw each),
-    // left column, right column (bh each)
+    // north rows
     const int n_w = west >= 0 ? h : 0, n_e = east >= 0 ? h : 0, n_s = south >= 0 ? w : 0, n_n = north >= 0 ? w : 0;
-    const int n_halo = n_w + n_e + n_s + n_n;  // also the number of cells published
-    const int cta_words = 9 * R.cells;
+    const int n_halo = n_w + n_e + n_s + n_n;
     for (int q = tid; q < n_halo; q += T) {
-        int k = q, from, at, dst, src, to;
-        if (k < n_w) {
-            from = west, at = 2 * R.bw + R.bh + k, dst = origin + k * RS - 1;
-            src = origin + k * RS, to = 2 * R.bw + k;
-        } else if ((k -= n_w) < n_e) {
-            from = east, at = 2 * R.bw + k, dst = origin + k * RS + w;
-            src = dst - 1, to = 2 * R.bw + R.bh + k;
-        } else if ((k -= n_e) < n_s) {
-            from = south, at = R.bw + k, dst = origin - RS + k;
-            src = origin + k, to = k;
+        int k = q, from, dst;
+        const int side = k < n_w ? S_LEFT : (k -= n_w) < n_e ? S_RIGHT : (k -= n_e) < n_s ? S_BOTTOM : S_TOP;
+        if (side == S_LEFT) {
+            from = west, dst = origin + k * RS - 1;
+        } else if (side == S_RIGHT) {
+            from = east, dst = origin + k * RS + w;
+        } else if (side == S_BOTTOM) {
+            from = south, dst = origin - RS + k;
         } else {
             k -= n_s;
-            from = north, at = k, dst = origin + h * RS + k;
-            src = dst - RS, to = R.bw + k;
+            from = north, dst = origin + h * RS + k;
         }
-        halo_src[q] = (unsigned)(from * cta_words + at);
+        // the node in the other CTA's tile
+        const int fw = min(R.bw, G.nx - from % R.px * R.bw), fh = min(R.bh, G.ny - from / R.px * R.bh);
+        const int lx = side == S_LEFT ? fw - 1 : side == S_RIGHT ? 0 : k;
+        const int ly = side == S_BOTTOM ? fh - 1 : side == S_TOP ? 0 : k;
+        halo_src[q] = (unsigned)(from * R.cells) + cell_id(R, lx, ly, fw, fh);
         halo_dst[q] = (unsigned short)dst;
-        send[q] = (unsigned)src | (unsigned)to << 16;
     }
     // ghost cells inside the tile: of physical sides, and of periodic sides
     // whose two ends the tile holds
@@ -327,29 +363,55 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncthreads();
 
-    constexpr int W = kWords<S>;
-    unsigned long long* const mine = A.xch + (size_t)cta * cta_words * W;
-    const size_t slot_words = (size_t)gridDim.x * cta_words * W;
-    // the first warps publish, the next fill ghost cells, the next poll
-    const int ghost_from = (n_halo + 31) / 32 * 32 % T, halo_from = (ghost_from + (n_ghost + 31) / 32 * 32) % T;
-    const int ghost_tid = (tid - ghost_from + T) % T, halo_tid = (tid - halo_from + T) % T;
+    constexpr int Q = kCellWords<S>;
+    const size_t slot_cells = (size_t)gridDim.x * R.cells;
+    // the last warps poll, those before them fill ghost cells; FP32: after the
+    // very last one, which follows the moving splits, beside the node updates
+    // (its few FP64 instructions take up to 1600 cycles)
+    const int T1 = sizeof(S) == 4 ? T - 32 : T;
+    const int halo_tid = tid < T1 ? T1 - 1 - tid : tid;
+    const int ghost_tid = (halo_tid - (n_halo + 31) / 32 * 32 % T + T) % T;
+    const int split_tid = sizeof(S) == 4 ? tid - T1 : tid;
     unsigned bits = 0;
     bool ok = true;
     for (int s = 0; s < A.nsteps; ++s) {
         const unsigned tag = epoch + (unsigned)s + 1u;
+        const bool more = s + 1 < A.nsteps, keep = s >= A.write_from;
+        const ResWord* in_box = A.xch + (tag & 1u) * slot_cells * Q;
+        ResWord* out_box = more ? A.xch + ((tag & 1u) * slot_cells + (size_t)cta * R.cells) * Q : nullptr;
+        if (more && split_tid >= 0 && split_tid < 4)
+            split_now[(s + 1) & 1][split_tid] = split_at(G, split_tid, A.level0 + s + 2);
         if constexpr (sizeof(S) == 8) {
             bits |= quad_update(M, cur, nxt, item, n_items, P);
+            __syncthreads();  // a node's values come from four warps
+            for (int q = tid; q < n_edge && more; q += T) {
+                const unsigned it = item[q];
+                ResWord* d = out_box + (size_t)(it >> 16) * Q;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    const double v = nxt[(it & 0xffffu) + i * P];
+                    st_word(d + i, (unsigned)__double2loint(v), (unsigned)__double2hiint(v), 0u, tag);
+                }
+            }
         } else {
-            for (int q = tid; q < n_items; q += T) {
-                const int at = item[q];
+            for (int q = tid < T1 ? tid : n_items; q < n_items; q += T1) {
+                const unsigned it = item[q];
+                const int at = (int)(it & 0xffffu);
                 S o[9];
                 bits |= node_update<TM>(M, cur + at, P, o);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) nxt[at + i * P] = o[i];
+                if (more && it >> 16 != kNoCell) {
+                    ResWord* d = out_box + (size_t)(it >> 16) * Q;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        st_word(d + k, __float_as_uint(o[3 * k]), __float_as_uint(o[3 * k + 1]),
+                                __float_as_uint(o[3 * k + 2]), tag);
+                }
             }
         }
-        __syncthreads();
-        if (s >= A.write_from) {
+        if (sizeof(S) == 4 && (keep || n_ghost)) __syncthreads();
+        if (keep) {
             // this level goes to the context's buffer too
             S* const fout = ((s & 1) ? A.out_odd : A.out_even) + (size_t)(s >> 1) * (size_t)A.out_stride;
             const int cols = 9 * w;
@@ -369,25 +431,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
-        if (s + 1 == A.nsteps) break;
-        unsigned long long* const out_box = mine + (tag & 1u) * slot_words;
-        for (int q = tid; q < n_halo; q += T) {
-            const unsigned e = send[q];
-            const S* v = nxt + (e & 0xffffu);
-            unsigned long long* d = out_box + (size_t)(e >> 16) * W;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) put(d + (size_t)(i * R.cells * W), v[i * P], tag);
-        }
+        if (!more) break;
+        for (int q = halo_tid; q < n_halo && ok; q += T)
+            ok = receive<S>(in_box + (size_t)halo_src[q] * Q, tag, nxt + halo_dst[q], P, A.status);
         for (int q = ghost_tid; q < n_ghost; q += T) {
             const uint2 e = ghost[q];
             const int side = e.y & 3u;
             fill_ghost(G, side, (int)(e.y >> 2) < split_now[s & 1][side] ? 0 : 1, nxt + (e.x & 0xffffu),
                        nxt + (e.x >> 16), P);
         }
-        const unsigned long long* in_box = A.xch + (tag & 1u) * slot_words;
-        for (int q = halo_tid; q < n_halo && ok; q += T)
-            ok = receive<S>(in_box + (size_t)halo_src[q] * W, R.cells * W, tag, nxt + halo_dst[q], P, A.status);
-        if (tid >= T - 4) split_now[(s + 1) & 1][T - 1 - tid] = split_at(G, T - 1 - tid, A.level0 + s + 2);
         if (__syncthreads_or(!ok)) {
             ok = false;
             break;
@@ -410,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 namespace {
-constexpr int kThreads32 = 512, kThreads64 = 128 * kQuadGroups;
+constexpr int kThreads32 = 768, kThreads64 = 128 * kQuadGroups;
 
 // The largest dynamic shared memory of a plan: 227 KB a CTA less the static
 // part; FP64 tiles are small.
@@ -418,7 +470,7 @@ template <typename S>
 constexpr size_t kSmemMax = sizeof(S) == 4 ? 226 * 1024 : 113 * 1024;
 
 size_t smem_bytes(const ResPlan& R, size_t esize) {
-    return 2 * (size_t)(R.bh + 2) * 9 * R.pitch * esize + 18 * (size_t)R.cells + 2 * (size_t)R.bw * R.bh;
+    return 2 * (size_t)(R.bh + 2) * 9 * R.pitch * esize + 14 * (size_t)R.cells + 4 * (size_t)R.bw * R.bh;
 }
 
 template <typename S, int TM>
@@ -456,14 +508,22 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
             R.bh = (ny + py - 1) / py;
             R.py = (ny + R.bh - 1) / R.bh;
             if (R.py != py) continue;
-            const int align = how == 0 ? 1 : how == 1 ? 32 : R.bh < 32 ? 32 / R.bh : 1;
             const int mx = sms / py;
-            R.bw = ((nx + mx - 1) / mx + align - 1) / align * align;
+            R.bw = (nx + mx - 1) / mx;
+            const int ends = R.bw < nx ? 2 : 0;  // columns updated apart from the rows
+            if (how == 1) R.bw = (R.bw - ends + 31) / 32 * 32 + ends;
+            if (how == 2 && R.bh < 32) R.bw = (R.bw + 32 / R.bh - 1) / (32 / R.bh) * (32 / R.bh);
             R.px = (nx + R.bw - 1) / R.bw;
-            // pitch: a warp that continues on the next row stays free of bank
-            // conflicts if 9 pitch = bw modulo 32 banks (9 x 25 = 1 mod 32)
+            // pitch: a warp that continues on the next row of the inner columns
+            // stays free of bank conflicts if 9 pitch = their number modulo 32
+            // banks (9 x 25 = 1 mod 32); if rows are whole warps, an odd pitch
+            // keeps the column updates free of them
+            const int inner = R.bw - (R.px > 1 ? 2 : 0);
             R.pitch = R.bw + 4;
-            if (R.bw % 32 != 0) R.pitch += ((25 * R.bw - R.pitch) % 32 + 32) % 32;
+            if (inner % 32 != 0)
+                R.pitch += ((25 * inner - R.pitch) % 32 + 32) % 32;
+            else
+                R.pitch |= 1;
             R.cells = 2 * R.bw + 2 * R.bh;
             const int warps = (R.bw * R.bh + 31) / 32;
             const int exchanged = R.py > 1 ? R.cells : 2 * R.bh;
@@ -471,17 +531,18 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
                 if (warps > kQuadGroups) continue;
                 R.threads = 128 * warps;
             } else {
-                const int rounds = (32 * warps + kThreads32 - 1) / kThreads32;
+                const int most = kThreads32 - 32, rounds = (32 * warps + most - 1) / most;
                 R.threads = (warps + rounds - 1) / rounds * 32;
-                // warps enough that no warp has to publish and poll as well
-                const int roles = 2 * ((exchanged + 31) / 32 * 32) + 64;
-                if (R.threads < roles) R.threads = roles < kThreads32 ? roles : kThreads32;
+                // warps enough to poll beside those that update the last nodes
+                const int roles = (exchanged + 31) / 32 * 32 + 64;
+                if (R.threads < roles) R.threads = roles < most ? roles : most;
+                R.threads += 32;
             }
             R.smem = smem_bytes(R, sizeof(S));
             // places in the tile are 16-bit
             if ((R.bh + 2) * 9 * R.pitch > 65535 || R.smem > kSmemMax<S>) continue;
-            const double each = f64 ? 1.25 : TM == T_INT64 ? 0.13 : R.bw % 32 == 0 ? 0.060 : 0.067;
-            const double c = each * warps + 0.002 * exchanged + (R.py > 1 ? 0.2 : 0.0) + 0.001 * R.px * R.py;
+            const double each = f64 ? 1.25 : TM == T_INT64 ? 0.13 : inner % 32 == 0 ? 0.060 : 0.067;
+            const double c = each * warps + (f64 ? 0.02 : 0.002) * exchanged + (R.py > 1 ? 0.2 : 0.0) + 0.001 * R.px * R.py;
             if (!found || c < cost) {
                 found = true;
                 cost = c;
@@ -489,7 +550,7 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
             }
         }
     if (!found) return false;
-    best->xch_bytes = 2 * (size_t)best->px * best->py * 9 * best->cells * 8 * (sizeof(S) / 4);
+    best->xch_bytes = 2 * (size_t)best->px * best->py * best->cells * kCellWords<S> * sizeof(ResWord);
     // resident all at once; sets the kernel's shared-memory limit on this device
     constexpr auto kern = kernel_of<S, TM>();
     int per_sm = 0;
