@@ -296,6 +296,9 @@ template <typename S> const Grid<S>& grid_of(const lbm_ctx* c);
 template <> const Grid<double>& grid_of<double>(const lbm_ctx* c) { return c->gd; }
 template <> const Grid<float>& grid_of<float>(const lbm_ctx* c) { return c->gf; }
 
+// Whether device_view copies p through the staging buffer.
+bool staged(const void* p) { return p && !is_device_ptr(p) && !pinned_alias(p); }
+
 // Copy `bytes` from a host or device pointer into the staging buffer at
 // `offset` (returns a device pointer to read from), or pass device pointers
 // through.
@@ -320,13 +323,25 @@ lbm_status device_view(lbm_ctx* c, const void* p, size_t bytes, size_t offset, c
 
 size_t level_bytes(const lbm_ctx* c) { return (size_t)(c->ny + 2) * (size_t)c->row * c->esize; }
 
+size_t level_stride(const lbm_ctx* c) { return (level_bytes(c) + 255) / 256 * 256; }
+
+// Make room for n checkpoints, the missing ones in one allocation (cudaMalloc
+// and cudaFree of a level cost about 40 us each, whatever its size up to tens
+// of MB).
+lbm_status reserve_checkpoints(lbm_ctx* c, size_t n) {
+    if (c->ck.size() >= n) return LBM_OK;
+    const size_t more = n - c->ck.size();
+    char* p = nullptr;
+    LBM_CUDA(c, dev_malloc(&p, more * level_stride(c)), "allocating checkpoints");
+    c->ck_mem.push_back(p);
+    for (size_t k = 0; k < more; ++k) c->ck.push_back(p + k * level_stride(c));
+    return LBM_OK;
+}
+
 // Keep a copy of the current level (padded, ghosts included) as checkpoint k.
 lbm_status save_checkpoint(lbm_ctx* c, size_t k) {
-    while (c->ck.size() <= k) {
-        void* p = nullptr;
-        LBM_CUDA(c, dev_malloc(&p, level_bytes(c)), "allocating a checkpoint");
-        c->ck.push_back(p);
-    }
+    const lbm_status s = reserve_checkpoints(c, k + 1);
+    if (s != LBM_OK) return s;
     LBM_CUDA(c, cudaMemcpyAsync(c->ck[k], c->f[c->cur], level_bytes(c), cudaMemcpyDeviceToDevice, c->stream),
              "saving a checkpoint");
     return LBM_OK;
@@ -403,19 +418,35 @@ bool plan_resident(lbm_ctx* c) {
 // step: it reads the level, exchanges n - 1 times and writes two levels.
 constexpr int kResidentMinSteps = 3;
 
-// n steps of the context in one launch (res_ok).
-cudaError_t step_resident(lbm_ctx* c, int n) {
+// The default launch shape: lbm_step and the adjoint's recomputation may run
+// several steps per launch.
+bool default_launch(const lbm_ctx* c) {
+    return c->cfg.grid == 0 && c->cfg.variant == (c->prec == LBM_FP64 ? STEP_SIMPLE : STEP_TILE);
+}
+
+// n steps from `level` in `fin` in one launch (res_ok).  seg = nullptr: fin is
+// the context's current buffer, the last two levels go to the two buffers in
+// turn; else every level, seg + k * level_stride() receiving level + k.
+cudaError_t step_resident(lbm_ctx* c, int n, const char* fin, char* seg, long long level) {
     return dispatch(c, [&](auto tag, auto tm) {
         using S = decltype(tag);
         ResRun<S> A{};
-        A.fin = static_cast<const S*>(c->f[c->cur]);
-        A.out_even = static_cast<S*>(c->f[c->cur ^ 1]);
-        A.out_odd = static_cast<S*>(c->f[c->cur]);
-        A.write_from = n - 2;
+        A.fin = reinterpret_cast<const S*>(fin);
+        if (seg) {
+            const size_t stride = level_stride(c);
+            A.out_even = reinterpret_cast<S*>(seg + stride);
+            A.out_odd = reinterpret_cast<S*>(seg + 2 * stride);
+            A.out_stride = (long long)(2 * stride / sizeof(S));
+            A.write_from = 0;
+        } else {
+            A.out_even = static_cast<S*>(c->f[c->cur ^ 1]);
+            A.out_odd = static_cast<S*>(c->f[c->cur]);
+            A.write_from = n - 2;
+        }
         A.nsteps = n;
-        A.level0 = c->step;
+        A.level0 = level;
         A.sync = c->d_res;
-        A.xch = reinterpret_cast<ResWord*>(c->d_res + 64);
+        A.xch = c->d_xch;
         A.status = c->d_status;
         return launch_resident<S, decltype(tm)::value>(c->res, model_of<S>(c), c->f64, grid_of<S>(c), A, c->stream);
     });
@@ -484,21 +515,25 @@ lbm_status create_context(int nx, int ny, double b, double tau, double dt, doubl
             c->f[k] = bufs[k];
         }
         c->f_owned = false;
-    } else {
-        for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = dev_malloc(&c->f[k], fbytes);
     }
     if (resident) c->res_ok = plan_resident(c);
+    const size_t xbytes = c->res_ok ? c->res.xch_bytes : 0;
+    // the exchange buffer of the resident steps lies behind the second level,
+    // or behind the status words if the levels are the caller's
+    if (!caller_f) {
+        e = dev_malloc(&c->f[0], fbytes);
+        if (e == cudaSuccess) e = dev_malloc(&c->f[1], level_stride(c) + xbytes);
+    }
     // status word, a spare, and the tile kernel's two scheduling counters; 256
-    // bytes on, the words and the exchange buffer of the resident steps
-    const size_t status_bytes = c->res_ok ? 512 + c->res.xch_bytes : 4 * sizeof(unsigned);
+    // bytes on, the tag counter and the leave count of the resident steps
+    const size_t status_bytes = 512 + (caller_f ? xbytes : 0);
     if (e == cudaSuccess) e = dev_malloc((void**)&c->d_status, status_bytes);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_status, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_sums, 6 * sizeof(double));
     const int np = c->prec == LBM_FP64 ? conservation_partials(c->gd) : conservation_partials(c->gf);
     if (e == cudaSuccess) e = dev_malloc((void**)&c->d_partials, sizeof(double) * 4 * np);
     if (e == cudaSuccess) e = dev_malloc((void**)&c->d_left, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_sums, sizeof(double) * 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->f[0], 0, fbytes, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, fbytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->f[1], 0, caller_f ? fbytes : level_stride(c) + xbytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, status_bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_left, 0, sizeof(unsigned), c->stream);
     if (e != cudaSuccess) {
@@ -506,10 +541,16 @@ lbm_status create_context(int nx, int ny, double b, double tau, double dt, doubl
         lbm_destroy(c);
         return r;
     }
+    c->h_tau = c->h_sums + 4;
+    c->h_status = reinterpret_cast<unsigned*>(c->h_sums + 5);
+    if (c->res_ok) {
+        c->d_res = c->d_status + 64;
+        c->d_xch = reinterpret_cast<ResWord*>(caller_f ? reinterpret_cast<char*>(c->d_status) + 512
+                                                       : static_cast<char*>(c->f[1]) + level_stride(c));
+    }
     if (c->prec != LBM_FP64)
         c->tmap_ok = make_tmap(&c->tmap[0], c->f[0], *c) && make_tmap(&c->tmap[1], c->f[1], *c);
     if (c->prec != LBM_FP64 && !c->tmap_ok) c->cfg = StepConfig{STEP_VEC, 4, 0, 0};
-    if (c->res_ok) c->d_res = c->d_status + 64;
     *out = c;
     return LBM_OK;
 }
@@ -617,17 +658,14 @@ void lbm_destroy(lbm_ctx* c) {
         cudaFree(c->f[1]);
     }
     cudaFree(c->d_status);
-    cudaFreeHost(c->h_status);
     cudaFree(c->d_partials);
     cudaFree(c->d_left);
     cudaFreeHost(c->h_sums);
     cudaFree(c->d_stage);
-    for (void* p : c->ck) cudaFree(p);
-    for (void* p : c->seg) cudaFree(p);
+    for (void* p : c->ck_mem) cudaFree(p);
+    cudaFree(c->seg);
     cudaFree(c->adj[0]);
-    cudaFree(c->adj[1]);
     cudaFree(c->d_taup);
-    cudaFreeHost(c->h_taup);
     cudaFree(c->d_astage);
     cudaGetLastError();
     delete c;
@@ -639,9 +677,10 @@ lbm_status lbm_init(lbm_ctx* c, const void* rho, const void* ux, const void* uy,
     if (s != LBM_OK) return s;
     if (!rho || !ux || !uy || !T) return fail(c, LBM_E_INVAL, "lbm_init: fields must not be NULL");
     const size_t fb = nodes(c) * c->esize;
-    if ((s = ensure_stage(c, 9 * fb)) != LBM_OK) return s;
     const void* d[4];
     const void* in[4] = {rho, ux, uy, T};
+    for (int k = 0; k < 4; ++k)
+        if (staged(in[k]) && (s = ensure_stage(c, 9 * fb)) != LBM_OK) return s;
     for (int k = 0; k < 4; ++k)
         if ((s = device_view(c, in[k], fb, k * fb, &d[k])) != LBM_OK) return s;
     c->cur = 0;
@@ -666,8 +705,11 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
     if (n < 0) return fail(c, LBM_E_INVAL, "lbm_step: n must be >= 0");
     if (!c->ready) return fail(c, LBM_E_STATE, "lbm_step before lbm_init / lbm_set_f / lbm_load");
     // the default launch shape: several steps per launch on small grids
-    const bool resident =
-        c->res_ok && c->cfg.grid == 0 && c->cfg.variant == (c->prec == LBM_FP64 ? STEP_SIMPLE : STEP_TILE);
+    bool resident = default_launch(c) && c->res_ok;
+    if (c->ck_every > 0) {
+        s = reserve_checkpoints(c, (size_t)((c->step + n - c->ck_base) / c->ck_every + 1));
+        if (s != LBM_OK) return s;
+    }
     for (int k = 0; k < n;) {
         int m = n - k;
         if (c->ck_every > 0) {  // up to the next level to be recorded
@@ -676,7 +718,13 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
         }
         cudaError_t e;
         if (resident && m >= kResidentMinSteps) {
-            e = step_resident(c, m);
+            e = step_resident(c, m, static_cast<const char*>(c->f[c->cur]), nullptr, c->step);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
+                // not all of the device's SMs are there for this context
+                cudaGetLastError();
+                resident = c->res_ok = false;
+                continue;
+            }
         } else {
             m = 1;
             c->cfg.tmap = c->tmap_ok ? &c->tmap[c->cur] : nullptr;
@@ -802,7 +850,7 @@ lbm_status lbm_set_f(lbm_ctx* c, const void* src, long long step) {
     if (!src) return fail(c, LBM_E_INVAL, "lbm_set_f: src must not be NULL");
     if (step < 0) return fail(c, LBM_E_INVAL, "lbm_set_f: step must be >= 0");
     const size_t bytes = 9 * nodes(c) * c->esize;
-    if (!is_device_ptr(src) && (s = ensure_stage(c, bytes)) != LBM_OK) return s;
+    if (staged(src) && (s = ensure_stage(c, bytes)) != LBM_OK) return s;
     const void* d;
     if ((s = device_view(c, src, bytes, 0, &d)) != LBM_OK) return s;
     LBM_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "clearing status");
@@ -843,9 +891,10 @@ lbm_status lbm_adjoint_seed(lbm_ctx* c, const void* qr, const void* qx, const vo
     if (!abar) return fail(c, LBM_E_INVAL, "lbm_adjoint_seed: abar must not be NULL");
     if (!c->ready) return fail(c, LBM_E_STATE, "lbm_adjoint_seed before lbm_init");
     const size_t fb = nodes(c) * c->esize;
-    if ((s = ensure_astage(c, 13 * fb)) != LBM_OK) return s;
     const void* in[4] = {qr, qx, qy, qT};
     const void* d[4];
+    for (const void* p : {in[0], in[1], in[2], in[3], (const void*)abar})
+        if (p && !is_device_ptr(p) && (s = ensure_astage(c, 13 * fb)) != LBM_OK) return s;
     for (int k = 0; k < 4; ++k) {
         if (!in[k] || is_device_ptr(in[k])) {
             d[k] = in[k];
@@ -886,34 +935,44 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
     const bool fp32 = c->prec != LBM_FP64;
     int abx = 0, aby = 0, afx = 0, afy = 0;
     adjoint_tile_boxes(&abx, &aby, &afx, &afy);
-    for (int k = 0; k < 2; ++k)
-        if (!c->adj[k]) {
-            LBM_CUDA(c, dev_malloc(&c->adj[k], lb), "allocating adjoint levels");
-            LBM_CUDA(c, cudaMemsetAsync(c->adj[k], 0, lb, c->stream), "clearing adjoint levels");
-            if (k == 1)
-                c->adj_tmaps_ok = fp32 && make_tmap_box(&c->adj_tmap[0], c->adj[0], *c, abx, aby) &&
-                                  make_tmap_box(&c->adj_tmap[1], c->adj[1], *c, abx, aby);
-        }
-    while ((int)c->seg.size() < c->ck_every) {
-        void* p = nullptr;
-        LBM_CUDA(c, dev_malloc(&p, lb), "allocating segment levels");
-        c->seg.push_back(p);
-        CUtensorMap mf{}, ms{};
-        if (c->adj_tmaps_ok && !(make_tmap_box(&mf, p, *c, afx, afy) && make_tmap(&ms, p, *c)))
-            c->adj_tmaps_ok = false;
-        c->seg_tmapF.push_back(mf);
-        c->seg_tmapS.push_back(ms);
+    const size_t stride = level_stride(c);
+    if (!c->adj[0]) {
+        char* p = nullptr;
+        LBM_CUDA(c, dev_malloc(&p, 2 * stride), "allocating adjoint levels");
+        c->adj[0] = p;
+        c->adj[1] = p + stride;
+        LBM_CUDA(c, cudaMemsetAsync(p, 0, 2 * stride, c->stream), "clearing adjoint levels");
+        c->adj_tmaps_ok = fp32 && make_tmap_box(&c->adj_tmap[0], c->adj[0], *c, abx, aby) &&
+                          make_tmap_box(&c->adj_tmap[1], c->adj[1], *c, abx, aby);
     }
+    // the segment's levels in one allocation: for 50 of 19 MB one cudaMalloc
+    // and one cudaFree take 0.5 ms, fifty of each 4 ms
+    if (c->seg_n < c->ck_every) {
+        if (c->seg) {
+            LBM_CUDA(c, cudaStreamSynchronize(c->stream), "synchronising the stream");
+            cudaFree(c->seg);
+        }
+        c->seg = nullptr;
+        c->seg_n = 0;
+        LBM_CUDA(c, dev_malloc(&c->seg, stride * (size_t)c->ck_every), "allocating segment levels");
+        c->seg_n = c->ck_every;
+        c->seg_tmapF.assign((size_t)c->seg_n, CUtensorMap{});
+        c->seg_tmapS.assign((size_t)c->seg_n, CUtensorMap{});
+        for (int k = 0; k < c->seg_n && c->adj_tmaps_ok; ++k) {
+            char* p = c->seg + stride * (size_t)k;
+            c->adj_tmaps_ok = make_tmap_box(&c->seg_tmapF[(size_t)k], p, *c, afx, afy) &&
+                              make_tmap(&c->seg_tmapS[(size_t)k], p, *c);
+        }
+    }
+    auto seg_level = [&](long long k) { return c->seg + stride * (size_t)k; };
     // the tile adjoint (and tile recomputation) with the tile step kernel
     const bool tile = c->adj_tmaps_ok && c->cfg.variant == STEP_TILE;
     const int np = c->prec == LBM_FP64 ? adjoint_partials(c->gd) : adjoint_partials(c->gf);
     if (c->ntaup < np) {
         cudaFree(c->d_taup);
-        cudaFreeHost(c->h_taup);
         c->d_taup = nullptr;
-        c->h_taup = nullptr;
+        c->ntaup = 0;
         LBM_CUDA(c, dev_malloc((void**)&c->d_taup, sizeof(double) * np), "allocating tau partials");
-        LBM_CUDA(c, cudaMallocHost((void**)&c->h_taup, sizeof(double) * np), "allocating tau partials");
         c->ntaup = np;
     }
     LBM_CUDA(c, cudaMemsetAsync(c->d_taup, 0, sizeof(double) * np, c->stream), "clearing tau partials");
@@ -941,15 +1000,27 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
         const long long k = (L - 1 - c->ck_base) / c->ck_every;
         c0 = c->ck_base + k * c->ck_every;
         const long long lo = c0 > target ? c0 : target;
-        LBM_CUDA(c, cudaMemcpyAsync(c->seg[0], c->ck[(size_t)k], lb, cudaMemcpyDeviceToDevice, c->stream),
+        LBM_CUDA(c, cudaMemcpyAsync(c->seg, c->ck[(size_t)k], lb, cudaMemcpyDeviceToDevice, c->stream),
                  "restoring a checkpoint");
-        for (long long l = c0; l < L - 1; ++l) {
+        long long l0 = c0;
+        if (c->res_ok && default_launch(c) && L - 1 - c0 >= kResidentMinSteps) {
+            e = step_resident(c, (int)(L - 1 - c0), c->seg, c->seg, c0);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
+                cudaGetLastError();
+                c->res_ok = false;
+            } else if (e != cudaSuccess) {
+                return cuda_fail(c, e, "lbm_adjoint_step: recomputing");
+            } else {
+                l0 = L - 1;
+            }
+        }
+        for (long long l = l0; l < L - 1; ++l) {
             if (tile) rcfg.tmap = &c->seg_tmapS[(size_t)(l - c0)];
             e = dispatch(c, [&](auto tag, auto tm) {
                 using S = decltype(tag);
                 constexpr int TM = decltype(tm)::value;
-                return launch_step<S, TM>(static_cast<const S*>(c->seg[(size_t)(l - c0)]),
-                                          static_cast<S*>(c->seg[(size_t)(l - c0 + 1)]), model_of<S>(c),
+                return launch_step<S, TM>(reinterpret_cast<const S*>(seg_level(l - c0)),
+                                          reinterpret_cast<S*>(seg_level(l - c0 + 1)), model_of<S>(c),
                                           grid_of<S>(c), l, c->d_status, c->stream, rcfg);
             });
             if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step: recomputing");
@@ -964,7 +1035,7 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
                                                        static_cast<float*>(c->adj[ac ^ 1]), model_of<S>(c),
                                                        grid_of<S>(c), l, c->d_taup, c->d_status, c->stream);
                 }
-                return launch_adjoint<S, TM>(static_cast<const S*>(c->seg[(size_t)(l - c0)]),
+                return launch_adjoint<S, TM>(reinterpret_cast<const S*>(seg_level(l - c0)),
                                              static_cast<const S*>(c->adj[ac]), static_cast<S*>(c->adj[ac ^ 1]),
                                              model_of<S>(c), grid_of<S>(c), l, c->d_taup, c->stream);
             });
@@ -974,7 +1045,7 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
         L = lo;
     }
     // the forward state moves back to level `target`
-    LBM_CUDA(c, cudaMemcpyAsync(c->f[c->cur], c->seg[(size_t)(target - c0)], lb, cudaMemcpyDeviceToDevice,
+    LBM_CUDA(c, cudaMemcpyAsync(c->f[c->cur], seg_level(target - c0), lb, cudaMemcpyDeviceToDevice,
                                 c->stream),
              "restoring the forward level");
     c->step = target;
@@ -986,14 +1057,10 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step: packing abar");
     if (!dev)
         LBM_CUDA(c, cudaMemcpyAsync(abar, c->d_astage, 9 * fb, cudaMemcpyDeviceToHost, c->stream), "copying abar out");
-    LBM_CUDA(c, cudaMemcpyAsync(c->h_taup, c->d_taup, sizeof(double) * np, cudaMemcpyDeviceToHost, c->stream),
-             "copying tau partials");
+    e = launch_sum(c->d_taup, np, c->h_tau, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step: summing the tau partials");
     LBM_CUDA(c, cudaStreamSynchronize(c->stream), "synchronising the stream");
-    if (dL_dtau) {
-        double t = 0.0;
-        for (int b = 0; b < np; ++b) t += c->h_taup[b];
-        *dL_dtau += -(c->dt / (c->tau * c->tau)) * t;
-    }
+    if (dL_dtau) *dL_dtau += -(c->dt / (c->tau * c->tau)) * *c->h_tau;
     return LBM_OK;
 }
 
@@ -1003,9 +1070,11 @@ lbm_status lbm_feq_vjp(lbm_ctx* c, const void* rho, const void* ux, const void* 
     if (s != LBM_OK) return s;
     if (!rho || !ux || !uy || !T || !abar) return fail(c, LBM_E_INVAL, "lbm_feq_vjp: NULL input");
     const size_t fb = nodes(c) * c->esize;
-    if ((s = ensure_astage(c, 17 * fb)) != LBM_OK) return s;
-    char* st = static_cast<char*>(c->d_astage);
     const void* in[5] = {rho, ux, uy, T, abar};
+    for (const void* p : {in[0], in[1], in[2], in[3], in[4], (const void*)grho, (const void*)gux, (const void*)guy,
+                          (const void*)gT})
+        if (p && !is_device_ptr(p) && (s = ensure_astage(c, 17 * fb)) != LBM_OK) return s;
+    char* st = static_cast<char*>(c->d_astage);
     const size_t sz[5] = {fb, fb, fb, fb, 9 * fb};
     const size_t off[5] = {0, fb, 2 * fb, 3 * fb, 4 * fb};
     const void* d[5];

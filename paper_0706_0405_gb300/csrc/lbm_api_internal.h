@@ -38,10 +38,11 @@ struct lbm_ctx {
     long long step = 0;     // step index of the current level
     bool ready = false;     // lbm_init / lbm_set_f / lbm_load done
     unsigned* d_status = nullptr;
-    unsigned* h_status = nullptr;
+    unsigned* h_status = nullptr;  // page-locked, one allocation: the sums, the tau derivative, the status word
     double* d_partials = nullptr;
     unsigned* d_left = nullptr;  // the totals kernel's count of finished CTAs (zero between launches)
     double* h_sums = nullptr;
+    double* h_tau = nullptr;
     void* d_stage = nullptr;
     size_t stage_bytes = 0;
     Model<double> md{};
@@ -53,22 +54,25 @@ struct lbm_ctx {
     // several steps of a small grid per launch (lbm_resident.cu)
     ResPlan res{};
     bool res_ok = false;
-    unsigned* d_res = nullptr;  // its tag counter and leave count, then (256 bytes on) its exchange buffer
+    unsigned* d_res = nullptr;  // its tag counter and leave count
+    ResWord* d_xch = nullptr;   // its exchange buffer (behind f[1], or behind the status words)
     CUtensorMap tmap[2];  // FP32: tensor maps of the two level buffers (tile kernel)
     bool tmap_ok = false;
     // adjoint: checkpoints every ck_every steps from level ck_base
     int ck_every = 0;
     long long ck_base = -1;
     std::vector<void*> ck;       // ck[k] holds level ck_base + k * ck_every (padded, with ghosts)
-    std::vector<void*> seg;      // recomputed levels of one segment
-    void* adj[2] = {nullptr, nullptr};
+    std::vector<void*> ck_mem;   // the allocations they lie in
+    // recomputed levels of one segment: seg_n of them, level_stride() bytes apart
+    char* seg = nullptr;
+    int seg_n = 0;
+    void* adj[2] = {nullptr, nullptr};  // one allocation
     // FP32 tile adjoint: tensor maps of the adjoint levels and, per segment
     // level, of its tile (adjoint) and of its halo box (tile recomputation)
     CUtensorMap adj_tmap[2];
     std::vector<CUtensorMap> seg_tmapF, seg_tmapS;
     bool adj_tmaps_ok = false;
-    double* d_taup = nullptr;
-    double* h_taup = nullptr;
+    double* d_taup = nullptr;    // tau partials, then their sum
     int ntaup = 0;
     void* d_astage = nullptr;    // staging of the adjoint calls' host arguments
     size_t astage_bytes = 0;
@@ -109,6 +113,9 @@ Model<double> build_model(double b, double tau, double dt, double dx, const lbm_
                           const lbm_dissipation& diss);
 size_t nodes(const lbm_ctx* c);
 size_t level_bytes(const lbm_ctx* c);
+// level_bytes rounded up so that levels placed one behind the other start on
+// 256-byte boundaries
+size_t level_stride(const lbm_ctx* c);
 // lbm_create; resident: prepare for several steps per launch where the grid
 // is small enough (a batch steps its problems itself and does without)
 lbm_status create_context(int nx, int ny, double b, double tau, double dt, double dx, const lbm_dvm* dvm,

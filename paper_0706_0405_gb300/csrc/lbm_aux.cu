@@ -486,6 +486,28 @@ cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S
     return cudaGetLastError();
 }
 
+// Sum of n doubles by one CTA: strided partial sums, then a fixed tree.
+__global__ void __launch_bounds__(1024) k_sum(const double* __restrict__ v, int n, double* out) {
+    __shared__ double sh[32];
+    double t = 0.0;
+    for (int k = threadIdx.x; k < n; k += 1024) t += v[k];
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) t += __shfl_down_sync(0xffffffffu, t, s);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x / 32] = t;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        t = sh[threadIdx.x];
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) t += __shfl_down_sync(0xffffffffu, t, s);
+        if (threadIdx.x == 0) *out = t;
+    }
+}
+
+cudaError_t launch_sum(const double* v, int n, double* out, cudaStream_t st) {
+    k_sum<<<1, 1024, 0, st>>>(v, n, out);
+    return cudaGetLastError();
+}
+
 // ----------------------------------------------------------- pack / unpack
 // Interior of a level <-> dense 9 x ny x nx array (kUnpack: dense to level),
 // one population row at a time in the level's order ([row][population]), V

@@ -551,15 +551,13 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
         }
     if (!found) return false;
     best->xch_bytes = 2 * (size_t)best->px * best->py * best->cells * kCellWords<S> * sizeof(ResWord);
-    // resident all at once; sets the kernel's shared-memory limit on this device
-    constexpr auto kern = kernel_of<S, TM>();
-    int per_sm = 0;
-    if (allow_smem<kernel_of<S, TM>()>(kSmemMax<S>) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, best->threads, best->smem) != cudaSuccess) {
+    // one CTA per SM is always resident: the launch bounds and kSmemMax see to
+    // it (a device with fewer SMs free refuses the cooperative launch)
+    if (allow_smem<kernel_of<S, TM>()>(kSmemMax<S>) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return best->px * best->py <= per_sm * sms;
+    return true;
 }
 
 template <typename S, int TM>
