@@ -19,57 +19,117 @@ __device__ __forceinline__ int kind_at(const Grid<S>& G, int side, int along_ind
     return side_part(G, side, along_index, level) ? G.kind_hi[side] : G.kind_lo[side];
 }
 
-// Adjoint of one node (gather form over the transposed star): from f at the
-// node (fv), the adjoint of level n + 1 at the node (av) and at its four star
-// neighbours (aL, aR, aD, aU; zero where the star leaves the grid through a
-// non-periodic side), the adjoint of level n at the node (o) before the ghost
-// links, and the node's tau term tn = sum_i a_i (f^eq_i - f_i).  Both adjoint
-// kernels use it, so they round alike.
-// The collision part: g = (df^eq/df)^T a at the node (through the moments)
-// and the tau term tn.
-template <typename S, int TM>
-__device__ __forceinline__ void adjoint_collision(const Model<S>& M, const S (&fv)[9], const S (&av)[9],
-                                                  S (&g)[9], S& tn) {
-    S rho, ux, uy, T;
-    moments<S, TM>(fv, M, rho, ux, uy, T);
-    S h[4];
+// Transposed collision of one node: from f (fv) and the adjoint of level
+// n + 1 (av) at the node, g = omega (df^eq/df)^T a, and the node's tau term
+// tn = sum_i a_i (f^eq_i - f_i).  FP32: through the moments (rho, u, T).
+template <int TM>
+__device__ __forceinline__ void adjoint_collision(const Model<float>& M, const float (&fv)[9], const float (&av)[9],
+                                                  float (&g)[9], float& tn) {
+    float rho, ux, uy, T;
+    moments<float, TM>(fv, M, rho, ux, uy, T);
+    float h[4];
     feq_vjp(M, rho, ux, uy, T, av, h);
     // tau term: f^eq is linear in rho, so sum_i a_i f^eq_i = rho dF/drho . a
     // = rho h[0]; no equilibrium needs evaluating
-    S af = mul_(av[0], fv[0]);
+    float af = mul_(av[0], fv[0]);
 #pragma unroll
     for (int i = 1; i < 9; ++i) af = fma_(av[i], fv[i], af);
     tn = fma_(rho, h[0], neg_(af));
     moments_vjp(M, rho, ux, uy, T, h, g);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = mul_(M.omega, g[i]);
+}
+
+// FP64, for the fewest instructions of the FP64 pipe.  With the variables of
+// lbm_fp64.cuh -- rho, g = rho u / c1, p = rho T, q = g.U,
+// V = ((b + 2) T + u^2) / c1^2, all functions of the linear sums rho, g and
+// e = (energy) / b -- the contraction L = omega sum_i a_i f^eq_i is
+//   k0 p a0 + A1 S1 + h1 (gx Ux P13 + gy Uy P24) + B1 (gx Q13 + gy Q24)
+//           + A5 S5 + k5 gx Uy D5               + B5 (gx Qp + gy Qm)
+// (P, Q: sums and differences of a over opposite pairs; S, D, Qp, Qm: of
+// those), and its derivatives come out by one backward pass over these few
+// intermediates: 33 operations, and 13 to spread them over the nine
+// populations.  L is homogeneous of degree one in f, so L itself is the
+// derivatives' product with the sums (Euler).  In all 150 instructions a node
+// with the transposed star, where the FP32 form takes about 215 (2048 x 256:
+// 211 -> 152 us a step).  (In FP32 it is no faster, the adjoint kernel there
+// waits on its boxes, and its rounding moves the tau derivative, a sum that
+// nearly cancels, by 1e-4.)
+template <int TM>
+__device__ __forceinline__ void adjoint_collision(const Fp64Adjoint& C, const double (&fv)[9],
+                                                  const double (&av)[9], double (&g)[9], double& tn) {
+    const double ar = fv[7] - fv[5], am = fv[6] - fv[8];
+    const double s14 = (fv[1] + fv[3]) + (fv[2] + fv[4]), s58 = (fv[5] + fv[7]) + (fv[6] + fv[8]);
+    const double rho = (fv[0] + s14) + s58;
+    const double inv = fp64_rcp(rho);
+    const double gx = fma_(C.kap, ar + am, fv[3] - fv[1]), gy = fma_(C.kap, ar - am, fv[4] - fv[2]);
+    const double Ux = gx * inv, Uy = gy * inv;
+    const double qr = fma_(Ux, Ux, Uy * Uy);                                       // q / rho
+    const double T = fma_(-C.t1, qr, fp64_energy(C, fv[0], s14, s58) * inv);
+    const double V = fma_(C.vp, T, qr);
+    const double B1 = fma_(C.b1v, V, C.b1c), B5 = fma_(C.b5v, V, C.b5c);
+    const double P13 = av[1] + av[3], Q13 = av[3] - av[1], P24 = av[2] + av[4], Q24 = av[4] - av[2];
+    const double P57 = av[5] + av[7], Q57 = av[7] - av[5], P68 = av[6] + av[8], Q68 = av[6] - av[8];
+    const double S1 = P13 + P24, S5 = P57 + P68, Qp = Q57 + Q68, Qm = Q57 - Q68;
+    // derivatives (d_x: of L with respect to x), backwards from L
+    const double dV = fma_(C.b1v, fma_(gx, Q13, gy * Q24), C.b5v * fma_(gx, Qp, gy * Qm));
+    const double v = dV * inv;
+    const double de = fma_(C.vp, v, fma_(C.k0, av[0], fma_(C.a1p, S1, C.a5p * S5)));
+    const double dq = fma_(-C.t1, de, v + fma_(C.a1q, S1, C.a5q * S5));
+    const double X = fma_(C.h1, P13, dq), Y = fma_(C.h1, P24, dq), W = C.k5h * (P57 - P68);
+    const double ex = fma_(Ux, X, Uy * W), ey = fma_(Uy, Y, Ux * W);
+    const double dx = fma_(2.0, ex, fma_(B1, Q13, B5 * Qp)), dy = fma_(2.0, ey, fma_(B1, Q24, B5 * Qm));
+    const double dr = fma_(-Ux, ex, fma_(-Uy, ey, fma_(-V, v, fma_(C.a1r, S1, C.a5r * S5))));
+    const double c1 = fma_(C.t1, de, dr), c5 = fma_(C.t2, de, dr), dp = dx + dy, dm = dx - dy;
+    g[0] = fma_(C.te, de, dr);
+    g[1] = c1 - dx;
+    g[2] = c1 - dy;
+    g[3] = c1 + dx;
+    g[4] = c1 + dy;
+    g[5] = fma_(-C.kap, dp, c5);
+    g[7] = fma_(C.kap, dp, c5);
+    g[6] = fma_(C.kap, dm, c5);
+    g[8] = fma_(-C.kap, dm, c5);
+    // L = rho (dr + dx Ux + dy Uy + de e / rho), e / rho = T + t1 q / rho
+    const double L = rho * fma_(dx, Ux, fma_(dy, Uy, fma_(de, fma_(C.t1, qr, T), dr)));
+    double af = av[0] * fv[0];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) af = fma_(av[i], fv[i], af);
+    tn = fma_(L, C.inv_omega, -af);
 }
 
 // Adjoint of population j of one node from the transposed star: its own
 // weight with the collision term, then the nodes left of, right of, below
 // and above it, which read it as their E, W, N and S neighbour.
-template <typename S>
-__device__ __forceinline__ S adjoint_star(const Model<S>& M, int j, S g, S a, S aL, S aR, S aD, S aU) {
-    S r = fma_(M.w[j][0], a, mul_(M.omega, g));
-    r = fma_(M.w[j][1], aL, r);
-    r = fma_(M.w[j][2], aR, r);
-    r = fma_(M.w[j][3], aD, r);
-    return fma_(M.w[j][4], aU, r);
+template <typename C_, typename S>
+__device__ __forceinline__ S adjoint_star(const C_& C, int j, S g, S a, S aL, S aR, S aD, S aU) {
+    S r = fma_(C.w[j][0], a, g);
+    r = fma_(C.w[j][1], aL, r);
+    r = fma_(C.w[j][2], aR, r);
+    r = fma_(C.w[j][3], aD, r);
+    return fma_(C.w[j][4], aU, r);
 }
 
-template <typename S, int TM>
-__device__ __forceinline__ void adjoint_core(const Model<S>& M, const S (&fv)[9], const S (&av)[9],
-                                             const S (&aL)[9], const S (&aR)[9], const S (&aD)[9],
-                                             const S (&aU)[9], S (&o)[9], S& tn) {
+// Adjoint of level n at one node (o) before the ghost links, from f at the
+// node, the adjoint of level n + 1 at the node and at its four star
+// neighbours (aL, aR, aD, aU; zero where the star leaves the grid through a
+// non-periodic side), and the node's tau term.  Both adjoint kernels use it,
+// so they round alike.
+template <typename S, int TM, typename C_>
+__device__ __forceinline__ void adjoint_core(const C_& C, const S (&fv)[9],
+                                             const S (&av)[9], const S (&aL)[9], const S (&aR)[9],
+                                             const S (&aD)[9], const S (&aU)[9], S (&o)[9], S& tn) {
     S g[9];
-    adjoint_collision<S, TM>(M, fv, av, g, tn);
+    adjoint_collision<TM>(C, fv, av, g, tn);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) o[j] = adjoint_star(M, j, g[j], av[j], aL[j], aR[j], aD[j], aU[j]);
+    for (int j = 0; j < 9; ++j) o[j] = adjoint_star(C, j, g[j], av[j], aL[j], aR[j], aD[j], aU[j]);
 }
 
 // Ghost links of an edge node: its own ghost cell on a non-periodic side is
 // made from it (outflow: copied; reflect: mirrored), so the weight that read
 // that ghost comes back to it.  Dirichlet ghosts depend on nothing.
-template <typename S>
-__device__ __forceinline__ void adjoint_ghost_links(const Model<S>& M, const Grid<S>& G, long long level,
+template <typename C_, typename S>
+__device__ __forceinline__ void adjoint_ghost_links(const C_& M, const Grid<S>& G, long long level,
                                                     int ix, int iy, const S (&av)[9], S (&o)[9]) {
     const int kl = ix == 0 ? kind_at(G, S_LEFT, iy, level) : -1;
     const int kr = ix == G.nx - 1 ? kind_at(G, S_RIGHT, iy, level) : -1;
@@ -128,23 +188,34 @@ __device__ __forceinline__ void star_neighbours(const Grid<S>& G, int ix, int iy
     yu = iy < G.ny - 1 ? iy + 1 : (pery ? 0 : -1);
 }
 
-// One adjoint step from level n + 1 back to level n, one thread per node.
-// a: adjoint of level n + 1, abar: adjoint of level n (interior of the
-// padded layout; ghost cells are never read or written).
-// taup[block] += sum over the block's nodes of the node tau terms (per node
-// in the storage precision, across nodes in FP64; the tau derivative is
-// -(dt / tau^2) times the total).
+// One adjoint step from level n + 1 back to level n, one thread per node, 32
+// nodes of the flattened grid per CTA: the FP64 adjoint is bound by the FP64
+// pipe (64 cycles a warp instruction on a quarter of an SM), so a small grid
+// wants its warps spread over all SMs (256 x 8, us a step: 20 with CTAs of
+// eight warps, 9.6 with one).  a: adjoint of level n + 1, abar: adjoint of
+// level n (interior of the padded layout; ghost cells are never read or
+// written).  taup[block] += sum over the block's nodes of the node tau terms
+// (per node in the storage precision, across nodes in FP64; the tau
+// derivative is -(dt / tau^2) times the total).
 template <typename S, int TM>
-__global__ void __launch_bounds__(kThreads) k_adjoint(const S* __restrict__ f, const S* __restrict__ a,
-                                                      S* __restrict__ abar, const Model<S> M,
-                                                      const Grid<S> G, long long level,
-                                                      double* __restrict__ taup) {
-    __shared__ double sh[kThreads / 32];
+__global__ void __launch_bounds__(32) k_adjoint(const S* __restrict__ f, const S* __restrict__ a,
+                                                S* __restrict__ abar, const AdjointModel<S> C,
+                                                const Grid<S> G, long long level, double* __restrict__ taup) {
+    // a programmatic dependent of the previous adjoint step
+    grid_dependency_wait();
+    grid_dependents_launch();
     const long long n = (long long)G.nx * G.ny;
-    const long long q = blockIdx.x * (long long)kThreads + threadIdx.x;
+    const long long q = blockIdx.x * 32LL + threadIdx.x;
     S tsum = S(0);
     if (q < n) {
-        const int iy = (int)(q / G.nx), ix = (int)(q % G.nx);
+        int ix, iy;
+        if (n <= 0xffffffffLL) {
+            iy = (int)((unsigned)q / (unsigned)G.nx);
+            ix = (int)((unsigned)q % (unsigned)G.nx);
+        } else {
+            iy = (int)(q / G.nx);
+            ix = (int)(q % G.nx);
+        }
         const size_t pl = (size_t)G.plane;
         const size_t c = cell(G, ix, iy);
         int xl, xr, yd, yu;
@@ -159,23 +230,16 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const S* __restrict__ f, c
             aD[i] = yd >= 0 ? a[i * pl + cell(G, ix, yd)] : S(0);
             aU[i] = yu >= 0 ? a[i * pl + cell(G, ix, yu)] : S(0);
         }
-        adjoint_core<S, TM>(M, fv, av, aL, aR, aD, aU, o, tsum);
+        adjoint_core<S, TM>(C, fv, av, aL, aR, aD, aU, o, tsum);
         if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1)
-            adjoint_ghost_links(M, G, level, ix, iy, av, o);
+            adjoint_ghost_links(C, G, level, ix, iy, av, o);
 #pragma unroll
         for (int j = 0; j < 9; ++j) abar[j * pl + c] = o[j];
     }
-    // warp sums in the storage precision (fixed shuffle tree), then the
-    // block's eight warp sums in FP64 in a fixed order
+    // the warp's sum in the storage precision (fixed shuffle tree)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tsum += __shfl_down_sync(0xffffffffu, tsum, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x / 32] = (double)tsum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) t += sh[w];
-        taup[blockIdx.x] += t;
-    }
+    if (threadIdx.x == 0) taup[blockIdx.x] += (double)tsum;
 }
 
 // Periodic ghost cells of an adjoint level written by something other than
@@ -207,14 +271,11 @@ __global__ void k_adjoint_wrap(float* __restrict__ a, const Grid<float> G) {
 #ifndef LBM_ADJ_TY
 #define LBM_ADJ_TY 4
 #endif
-#ifndef LBM_ADJ_NPT
-#define LBM_ADJ_NPT 1
-#endif
 #ifndef LBM_ADJ_MIN_BLOCKS
-#define LBM_ADJ_MIN_BLOCKS (LBM_ADJ_NPT == 2 ? 4 : 3)
+#define LBM_ADJ_MIN_BLOCKS 3
 #endif
-constexpr int kAdjTX = 64, kAdjTY = LBM_ADJ_TY, kAdjNpt = LBM_ADJ_NPT;
-constexpr int kAdjThreads = kAdjTX / kAdjNpt * kAdjTY;  // kAdjNpt x-adjacent nodes per thread
+constexpr int kAdjTX = 64, kAdjTY = LBM_ADJ_TY;
+constexpr int kAdjThreads = kAdjTX * kAdjTY;  // one node per thread
 constexpr int kAdjBoxX = kAdjTX + 8, kAdjBoxY = kAdjTY + 2;
 constexpr int kAdjAFloats = kAdjBoxX * kAdjBoxY * 9;
 constexpr int kAdjAPad = (kAdjAFloats + 31) / 32 * 32;  // the f box starts on a 128-byte boundary
@@ -235,8 +296,7 @@ __global__ void __launch_bounds__(kAdjThreads, LBM_ADJ_MIN_BLOCKS)
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + sizeof(float) * 2 * kAdjStageFloats);
     __shared__ int abort_flag;
     __shared__ double wsum_sh[kAdjThreads / 32];
-    constexpr int kLanesX = kAdjTX / kAdjNpt;
-    const int tid = threadIdx.x, tx = tid % kLanesX, ty = tid / kLanesX;
+    const int tid = threadIdx.x, tx = tid % kAdjTX, ty = tid / kAdjTX;
     // launched as a programmatic dependent of the previous adjoint step: no
     // level, adjoint level or tau slot is touched before that grid is done
     grid_dependency_wait();
@@ -296,97 +356,32 @@ __global__ void __launch_bounds__(kAdjThreads, LBM_ADJ_MIN_BLOCKS)
             issued = k + 1;
         }
         float tn = 0.0f;
-        if constexpr (kAdjNpt == 1) {
-            const int ix = tile_x * kAdjTX + tx, iy = tile_y * kAdjTY + ty;
-            if (ix < G.nx && iy < G.ny) {
-                const float* sA = stage0 + (k & 1) * kAdjStageFloats + (ty + 1) * RA + (tx + 4);
-                const float* sF = stage0 + (k & 1) * kAdjStageFloats + kAdjAPad + ty * RF + tx;
-                // the box holds the star of every node: interior neighbours, the
-                // wrapped values in the ghost cells of periodic sides, zeros in
-                // the ghost cells of the others
-                float fv[9], av[9], aL[9], aR[9], aD[9], aU[9], o[9];
+        const int ix = tile_x * kAdjTX + tx, iy = tile_y * kAdjTY + ty;
+        if (ix < G.nx && iy < G.ny) {
+            const float* sA = stage0 + (k & 1) * kAdjStageFloats + (ty + 1) * RA + (tx + 4);
+            const float* sF = stage0 + (k & 1) * kAdjStageFloats + kAdjAPad + ty * RF + tx;
+            // the box holds the star of every node: interior neighbours, the
+            // wrapped values in the ghost cells of periodic sides, zeros in
+            // the ghost cells of the others
+            float fv[9], av[9], aL[9], aR[9], aD[9], aU[9], o[9];
 #pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    const float* pA = sA + i * PA;
-                    fv[i] = sF[i * PF];
-                    av[i] = pA[0];
-                    aL[i] = pA[-1];
-                    aR[i] = pA[1];
-                    aD[i] = pA[-RA];
-                    aU[i] = pA[RA];
-                }
-                adjoint_core<float, TM>(M, fv, av, aL, aR, aD, aU, o, tn);
-                const size_t c = cell(G, ix, iy);
-                if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) {
-                    adjoint_ghost_links(M, G, level, ix, iy, av, o);
-                    write_periodic_ghosts(G, abar, ix, iy, o);
-                }
-#pragma unroll
-                for (int j = 0; j < 9; ++j) abar[j * pl + c] = o[j];
+            for (int i = 0; i < 9; ++i) {
+                const float* pA = sA + i * PA;
+                fv[i] = sF[i * PF];
+                av[i] = pA[0];
+                aL[i] = pA[-1];
+                aR[i] = pA[1];
+                aD[i] = pA[-RA];
+                aU[i] = pA[RA];
             }
-        } else {  // two x-adjacent nodes per thread: 8-byte shared loads and stores
-            const int ix0 = tile_x * kAdjTX + 2 * tx, iy = tile_y * kAdjTY + ty;
-            if (ix0 < G.nx && iy < G.ny) {
-                const int nvalid = min(2, G.nx - ix0);
-                const float* sA = stage0 + (k & 1) * kAdjStageFloats + (ty + 1) * RA + (2 * tx + 4);
-                const float* sF = stage0 + (k & 1) * kAdjStageFloats + kAdjAPad + ty * RF + 2 * tx;
-                float2 A2[9];
-                float g[2][9];
-                float tt[2];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) A2[i] = *reinterpret_cast<const float2*>(sA + i * PA);
-#pragma unroll
-                for (int n = 0; n < 2; ++n) {
-                    float fv[9], av[9];
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        fv[i] = sF[i * PF + n];
-                        av[i] = n ? A2[i].y : A2[i].x;
-                    }
-                    adjoint_collision<float, TM>(M, fv, av, g[n], tt[n]);
-                }
-                // a node past the right edge (odd nx) has f = 0 in the box:
-                // its terms are not used
-                tn = nvalid == 2 ? add_(tt[0], tt[1]) : tt[0];
-                float o[2][9];
-#pragma unroll
-                for (int j = 0; j < 9; ++j) {
-                    const float* pA = sA + j * PA;
-                    const float2 Nn = *reinterpret_cast<const float2*>(pA + RA);
-                    const float2 Ss = *reinterpret_cast<const float2*>(pA - RA);
-                    const float Wv = pA[-1], Ev = pA[2];
-                    o[0][j] = adjoint_star(M, j, g[0][j], A2[j].x, Wv, A2[j].y, Ss.x, Nn.x);
-                    o[1][j] = adjoint_star(M, j, g[1][j], A2[j].y, A2[j].x, Ev, Ss.y, Nn.y);
-                }
-                float* out = abar + cell(G, ix0, iy);  // 8-byte aligned: ix0 + PADX is even
-#pragma unroll
-                for (int j = 0; j < 9; ++j) {
-                    if (nvalid == 2)
-                        *reinterpret_cast<float2*>(out + j * pl) = make_float2(o[0][j], o[1][j]);
-                    else
-                        out[j * pl] = o[0][j];
-                }
-                // edge nodes: the ghost links, on the values just stored (read
-                // back) and the node's adjoint from the box
-                const bool edge_row = iy == 0 || iy == G.ny - 1;
-                if (edge_row || ix0 == 0 || ix0 + nvalid == G.nx) {
-#pragma unroll 1
-                    for (int n = 0; n < nvalid; ++n) {
-                        const int ix = ix0 + n;
-                        if (!(edge_row || ix == 0 || ix == G.nx - 1)) continue;
-                        float av[9], on[9];
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) {
-                            av[i] = sA[i * PA + n];
-                            on[i] = out[i * pl + n];
-                        }
-                        adjoint_ghost_links(M, G, level, ix, iy, av, on);
-                        write_periodic_ghosts(G, abar, ix, iy, on);
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) out[i * pl + n] = on[i];
-                    }
-                }
+            adjoint_core<float, TM>(M, fv, av, aL, aR, aD, aU, o, tn);
+            const size_t c = cell(G, ix, iy);
+            if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) {
+                adjoint_ghost_links(M, G, level, ix, iy, av, o);
+                write_periodic_ghosts(G, abar, ix, iy, o);
             }
+#pragma unroll
+            for (int j = 0; j < 9; ++j) abar[j * pl + c] = o[j];
         }
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) tn += __shfl_down_sync(0xffffffffu, tn, s);
@@ -447,11 +442,18 @@ __global__ void k_feq_vjp(const S* __restrict__ r, const S* __restrict__ ux, con
 }  // namespace
 
 template <typename S, int TM>
-cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const Model<S>& M, const Grid<S>& G,
+cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const AdjointModel<S>& C, const Grid<S>& G,
                            long long level, double* taup, cudaStream_t st) {
-    const long long n = (long long)G.nx * G.ny;
-    k_adjoint<S, TM><<<blocks_for(n, kThreads), kThreads, 0, st>>>(f, a, abar, M, G, level, taup);
-    return cudaGetLastError();
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(blocks_for((long long)G.nx * G.ny, 32));
+    lc.blockDim = dim3(32);
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, k_adjoint<S, TM>, f, a, abar, C, G, level, taup);
 }
 
 template <int TM>
@@ -502,7 +504,7 @@ void adjoint_tile_boxes(int* ax, int* ay, int* fx, int* fy) {
 // tile count).
 template <typename S>
 int adjoint_partials(const Grid<S>& G) {
-    const int simple = (int)blocks_for((long long)G.nx * G.ny, kThreads);
+    const int simple = (int)blocks_for((long long)G.nx * G.ny, 32);
     const int tiles = ((G.nx + kAdjTX - 1) / kAdjTX) * ((G.ny + kAdjTY - 1) / kAdjTY);
     return simple > tiles ? simple : tiles;
 }
@@ -526,8 +528,8 @@ cudaError_t launch_feq_vjp(const S* r, const S* ux, const S* uy, const S* T, con
 }
 
 #define LBM_ADJ_INST(S, TM)                                                                             \
-    template cudaError_t launch_adjoint<S, TM>(const S*, const S*, S*, const Model<S>&, const Grid<S>&, \
-                                               long long, double*, cudaStream_t);                       \
+    template cudaError_t launch_adjoint<S, TM>(const S*, const S*, S*, const AdjointModel<S>&,          \
+                                               const Grid<S>&, long long, double*, cudaStream_t);       \
     template cudaError_t launch_moments_vjp<S, TM>(const S*, const S*, const S*, const S*, const S*, S*, \
                                                    const Model<S>&, const Grid<S>&, cudaStream_t);
 LBM_ADJ_INST(double, T_PLAIN)

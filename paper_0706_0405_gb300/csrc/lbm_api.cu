@@ -299,6 +299,19 @@ template <> const Grid<float>& grid_of<float>(const lbm_ctx* c) { return c->gf; 
 // Whether device_view copies p through the staging buffer.
 bool staged(const void* p) { return p && !is_device_ptr(p) && !pinned_alias(p); }
 
+template <typename S>
+AdjointModel<S> adjoint_model(const lbm_ctx* c) {
+    if constexpr (sizeof(S) == 8) {
+        Fp64Adjoint A;
+        static_cast<Fp64Step&>(A) = c->f64;
+        A.k5h = 0.5 * c->f64.k5;
+        A.inv_omega = c->tau / c->dt;
+        return A;
+    } else {
+        return c->mf;
+    }
+}
+
 // Copy `bytes` from a host or device pointer into the staging buffer at
 // `offset` (returns a device pointer to read from), or pass device pointers
 // through.
@@ -1037,7 +1050,7 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
                 }
                 return launch_adjoint<S, TM>(reinterpret_cast<const S*>(seg_level(l - c0)),
                                              static_cast<const S*>(c->adj[ac]), static_cast<S*>(c->adj[ac ^ 1]),
-                                             model_of<S>(c), grid_of<S>(c), l, c->d_taup, c->stream);
+                                             adjoint_model<S>(c), grid_of<S>(c), l, c->d_taup, c->stream);
             });
             if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step");
             ac ^= 1;

@@ -104,6 +104,12 @@ inline Fp64Step fp64_step(const Model<double>& M, double b_, double tau, double 
     return C;
 }
 
+// The constants of the FP64 adjoint step (adjoint_collision).
+struct Fp64Adjoint : Fp64Step {
+    double k5h;        // k5 / 2
+    double inv_omega;  // tau / dt
+};
+
 // 1 / a: the hardware approximation x (its error e = 1 - a x is about 2^-20)
 // and one step of Newton's iteration carried to third order,
 // x (1 + e + e^2), whose error is e^3.

@@ -150,8 +150,10 @@ cudaError_t launch_unpack(S* f, const S* dense, const Grid<S>& G, cudaStream_t s
 
 // Adjoint (lbm_adjoint.cu).  a, abar: padded layout; taup: one FP64 slot per
 // block (adjoint_partials of them), accumulated across calls.
+template <typename S>
+using AdjointModel = std::conditional_t<sizeof(S) == 8, Fp64Adjoint, Model<float>>;
 template <typename S, int TM>
-cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const Model<S>& M, const Grid<S>& G,
+cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const AdjointModel<S>& C, const Grid<S>& G,
                            long long level, double* taup, cudaStream_t st);
 template <typename S>
 int adjoint_partials(const Grid<S>& G);
