@@ -7,9 +7,17 @@
 // Computations, Sec. 7.5), restricted to what the spectral radius needs: the
 // rotations act only on the active diagonal block, since the eigenvalues do
 // not depend on the blocks outside it.  Compiles for host and device.
+//
+// On the GPU the FP64 pipe bounds it (1/64 of the FP32 rate), comparisons and
+// conversions included, so everything but the rotations themselves is kept
+// off it or short: a rotation is formed with two reciprocal square roots (24
+// instructions; hypot and divisions took about 135, more than applying it to
+// a 9 x 9 matrix's columns), deflation is decided in FP32, and zero tests
+// look at the exponent.
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #ifdef __CUDACC__
 #define LBM_HD __host__ __device__ __forceinline__
@@ -23,37 +31,81 @@ struct cplx {
     double re, im;
 };
 
-LBM_HD cplx cmake(double re, double im) { return cplx{re, im}; }
 LBM_HD cplx cadd(cplx a, cplx b) { return cplx{a.re + b.re, a.im + b.im}; }
 LBM_HD cplx csub(cplx a, cplx b) { return cplx{a.re - b.re, a.im - b.im}; }
 LBM_HD cplx cmul(cplx a, cplx b) { return cplx{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
 LBM_HD cplx cconj(cplx a) { return cplx{a.re, -a.im}; }
 LBM_HD cplx cscale(cplx a, double s) { return cplx{a.re * s, a.im * s}; }
 LBM_HD double cabs2(cplx a) { return a.re * a.re + a.im * a.im; }
-LBM_HD double cabs(cplx a) { return hypot(a.re, a.im); }
-LBM_HD double cabs1(cplx a) { return fabs(a.re) + fabs(a.im); }
 
-// a / b by scaling with the larger component of b (Smith's method).
+// The upper half of a double's bits: its sign, exponent and leading digits.
+LBM_HD int high_bits(double a) {
+#ifdef __CUDA_ARCH__
+    return __double2hiint(a);
+#else
+    long long v;
+    memcpy(&v, &a, sizeof v);
+    return (int)(v >> 32);
+#endif
+}
+
+// |a| rounded towards zero to FP32 by integer operations: 0 below 2^-126,
+// infinite or NaN from 2^128.
+LBM_HD float narrow_abs(double a) {
+    unsigned long long v;
+#ifdef __CUDA_ARCH__
+    v = (unsigned long long)__double_as_longlong(a);
+#else
+    memcpy(&v, &a, sizeof v);
+#endif
+    v &= 0x7fffffffffffffffull;
+    const unsigned long long low = 897ull << 52, high = (896ull + 255ull) << 52;
+    const unsigned bits = v < low ? 0u : v >= high ? 0x7fc00000u : (unsigned)((v - (896ull << 52)) >> 29);
+    float f;
+#ifdef __CUDA_ARCH__
+    f = __uint_as_float(bits);
+#else
+    memcpy(&f, &bits, sizeof f);
+#endif
+    return f;
+}
+LBM_HD float narrow_abs1(cplx a) { return narrow_abs(a.re) + narrow_abs(a.im); }
+
+// A square so small (below about 2^-960) that the number counts as zero; a
+// NaN of either sign does not.
+LBM_HD bool tiny_square(double a2) { return (unsigned)high_bits(a2) < (63u << 20); }
+
+// 1 / sqrt(a), a > 0 and not tiny: the hardware approximation y (its error
+// e = 1 - a y^2 is about 2^-20) and one step of Newton's iteration carried to
+// third order, y (1 + e / 2 + 3 e^2 / 8).
+LBM_HD double rsqrt_pos(double a) {
+#ifdef __CUDA_ARCH__
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = __fma_rn(-(a * y), y, 1.0);
+    return __fma_rn(y * e, __fma_rn(0.375, e, 0.5), y);
+#else
+    return 1.0 / sqrt(a);
+#endif
+}
+
+// a / b as a conj(b) / |b|^2 (b not tiny; the quotients here are of order
+// one, so the squares neither overflow nor lose b).
 LBM_HD cplx cdiv(cplx a, cplx b) {
-    if (fabs(b.re) >= fabs(b.im)) {
-        const double r = b.im / b.re, d = b.re + b.im * r;
-        return cplx{(a.re + a.im * r) / d, (a.im - a.re * r) / d};
-    }
-    const double r = b.re / b.im, d = b.re * r + b.im;
-    return cplx{(a.re * r + a.im) / d, (a.im * r - a.re) / d};
+    const double ri = rsqrt_pos(cabs2(b));
+    return cscale(cmul(a, cconj(b)), ri * ri);
 }
 
 // Principal square root: sqrt(z) = sqrt((|z| + x) / 2) + i sgn(y) sqrt((|z| - x) / 2),
 // with the smaller part formed as y / (2 * larger) to avoid cancellation.
 LBM_HD cplx csqrt_p(cplx z) {
-    if (z.re == 0.0 && z.im == 0.0) return cplx{0.0, 0.0};
-    const double m = cabs(z);
-    if (z.re >= 0.0) {
-        const double t = sqrt(0.5 * (m + z.re));
-        return cplx{t, z.im / (2.0 * t)};
-    }
-    const double t = sqrt(0.5 * (m - z.re));
-    return cplx{fabs(z.im) / (2.0 * t), z.im >= 0.0 ? t : -t};
+    const double m2 = cabs2(z);
+    if (tiny_square(m2)) return cplx{0.0, 0.0};
+    const double m = m2 * rsqrt_pos(m2);
+    const double h = 0.5 * (m + fabs(z.re)), ri = rsqrt_pos(h);
+    const double big = h * ri, small = 0.5 * z.im * ri;
+    if (high_bits(z.re) >= 0) return cplx{big, small};
+    return high_bits(z.im) >= 0 ? cplx{small, big} : cplx{-small, -big};
 }
 
 // Rotation G = [[c, s], [-conj(s), c]] (c real, c^2 + |s|^2 = 1) with
@@ -64,13 +116,13 @@ struct Givens {
 };
 
 LBM_HD Givens givens(cplx x, cplx y) {
-    const double ay = cabs(y);
-    if (ay == 0.0) return Givens{1.0, cplx{0.0, 0.0}};
-    const double ax = cabs(x);
-    if (ax == 0.0) return Givens{0.0, cconj(cscale(y, 1.0 / ay))};  // s = conj(y) / |y|
-    const double r = hypot(ax, ay);
-    const cplx ph = cscale(x, 1.0 / ax);                              // x / |x|
-    return Givens{ax / r, cscale(cmul(ph, cconj(y)), 1.0 / r)};
+    const double y2 = cabs2(y);
+    if (tiny_square(y2)) return Givens{1.0, cplx{0.0, 0.0}};
+    const double x2 = cabs2(x);
+    if (tiny_square(x2)) return Givens{0.0, cconj(cscale(y, rsqrt_pos(y2)))};  // s = conj(y) / |y|
+    const double ri = rsqrt_pos(x2 + y2), xi = rsqrt_pos(x2);
+    // c = |x| / r, s = (x / |x|) conj(y) / r
+    return Givens{x2 * xi * ri, cmul(cscale(x, xi * ri), cconj(y))};
 }
 
 // Rows p, p + 1 of H (n x n, row-major, leading dimension ld), columns
@@ -109,9 +161,9 @@ LBM_HD void hessenberg(cplx* H, int n) {
 // kMaxSweeps sweeps (the unconverged eigenvalues are then NaN).
 LBM_HD int hessenberg_eigenvalues(cplx* H, int n, cplx* ev) {
     constexpr int kMaxSweeps = 60;  // per eigenvalue
-    constexpr double kEps = 2.220446049250313e-16;
-    double anorm = 0.0;
-    for (int k = 0; k < n * n; ++k) anorm = fmax(anorm, cabs1(H[k]));
+    constexpr float kEps = 2.220446049250313e-16f;
+    float anorm = 0.0f;
+    for (int k = 0; k < n * n; ++k) anorm = fmaxf(anorm, narrow_abs1(H[k]));
     int hi = n - 1, its = 0, total = 0;
     while (hi >= 0) {
         if (hi == 0) {
@@ -121,9 +173,9 @@ LBM_HD int hessenberg_eigenvalues(cplx* H, int n, cplx* ev) {
         // smallest l such that the block l..hi has no negligible subdiagonal
         int l = hi;
         while (l > 0) {
-            double s = cabs1(H[(l - 1) * n + l - 1]) + cabs1(H[l * n + l]);
-            if (s == 0.0) s = anorm;
-            if (cabs1(H[l * n + l - 1]) <= kEps * s) {
+            float s = narrow_abs1(H[(l - 1) * n + l - 1]) + narrow_abs1(H[l * n + l]);
+            if (s == 0.0f) s = anorm;
+            if (narrow_abs1(H[l * n + l - 1]) <= kEps * s) {
                 H[l * n + l - 1] = cplx{0.0, 0.0};
                 break;
             }
@@ -144,16 +196,16 @@ LBM_HD int hessenberg_eigenvalues(cplx* H, int n, cplx* ev) {
         const cplx a = H[(hi - 1) * n + hi - 1], b = H[(hi - 1) * n + hi];
         const cplx c = H[hi * n + hi - 1], d = H[hi * n + hi];
         if (its == 10 || its == 20) {
-            mu = cadd(d, cmake(fabs(c.re) + (hi >= 2 ? fabs(H[(hi - 1) * n + hi - 2].re) : 0.0), 0.0));
+            mu = cadd(d, cplx{fabs(c.re) + (hi >= 2 ? fabs(H[(hi - 1) * n + hi - 2].re) : 0.0), 0.0});
         } else {
             // eigenvalue of [[a, b], [c, d]] nearer to d: d - bc / (p + disc),
             // p = (a - d) / 2, disc = sqrt(p^2 + bc) signed to enlarge |p + disc|
             const cplx p = cscale(csub(a, d), 0.5);
             const cplx bc = cmul(b, c);
             cplx disc = csqrt_p(cadd(cmul(p, p), bc));
-            if (p.re * disc.re + p.im * disc.im < 0.0) disc = cscale(disc, -1.0);
+            if (high_bits(p.re * disc.re + p.im * disc.im) < 0) disc = cplx{-disc.re, -disc.im};
             const cplx den = cadd(p, disc);
-            mu = (den.re == 0.0 && den.im == 0.0) ? d : csub(d, cdiv(bc, den));
+            mu = tiny_square(cabs2(den)) ? d : csub(d, cdiv(bc, den));
         }
         // one explicit-shift QR sweep on the block l..hi: H - mu I = Q R, H <- R Q + mu I
         for (int k = l; k <= hi; ++k) H[k * n + k] = csub(H[k * n + k], mu);
@@ -169,6 +221,30 @@ LBM_HD int hessenberg_eigenvalues(cplx* H, int n, cplx* ev) {
         ++total;
     }
     return total;
+}
+
+// Spectral radius of H (n x n, n <= 9, destroyed); NaN if the iteration does
+// not converge.  Entries far from one are scaled by a power of two, so that
+// squares stay in range.
+LBM_HD double spectral_radius(cplx* H, int n) {
+    int m = 0;
+    for (int k = 0; k < n * n; ++k) {
+        const int re = high_bits(H[k].re) & 0x7fffffff, im = high_bits(H[k].im) & 0x7fffffff;
+        m = m > re ? m : re;
+        m = m > im ? m : im;
+    }
+    if (m >= 0x7ff00000) return NAN;
+    const int e = (m >> 20) - 1023;
+    const int shift = e > 60 || e < -60 ? e : 0;
+    if (shift)
+        for (int k = 0; k < n * n; ++k) H[k] = cplx{scalbn(H[k].re, -shift), scalbn(H[k].im, -shift)};
+    hessenberg(H, n);
+    cplx ev[9];
+    if (hessenberg_eigenvalues(H, n, ev) < 0) return NAN;
+    double r2 = 0.0;
+    for (int k = 0; k < n; ++k) r2 = fmax(r2, cabs2(ev[k]));
+    const double r = sqrt(r2);
+    return shift ? scalbn(r, shift) : r;
 }
 
 }  // namespace lbm

@@ -63,12 +63,7 @@ __global__ void __launch_bounds__(kVnThreads)
         H[i * 9 + i].re += w[0] + (w[1] + w[2]) * cx + (w[3] + w[4]) * cy;
         H[i * 9 + i].im += (w[1] - w[2]) * sx + (w[3] - w[4]) * sy;
     }
-    hessenberg(H, 9);
-    cplx ev[9];
-    const int sweeps = hessenberg_eigenvalues(H, 9, ev);
-    double r = 0.0;
-    for (int k = 0; k < 9; ++k) r = fmax(r, cabs(ev[k]));
-    radius[t] = sweeps < 0 ? NAN : r;
+    radius[t] = spectral_radius(H, 9);
 }
 
 // growth[c] = max over the case's directions and wave numbers (NaN if any is NaN).
