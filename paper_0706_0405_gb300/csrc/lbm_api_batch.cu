@@ -278,7 +278,33 @@ lbm_status lbm_batch_create(int nprob, const lbm_problem* probs, lbm_precision p
 lbm_status lbm_batch_init(lbm_batch* b, const void* const* rho, const void* const* ux, const void* const* uy,
                           const void* const* T) {
     if (!b || !rho || !ux || !uy || !T) return bfail(b, LBM_E_INVAL, "lbm_batch_init: NULL argument");
-    for (size_t p = 0; p < b->ctx.size(); ++p) {
+    const void* const* in[4] = {rho, ux, uy, T};
+    const size_t n = b->ctx.size();
+    // arrays that all lie on the device: a launch per kInitProblems problems
+    bool device = true;
+    for (size_t p = 0; p < n && device; ++p)
+        for (int k = 0; k < 4 && device; ++k) device = in[k][p] && is_device_ptr(in[k][p]);
+    if (device) cudaSetDevice(b->device);
+    for (size_t p0 = 0; device && p0 < n; p0 += kInitProblems) {
+        BatchInit args;
+        const size_t p1 = p0 + kInitProblems < n ? p0 + kInitProblems : n;
+        for (size_t p = p0; p < p1; ++p) {
+            for (int k = 0; k < 4; ++k) args.of[p - p0].in[k] = static_cast<const float*>(in[k][p]);
+            args.of[p - p0].status = b->ctx[p]->d_status;
+        }
+        const int t0 = b->tile_base[p0], t1 = p1 < n ? b->tile_base[p1] : b->ntiles;
+        const cudaError_t e = launch_init_batch(args, b->d_probs, b->d_tiles, t0, t1 - t0, (int)p0, b->stream);
+        if (e != cudaSuccess) return bfail(b, LBM_E_CUDA, std::string("lbm_batch_init: ") + cudaGetErrorString(e));
+        for (size_t p = p0; p < p1; ++p) {
+            lbm_ctx* c = b->ctx[p];
+            c->cur = 0;
+            c->step = 0;
+            c->ck_every = 0;
+            c->ck_base = -1;
+            c->ready = true;
+        }
+    }
+    for (size_t p = 0; p < n && !device; ++p) {
         lbm_status s = lbm_init(b->ctx[p], rho[p], ux[p], uy[p], T[p]);
         if (s != LBM_OK) return bfail(b, s, "problem " + std::to_string(p) + ": " + b->ctx[p]->err);
     }

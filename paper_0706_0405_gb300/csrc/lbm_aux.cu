@@ -70,8 +70,41 @@ __device__ __forceinline__ void store_run(float* p, const Run<V>& o, bool wide, 
 // grid with V = 4 against 48 with one node a thread, its index divided, and
 // the ghost cells in a launch of their own.  Latency-bound on small ones,
 // where V = 2 has twice the threads: 256 tubes of 4 rows one after the other
-// 1.7-1.9 ms against 2.1 (V = 4) and 2.4 (two launches each).
+// 1.7-1.9 ms against 2.1 (V = 4) and 2.4 (two launches each); a batch takes
+// k_init_batch.
 constexpr long long kInitWideNodes = 1 << 20;
+// V x-adjacent nodes from (ix, iy) on, and the ghost cells they write.
+template <int V>
+__device__ __forceinline__ void init_run(float* __restrict__ f, const float* __restrict__ rho,
+                                         const float* __restrict__ ux, const float* __restrict__ uy,
+                                         const float* __restrict__ T, const Model<float>& M, const Grid<float>& G,
+                                         bool wide, int ix, int iy) {
+    const int n = min(V, G.nx - ix);
+    const size_t pl = (size_t)G.plane;
+    const size_t q = (size_t)iy * G.nx + ix;
+    const Run<V> r = load_run<V>(rho + q, wide, n), u = load_run<V>(ux + q, wide, n),
+                 w = load_run<V>(uy + q, wide, n), t = load_run<V>(T + q, wide, n);
+    F2 fe[V / 2][9];
+#pragma unroll
+    for (int k = 0; k < V / 2; ++k) equilibrium_scaled<float, F2>(M, r.h[k], u.h[k], w.h[k], t.h[k], fe[k]);
+    float* out = f + cell(G, ix, iy);  // 4 V-byte aligned: ix + PADX is a multiple of V
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        Run<V> o;
+#pragma unroll
+        for (int k = 0; k < V / 2; ++k) o.h[k] = fe[k][i];
+        store_run<V>(out + i * pl, o, n == V, n);
+    }
+    if (ix == 0 || iy == 0 || ix + n == G.nx || iy == G.ny - 1) {
+        for (int j = 0; j < n; ++j) {
+            float v[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = out[i * pl + j];
+            write_ghosts(G, f, ix + j, iy, v, 0);
+        }
+    }
+}
+
 template <int V>
 __global__ void __launch_bounds__(kThreads) k_init32(float* __restrict__ f, const float* __restrict__ rho,
                                                      const float* __restrict__ ux, const float* __restrict__ uy,
@@ -79,32 +112,26 @@ __global__ void __launch_bounds__(kThreads) k_init32(float* __restrict__ f, cons
                                                      const Grid<float> G, bool wide) {
     const int ix = (blockIdx.x * kRowX + threadIdx.x) * V;
     if (ix >= G.nx) return;
-    const int n = min(V, G.nx - ix);
-    const size_t pl = (size_t)G.plane;
-    for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
-        const size_t q = (size_t)iy * G.nx + ix;
-        const Run<V> r = load_run<V>(rho + q, wide, n), u = load_run<V>(ux + q, wide, n),
-                     w = load_run<V>(uy + q, wide, n), t = load_run<V>(T + q, wide, n);
-        F2 fe[V / 2][9];
-#pragma unroll
-        for (int k = 0; k < V / 2; ++k) equilibrium_scaled<float, F2>(M, r.h[k], u.h[k], w.h[k], t.h[k], fe[k]);
-        float* out = f + cell(G, ix, iy);  // 4 V-byte aligned: ix + PADX is a multiple of V
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            Run<V> o;
-#pragma unroll
-            for (int k = 0; k < V / 2; ++k) o.h[k] = fe[k][i];
-            store_run<V>(out + i * pl, o, n == V, n);
-        }
-        if (ix == 0 || iy == 0 || ix + n == G.nx || iy == G.ny - 1) {
-            for (int j = 0; j < n; ++j) {
-                float v[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) v[i] = out[i * pl + j];
-                write_ghosts(G, f, ix + j, iy, v, 0);
-            }
-        }
-    }
+    for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY)
+        init_run<V>(f, rho, ux, uy, T, M, G, wide, ix, iy);
+}
+
+// A batch's problems, one 64 x 4 tile of its tile list a CTA, the arrays'
+// addresses in the launch's parameters: 256 tubes 0.50 ms
+// (the kinds of 1024 addresses looked up by the host), 1.9 with a launch and a
+// clearing of the status word per problem.
+__global__ void __launch_bounds__(128) k_init_batch(const __grid_constant__ BatchInit A,
+                                                    const BatchProb* __restrict__ probs,
+                                                    const int4* __restrict__ tiles, int t0, int p0) {
+    const int4 t = tiles[t0 + blockIdx.x];
+    const BatchProb& P = probs[t.x];
+    const BatchInit::Fields& a = A.of[t.x - p0];
+    if (t.y == 0 && t.z == 0 && threadIdx.x == 0 && threadIdx.y == 0) *a.status = 0u;
+    const int ix = t.y + 2 * threadIdx.x, iy = t.z + threadIdx.y;
+    if (ix >= P.G.nx || iy >= P.G.ny) return;
+    const bool wide = P.G.nx % 2 == 0 && (((uintptr_t)a.in[0] | (uintptr_t)a.in[1] | (uintptr_t)a.in[2] |
+                                           (uintptr_t)a.in[3]) & 7) == 0;
+    init_run<2>(P.f[0], a.in[0], a.in[1], a.in[2], a.in[3], P.M, P.G, wide, ix, iy);
 }
 
 template <int V>
@@ -143,6 +170,12 @@ cudaError_t launch_init(S* f, const S* rho, const S* ux, const S* uy, const S* T
     } else {
         k_init64<<<row_grid(G.nx, G.ny, 1), dim3(kRowX, kRowY), 0, st>>>(f, rho, ux, uy, T, M, G);
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_batch(const BatchInit& args, const BatchProb* probs, const int4* tiles, int t0, int ntiles,
+                              int p0, cudaStream_t st) {
+    k_init_batch<<<ntiles, dim3(32, 4), 0, st>>>(args, probs, tiles, t0, p0);
     return cudaGetLastError();
 }
 

@@ -189,6 +189,18 @@ struct BatchProb {  // 128-byte aligned by its tensor maps
     int wrap;           // batch_wraps_in_tile(G): boxes start at the first interior row
     unsigned box_bytes; // bytes of one box
 };
+// Initial levels (f[0]) of up to kInitProblems consecutive problems from
+// device arrays: the tiles t0 .. t0 + ntiles - 1 of the batch, which are those
+// of the problems from p0 on.  Also clears the problems' status words.
+constexpr int kInitProblems = 100;  // the fields fit in 4 KB of launch parameters
+struct BatchInit {
+    struct Fields {
+        const float* in[4];  // rho, ux, uy, T
+        unsigned* status;
+    } of[kInitProblems];
+};
+cudaError_t launch_init_batch(const BatchInit& args, const BatchProb* probs, const int4* tiles, int t0, int ntiles,
+                              int p0, cudaStream_t st);
 // The problem's height fits in one tile row and its y sides are periodic:
 // the batch kernel takes the wrapped y neighbours from inside the tile.
 bool batch_wraps_in_tile(const Grid<float>& G);
