@@ -1,6 +1,8 @@
 // lbm_api_batch.cu -- the batch calls of the C ABI (include/lbm.h): many
 // problems advanced by one persistent launch, its launch shape and
 // autotuner, the neighbour lists that order its steps, and its test hooks.
+#include <algorithm>
+
 #include "lbm_api_internal.h"
 #include "lbm_batch_plan.h"
 
@@ -24,7 +26,7 @@ struct lbm_batch {
     int nbr_grid = -1;  // grid the lists were made for
     bool nbr_ok = false;
     long long* d_level = nullptr;
-    unsigned* d_bar = nullptr;     // [0] arrivals, [1] generation
+    unsigned* d_bar = nullptr;     // [0] arrivals, [1] generation, [2] strip tickets
     unsigned* d_status = nullptr;
     unsigned* h_status = nullptr;
     long long step = 0;
@@ -38,6 +40,14 @@ struct lbm_batch {
     int4* d_segs = nullptr;
     int nsegs = 0;
     int tb_max_grid[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // per odd steps-per-pass 3, 5, 7
+    // temporal blocking with the columns in registers (lbm_strip.cu): every
+    // problem has strip_rows rows (2 or 4), periodic in y
+    int strip_rows = 0;           // 0: not applicable
+    int strip_max = 0;            // resident CTAs
+    StripWarp* d_strips = nullptr;
+    size_t strip_cap = 0;         // entries it holds
+    int strip_rounds = 0;
+    int strip_ns = 0, strip_grid = 0;  // steps a pass and CTAs the plan was made for
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int graph_n = -1;
@@ -74,10 +84,40 @@ bool batch_neighbour_lists(const lbm_batch* b, int grid, std::vector<int>& out) 
                                  [&](int t) { return batch_tile_owner(t, n, grid); }, kBatchMaxNbr, out);
 }
 
-// Make the neighbour lists match the current grid (outside graph capture:
-// waits for the stream, then copies synchronously).
+// Full wave of a blocking launch, in CTAs of the shared-memory kernel.
+int tb_full(const lbm_batch* b, int ns) {
+    return b->tb_max_grid[ns] < b->nsegs ? b->tb_max_grid[ns] : b->nsegs;
+}
+
+// CTAs of a strip launch: a full wave for a full wave, else the chosen grid or
+// as many of it as are resident.
+int strip_launch_grid(const lbm_batch* b) {
+    return b->grid < b->strip_max && b->grid != tb_full(b, b->block) ? b->grid : b->strip_max;
+}
+
+// Make the strip plan match the current steps a pass and grid.
+cudaError_t batch_prepare_strips(lbm_batch* b) {
+    const int grid = strip_launch_grid(b);
+    if (b->strip_ns == b->block && b->strip_grid == grid) return cudaSuccess;
+    std::vector<int> nx;
+    for (const lbm_ctx* c : b->ctx) nx.push_back(c->gf.nx);
+    std::vector<StripWarp> plan;
+    const int rounds = strip_plan((int)nx.size(), nx.data(), b->block, grid, kStripWarps, plan);
+    if (plan.size() > b->strip_cap) return cudaErrorInvalidValue;
+    cudaError_t e = cudaStreamSynchronize(b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(b->d_strips, plan.data(), sizeof(StripWarp) * plan.size(), cudaMemcpyHostToDevice);
+    b->strip_ns = e == cudaSuccess ? b->block : 0;
+    b->strip_grid = grid;
+    b->strip_rounds = rounds;
+    return e;
+}
+
+// Make the neighbour lists, or the strip plan, match the current launch shape
+// (outside graph capture: waits for the stream, then copies synchronously).
 cudaError_t batch_prepare_sync(lbm_batch* b) {
-    if (b->block > 1 || b->nbr_grid == b->grid) return cudaSuccess;
+    if (b->block > 1) return b->strip_rows ? batch_prepare_strips(b) : cudaSuccess;
+    if (b->nbr_grid == b->grid) return cudaSuccess;
     std::vector<int> lists;
     b->nbr_ok = b->grid <= b->nbr_cap && batch_neighbour_lists(b, b->grid, lists);
     b->nbr_grid = b->grid;
@@ -91,6 +131,10 @@ cudaError_t batch_prepare_sync(lbm_batch* b) {
 cudaError_t batch_launch(lbm_batch* b, int n) {
     auto go = [&](auto tm) {
         constexpr int TM = decltype(tm)::value;
+        if (b->block > 1 && b->strip_rows)
+            return launch_strip<TM>(b->d_probs, b->d_strips, b->strip_rounds, b->strip_rows, n, b->block, b->d_level,
+                                    b->d_bar, b->d_bar + 1, b->d_bar + 2, b->d_status, strip_launch_grid(b),
+                                    b->stream);
         if (b->block > 1)
             return launch_batch_tb<TM>(b->d_probs, b->d_segs, b->nsegs, n, b->block, b->rows_max, b->d_level,
                                        b->d_bar, b->d_bar + 1, b->d_status, b->grid, b->stream);
@@ -127,6 +171,7 @@ void lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->d_done);
     cudaFree(b->d_epoch);
     cudaFree(b->d_segs);
+    cudaFree(b->d_strips);
     cudaFree(b->d_level);
     cudaFree(b->d_bar);
     cudaFree(b->d_status);
@@ -223,7 +268,7 @@ lbm_status lbm_batch_create(int nprob, const lbm_problem* probs, lbm_precision p
     if (e == cudaSuccess) e = dev_malloc((void**)&b->d_tiles, sizeof(int4) * tiles.size());
     if (e == cudaSuccess && b->tb_ok) e = dev_malloc((void**)&b->d_segs, sizeof(int4) * segs.size());
     if (e == cudaSuccess) e = dev_malloc((void**)&b->d_level, sizeof(long long));
-    if (e == cudaSuccess) e = dev_malloc((void**)&b->d_bar, 2 * sizeof(unsigned));
+    if (e == cudaSuccess) e = dev_malloc((void**)&b->d_bar, 3 * sizeof(unsigned));
     if (e == cudaSuccess) e = dev_malloc((void**)&b->d_status, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_status, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->gstream, cudaStreamNonBlocking);
@@ -236,7 +281,7 @@ lbm_status lbm_batch_create(int nprob, const lbm_problem* probs, lbm_precision p
                             b->stream);
     if (e == cudaSuccess && b->tb_ok)
         e = cudaMemcpyAsync(b->d_segs, segs.data(), sizeof(int4) * segs.size(), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, 2 * sizeof(unsigned), b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, 3 * sizeof(unsigned), b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_status, 0, sizeof(unsigned), b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_level, 0, sizeof(long long), b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -271,6 +316,35 @@ lbm_status lbm_batch_create(int nprob, const lbm_problem* probs, lbm_precision p
                                  : prec == LBM_FP32_TDF  ? batch_tb_max_grid<T_DF>(ns, b->rows_max)
                                  : prec == LBM_FP32_CONS ? batch_tb_max_grid<T_CONS>(ns, b->rows_max)
                                                          : batch_tb_max_grid<T_INT32>(ns, b->rows_max);
+    // columns in registers: two or four rows, periodic in y
+    if (b->tb_ok && (b->rows_max == 2 || b->rows_max == 4)) {
+        bool ok = true;
+        std::vector<int> nx;
+        for (int p = 0; p < nprob; ++p) {
+            ok = ok && probs[p].ny == b->rows_max && batch_wraps_in_tile(hp[p].G);
+            nx.push_back(probs[p].nx);
+        }
+        if (ok)
+            b->strip_max = prec == LBM_FP32_T64    ? strip_max_grid<T_INT64>(b->rows_max)
+                           : prec == LBM_FP32_TDF  ? strip_max_grid<T_DF>(b->rows_max)
+                           : prec == LBM_FP32_CONS ? strip_max_grid<T_CONS>(b->rows_max)
+                                                   : strip_max_grid<T_INT32>(b->rows_max);
+        if (b->strip_max > 0) {
+            // a plan has at most as many rounds more than full ones as CTAs
+            std::vector<StripWarp> plan;
+            int rounds = 0;
+            for (int ns = 3; ns <= 7; ns += 2)
+                rounds = std::max(rounds, strip_pack(nprob, nx.data(), ns, kStripWarps, kStripWarps, plan));
+            b->strip_cap = (size_t)(rounds + b->strip_max) * kStripWarps;
+            e = dev_malloc((void**)&b->d_strips, sizeof(StripWarp) * b->strip_cap);
+            if (e != cudaSuccess) {
+                std::string m = std::string("lbm_batch_create: ") + cudaGetErrorString(e);
+                lbm_batch_destroy(b);
+                return bfail(nullptr, e == cudaErrorMemoryAllocation ? LBM_E_NOMEM : LBM_E_CUDA, m);
+            }
+            b->strip_rows = b->rows_max;
+        }
+    }
     *out = b;
     return LBM_OK;
 }
@@ -314,7 +388,7 @@ lbm_status lbm_batch_init(lbm_batch* b, const void* const* rho, const void* cons
     // arrivals that never completed
     if (cudaMemsetAsync(b->d_level, 0, sizeof(long long), b->stream) != cudaSuccess ||
         cudaMemsetAsync(b->d_status, 0, sizeof(unsigned), b->stream) != cudaSuccess ||
-        cudaMemsetAsync(b->d_bar, 0, 2 * sizeof(unsigned), b->stream) != cudaSuccess ||
+        cudaMemsetAsync(b->d_bar, 0, 3 * sizeof(unsigned), b->stream) != cudaSuccess ||
         cudaMemsetAsync(b->d_done, 0, sizeof(unsigned long long) * (size_t)(b->nbr_cap + 1), b->stream) !=
             cudaSuccess ||
         cudaMemsetAsync(b->d_epoch, 0, sizeof(unsigned long long), b->stream) != cudaSuccess)
@@ -434,7 +508,7 @@ lbm_status lbm_batch_set_launch(lbm_batch* b, const lbm_batch_launch* l) {
             return bfail(b, LBM_E_INVAL,
                          "lbm_batch_set_launch: temporal blocking needs problems of at most " +
                              std::to_string(kBatchTbRowsMax) + " rows and no periodic x sides");
-        full = b->tb_max_grid[l->block] < b->nsegs ? b->tb_max_grid[l->block] : b->nsegs;
+        full = tb_full(b, l->block);
         if (full < 1) return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: the blocking kernel does not fit");
     } else {
         if (l->block < 0) return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: block must be 0, 1, 3, 5 or 7");
@@ -449,6 +523,10 @@ lbm_status lbm_batch_set_launch(lbm_batch* b, const lbm_batch_launch* l) {
     b->npt = l->block > 1 ? 1 : l->npt;
     b->grid = l->grid == 0 ? full : l->grid;
     batch_drop_graph(b);
+    if (b->block > 1 && batch_prepare_sync(b) != cudaSuccess) {
+        cudaGetLastError();
+        return bfail(b, LBM_E_CUDA, "lbm_batch_set_launch: copying the plan failed");
+    }
     return LBM_OK;
 }
 
@@ -519,7 +597,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps, lbm_batch_launch* best, d
     }
     if (b->tb_ok)
         for (int ns = 3; ns <= 7; ns += 2) {
-            const int full = b->tb_max_grid[ns] < b->nsegs ? b->tb_max_grid[ns] : b->nsegs;
+            const int full = tb_full(b, ns);
             if (full >= 1) cand[nc++] = {1, full, ns};
         }
     // save every problem's current level, the level counter and the status
@@ -598,6 +676,10 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps, lbm_batch_launch* best, d
     b->grid = cand[bi].grid;
     b->block = cand[bi].block;
     batch_drop_graph(b);
+    if (b->block > 1 && batch_prepare_sync(b) != cudaSuccess) {
+        cudaGetLastError();
+        return bfail(b, LBM_E_CUDA, "lbm_batch_autotune: copying the plan failed");
+    }
     if (best) *best = cand[bi];
     if (n_candidates) *n_candidates = nc;
     return LBM_OK;

@@ -12,6 +12,7 @@
 // each problem's levels are bit-identical to stepping it alone.
 #include <cstddef>
 
+#include "lbm_gridsync.cuh"
 #include "lbm_launch.h"
 #include "lbm_ptx.cuh"
 
@@ -25,50 +26,7 @@ template <int NPT>
 constexpr int batch_threads() {
     return kTileW / NPT * kTileH;
 }
-constexpr long long kBarrierCycles = 4000000000LL;  // ~2 s at 2 GHz, then give up
-// SM cycles an inter-CTA wait (grid barrier, neighbour wait) lasts before it
-// gives up (batch_set_wait_cycles)
-__device__ long long g_wait_cycles = kBarrierCycles;
 constexpr uint32_t kBatchWaitLimit = 1u << 22;       // mbarrier probes before a wait gives up
-
-// Bounded grid-wide barrier for a cooperative launch.  Returns false (and
-// sets ST_TIMEOUT) if the barrier did not complete in time or another CTA
-// has given up (ST_TIMEOUT already set); the decision is the CTA's, taken
-// by one thread and passed on by the CTA barrier, so all its threads leave
-// together.  The stores of
-// the step are ordered before the async-proxy reads (tensor copies) of the
-// next step on both sides: every thread fences after its stores, and the
-// thread that issues the copies fences after the barrier.
-__device__ bool grid_barrier(unsigned* count, volatile unsigned* gen, unsigned* status) {
-    __shared__ int ok;
-    fence_proxy_async_global();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ok = 1;
-        const unsigned g = *gen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(count, 1u);
-        if (arrived == gridDim.x - 1) {
-            *count = 0u;
-            __threadfence();
-            atomicAdd(const_cast<unsigned*>(gen), 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*gen == g) {
-                if (clock64() - t0 > g_wait_cycles || (*(volatile unsigned*)status & ST_TIMEOUT)) {
-                    atomicOr(status, ST_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-        fence_proxy_async_global();
-    }
-    __syncthreads();
-    return ok != 0;
-}
 
 // Point-to-point step ordering between CTAs.  After its last tile of a
 // step, a CTA publishes the step count it has completed (a value that only
@@ -534,7 +492,8 @@ int batch_tile_owner(int t, int ntiles, int grid) {
 }
 
 cudaError_t batch_set_wait_cycles(long long cycles) {
-    return cudaMemcpyToSymbol(g_wait_cycles, &cycles, sizeof(cycles));
+    const cudaError_t e = strip_set_wait_cycles(cycles);
+    return e != cudaSuccess ? e : cudaMemcpyToSymbol(g_wait_cycles, &cycles, sizeof(cycles));
 }
 
 int batch_tile_dims(int* w, int* h) {

@@ -157,6 +157,8 @@ __device__ __forceinline__ float2 lanes(F2 a) {
 }
 __device__ __forceinline__ float lane0(F2 a) { return lanes(a).x; }
 __device__ __forceinline__ float lane1(F2 a) { return lanes(a).y; }
+__device__ __forceinline__ float lane0(float a) { return a; }
+__device__ __forceinline__ double lane0(double a) { return a; }
 __device__ __forceinline__ F2 add2_(F2 a, F2 b) {
     F2 r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
@@ -258,10 +260,13 @@ __device__ __forceinline__ V df_energy(const V (&f)[9], const V (&w)[9]) {
     return add_(hi, lo);
 }
 
+// The node update below takes its constants from a Model<S>, or, for two nodes
+// at once (V = F2), from a Model<F2> that holds every constant in both lanes.
+
 // ---------------------------------------------------------------- moments
 // rho = sum f (Eq. e4), rho u = sum f v (Eq. e5), T from Eq. (e7).
-template <typename S, int TM, typename V = S>
-__device__ __forceinline__ void moments(const V (&f)[9], const Model<S>& M, V& rho, V& ux, V& uy,
+template <typename S, int TM, typename V = S, typename MT>
+__device__ __forceinline__ void moments(const V (&f)[9], const MT& M, V& rho, V& ux, V& uy,
                                         V& T) {
     const V s14 = add_(add_(f[1], f[3]), add_(f[2], f[4]));
     const V s58 = add_(add_(f[5], f[7]), add_(f[6], f[8]));
@@ -302,8 +307,8 @@ __device__ __forceinline__ void moments(const V (&f)[9], const Model<S>& M, V& r
 // Equilibrium of Eqs. (e16)-(e18) times a factor:
 // fe_i = scale (A_i + B_i v.u + D_i (v.u)^2); scale = rho gives f^eq, scale =
 // omega rho gives the relaxation term omega f^eq of the update directly.
-template <typename S, typename V = S>
-__device__ __forceinline__ void equilibrium_scaled(const Model<S>& M, V scale, V ux, V uy, V T, V (&fe)[9]) {
+template <typename S, typename V = S, typename MT>
+__device__ __forceinline__ void equilibrium_scaled(const MT& M, V scale, V ux, V uy, V T, V (&fe)[9]) {
     const V rho = scale;
     const V u2 = fma_(ux, ux, mul_(uy, uy));
     fe[0] = mul_(rho, mul_(M.k0, T));
@@ -334,12 +339,12 @@ __device__ __forceinline__ void equilibrium_scaled(const Model<S>& M, V scale, V
 
 template <typename S>
 __device__ __forceinline__ void equilibrium(const Model<S>& M, S rho, S ux, S uy, S T, S (&fe)[9]) {
-    equilibrium_scaled(M, rho, ux, uy, T, fe);
+    equilibrium_scaled<S, S>(M, rho, ux, uy, T, fe);
 }
 
 // omega f^eq (the relaxation term of Eq. SEC-VON-11 with omega = dt / tau).
-template <typename S, typename V = S>
-__device__ __forceinline__ void omega_equilibrium(const Model<S>& M, V rho, V ux, V uy, V T, V (&ofe)[9]) {
+template <typename S, typename V = S, typename MT>
+__device__ __forceinline__ void omega_equilibrium(const MT& M, V rho, V ux, V uy, V T, V (&ofe)[9]) {
     equilibrium_scaled<S, V>(M, mul_(M.omega, rho), ux, uy, T, ofe);
 }
 
@@ -363,24 +368,24 @@ __device__ __forceinline__ void omega_equilibrium(const Model<S>& M, V rho, V ux
 // Then d carries no mass, momentum or energy (up to its own final roundings,
 // relative to the small increments), as in exact arithmetic, and the
 // collision conserves them (Eqs. e4, e5, e7).
-template <typename S, int TM, typename V = S>
-__device__ __forceinline__ void conserve_increment(const Model<S>& M, V (&d)[9]) {
+template <typename S, int TM, typename V = S, typename MT>
+__device__ __forceinline__ void conserve_increment(const MT& M, V (&d)[9]) {
     if constexpr (moment_exact<TM>()) {
         const V sa = add_(add_(d[1], d[3]), add_(d[2], d[4]));
         const V sd = add_(add_(d[5], d[7]), add_(d[6], d[8]));
         const V djx = fma_(M.c1, sub_(d[3], d[1]), mul_(M.d, sub_(add_(d[6], d[7]), add_(d[5], d[8]))));
         const V djy = fma_(M.c1, sub_(d[4], d[2]), mul_(M.d, sub_(add_(d[7], d[8]), add_(d[5], d[6]))));
         const V gx = mul_(djx, M.h1), gy = mul_(djy, M.h1);
-        if (M.cons_diag == S(0)) {
+        if (lane0(M.cons_diag) == S(0)) {
             const V t = fma_(sd, M.kcons, mul_(sa, S(0.25)));  // -delta_s
-            d[0] = mul_(sd, -M.kzero);
+            d[0] = mul_(sd, neg_(M.kzero));
             d[1] = sub_(add_(d[1], gx), t);
             d[3] = sub_(sub_(d[3], gx), t);
             d[2] = sub_(add_(d[2], gy), t);
             d[4] = sub_(sub_(d[4], gy), t);
         } else {
             const V t = fma_(sa, M.kcons, mul_(sd, S(0.25)));
-            d[0] = mul_(sa, -M.kzero);
+            d[0] = mul_(sa, neg_(M.kzero));
             d[1] = add_(d[1], gx);
             d[3] = sub_(d[3], gx);
             d[2] = add_(d[2], gy);
@@ -394,13 +399,13 @@ __device__ __forceinline__ void conserve_increment(const Model<S>& M, V (&d)[9])
 // The relaxation term of Eq. (SEC-VON-11) at a node, in the form update()
 // takes it.  FP32 (increment form): r_i = omega (f^eq_i - f_i), moment-exact
 // in the modes that ask for it.  FP64: r_i = omega f^eq_i.
-template <typename S, int TM, typename V = S>
-__device__ __forceinline__ void relaxation(const Model<S>& M, const V (&f)[9], V rho, V ux, V uy, V T,
+template <typename S, int TM, typename V = S, typename MT>
+__device__ __forceinline__ void relaxation(const MT& M, const V (&f)[9], V rho, V ux, V uy, V T,
                                            V (&r)[9]) {
     omega_equilibrium<S, V>(M, rho, ux, uy, T, r);
     if constexpr (std::is_same<S, float>::value) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) r[i] = fma_(-M.omega, f[i], r[i]);
+        for (int i = 0; i < 9; ++i) r[i] = fma_(neg_(M.omega), f[i], r[i]);
         conserve_increment<S, TM, V>(M, r);
     }
 }
@@ -412,9 +417,9 @@ __device__ __forceinline__ void relaxation(const Model<S>& M, const V (&f)[9], V
 // whose increment rounds away keeps its bits (a uniform state stays put
 // instead of drifting by the roundings of a full recomputation every step).
 // FP64: f' = w0 c + w1 e + w2 w + w3 n + w4 s + r.
-template <typename S, typename V = S>
-__device__ __forceinline__ V update(const Model<S>& M, int i, V r, V c, V e, V w, V n, V s) {
-    if constexpr (std::is_same<S, float>::value) {
+template <typename V, typename MT>
+__device__ __forceinline__ V update(const MT& M, int i, V r, V c, V e, V w, V n, V s) {
+    if constexpr (!std::is_same<V, double>::value) {
         V acc = fma_(M.wi[i], c, r);
         acc = fma_(M.w[i][1], e, acc);
         acc = fma_(M.w[i][2], w, acc);
@@ -604,7 +609,7 @@ __device__ __forceinline__ unsigned pair_update(const Model<float>& M, const flo
             Nn.v = *reinterpret_cast<const unsigned long long*>(bp + dn);
             Ss.v = *reinterpret_cast<const unsigned long long*>(bp + ds);
             const F2 Ev = pair(lane1(C[i]), bp[2]), Wv = pair(bp[-1], lane0(C[i]));
-            o[i] = lanes(update<float, F2>(M, i, acc[i], C[i], Ev, Wv, Nn, Ss));
+            o[i] = lanes(update(M, i, acc[i], C[i], Ev, Wv, Nn, Ss));
         }
     } else {
         float2 C[9];

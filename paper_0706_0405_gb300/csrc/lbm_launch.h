@@ -242,6 +242,19 @@ cudaError_t launch_batch_tb(const BatchProb* probs, const int4* segs, int nsegs,
 template <int TM>
 int batch_tb_max_grid(int ns, int rows_max);
 
+// Temporal blocking for problems of two or four rows, periodic in y and not in
+// x (lbm_strip.cu): the populations of a column in registers, `warps` holds
+// `rounds` rounds of kStripWarps entries (strip_plan), one CTA's work at a time.
+constexpr int kStripWarps = 4;
+struct StripWarp;
+template <int TM>
+cudaError_t launch_strip(const BatchProb* probs, const StripWarp* warps, int rounds, int rows, int nsteps, int ns,
+                         long long* level, unsigned* bar_count, unsigned* bar_gen, unsigned* ticket, unsigned* status,
+                         int grid, cudaStream_t st);
+template <int TM>
+int strip_max_grid(int rows);
+cudaError_t strip_set_wait_cycles(long long cycles);
+
 // von Neumann scan (lbm_vonneumann.cu): one case is the step's constants
 // (folded weights, omega, equilibrium coefficients) and a uniform state.
 struct VnCase {
