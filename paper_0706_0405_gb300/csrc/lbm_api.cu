@@ -451,10 +451,13 @@ cudaError_t step_resident(lbm_ctx* c, int n, const char* fin, char* seg, long lo
             A.out_odd = reinterpret_cast<S*>(seg + 2 * stride);
             A.out_stride = (long long)(2 * stride / sizeof(S));
             A.write_from = 0;
+            A.first = c->res.depth;  // (no level goes to fin)
         } else {
             A.out_even = static_cast<S*>(c->f[c->cur ^ 1]);
             A.out_odd = static_cast<S*>(c->f[c->cur]);
             A.write_from = n - 2;
+            const int back = n % 2 ? n - 2 : n - 1;  // the odd step that writes to fin
+            A.first = back < c->res.depth ? back : c->res.depth;
         }
         A.nsteps = n;
         A.level0 = level;

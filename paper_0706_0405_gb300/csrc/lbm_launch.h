@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "lbm_device.cuh"
+#include "lbm_resident_plan.h"
 #include "lbm_fp64.cuh"
 
 namespace lbm {
@@ -79,15 +80,6 @@ cudaError_t launch_step(const S* fin, S* fout, const Model<S>& M, const Grid<S>&
                         long long level, unsigned* status, cudaStream_t st, const StepConfig& cfg);
 
 // Several steps of a small grid in one cooperative launch (lbm_resident.cu).
-struct ResPlan {
-    int px, py;        // CTAs along x and y
-    int bw, bh;        // nodes of a tile (the last ones along x, y may be smaller)
-    int pitch;         // columns per population row of a tile in shared memory
-    int cells;         // cells a CTA publishes: 2 bw + 2 bh
-    int threads;       // per CTA
-    size_t smem;       // dynamic shared memory
-    size_t xch_bytes;  // exchange buffer, zeroed by its owner before the first launch
-};
 struct alignas(16) ResWord {
     unsigned long long lo, hi;  // three 32-bit values, then the tag
 };
@@ -99,6 +91,8 @@ struct ResRun {
     S *out_even, *out_odd;
     long long out_stride;
     int write_from, nsteps;
+    int first;                   // steps to the first exchange, 1 .. depth: the CTAs that read a tile's
+                                 // nodes from fin must have done so before the tile overwrites them
     long long level0;
     ResWord* xch;                // exchange buffer
     unsigned* sync;              // tag counter, count of CTAs that have left (both zero at first)

@@ -8,15 +8,20 @@
 // a fixed tile, keeps its level in shared memory for all the steps and
 // exchanges only the tile's edge nodes with the CTAs next to it.  Measured, us
 // a step, launch a step -> here (FP32_TDF / FP32_CONS / FP32_T64): 400 x 4
-// 5.3 -> 1.3 / 3.6 -> 1.2 / 4.5 -> 1.6, 2000 x 4 5.4 -> 1.3 / 3.7 -> 1.2 /
-// 4.5 -> 1.6, 400 x 100 6.1 -> 1.9 / 4.7 -> 1.7 / 5.8 -> 2.4, 1024 x 256
-// 8.8 -> 4.5 / 7.3 -> 3.8 / 11.4 -> 6.8; FP64: 400 x 4 6.1 -> 3.1,
-// 2000 x 4 6.0 -> 4.0.  A small tile's step is a chain of latencies: the node
+// 5.3 -> 1.0 / 3.6 -> 0.9 / 4.5 -> 1.3, 2000 x 4 5.4 -> 1.0 / 3.7 -> 0.9 /
+// 4.5 -> 1.4, 400 x 100 6.1 -> 1.8 / 4.7 -> 1.7 / 5.8 -> 2.4, 1024 x 256
+// 8.8 -> 4.3 / 7.3 -> 3.8 / 11.4 -> 6.7; FP64: 400 x 4 6.1 -> 2.6,
+// 2000 x 4 6.0 -> 3.6.  A small tile's step is a chain of latencies: the node
 // update 950 cycles, the exchange about 1300 (of which 1000 from one CTA's
 // store to another's poll, measured between neighbours among 50 to 125 CTAs),
 // barriers 150; a large one's is issue- and shared-memory-bound.
-//  * two copies of the tile with a one-cell halo, [row][population][column]
-//    like a level; a step reads one and writes the other;
+//  * two copies of the tile with a halo, [row][population][column] like a
+//    level; a step reads one and writes the other;
+//  * tiles that span the grid's height keep a halo of up to four columns and
+//    exchange every fourth step only, updating the columns of the halo that
+//    later steps need in between (lbm_resident_plan.h has the index
+//    arithmetic); where such a grid is periodic in y, a node at its bottom or
+//    top finds the row around the edge in the tile, without ghost cells;
 //  * a step is: the threads update the tile's nodes, its edge nodes first,
 //    and publish the edge nodes' values from registers as they go; the
 //    last warps poll the halo cells, one cell (nine values) a thread, while
@@ -25,13 +30,12 @@
 //    any.  (Publishing in a phase of its own after a barrier cost 0.35 us a
 //    step; ghost rules and polls in the edge nodes' own threads up to 3600
 //    cycles, where the node update takes 900);
-//  * edge values travel as 128-bit words of three 32-bit values and the step
-//    they belong to (FP64: one value), written and polled with relaxed
-//    GPU-scope accesses.  The tag makes a word its own flag: no fence, no
-//    second round trip.  Slots
-//    alternate by the step's parity: a CTA publishes step t + 2 only after it
-//    has received its neighbours' t + 1, which they publish after a barrier
-//    that follows their reads of t.  Tags come from a counter in device memory
+//  * edge values travel as 128-bit words of three 32-bit values and the
+//    exchange they belong to (FP64: one value), written and polled with
+//    relaxed GPU-scope accesses.  The tag makes a word its own flag: no fence,
+//    no second round trip.  Slots alternate by the exchange's parity: a CTA
+//    publishes exchange t + 2 only after it has received its neighbours'
+//    t + 1, which they publish after a barrier that follows their reads of t.  Tags come from a counter in device memory
 //    that only grows, advanced by the last CTA to leave, so replays of a
 //    captured launch work;
 //  * the place of a moving split (the double Mach reflection's top boundary)
@@ -47,7 +51,7 @@ namespace lbm {
 
 namespace {
 constexpr long long kPollCycles = 4000000000LL;  // ~2 s, then a poll gives up
-constexpr int kPadL = 2;                         // columns left of the tile in shared memory (pairs stay aligned)
+constexpr int kMaxDepth = 4;                     // steps between exchanges at most
 
 __device__ __forceinline__ void st_word(ResWord* p, unsigned a, unsigned b, unsigned c, unsigned tag) {
     asm volatile(
@@ -71,26 +75,18 @@ __device__ __forceinline__ unsigned word_tag(const ResWord& w) { return (unsigne
 template <typename S>
 constexpr int kCellWords = sizeof(S) == 4 ? 3 : 9;
 
-constexpr unsigned kNoCell = 0xffffu;
-// The exchange cell of node (lx, ly) of a tile of w x h nodes: the bottom
-// row, the top row, the left and the right column, where there are CTAs on
-// that axis.
-__host__ __device__ __forceinline__ unsigned cell_id(const ResPlan& R, int lx, int ly, int w, int h) {
-    if (R.py > 1) {
-        if (ly == 0) return lx;
-        if (ly == h - 1) return R.bw + lx;
-    }
-    if (R.px > 1) {
-        if (lx == 0) return 2 * R.bw + ly;
-        if (lx == w - 1) return 2 * R.bw + R.bh + ly;
-    }
-    return kNoCell;
-}
+// A node's entry in the table of the nodes to update: its place in the tile,
+// its exchange cell, and whether the row above (below) it is the bottom (top)
+// one of a tile that wraps around.
+constexpr unsigned kWrapUp = 1u << 30, kWrapDown = 1u << 31;
+__device__ __forceinline__ int item_place(unsigned e) { return (int)(e & 0xffffu); }
+__device__ __forceinline__ unsigned item_cell(unsigned e) { return e >> 16 & kNoCell; }
 
 // Values of one node after a step, FP32 modes, from the box b (populations P
-// apart, rows 9 P).
+// apart, the rows above and below dn and ds away).
 template <int TM>
-__device__ __forceinline__ unsigned node_update(const Model<float>& M, const float* b, int P, float (&o)[9]) {
+__device__ __forceinline__ unsigned node_update(const Model<float>& M, const float* b, int P, int dn, int ds,
+                                                float (&o)[9]) {
     float f[9], rho, ux, uy, T;
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = b[i * P];
@@ -99,7 +95,7 @@ __device__ __forceinline__ unsigned node_update(const Model<float>& M, const flo
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const float* p = b + i * P;
-        o[i] = update(M, i, o[i], f[i], p[1], p[-1], p[9 * P], p[-9 * P]);
+        o[i] = update(M, i, o[i], f[i], p[1], p[-1], p[dn], p[ds]);
     }
     return health(rho, ux, uy, T);
 }
@@ -116,13 +112,15 @@ __device__ __forceinline__ unsigned node_update(const Model<float>& M, const flo
 // fp64_relaxation and fp64_update, so the bits are too.
 constexpr int kQuadGroups = 3;  // 32-node groups per CTA at most
 __device__ __forceinline__ unsigned quad_update(const Fp64Step& C, const double* cur, double* nxt,
-                                                const unsigned* item, int n_items, int P) {
+                                                const unsigned* item, int n_items, int P, int around) {
     __shared__ double pairs[kQuadGroups][8][32];  // differences (0..3) and sums (4..7) of the warps' pairs
     __shared__ double mom[kQuadGroups][5][32];    // 1 / rho, rho, gx, gy, E / b
     const int lane = threadIdx.x & 31, role = threadIdx.x / 32 & 3, group = threadIdx.x / 128;
     const int q = group * 32 + lane;
     const bool in = q < n_items;
-    const int at = (int)(item[in ? q : 0] & 0xffffu);
+    const unsigned it = item[in ? q : 0];
+    const int at = item_place(it);
+    const int dn = it & kWrapUp ? -around : 9 * P, ds = it & kWrapDown ? around : -9 * P;
     const double* b = cur + at;
     // the pair's populations against and along its direction
     const int lo = role == 0 ? 1 : role == 1 ? 2 : role == 2 ? 5 : 8, hi = role == 0 ? 3 : role == 1 ? 4 : role == 2 ? 7 : 6;
@@ -164,7 +162,7 @@ __device__ __forceinline__ unsigned quad_update(const Fp64Step& C, const double*
     if (!in) return 0u;
     auto store = [&](int i, double r, double c) {
         const double* n = b + i * P;
-        nxt[at + i * P] = fp64_update(C, i, r, c, n[1], n[-1], n[9 * P], n[-9 * P]);
+        nxt[at + i * P] = fp64_update(C, i, r, c, n[1], n[-1], n[dn], n[ds]);
     };
     store(lo, __fma_rn(-B, g, sum), fl);
     store(hi, __fma_rn(B, g, sum), fh);
@@ -259,106 +257,71 @@ __global__ void __launch_bounds__(kThreads, 1)
                const __grid_constant__ ResRun<S> A) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int P = R.pitch, RS = 9 * R.pitch;
-    const int T = blockDim.x, tid = threadIdx.x;
-    const int cta = blockIdx.x, bx = cta % R.px, by = cta / R.px;
-    const int x0 = bx * R.bw, y0 = by * R.bh;
-    const int w = min(R.bw, G.nx - x0), h = min(R.bh, G.ny - y0);
-    const size_t buf = (size_t)(R.bh + 2) * RS;
+    const int T = blockDim.x, tid = threadIdx.x, cta = blockIdx.x;
+    const bool perx = G.kind_lo[S_LEFT] == BC_PERIODIC, pery = G.kind_lo[S_BOTTOM] == BC_PERIODIC;
+    const ResTile t = res_tile(R, G.nx, G.ny, perx, pery, cta);
+    const int x0 = t.x0, y0 = t.y0, w = t.w, h = t.h;
+    const int pad_x = res_pad_x(R), pad_y = res_pad_y(R);
+    const size_t buf = (size_t)(R.bh + 2 * pad_y) * RS;
     S* cur = reinterpret_cast<S*>(smem);
     S* nxt = cur + buf;
     // tables: per ghost cell its place, its source's, its side and along-side
-    // index; per halo cell its source's cell; per node its place and the cell
-    // it is published as; per halo cell its place
+    // index; per received cell its source's; per node its place and the cell
+    // it is published as; per received cell its place
+    const ResTile full = res_full_tile(R);
+    const int max_halo = res_nodes(full, R.depth) - R.bw * R.bh;
     uint2* ghost = reinterpret_cast<uint2*>(nxt + buf);
-    unsigned* halo_src = reinterpret_cast<unsigned*>(ghost + R.cells);
-    unsigned* item = halo_src + R.cells;
-    unsigned short* halo_dst = reinterpret_cast<unsigned short*>(item + R.bw * R.bh);
+    unsigned* halo_src = reinterpret_cast<unsigned*>(ghost + res_max_ghosts(R));
+    unsigned* item = halo_src + max_halo;
+    unsigned short* halo_dst = reinterpret_cast<unsigned short*>(item + res_nodes(full, R.depth - 1));
     __shared__ int split_now[2][4];  // by the step's parity
-    const int origin = RS + kPadL;  // node (0, 0), population 0, in a buffer
+    __shared__ int upto[kMaxDepth];  // nodes of the core and the shells up to d
+    const int origin = pad_y * RS + pad_x;  // node (0, 0), population 0, in a buffer
     const unsigned epoch = *(volatile unsigned*)A.sync;
     const size_t pl = (size_t)G.plane;
 
-    // neighbours: CTA index, -1 at a physical side or where the tile meets itself
-    const bool perx = G.kind_lo[S_LEFT] == BC_PERIODIC, pery = G.kind_lo[S_BOTTOM] == BC_PERIODIC;
-    const int west = bx > 0 ? cta - 1 : (perx && R.px > 1 ? cta + R.px - 1 : -1);
-    const int east = bx < R.px - 1 ? cta + 1 : (perx && R.px > 1 ? cta - (R.px - 1) : -1);
-    const int south = by > 0 ? cta - R.px : (pery && R.py > 1 ? cta + (R.py - 1) * R.px : -1);
-    const int north = by < R.py - 1 ? cta + R.px : (pery && R.py > 1 ? cta - (R.py - 1) * R.px : -1);
-
-    // the tile's nodes in the order of their update: those that are published
-    // first (bottom and top row, left and right column, on the axes with other
-    // CTAs), so that few warps publish, then the rest row by row
-    const int n_items = w * h;
-    const int ey = R.py > 1, ex = R.px > 1;
-    const int n_rows = ey ? w * min(h, 2) : 0, rest_h = ey ? max(h - 2, 0) : h;
-    const int n_cols = ex ? rest_h * min(w, 2) : 0, rest_w = ex ? w - 2 : w;
-    const int n_edge = n_rows + n_cols;
+    const bool wraps = res_wraps(R, pery);
+    const int around = (h - 1) * RS;  // from the bottom row to the top row
+    const int n_core = w * h, n_edge = res_edges(R, t), n_items = res_nodes(t, R.depth - 1);
     for (int q = tid; q < n_items; q += T) {
-        int r, c, k = q;
-        if (k < n_rows) {
-            r = k < w ? 0 : h - 1;
-            c = k < w ? k : k - w;
-        } else if ((k -= n_rows) < n_cols) {
-            r = ey + k % rest_h;
-            c = k < rest_h ? 0 : w - 1;
-        } else {
-            k -= n_cols;
-            r = ey + k / rest_w;
-            c = ex + k % rest_w;
-        }
-        item[q] = (unsigned)(origin + r * RS + c) | cell_id(R, c, r, w, h) << 16;
+        int c, r;
+        if (q < n_core)
+            res_core_node(R, t, q, &c, &r);
+        else
+            res_shell_node(t, q - n_core, &c, &r);
+        item[q] = (unsigned)(origin + r * RS + c) | (q < n_edge ? res_cell(R, t, c, r) : kNoCell) << 16 |
+                  (wraps && r == h - 1 ? kWrapUp : 0u) | (wraps && r == 0 ? kWrapDown : 0u);
     }
-    // halo cells that come from other CTAs: west and east columns, south and
-    // north rows
-    const int n_w = west >= 0 ? h : 0, n_e = east >= 0 ? h : 0, n_s = south >= 0 ? w : 0, n_n = north >= 0 ? w : 0;
-    const int n_halo = n_w + n_e + n_s + n_n;
+    const int n_halo = R.cells > 0 ? res_nodes(t, R.depth) - n_core : 0;
     for (int q = tid; q < n_halo; q += T) {
-        int k = q, from, dst;
-        const int side = k < n_w ? S_LEFT : (k -= n_w) < n_e ? S_RIGHT : (k -= n_e) < n_s ? S_BOTTOM : S_TOP;
-        if (side == S_LEFT) {
-            from = west, dst = origin + k * RS - 1;
-        } else if (side == S_RIGHT) {
-            from = east, dst = origin + k * RS + w;
-        } else if (side == S_BOTTOM) {
-            from = south, dst = origin - RS + k;
-        } else {
-            k -= n_s;
-            from = north, dst = origin + h * RS + k;
-        }
-        // the node in the other CTA's tile
-        const int fw = min(R.bw, G.nx - from % R.px * R.bw), fh = min(R.bh, G.ny - from / R.px * R.bh);
-        const int lx = side == S_LEFT ? fw - 1 : side == S_RIGHT ? 0 : k;
-        const int ly = side == S_BOTTOM ? fh - 1 : side == S_TOP ? 0 : k;
-        halo_src[q] = (unsigned)(from * R.cells) + cell_id(R, lx, ly, fw, fh);
-        halo_dst[q] = (unsigned short)dst;
+        int c, r;
+        res_shell_node(t, q, &c, &r);
+        unsigned cell;
+        const int from = res_owner(R, G.nx, G.ny, perx, pery, t, c, r, &cell);
+        halo_src[q] = (unsigned)(from * R.cells) + cell;
+        halo_dst[q] = (unsigned short)(origin + r * RS + c);
     }
-    // ghost cells inside the tile: of physical sides, and of periodic sides
-    // whose two ends the tile holds
-    const int g_w = x0 == 0 && west < 0 ? h : 0, g_e = x0 + w == G.nx && east < 0 ? h : 0;
-    const int g_s = y0 == 0 && south < 0 ? w : 0, g_n = y0 + h == G.ny && north < 0 ? w : 0;
-    const int n_ghost = g_w + g_e + g_s + g_n;
+    const ResGhosts ghosts = res_ghosts(R, G.nx, G.ny, perx, pery, t);
+    const int n_ghost = ghosts.w + ghosts.e + ghosts.s + ghosts.n;
     for (int q = tid; q < n_ghost; q += T) {
-        int k = q, side, dst, src, along;
-        if (k < g_w) {
-            side = S_LEFT, dst = origin + k * RS - 1, src = perx ? dst + w : dst + 1, along = y0 + k;
-        } else if ((k -= g_w) < g_e) {
-            side = S_RIGHT, dst = origin + k * RS + w, src = perx ? dst - w : dst - 1, along = y0 + k;
-        } else if ((k -= g_e) < g_s) {
-            side = S_BOTTOM, dst = origin - RS + k, src = pery ? dst + h * RS : dst + RS, along = x0 + k;
-        } else {
-            k -= g_s;
-            side = S_TOP, dst = origin + h * RS + k, src = pery ? dst - h * RS : dst - RS, along = x0 + k;
-        }
-        ghost[q] = make_uint2((unsigned)dst | (unsigned)src << 16, (unsigned)side | (unsigned)along << 2);
+        const ResGhost g = res_ghost(ghosts, G.nx, G.ny, perx, pery, t, q);
+        const int dst = origin + g.r * RS + g.c, src = origin + g.sr * RS + g.sc;
+        ghost[q] = make_uint2((unsigned)dst | (unsigned)src << 16, (unsigned)g.side | (unsigned)g.along << 2);
     }
+    if (tid < R.depth) upto[tid] = res_nodes(t, tid);
     if (tid < 4) split_now[0][tid] = split_at(G, tid, A.level0 + 1);
-    // the tile and its halo, ghost cells of the level included
+    // the tile, ghost cells of the level included
     {
-        const int cols = w + 2, per = 9 * cols, n = (h + 2) * per;
+        const int c0 = -min(t.l + 1, pad_x), c1 = min(w + t.r, w + pad_x - 1);
+        const int r0 = -min(t.b + 1, pad_y), r1 = min(h + t.t, h + pad_y - 1);
+        const int cols = c1 - c0 + 1, per = 9 * cols, n = (r1 - r0 + 1) * per;
         for (int q = tid; q < n; q += T) {
-            const int r = q / per, k = q - r * per, i = k / cols, c = k - i * cols;
-            cur[r * RS + i * P + (kPadL - 1) + c] =
-                A.fin[(size_t)(y0 + r) * (size_t)G.row + i * pl + (size_t)(x0 + c + PADX - 1)];
+            const int j = q / per, k = q - j * per, i = k / cols, c = c0 + k - i * cols, r = r0 + j;
+            int gx = x0 + c, gy = y0 + r;
+            if (R.px > 1 && perx) gx = (gx + G.nx * R.depth) % G.nx;
+            if (R.py > 1 && pery) gy = (gy + G.ny * R.depth) % G.ny;
+            cur[origin + r * RS + i * P + c] =
+                A.fin[(size_t)(gy + 1) * (size_t)G.row + i * pl + (size_t)(gx + PADX)];
         }
     }
     __syncthreads();
@@ -374,35 +337,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int split_tid = sizeof(S) == 4 ? tid - T1 : tid;
     unsigned bits = 0;
     bool ok = true;
-    for (int s = 0; s < A.nsteps; ++s) {
-        const unsigned tag = epoch + (unsigned)s + 1u;
+    // j: the step's place since the last exchange, round: exchanges so far
+    for (int s = 0, j = R.depth - A.first, round = 0; s < A.nsteps; ++s) {
+        const unsigned tag = epoch + (unsigned)round + 1u;
         const bool more = s + 1 < A.nsteps, keep = s >= A.write_from;
+        const bool publish = more && j == R.depth - 1;
+        // steps from here to the next exchange, or to the end, this one included
+        const int n_now = upto[min(R.depth - j, A.nsteps - s) - 1];
         const ResWord* in_box = A.xch + (tag & 1u) * slot_cells * Q;
-        ResWord* out_box = more ? A.xch + ((tag & 1u) * slot_cells + (size_t)cta * R.cells) * Q : nullptr;
+        ResWord* out_box = publish ? A.xch + ((tag & 1u) * slot_cells + (size_t)cta * R.cells) * Q : nullptr;
         if (more && split_tid >= 0 && split_tid < 4)
             split_now[(s + 1) & 1][split_tid] = split_at(G, split_tid, A.level0 + s + 2);
         if constexpr (sizeof(S) == 8) {
-            bits |= quad_update(M, cur, nxt, item, n_items, P);
+            bits |= quad_update(M, cur, nxt, item, n_now, P, around);
             __syncthreads();  // a node's values come from four warps
-            for (int q = tid; q < n_edge && more; q += T) {
+            for (int q = tid; q < n_edge && publish; q += T) {
                 const unsigned it = item[q];
-                ResWord* d = out_box + (size_t)(it >> 16) * Q;
+                ResWord* d = out_box + (size_t)item_cell(it) * Q;
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
-                    const double v = nxt[(it & 0xffffu) + i * P];
+                    const double v = nxt[item_place(it) + i * P];
                     st_word(d + i, (unsigned)__double2loint(v), (unsigned)__double2hiint(v), 0u, tag);
                 }
             }
         } else {
-            for (int q = tid < T1 ? tid : n_items; q < n_items; q += T1) {
+            for (int q = tid < T1 ? tid : n_now; q < n_now; q += T1) {
                 const unsigned it = item[q];
-                const int at = (int)(it & 0xffffu);
+                const int at = item_place(it);
                 S o[9];
-                bits |= node_update<TM>(M, cur + at, P, o);
+                bits |= node_update<TM>(M, cur + at, P, it & kWrapUp ? -around : RS, it & kWrapDown ? around : -RS, o);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) nxt[at + i * P] = o[i];
-                if (more && it >> 16 != kNoCell) {
-                    ResWord* d = out_box + (size_t)(it >> 16) * Q;
+                if (publish && item_cell(it) != kNoCell) {
+                    ResWord* d = out_box + (size_t)item_cell(it) * Q;
 #pragma unroll
                     for (int k = 0; k < 3; ++k)
                         st_word(d + k, __float_as_uint(o[3 * k]), __float_as_uint(o[3 * k + 1]),
@@ -432,8 +399,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         if (!more) break;
-        for (int q = halo_tid; q < n_halo && ok; q += T)
+        for (int q = halo_tid; q < n_halo && ok && publish; q += T)
             ok = receive<S>(in_box + (size_t)halo_src[q] * Q, tag, nxt + halo_dst[q], P, A.status);
+        // (ghost cells beside the shells are made from received cells)
+        if (publish && n_ghost && R.depth > 1) __syncthreads();
         for (int q = ghost_tid; q < n_ghost; q += T) {
             const uint2 e = ghost[q];
             const int side = e.y & 3u;
@@ -444,9 +413,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = false;
             break;
         }
-        S* t = cur;
+        S* swap = cur;
         cur = nxt;
-        nxt = t;
+        nxt = swap;
+        j = publish ? 0 : j + 1;
+        round += publish;
     }
     if (!ok) bits |= ST_TIMEOUT;
     report(A.status, bits);
@@ -470,7 +441,9 @@ template <typename S>
 constexpr size_t kSmemMax = sizeof(S) == 4 ? 226 * 1024 : 113 * 1024;
 
 size_t smem_bytes(const ResPlan& R, size_t esize) {
-    return 2 * (size_t)(R.bh + 2) * 9 * R.pitch * esize + 14 * (size_t)R.cells + 4 * (size_t)R.bw * R.bh;
+    const ResTile full = res_full_tile(R);
+    return 2 * (size_t)(R.bh + 2 * res_pad_y(R)) * 9 * R.pitch * esize + 8 * (size_t)res_max_ghosts(R) +
+           6 * (size_t)(res_nodes(full, R.depth) - R.bw * R.bh) + 4 * (size_t)res_nodes(full, R.depth - 1);
 }
 
 template <typename S, int TM>
@@ -484,10 +457,15 @@ constexpr auto kernel_of() {
 
 // The split of a grid over at most one CTA per SM: for every number of tiles
 // in y the fewest columns that fit, as they are, rounded up to 32 (a warp's
-// nodes then lie in one row) or to whole warps; the cheapest by an estimate of the step's time
-// in us, fitted to 260 splits of grids from 400 x 4 to 1240 x 310 (7 % rms):
-// per warp of nodes, per cell exchanged, for neighbours in y, and per CTA (the
-// more, the more often one lags).  FP64: only up to kQuadGroups groups of 32
+// nodes then lie in one row) or to whole warps; the cheapest by an estimate of
+// the step's time in us, fitted to 260 splits of grids from 400 x 4 to 1240 x
+// 310 (7 % rms): per warp of nodes, per cell exchanged, for neighbours in y,
+// and per CTA (the more, the more often one lags).  Tiles that span the grid's
+// height exchange every depth-th step, at 0.4 us (0.7 in FP64) an exchange
+// besides: one to four steps, 2000 x 4 1.35 / 1.11 / 1.02 / 0.99 us a step, FP64
+// 400 x 4 3.05 / 2.67 / 2.60 / 3.25 (the fourth takes another 32 nodes); six
+// and eight gain nothing more.  With neighbours on both axes deeper tiles gain
+// at most 6 % (128 x 32) and lose from 512 x 128 on.  FP64: only up to kQuadGroups groups of 32
 // nodes per SM (beyond, a launch a step keeps the FP64 pipe as busy: 400 x 100
 // 11.1 us a step, 12.6 in a resident kernel of one node a thread).
 template <typename S, int TM>
@@ -514,39 +492,47 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
             if (how == 1) R.bw = (R.bw - ends + 31) / 32 * 32 + ends;
             if (how == 2 && R.bh < 32) R.bw = (R.bw + 32 / R.bh - 1) / (32 / R.bh) * (32 / R.bh);
             R.px = (nx + R.bw - 1) / R.bw;
-            // pitch: a warp that continues on the next row of the inner columns
-            // stays free of bank conflicts if 9 pitch = their number modulo 32
-            // banks (9 x 25 = 1 mod 32); if rows are whole warps, an odd pitch
-            // keeps the column updates free of them
-            const int inner = R.bw - (R.px > 1 ? 2 : 0);
-            R.pitch = R.bw + 4;
-            if (inner % 32 != 0)
-                R.pitch += ((25 * inner - R.pitch) % 32 + 32) % 32;
-            else
-                R.pitch |= 1;
-            R.cells = 2 * R.bw + 2 * R.bh;
-            const int warps = (R.bw * R.bh + 31) / 32;
-            const int exchanged = R.py > 1 ? R.cells : 2 * R.bh;
-            if (f64) {
-                if (warps > kQuadGroups) continue;
-                R.threads = 128 * warps;
-            } else {
-                const int most = kThreads32 - 32, rounds = (32 * warps + most - 1) / most;
-                R.threads = (warps + rounds - 1) / rounds * 32;
-                // warps enough to poll beside those that update the last nodes
-                const int roles = (exchanged + 31) / 32 * 32 + 64;
-                if (R.threads < roles) R.threads = roles < most ? roles : most;
-                R.threads += 32;
-            }
-            R.smem = smem_bytes(R, sizeof(S));
-            // places in the tile are 16-bit
-            if ((R.bh + 2) * 9 * R.pitch > 65535 || R.smem > kSmemMax<S>) continue;
-            const double each = f64 ? 1.25 : TM == T_INT64 ? 0.13 : inner % 32 == 0 ? 0.060 : 0.067;
-            const double c = each * warps + (f64 ? 0.02 : 0.002) * exchanged + (R.py > 1 ? 0.2 : 0.0) + 0.001 * R.px * R.py;
-            if (!found || c < cost) {
-                found = true;
-                cost = c;
-                *best = R;
+            for (R.depth = 1; R.depth <= (R.py == 1 && R.px > 1 ? kMaxDepth : 1); ++R.depth) {
+                // pitch: a warp that continues on the next row of the inner
+                // columns stays free of bank conflicts if 9 pitch = their
+                // number modulo 32 banks (9 x 25 = 1 mod 32); if rows are whole
+                // warps, an odd pitch keeps the column updates free of them
+                const int inner = R.bw - (R.px > 1 ? min(2 * R.depth, R.bw) : 0);
+                R.pitch = R.bw + 2 * res_pad_x(R);
+                if (inner % 32 != 0)
+                    R.pitch += ((25 * inner - R.pitch) % 32 + 32) % 32;
+                else
+                    R.pitch |= 1;
+                R.cells = res_cells(R);
+                const ResTile full = res_full_tile(R);
+                const int warps = (res_nodes(full, R.depth - 1) + 31) / 32;
+                const int received = res_nodes(full, R.depth) - R.bw * R.bh;
+                if (f64) {
+                    if (warps > kQuadGroups) continue;
+                    R.threads = 128 * warps;
+                } else {
+                    const int most = kThreads32 - 32, rounds = (32 * warps + most - 1) / most;
+                    R.threads = (warps + rounds - 1) / rounds * 32;
+                    // warps enough to poll beside those that update the last nodes
+                    const int roles = (received + 31) / 32 * 32 + 64;
+                    if (R.threads < roles) R.threads = roles < most ? roles : most;
+                    R.threads += 32;
+                }
+                R.smem = smem_bytes(R, sizeof(S));
+                // places in the tile are 16-bit, and cells but for one value
+                if ((R.bh + 2 * res_pad_y(R)) * 9 * R.pitch > 65535 || R.cells >= (int)kNoCell ||
+                    R.smem > kSmemMax<S>)
+                    continue;
+                double sum = 0.0;  // warps of nodes over the steps to an exchange
+                for (int d = 0; d < R.depth; ++d) sum += f64 ? warps : (res_nodes(full, d) + 31) / 32;
+                const double each = f64 ? 1.25 : TM == T_INT64 ? 0.13 : inner % 32 == 0 ? 0.060 : 0.067;
+                const double c = (each * sum + (f64 ? 0.02 : 0.002) * received + (R.py > 1 ? 0.2 : 0.0) +
+                                  (f64 ? 0.7 : 0.4)) / R.depth + 0.001 * R.px * R.py;
+                if (!found || c < cost) {
+                    found = true;
+                    cost = c;
+                    *best = R;
+                }
             }
         }
     if (!found) return false;
