@@ -9,13 +9,15 @@
 // constant in shared memory in both lanes, ready to be an operand: 298 warp
 // instructions per 32 nodes in the double-float mode, the columns computed
 // twice included, where the tile kernel (one tensor copy per tile and step)
-// issues 414.  Bound by the latency of a warp's own chain: 128 registers a
-// thread leave four warps to a scheduler, which keep the FP32 pipe 58 % busy
-// (fewer registers spill: 24.6 us with five warps).  Four CTAs of four warps
+// issues 414.  Bound by the FP32 pipe's register reads: a packed FMA of three
+// different operands takes three cycles on a quarter of an SM, two with one
+// that the instruction before used too (measured), so that two, three and four
+// warps to a scheduler take 24.6, 22.0 and 21.1 us a step on 256 tubes, and a
+// fifth, whose 96 registers a thread spill, 24.6.  Four CTAs of four warps
 // to an SM, so that some load or store their columns while others compute: two
-// of eight and one of sixteen take 21.9 and 22.6 us.  Against the tile kernel,
-// us a step: 256 Riemann tubes 21.6 / 24.9 (total-energy mode 17.8 / 22.8), 64
-// tubes 6.7 / 8.8, 4 tubes 2.0 / 4.0; with the FP64 sum of the temperature it
+// of eight and one of sixteen take 3 and 5 % longer.  Against the tile kernel,
+// us a step: 256 Riemann tubes 21.1 / 24.9 (total-energy mode 17.1 / 22.8), 64
+// tubes 6.7 / 8.8, 4 tubes 1.9 / 4.0; with the FP64 sum of the temperature it
 // is slower from 16 tubes on (40.6 / 34.9 us on 256), so the launch shape is
 // left to lbm_batch_autotune.
 #include "lbm_batch_plan.h"
@@ -85,20 +87,6 @@ __device__ __noinline__ void split_ghost(const Grid<float>& G, int side, const C
     }
 }
 
-// Exchange counters of a CTA's warps in shared memory: a warp that has put its
-// edge columns there raises its own, and waits (bounded) for its neighbours'.
-__device__ __forceinline__ void post(int* flag, int value) {
-    asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(flag)), "r"(value) : "memory");
-}
-__device__ __forceinline__ bool await(const int* flag, int value) {
-    for (int tries = 0; tries < (1 << 24); ++tries) {
-        int v;
-        asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(flag)) : "memory");
-        if (v >= value) return true;
-    }
-    return false;
-}
-
 // NP pairs of rows.
 template <int TM, int NP>
 __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
@@ -112,11 +100,8 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
     // the column beside the left and the right ghost column, or the ghost
     // column itself where it stays the same; then room for split sides'
     __shared__ Column<NP> sX[kStripWarps][2], sY[kStripWarps][2];
-    __shared__ int sFlag[kStripWarps], sRound;
+    __shared__ int sRound;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sFlag[w] = 0;
-    __syncthreads();
-    int exchanges = 0;
     const long long level0 = *(volatile long long*)level_ptr;
     unsigned bits = 0;
     // More rounds than CTAs: each CTA draws its next round while it works on
@@ -140,18 +125,6 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
             const bool busy = W.prob >= 0;
             const BatchProb& P = probs[busy ? W.prob : 0];
             const Grid<float>& G = P.G;
-            if (loaded != round) {  // the windows' constants, by their first warps
-                if (busy && !(W.links & 1)) {
-                    const float* m = reinterpret_cast<const float*>(&P.M);
-                    F2* d = reinterpret_cast<F2*>(&sM[W.slot]);
-                    for (int q = lane; q < kModelWords; q += 32) d[q] = bcast(__ldg(m + q));
-                }
-                __syncthreads();
-                loaded = round;
-            }
-            int next = rounds;
-            if (drawn && threadIdx.x == 0) next = (int)(atomicAdd(ticket, 1u) - base);
-            const Model<F2>& M = sM[W.slot];
             const int nx = G.nx, col = W.col0 + lane;
             const size_t pl = (size_t)G.plane, row = (size_t)G.row;
             // ghost columns of this warp: the left one in lane 0, the right one in lane gr
@@ -175,6 +148,18 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
                         f[i][k] = in_range ? pair(__ldcg(p), __ldcg(p + row)) : bcast(1.0f);
                     }
             }
+            int next = rounds;
+            if (drawn && threadIdx.x == 0) next = (int)(atomicAdd(ticket, 1u) - base);
+            if (loaded != round) {  // the windows' constants, by their first warps, while the columns arrive
+                if (busy && !(W.links & 1)) {
+                    const float* m = reinterpret_cast<const float*>(&P.M);
+                    F2* d = reinterpret_cast<F2*>(&sM[W.slot]);
+                    for (int q = lane; q < kModelWords; q += 32) d[q] = bcast(__ldg(m + q));
+                }
+                __syncthreads();
+                loaded = round;
+            }
+            const Model<F2>& M = sM[W.slot];
             if (has_left && lane == 0 && rule_l == BC_DIRICHLET) sX[w][0].put(f);
             if (has_right && lane == gr && rule_r == BC_DIRICHLET) sX[w][1].put(f);
             for (int j = 0; j < n; ++j) {
@@ -229,14 +214,9 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
                 if (j + 1 < n) {
                     Column<NP>(&E)[kStripWarps][2] = sE[j & 1];
                     if (busy && (lane == 1 || lane == 30)) E[w][lane == 30].put(f);
-                    __syncwarp();
-                    ++exchanges;
-                    if (busy && lane == 0) post(&sFlag[w], exchanges);
-                    if (busy && ((lane == 0 && (W.links & 1)) || (lane == 31 && (W.links & 2)))) {
-                        if (!await(&sFlag[lane == 0 ? w - 1 : w + 1], exchanges)) bits |= ST_TIMEOUT;
+                    __syncthreads();
+                    if (busy && ((lane == 0 && (W.links & 1)) || (lane == 31 && (W.links & 2))))
                         (lane == 0 ? E[w - 1][1] : E[w + 1][0]).get(f);
-                    }
-                    __syncwarp();
                 }
             }
             const bool ghost = (has_left && lane == 0 && W.c0 == 0) || (has_right && lane == gr && W.c1 == nx);
@@ -264,7 +244,6 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
             round = sRound;
         }
         base += (unsigned)rounds + gridDim.x;
-        if (bits & ST_TIMEOUT) atomicOr(status, ST_TIMEOUT);
         if (!grid_barrier(bar_count, bar_gen, status)) return;
         done += n;
     }
