@@ -290,13 +290,18 @@ cudaError_t launch_moments(const S* f, S* rho, S* ux, S* uy, S* T, const Model<S
 // CTA to finish adds the CTAs' partials in a fixed order, so the result does
 // not depend on scheduling, and writes it with the health word straight to
 // the caller's page-locked memory.  (With a second kernel and two
-// copies back a call took 30 us on the smallest grids, now 20.)
-constexpr int kConsSeg = 512;
+// copies back a call took 30 us on the smallest grids.)  On those the
+// kernel's time is that of its FP64 instructions one after the other, 64 cycles
+// each: the reductions share the totals out over the lanes, and an FP64 CTA
+// has one warp to each quarter of its SM (400 x 4, us a call: FP64 15.3 against
+// 21.0, FP32 15.9 against 18.5).
+constexpr int kConsSeg = 512, kConsSeg64 = 128;
 constexpr int kConsBlocks = 608;  // 4 per SM
 
 template <typename S>
 int conservation_partials(const Grid<S>& G) {
-    const long long units = (long long)G.ny * ((G.nx + kConsSeg - 1) / kConsSeg);
+    const int seg = sizeof(S) == 4 ? kConsSeg : kConsSeg64;
+    const long long units = (long long)G.ny * ((G.nx + seg - 1) / seg);
     return (int)(units < kConsBlocks ? units : kConsBlocks);
 }
 
@@ -311,33 +316,44 @@ __device__ __forceinline__ void totals_of(const Model<double>& M, const double (
     t[3] = M.eta2 * v[0] + M.c1s * s14 + M.c2s * s58;
 }
 
-// Called by one whole warp of a CTA, with the CTA's totals in lane 0: writes
-// the partials, and in the last CTA the totals and the health word.  left:
-// CTAs that have finished, zero between launches.
-__device__ __forceinline__ void finish_totals(const double (&t)[4], double* __restrict__ partials, unsigned* left,
-                                              const unsigned* status, double* out, unsigned* out_status) {
-    const int lane = threadIdx.x & 31;
-    const int nb = gridDim.x;
-    unsigned last = 0;
-    if (lane == 0) {
+// Sum over the eight lanes that share a total.
+__device__ __forceinline__ double sum8(double v) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) __stcg(partials + q * nb + blockIdx.x, t[q]);
+    for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+// Sums of four quantities over a warp: the lanes 8 q .. 8 q + 7 get the q-th.
+// Halves of the warp first take two of the four each, quarters one: six
+// additions, where four shuffle trees take twenty.
+__device__ __forceinline__ double warp_totals(const double (&t)[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool up = lane & 16, odd = lane & 8;
+    const double a = (up ? t[2] : t[0]) + __shfl_xor_sync(0xffffffffu, up ? t[0] : t[2], 16);
+    const double b = (up ? t[3] : t[1]) + __shfl_xor_sync(0xffffffffu, up ? t[1] : t[3], 16);
+    return sum8((odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8));
+}
+
+// Called by one whole warp of a CTA, with the CTA's q-th total in the lanes 8 q
+// .. 8 q + 7: writes the partials, and in the last CTA the totals and the
+// health word.  left: CTAs that have finished, zero between launches.
+__device__ __forceinline__ void finish_totals(double t, double* __restrict__ partials, unsigned* left,
+                                              const unsigned* status, double* out, unsigned* out_status) {
+    const int lane = threadIdx.x & 31, q = lane >> 3, k = lane & 7;
+    const int nb = gridDim.x;
+    if (k == 0) {
+        __stcg(partials + q * nb + blockIdx.x, t);
         __threadfence();
-        last = atomicAdd(left, 1u) == (unsigned)nb - 1;
     }
+    __syncwarp();
+    unsigned last = 0;
+    if (lane == 0) last = atomicAdd(left, 1u) == (unsigned)nb - 1;
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = lane; b < nb; b += 32)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] += __ldcg(partials + q * nb + b);
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] += __shfl_down_sync(0xffffffffu, acc[q], s);
+    double acc = 0.0;
+    for (int b = k; b < nb; b += 8) acc += __ldcg(partials + q * nb + b);
+    acc = sum8(acc);
+    if (k == 0) out[q] = acc;
     if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) out[q] = acc[q];
         *out_status = *status;
         *left = 0;
     }
@@ -441,39 +457,32 @@ __global__ void __launch_bounds__(kConsThreads32, 4)
         for (int k = 0; k < 3; ++k) sums[k][pop] = part[k];
     __syncthreads();
     if (pop == 0) {
-        // linear in the sums: each part's totals, the small parts first
-        double t[4] = {0.0, 0.0, 0.0, 0.0};
-        if (lane == 0) {
+        // linear in the sums: the totals of each part in a lane of its own
+        double v[9], t[4];
 #pragma unroll
-            for (int k = 2; k >= 0; --k) {
-                double v[9], q[4];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) v[i] = sums[k][i];
-                totals_of(M, v, q);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) t[m] += q[m];
-            }
-        }
-        finish_totals(t, partials, left, status, out, out_status);
+        for (int i = 0; i < 9; ++i) v[i] = lane < 3 ? sums[lane][i] : 0.0;
+        totals_of(M, v, t);
+        finish_totals(warp_totals(t), partials, left, status, out, out_status);
     }
 }
 
 // FP64 levels: one node per thread, FP64 sums of the pair differences and of
 // the three speed classes (17 FP64 instructions a node; forming the totals
 // node by node takes 27), combined once per thread.
-__global__ void __launch_bounds__(kThreads)
+constexpr int kConsThreads64 = 128;
+__global__ void __launch_bounds__(kConsThreads64)
     k_cons64(const double* __restrict__ f, const Model<double> M, const Grid<double> G, double* __restrict__ partials,
              unsigned* left, const unsigned* status, double* out, unsigned* out_status) {
-    __shared__ double sh[4][kThreads / 32];
-    const int segs = (G.nx + kConsSeg - 1) / kConsSeg;
+    __shared__ double sh[4][kConsThreads64 / 32];
+    const int segs = (G.nx + kConsSeg64 - 1) / kConsSeg64;
     const long long units = (long long)G.ny * segs;
     const size_t pl = (size_t)G.plane;
     double s0 = 0.0, s14 = 0.0, s58 = 0.0, ax = 0.0, ay = 0.0, ar = 0.0, am = 0.0;
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-        const int row = (int)(u / segs), x0 = (int)(u % segs) * kConsSeg;
-        const int n = min(kConsSeg, G.nx - x0);
+        const int row = (int)(u / segs), x0 = (int)(u % segs) * kConsSeg64;
+        const int n = min(kConsSeg64, G.nx - x0);
         const double* p = f + cell(G, x0, row);
-        for (int x = threadIdx.x; x < n; x += kThreads) {
+        for (int x = threadIdx.x; x < n; x += kConsThreads64) {
             double v[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) v[i] = __ldg(p + i * pl + x);
@@ -488,22 +497,13 @@ __global__ void __launch_bounds__(kThreads)
     }
     double t[4] = {s0 + s14 + s58, M.c1 * ax + M.d * (ar + am), M.c1 * ay + M.d * (ar - am),
                    M.eta2 * s0 + M.c1s * s14 + M.c2s * s58};
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] += __shfl_down_sync(0xffffffffu, t[q], d);
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) sh[q][warp] = t[q];
+    const double sum = warp_totals(t);
+    if ((lane & 7) == 0) sh[lane >> 3][warp] = sum;
     __syncthreads();
     if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            t[q] = 0.0;
-            for (int w = 0; w < kThreads / 32; ++w) t[q] += sh[q][w];
-        }
-        finish_totals(t, partials, left, status, out, out_status);
+        const double part = (lane & 7) < kConsThreads64 / 32 ? sh[lane >> 3][lane & 7] : 0.0;
+        finish_totals(sum8(part), partials, left, status, out, out_status);
     }
 }
 
@@ -515,7 +515,7 @@ cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S
     if constexpr (sizeof(S) == 4)
         k_cons32<<<nb, kConsThreads32, 0, st>>>(f, M, G, partials, left, status, out, out_status);
     else
-        k_cons64<<<nb, kThreads, 0, st>>>(f, M, G, partials, left, status, out, out_status);
+        k_cons64<<<nb, kConsThreads64, 0, st>>>(f, M, G, partials, left, status, out, out_status);
     return cudaGetLastError();
 }
 
