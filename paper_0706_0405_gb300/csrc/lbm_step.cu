@@ -152,9 +152,10 @@ constexpr int kStageFloats = (kBoxFloats + 31) / 32 * 32;  // stages start on 12
 // Shared-memory stages per CTA (boxes in flight + the one being computed) and
 // the resident CTAs per SM the register budget is set for: 6 (80 registers)
 // in every mode but the double-float one, whose packed update with the
-// centre pairs re-read from shared memory fits 72 registers and so 7 CTAs
-// (measured on the 4096 x 1024 double Mach reflection: double-float T 69.6
-// -> 70.9 GLUPS from 6 to 7 CTAs; FP32 total-energy T 78.1 -> 74.9).
+// centre pairs re-read from shared memory fits 64 registers and so 8 CTAs
+// (4096 x 1024 double Mach reflection, us a step: 57.7 with 6 CTAs, 53.6 with
+// 7, 53.3 with 8; the FP32 total-energy mode takes 4 % longer with 7 than with
+// 6).
 #ifndef LBM_TILE_STAGES
 #define LBM_TILE_STAGES 2
 #endif
@@ -162,23 +163,11 @@ constexpr int kStageFloats = (kBoxFloats + 31) / 32 * 32;  // stages start on 12
 #define LBM_TILE_MIN_BLOCKS 6
 #endif
 #ifndef LBM_TILE_MIN_BLOCKS_DF
-#define LBM_TILE_MIN_BLOCKS_DF 7
+#define LBM_TILE_MIN_BLOCKS_DF 8
 #endif
 template <int TM>
 constexpr int tile_min_blocks() {
     return TM == T_DF ? LBM_TILE_MIN_BLOCKS_DF : LBM_TILE_MIN_BLOCKS;
-}
-#ifndef LBM_TILE_DYNAMIC
-#define LBM_TILE_DYNAMIC 1  // 0: static walk everywhere, 1: as measured below, 2: claims everywhere
-#endif
-// Tiles claimed at run time (see below) where the grid's CTAs do not divide
-// the tiles evenly: with 7 CTAs per SM on the 4096 x 1024 grid (16384 tiles,
-// 1064 CTAs) a static walk gives 16 tiles to some CTAs and 15 to others
-// (70.9 -> 72.4 GLUPS with run-time claims); with 6 (912 CTAs, 17.96 each)
-// the static walk is already even and the claims only cost (78.1 -> 75.7).
-template <int TM>
-constexpr bool dynamic_tiles() {
-    return LBM_TILE_DYNAMIC == 2 || (LBM_TILE_DYNAMIC == 1 && tile_min_blocks<TM>() != LBM_TILE_MIN_BLOCKS);
 }
 constexpr int kStages = LBM_TILE_STAGES;
 static_assert(kStages >= 2 && kStages <= 8, "2 to 8 stages");
@@ -190,24 +179,25 @@ constexpr int kNoTile = 0x7fffffff;
 #ifndef LBM_TILE_PDL
 #define LBM_TILE_PDL 1
 #endif
-// Run-time claims one tile ahead of the copies, the claim's result held in
-// a register of thread 0 (1: 75.2 -> 76.2 GLUPS over 400 steps in the
-// double-float mode), or each tile claimed just before its copy (0).  (Held
-// in shared memory instead, the claim stalls warp 0 right after the copy:
-// 73.3.)
-#ifndef LBM_TILE_CLAIM_AHEAD
-#define LBM_TILE_CLAIM_AHEAD 1
+// Tiles claimed at run time instead of walked in a fixed stride, from this many
+// tiles a CTA on (double-float mode, us a step with claims / without: 2048 x
+// 256, 1.7 tiles a CTA, 11.5 / 9.7, a CTA that starts late still taking its
+// full share; 2048 x 640, 4.2, 19.8 / 19.8; 2048 x 768, 5.1, 22.7 / 23.3; 4096 x
+// 1024, 13.5, 52.0 / 54.9; 8192 x 2048, 54, 240 / 243; of the sizes between some
+// gain from the stride, 6000 x 1600 130 / 126).  The other modes' 912 CTAs have
+// 17.96 tiles each on 4096 x 1024, where claims only cost (78.1 -> 75.7 GLUPS).
+#ifndef LBM_TILE_CLAIM_TILES
+#define LBM_TILE_CLAIM_TILES 5
 #endif
-// Claims ahead are taken only where each CTA walks at least this many tiles
-// (chosen at launch): on a small grid a CTA that starts late would still take
-// its full share instead of leaving tiles to the CTAs that are free first
-// (the Mach-3 2048 x 256 tube, 1.9 tiles a CTA: 12.5 us a step with claims
-// ahead, 11.4 without).
-constexpr int kClaimAheadTiles = 8;
+constexpr int kClaimTiles = LBM_TILE_CLAIM_TILES;
+template <int TM>
+constexpr bool may_claim() {
+    return TM == T_DF;
+}
 
 // status[0]: health bits; status[2], status[3]: the tile counter and the
 // count of CTAs that have left (both zero between launches).
-template <int TM, bool kClaimAhead>
+template <int TM, bool kClaim>
 __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<TM>())
     k_step_tile(const __grid_constant__ CUtensorMap tmap, float* __restrict__ fout, const Model<float> M,
                 const Grid<float> G, long long level, unsigned* status, int tiles_x, int ntiles) {
@@ -227,6 +217,13 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<TM>())
     // its output buffer) or of the counters is touched before the previous
     // grid has completed; the next step may be scheduled from here on, its
     // CTAs taking SM slots as this grid's CTAs leave.
+    if (tid == 0) {
+        prefetch_tensormap(&tmap);
+        for (int j = 0; j < kStages; ++j) mbar_init(&bar[j], 1);
+        fence_mbar_init();
+        abort_flag = 0;
+        for (int j = 0; j < kStages; ++j) tile_of[j] = kNoTile;
+    }
     grid_dependency_wait();
     grid_dependents_launch();
     auto issue = [&](int tile, int stage) {
@@ -235,11 +232,10 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<TM>())
         // array column x0 is interior column x0 - 4; array row y0 is interior row y0 - 1
         tma_load_3d(box + stage * kStageFloats, &tmap, x0, 0, y0, &bar[stage]);
     };
-    constexpr bool kDyn = dynamic_tiles<TM>();
     // the tile of this CTA's local tile k: static walk, or (run-time claims)
     // the one held in k's stage
     auto tile_at = [&](int k) {
-        if constexpr (kDyn) {
+        if constexpr (kClaim) {
             return tile_of[k % kStages];
         } else {
             const int t = blockIdx.x + k * gridDim.x;
@@ -249,30 +245,20 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<TM>())
     // take the tile of local tile k into its stage and start its copy (thread 0)
     auto claim = [&](int k) {
         const int stage = k % kStages;
-        if constexpr (!kDyn) {
+        if constexpr (!kClaim) {
             const int t = tile_at(k);
             if (t != kNoTile) issue(t, stage);
             return;
         }
-        if constexpr (kClaimAhead) {
-            // the tile was claimed one round earlier: its copy starts now; the
-            // next claim's atomic is issued after the copy, and its result is
-            // first needed a tile later, so its round trip overlaps the tile's
-            // arithmetic instead of delaying the copy
-            const unsigned t = ahead;
-            if (t < (unsigned)ntiles) {
-                tile_of[stage] = (int)t;
-                issue((int)t, stage);
-                ahead = atomicAdd(counter, 1u);
-            } else {
-                tile_of[stage] = kNoTile;
-            }
-            return;
-        }
-        const unsigned t = atomicAdd(counter, 1u);
+        // the tile was claimed one round earlier: its copy starts now; the next
+        // claim's atomic is issued after the copy, and its result, in a register
+        // (in shared memory it would stall warp 0 right after the copy), is first
+        // needed a tile later, so its round trip overlaps the tile's arithmetic
+        const unsigned t = ahead;
         if (t < (unsigned)ntiles) {
             tile_of[stage] = (int)t;
             issue((int)t, stage);
+            ahead = atomicAdd(counter, 1u);
         } else {
             tile_of[stage] = kNoTile;
         }
@@ -283,11 +269,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<TM>())
         return mbar_wait_bounded(&bar[k % kStages], (uint32_t)((k / kStages) & 1), kWaitLimit);
     };
     if (tid == 0) {
-        for (int j = 0; j < kStages; ++j) mbar_init(&bar[j], 1);
-        fence_mbar_init();
-        abort_flag = 0;
-        for (int j = 0; j < kStages; ++j) tile_of[j] = kNoTile;
-        if constexpr (kDyn && kClaimAhead) ahead = atomicAdd(counter, 1u);
+        if constexpr (kClaim) ahead = atomicAdd(counter, 1u);
         for (int j = 0; j < kStages - 1; ++j) claim(j);  // fill all stages but one
     }
     __syncthreads();
@@ -345,7 +327,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<TM>())
                 if (tile_at(k + j) != kNoTile) wait(k + j);
             atomicOr(status, ST_TIMEOUT);
         }
-        if constexpr (kDyn) {
+        if constexpr (kClaim) {
             // every claim of this CTA is made; the last CTA out resets the
             // counters for the next launch
             __threadfence();
@@ -448,7 +430,7 @@ cudaError_t launch_tile(const CUtensorMap& tmap, float* fout, const Model<float>
     constexpr size_t smem = kTileSmem;
     // both instances have the same launch bounds, so the same occupancy
     cudaError_t e = allow_smem<k_step_tile<TM, false>>(smem);
-    if constexpr (dynamic_tiles<TM>())
+    if constexpr (may_claim<TM>())
         if (e == cudaSuccess) e = allow_smem<k_step_tile<TM, true>>(smem);
     if (e != cudaSuccess) return e;
     const int tiles_x = (G.nx + kTileX - 1) / kTileX;
@@ -457,8 +439,8 @@ cudaError_t launch_tile(const CUtensorMap& tmap, float* fout, const Model<float>
     if (grid <= 0) grid = full_wave<k_step_tile<TM, false>>(kTileThreads, smem);
     if (grid > ntiles) grid = ntiles;
     auto kern = k_step_tile<TM, false>;
-    if constexpr (dynamic_tiles<TM>())
-        if (LBM_TILE_CLAIM_AHEAD && ntiles >= kClaimAheadTiles * grid) kern = k_step_tile<TM, true>;
+    if constexpr (may_claim<TM>())
+        if (ntiles >= kClaimTiles * grid) kern = k_step_tile<TM, true>;
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(grid);
     lc.blockDim = dim3(kTileThreads);
