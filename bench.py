@@ -241,7 +241,7 @@ def run_ours(args, world, dist):
     glups = rate / 1e9
     bpn = BYTES_PER_NODE[args.precision]
     achieved = bpn * p.nodes / (kernel_ms / 1e3) / 1e9
-    kname = {0: "k_step_simple", 1: "k_step_ring", 2: "k_step_vec", 3: "k_step_tile"}[launch[0]]
+    kname = {0: "k_step_fp64" if args.precision == "fp64" else "k_step_simple", 1: "k_step_ring", 2: "k_step_vec", 3: "k_step_tile"}[launch[0]]
     # the tile kernel's data movement alone (same boxes, same stores, no
     # arithmetic) on the same grid: the ceiling of its access pattern
     pattern = lbm.lbm_probe_tile_copy(p.nx, p.ny, 10) if kname == "k_step_tile" else None

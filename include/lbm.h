@@ -392,7 +392,10 @@ lbm_status lbm_batch_info(const lbm_batch* batch, int* grid, int* ntiles, int* g
  * batches whose problems all have at most 8 rows and no periodic x sides):
  * one pass advances a 128-column segment of a problem by `block` steps in
  * shared memory (halo of `block` columns each side, recomputed), so DRAM
- * traffic and grid barriers drop by that factor; npt is then ignored.
+ * traffic and grid barriers drop by that factor; npt is then ignored.  If all
+ * problems have two or all four rows, periodic in y, the columns are held in
+ * registers instead, on as many CTAs as are resident for a full wave, at most
+ * grid otherwise.
  * block = 0 or 1 is the one-step tile kernel.  Every shape computes the same
  * bits.  Setting a shape drops the captured graph (the next lbm_batch_step
  * captures a new one). */

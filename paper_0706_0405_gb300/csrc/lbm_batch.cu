@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(batch_threads<NPT>(), batch_min_blocks<NPT>())
 }
 // ------------------------------------------------- temporal blocking
 // For batches of thin problems (at most kTbRowsMax rows, no periodic x
-// sides) one pass advances a segment of kTbW columns (all rows) by NS steps
+// sides; those of two or four rows, periodic in y, are lbm_strip.cu's) one
+// pass advances a segment of kTbW columns (all rows) by NS steps
 // (NS odd) inside shared memory: it loads the level with a halo of NS columns
 // on each side (the ghost cells included), then each sub-step j updates the
 // columns within NS - 1 - j of the segment and fills the ghost cells of the

@@ -1,5 +1,5 @@
-// lbm_reduce.cuh -- block-wide FP64 reduction shared by the conservation
-// kernels of liblbm (internal).
+// lbm_reduce.cuh -- block-wide FP64 reduction of the allocation-free totals
+// (lbm_noalloc.cu).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -152,10 +152,10 @@ constexpr int kStageFloats = (kBoxFloats + 31) / 32 * 32;  // stages start on 12
 // Shared-memory stages per CTA (boxes in flight + the one being computed) and
 // the resident CTAs per SM the register budget is set for: 6 (80 registers)
 // in every mode but the double-float one, whose packed update with the
-// centre pairs re-read from shared memory fits 64 registers and so 8 CTAs
-// (4096 x 1024 double Mach reflection, us a step: 57.7 with 6 CTAs, 53.6 with
-// 7, 53.3 with 8; the FP32 total-energy mode takes 4 % longer with 7 than with
-// 6).
+// centre pairs re-read from shared memory fits the 64 registers of 8 CTAs (of
+// which the stages leave room for 7; 4096 x 1024 double Mach reflection, us a
+// step: 57.7 with 6 CTAs of 80 registers, 53.6 with 7 of 72, 53.3 with 7 of
+// 64; the FP32 total-energy mode takes 4 % longer with 7 than with 6).
 #ifndef LBM_TILE_STAGES
 #define LBM_TILE_STAGES 2
 #endif
@@ -181,9 +181,9 @@ constexpr int kNoTile = 0x7fffffff;
 #endif
 // Tiles claimed at run time instead of walked in a fixed stride, from this many
 // tiles a CTA on (double-float mode, us a step with claims / without: 2048 x
-// 256, 1.7 tiles a CTA, 11.5 / 9.7, a CTA that starts late still taking its
-// full share; 2048 x 640, 4.2, 19.8 / 19.8; 2048 x 768, 5.1, 22.7 / 23.3; 4096 x
-// 1024, 13.5, 52.0 / 54.9; 8192 x 2048, 54, 240 / 243; of the sizes between some
+// 256, 1.9 tiles a CTA, 11.5 / 9.7, a CTA that starts late still taking its
+// full share; 2048 x 640, 4.8, 19.8 / 19.8; 2048 x 768, 5.8, 22.7 / 23.3; 4096 x
+// 1024, 15.4, 52.0 / 54.9; 8192 x 2048, 62, 240 / 243; of the sizes between some
 // gain from the stride, 6000 x 1600 130 / 126).  The other modes' 912 CTAs have
 // 17.96 tiles each on 4096 x 1024, where claims only cost (78.1 -> 75.7 GLUPS).
 #ifndef LBM_TILE_CLAIM_TILES
