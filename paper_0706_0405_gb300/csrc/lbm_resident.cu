@@ -75,6 +75,13 @@ __device__ __forceinline__ unsigned word_tag(const ResWord& w) { return (unsigne
 template <typename S>
 constexpr int kCellWords = sizeof(S) == 4 ? 3 : 9;
 
+// Modes that repeat a node for the sake of shared-memory banks (res_fill); where
+// the FP64 pipe is the bound, a warp more costs 1 %.
+template <typename S, int TM>
+constexpr bool fills() {
+    return sizeof(S) == 4 && TM != T_INT64;
+}
+
 // A node's entry in the table of the nodes to update: its place in the tile,
 // its exchange cell, and whether the row above (below) it is the bottom (top)
 // one of a tile that wraps around.
@@ -273,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint2* ghost = reinterpret_cast<uint2*>(nxt + buf);
     unsigned* halo_src = reinterpret_cast<unsigned*>(ghost + res_max_ghosts(R));
     unsigned* item = halo_src + max_halo;
-    unsigned short* halo_dst = reinterpret_cast<unsigned short*>(item + res_nodes(full, R.depth - 1));
+    unsigned short* halo_dst = reinterpret_cast<unsigned short*>(item + res_nodes(full, R.depth - 1) + kMaxFill);
     __shared__ int split_now[2][4];  // by the step's parity
     __shared__ int upto[kMaxDepth];  // nodes of the core and the shells up to d
     const int origin = pad_y * RS + pad_x;  // node (0, 0), population 0, in a buffer
@@ -282,14 +289,21 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const bool wraps = res_wraps(R, pery);
     const int around = (h - 1) * RS;  // from the bottom row to the top row
-    const int n_core = w * h, n_edge = res_edges(R, t), n_items = res_nodes(t, R.depth - 1);
-    for (int q = tid; q < n_items; q += T) {
+    // (fills(): the first of the other nodes is entered and updated more than
+    // once where that lets warps begin with the rows of a core whose inner
+    // columns are whole warps: shared-memory wavefronts of 900 x 300, 66 x 30 nodes a
+    // CTA, 5.0 -> 3.5 k a step, 4.2 -> 3.9 us in the total-energy mode; 700 x 200
+    // 2.9 -> 2.4)
+    const int n_core = w * h, n_edge = res_edges(R, t), n_nodes = res_nodes(t, R.depth - 1);
+    const int fill = fills<S, TM>() ? res_fill(R, t) : 0, n_items = n_nodes + fill;
+    for (int e = tid; e < n_items; e += T) {
+        const int q = e < n_edge ? e : max(e - fill, n_edge);
         int c, r;
         if (q < n_core)
             res_core_node(R, t, q, &c, &r);
         else
             res_shell_node(t, q - n_core, &c, &r);
-        item[q] = (unsigned)(origin + r * RS + c) | (q < n_edge ? res_cell(R, t, c, r) : kNoCell) << 16 |
+        item[e] = (unsigned)(origin + r * RS + c) | (q < n_edge ? res_cell(R, t, c, r) : kNoCell) << 16 |
                   (wraps && r == h - 1 ? kWrapUp : 0u) | (wraps && r == 0 ? kWrapDown : 0u);
     }
     const int n_halo = R.cells > 0 ? res_nodes(t, R.depth) - n_core : 0;
@@ -308,7 +322,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int dst = origin + g.r * RS + g.c, src = origin + g.sr * RS + g.sc;
         ghost[q] = make_uint2((unsigned)dst | (unsigned)src << 16, (unsigned)g.side | (unsigned)g.along << 2);
     }
-    if (tid < R.depth) upto[tid] = res_nodes(t, tid);
+    if (tid < R.depth) upto[tid] = res_nodes(t, tid) + fill;
     if (tid < 4) split_now[0][tid] = split_at(G, tid, A.level0 + 1);
     // the tile, ghost cells of the level included
     {
@@ -443,7 +457,7 @@ constexpr size_t kSmemMax = sizeof(S) == 4 ? 226 * 1024 : 113 * 1024;
 size_t smem_bytes(const ResPlan& R, size_t esize) {
     const ResTile full = res_full_tile(R);
     return 2 * (size_t)(R.bh + 2 * res_pad_y(R)) * 9 * R.pitch * esize + 8 * (size_t)res_max_ghosts(R) +
-           6 * (size_t)(res_nodes(full, R.depth) - R.bw * R.bh) + 4 * (size_t)res_nodes(full, R.depth - 1);
+           6 * (size_t)(res_nodes(full, R.depth) - R.bw * R.bh) + 4 * (size_t)(res_nodes(full, R.depth - 1) + kMaxFill);
 }
 
 template <typename S, int TM>
@@ -505,7 +519,7 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
                     R.pitch |= 1;
                 R.cells = res_cells(R);
                 const ResTile full = res_full_tile(R);
-                const int warps = (res_nodes(full, R.depth - 1) + 31) / 32;
+                const int warps = (res_nodes(full, R.depth - 1) + (fills<S, TM>() ? res_fill(R, full) : 0) + 31) / 32;
                 const int received = res_nodes(full, R.depth) - R.bw * R.bh;
                 if (f64) {
                     if (warps > kQuadGroups) continue;

@@ -108,6 +108,15 @@ LBM_PLAN_HD void res_core_node(const ResPlan& R, const ResTile& t, int k, int* c
 }
 
 constexpr unsigned kNoCell = 0x3fffu;
+// Entries to repeat after the edge nodes: where the inner columns are whole
+// warps, as many as let the rows begin a warp (whose 32 nodes then lie in 32
+// banks).
+constexpr int kMaxFill = 31;
+LBM_PLAN_HD int res_fill(const ResPlan& R, const ResTile& t) {
+    const int inner = t.w - res_edge_cols(R, t);
+    const int edges = res_edges(R, t);
+    return inner > 0 && inner % 32 == 0 && edges < t.w * t.h ? (32 - edges % 32) % 32 : 0;
+}
 // The exchange cell of core node (c, r), kNoCell for one that no CTA needs.
 LBM_PLAN_HD unsigned res_cell(const ResPlan& R, const ResTile& t, int c, int r) {
     const int n = R.depth;
