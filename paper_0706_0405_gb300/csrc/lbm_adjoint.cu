@@ -192,7 +192,7 @@ __device__ __forceinline__ void star_neighbours(const Grid<S>& G, int ix, int iy
 // nodes of the flattened grid per CTA: the FP64 adjoint is bound by the FP64
 // pipe (64 cycles a warp instruction on a quarter of an SM), so a small grid
 // wants its warps spread over all SMs (256 x 8, us a step: 20 with CTAs of
-// eight warps, 9.6 with one).  a: adjoint of level n + 1, abar: adjoint of
+// eight warps, 9.6 with one, 6.6 with k_adjoint_quad).  a: adjoint of level n + 1, abar: adjoint of
 // level n (interior of the padded layout; ghost cells are never read or
 // written).  taup[block] += sum over the block's nodes of the node tau terms
 // (per node in the storage precision, across nodes in FP64; the tau
@@ -240,6 +240,122 @@ __global__ void __launch_bounds__(32) k_adjoint(const S* __restrict__ f, const S
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tsum += __shfl_down_sync(0xffffffffu, tsum, o);
     if (threadIdx.x == 0) taup[blockIdx.x] += (double)tsum;
+}
+
+// The FP64 adjoint on small grids: four warps, on the four quarters of an SM,
+// share 32 nodes by population pairs, as the resident FP64 step does
+// (lbm_resident.cu).  Alone, a warp spends 150 x 64 cycles on them; here each
+// spends about 80, pair sums and linear combinations formed by one warp each
+// and handed over in shared memory, the rest of the backward pass by all.  The
+// operations are those of adjoint_collision and adjoint_star.
+__global__ void __launch_bounds__(128) k_adjoint_quad(const double* __restrict__ f, const double* __restrict__ a,
+                                                      double* __restrict__ abar, const Fp64Adjoint C,
+                                                      const Grid<double> G, long long level,
+                                                      double* __restrict__ taup) {
+    grid_dependency_wait();
+    grid_dependents_launch();
+    __shared__ double pf[2][4][32], pa[2][4][32], paf[4][32];  // [difference, sum] of f and a; products
+    __shared__ double m[12][32];
+    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+    const long long n = (long long)G.nx * G.ny;
+    const long long k = blockIdx.x * 32LL + lane;
+    const bool in = k < n;
+    const unsigned q = (unsigned)(in ? k : n - 1);  // small grids: 32 bits
+    const int iy = (int)(q / (unsigned)G.nx), ix = (int)(q % (unsigned)G.nx);
+    const size_t pl = (size_t)G.plane, c = cell(G, ix, iy);
+    int xl, xr, yd, yu;
+    star_neighbours(G, ix, iy, xl, xr, yd, yu);
+    // the pair's populations against and along its direction
+    const int lo = role == 0 ? 1 : role == 1 ? 2 : role == 2 ? 5 : 8, hi = role == 0 ? 3 : role == 1 ? 4 : role == 2 ? 7 : 6;
+    struct Star {
+        double a, l, r, d, u;
+    };
+    auto star = [&](int j) {
+        const double* p = a + j * pl;
+        return Star{p[c], xl >= 0 ? p[cell(G, xl, iy)] : 0.0, xr >= 0 ? p[cell(G, xr, iy)] : 0.0,
+                    yd >= 0 ? p[cell(G, ix, yd)] : 0.0, yu >= 0 ? p[cell(G, ix, yu)] : 0.0};
+    };
+    const double fl = f[lo * pl + c], fh = f[hi * pl + c], f0 = f[c], a0 = a[c];
+    const Star sl = star(lo), sh = star(hi), s0 = star(0);
+    pf[0][role][lane] = fh - fl;
+    pf[1][role][lane] = fl + fh;
+    pa[0][role][lane] = sh.a - sl.a;
+    pa[1][role][lane] = sl.a + sh.a;
+    paf[role][lane] = fma_(sh.a, fh, sl.a * fl);
+    __syncthreads();
+    auto fd = [&](int r) { return pf[0][r][lane]; };
+    auto fs = [&](int r) { return pf[1][r][lane]; };
+    auto Q = [&](int r) { return pa[0][r][lane]; };
+    auto P = [&](int r) { return pa[1][r][lane]; };
+    if (role == 0) {
+        const double rho = (f0 + (fs(0) + fs(1))) + (fs(2) + fs(3));
+        m[0][lane] = rho;
+        m[1][lane] = fp64_rcp(rho);
+    } else if (role == 1) {
+        m[2][lane] = fma_(C.kap, fd(2) + fd(3), fd(0));
+        m[3][lane] = fma_(C.kap, fd(2) - fd(3), fd(1));
+        m[4][lane] = fp64_energy(C, f0, fs(0) + fs(1), fs(2) + fs(3));
+    } else if (role == 2) {
+        const double S1 = P(0) + P(1), S5 = P(2) + P(3);
+        m[5][lane] = fma_(C.k0, a0, fma_(C.a1p, S1, C.a5p * S5));
+        m[6][lane] = fma_(C.a1q, S1, C.a5q * S5);
+        m[7][lane] = fma_(C.a1r, S1, C.a5r * S5);
+    } else {
+        m[8][lane] = Q(2) + Q(3);
+        m[9][lane] = Q(2) - Q(3);
+        m[10][lane] = C.k5h * (P(2) - P(3));
+        m[11][lane] = fma_(a0, f0, (paf[0][lane] + paf[1][lane]) + (paf[2][lane] + paf[3][lane]));
+    }
+    __syncthreads();
+    const double rho = m[0][lane], inv = m[1][lane], gx = m[2][lane], gy = m[3][lane];
+    const double Qp = m[8][lane], Qm = m[9][lane], W = m[10][lane];
+    const double Ux = gx * inv, Uy = gy * inv;
+    const double qr = fma_(Ux, Ux, Uy * Uy);
+    const double T = fma_(-C.t1, qr, m[4][lane] * inv);
+    const double V = fma_(C.vp, T, qr);
+    const double B1 = fma_(C.b1v, V, C.b1c), B5 = fma_(C.b5v, V, C.b5c);
+    const double dV = fma_(C.b1v, fma_(gx, Q(0), gy * Q(1)), C.b5v * fma_(gx, Qp, gy * Qm));
+    const double v = dV * inv;
+    const double de = fma_(C.vp, v, m[5][lane]);
+    const double dq = fma_(-C.t1, de, v + m[6][lane]);
+    const double X = fma_(C.h1, P(0), dq), Y = fma_(C.h1, P(1), dq);
+    const double ex = fma_(Ux, X, Uy * W), ey = fma_(Uy, Y, Ux * W);
+    const double dx = fma_(2.0, ex, fma_(B1, Q(0), B5 * Qp)), dy = fma_(2.0, ey, fma_(B1, Q(1), B5 * Qm));
+    const double dr = fma_(-Ux, ex, fma_(-Uy, ey, fma_(-V, v, m[7][lane])));
+    const bool edge = ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1;
+    // population j from its collision term and star, with the ghost links
+    auto store = [&](int j, double g, const Star& s) {
+        double r = adjoint_star(C, j, g, s.a, s.l, s.r, s.d, s.u);
+        if (edge) {
+            auto link = [&](int side, int along, int weight, int mirrored) {
+                const int kind = kind_at(G, side, along, level);
+                if (kind == BC_OUTFLOW) r = fma_(C.w[j][weight], s.a, r);
+                if (kind == BC_REFLECT) r = fma_(C.w[mirrored][weight], a[mirrored * pl + c], r);
+            };
+            if (ix == 0) link(S_LEFT, iy, 2, mirror_x(j));
+            if (ix == G.nx - 1) link(S_RIGHT, iy, 1, mirror_x(j));
+            if (iy == 0) link(S_BOTTOM, ix, 4, mirror_y(j));
+            if (iy == G.ny - 1) link(S_TOP, ix, 3, mirror_y(j));
+        }
+        if (in) abar[j * pl + c] = r;
+    };
+    if (role < 2) {
+        const double c1 = fma_(C.t1, de, dr), d = role == 0 ? dx : dy;
+        store(lo, c1 - d, sl);
+        store(hi, c1 + d, sh);
+        if (role == 1) store(0, fma_(C.te, de, dr), s0);
+    } else {
+        const double c5 = fma_(C.t2, de, dr), d = role == 2 ? dx + dy : dx - dy;
+        store(lo, fma_(-C.kap, d, c5), sl);
+        store(hi, fma_(C.kap, d, c5), sh);
+    }
+    if (role == 0) {  // the node's tau term, summed over the 32 nodes
+        const double L = rho * fma_(dx, Ux, fma_(dy, Uy, fma_(de, fma_(C.t1, qr, T), dr)));
+        double t = in ? fma_(L, C.inv_omega, -m[11][lane]) : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) taup[blockIdx.x] += t;
+    }
 }
 
 // Periodic ghost cells of an adjoint level written by something other than
@@ -441,11 +557,19 @@ __global__ void k_feq_vjp(const S* __restrict__ r, const S* __restrict__ ux, con
 }
 }  // namespace
 
+// Up to 64 nodes an SM a node's chain of FP64 instructions is the step's time;
+// larger grids keep the pipe busy with a warp to 32 nodes, and fewer
+// instructions in all (us a step of lbm_adjoint_step with every level
+// recorded, four warps / one: 256 x 8 8.8 / 12.9, 512 x 16 10.9 / 12.9, 160 x 100
+// 19.8 / 17.0).
+constexpr long long kQuadNodes = 64 * 152;
+
 template <typename S, int TM>
 cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const AdjointModel<S>& C, const Grid<S>& G,
                            long long level, double* taup, cudaStream_t st) {
+    const long long n = (long long)G.nx * G.ny;
     cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(blocks_for((long long)G.nx * G.ny, 32));
+    lc.gridDim = dim3(blocks_for(n, 32));
     lc.blockDim = dim3(32);
     lc.stream = st;
     cudaLaunchAttribute at[1];
@@ -453,6 +577,12 @@ cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const AdjointModel<S
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
+    if constexpr (sizeof(S) == 8) {
+        if (n <= kQuadNodes) {
+            lc.blockDim = dim3(128);
+            return cudaLaunchKernelEx(&lc, k_adjoint_quad, f, a, abar, C, G, level, taup);
+        }
+    }
     return cudaLaunchKernelEx(&lc, k_adjoint<S, TM>, f, a, abar, C, G, level, taup);
 }
 
