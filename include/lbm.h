@@ -394,8 +394,10 @@ lbm_status lbm_batch_info(const lbm_batch* batch, int* grid, int* ntiles, int* g
  * shared memory (halo of `block` columns each side, recomputed), so DRAM
  * traffic and grid barriers drop by that factor; npt is then ignored.  If all
  * problems have two or all four rows, periodic in y, the columns are held in
- * registers instead, on as many CTAs as are resident for a full wave, at most
- * grid otherwise.
+ * registers instead; a full wave is then as many CTAs as are resident and have
+ * work, and a larger grid (up to the shared-memory kernel's full wave, where
+ * that is the larger one) launches that many.  lbm_batch_get_launch,
+ * lbm_batch_info and lbm_batch_autotune give the CTAs that are launched.
  * block = 0 or 1 is the one-step tile kernel.  Every shape computes the same
  * bits.  Setting a shape drops the captured graph (the next lbm_batch_step
  * captures a new one). */

@@ -48,6 +48,7 @@ struct lbm_batch {
     size_t strip_cap = 0;         // entries it holds
     int strip_rounds = 0;
     int strip_ns = 0, strip_grid = 0;  // steps a pass and CTAs the plan was made for
+    int strip_full[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // CTAs of a full wave per steps a pass (0: not planned yet)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int graph_n = -1;
@@ -84,31 +85,42 @@ bool batch_neighbour_lists(const lbm_batch* b, int grid, std::vector<int>& out) 
                                  [&](int t) { return batch_tile_owner(t, n, grid); }, kBatchMaxNbr, out);
 }
 
-// Full wave of a blocking launch, in CTAs of the shared-memory kernel.
+// Full wave of the shared-memory blocking kernel.
 int tb_full(const lbm_batch* b, int ns) {
     return b->tb_max_grid[ns] < b->nsegs ? b->tb_max_grid[ns] : b->nsegs;
 }
 
-// CTAs of a strip launch: a full wave for a full wave, else the chosen grid or
-// as many of it as are resident.
-int strip_launch_grid(const lbm_batch* b) {
-    return b->grid < b->strip_max && b->grid != tb_full(b, b->block) ? b->grid : b->strip_max;
-}
-
-// Make the strip plan match the current steps a pass and grid.
-cudaError_t batch_prepare_strips(lbm_batch* b) {
-    const int grid = strip_launch_grid(b);
-    if (b->strip_ns == b->block && b->strip_grid == grid) return cudaSuccess;
+// Plan the strips of `ns` steps a pass for at most `grid` CTAs; `ctas` is how
+// many of them get work, the grid to launch (a plan for that many is the same
+// plan).
+int plan_strips(const lbm_batch* b, int ns, int grid, std::vector<StripWarp>& plan, int* ctas) {
     std::vector<int> nx;
     for (const lbm_ctx* c : b->ctx) nx.push_back(c->gf.nx);
+    const int rounds = strip_plan((int)nx.size(), nx.data(), ns, grid, kStripWarps, plan);
+    *ctas = std::min(grid, rounds);
+    return rounds;
+}
+
+// Full wave of a blocking launch.
+int blocking_full(lbm_batch* b, int ns) {
+    if (!b->strip_rows) return tb_full(b, ns);
     std::vector<StripWarp> plan;
-    const int rounds = strip_plan((int)nx.size(), nx.data(), b->block, grid, kStripWarps, plan);
+    if (b->strip_full[ns] == 0) plan_strips(b, ns, b->strip_max, plan, &b->strip_full[ns]);
+    return b->strip_full[ns];
+}
+
+// Make the strip plan match the current steps a pass and grid, which becomes
+// the number of CTAs with work.
+cudaError_t batch_prepare_strips(lbm_batch* b) {
+    if (b->strip_ns == b->block && b->strip_grid == b->grid) return cudaSuccess;
+    std::vector<StripWarp> plan;
+    const int rounds = plan_strips(b, b->block, b->grid, plan, &b->grid);
     if (plan.size() > b->strip_cap) return cudaErrorInvalidValue;
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_strips, plan.data(), sizeof(StripWarp) * plan.size(), cudaMemcpyHostToDevice);
     b->strip_ns = e == cudaSuccess ? b->block : 0;
-    b->strip_grid = grid;
+    b->strip_grid = b->grid;
     b->strip_rounds = rounds;
     return e;
 }
@@ -133,8 +145,7 @@ cudaError_t batch_launch(lbm_batch* b, int n) {
         constexpr int TM = decltype(tm)::value;
         if (b->block > 1 && b->strip_rows)
             return launch_strip<TM>(b->d_probs, b->d_strips, b->strip_rounds, b->strip_rows, n, b->block, b->d_level,
-                                    b->d_bar, b->d_bar + 1, b->d_bar + 2, b->d_status, strip_launch_grid(b),
-                                    b->stream);
+                                    b->d_bar, b->d_bar + 1, b->d_bar + 2, b->d_status, b->grid, b->stream);
         if (b->block > 1)
             return launch_batch_tb<TM>(b->d_probs, b->d_segs, b->nsegs, n, b->block, b->rows_max, b->d_level,
                                        b->d_bar, b->d_bar + 1, b->d_status, b->grid, b->stream);
@@ -500,7 +511,7 @@ extern "C" {
 
 lbm_status lbm_batch_set_launch(lbm_batch* b, const lbm_batch_launch* l) {
     if (!b || !l) return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: NULL argument");
-    int full = 0;
+    int full = 0, most = 0;
     if (l->block > 1) {
         if (l->block != 3 && l->block != 5 && l->block != 7)
             return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: block must be 0, 1, 3, 5 or 7");
@@ -508,20 +519,22 @@ lbm_status lbm_batch_set_launch(lbm_batch* b, const lbm_batch_launch* l) {
             return bfail(b, LBM_E_INVAL,
                          "lbm_batch_set_launch: temporal blocking needs problems of at most " +
                              std::to_string(kBatchTbRowsMax) + " rows and no periodic x sides");
-        full = tb_full(b, l->block);
+        full = blocking_full(b, l->block);
         if (full < 1) return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: the blocking kernel does not fit");
+        // every grid that the shared-memory kernel takes is taken
+        most = std::max(full, tb_full(b, l->block));
     } else {
         if (l->block < 0) return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: block must be 0, 1, 3, 5 or 7");
         if (l->npt != 1 && l->npt != 2) return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: npt must be 1 or 2");
-        full = b->max_grid[l->npt] < b->ntiles ? b->max_grid[l->npt] : b->ntiles;
+        most = full = b->max_grid[l->npt] < b->ntiles ? b->max_grid[l->npt] : b->ntiles;
     }
-    if (l->grid < 0 || l->grid > full)
-        return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: grid must lie in [0, " + std::to_string(full) + "]");
+    if (l->grid < 0 || l->grid > most)
+        return bfail(b, LBM_E_INVAL, "lbm_batch_set_launch: grid must lie in [0, " + std::to_string(most) + "]");
     cudaSetDevice(b->device);
     cudaStreamSynchronize(b->stream);
     b->block = l->block > 1 ? l->block : 0;
     b->npt = l->block > 1 ? 1 : l->npt;
-    b->grid = l->grid == 0 ? full : l->grid;
+    b->grid = l->grid == 0 ? full : std::min(l->grid, full);
     batch_drop_graph(b);
     if (b->block > 1 && batch_prepare_sync(b) != cudaSuccess) {
         cudaGetLastError();
@@ -597,7 +610,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps, lbm_batch_launch* best, d
     }
     if (b->tb_ok)
         for (int ns = 3; ns <= 7; ns += 2) {
-            const int full = tb_full(b, ns);
+            const int full = blocking_full(b, ns);
             if (full >= 1) cand[nc++] = {1, full, ns};
         }
     // save every problem's current level, the level counter and the status

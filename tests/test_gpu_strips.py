@@ -47,3 +47,52 @@ def test_columns_in_registers_equal_problems_stepped_alone(prec, rows):
             lat.init(*fl).step(60)
             want = lat.get_f().cpu().numpy()
         assert np.isfinite(want).all() and np.array_equal(g, want), (p.nx, p.sides)
+
+
+def _launched(run, kernel):
+    """CTAs of the launches of `kernel` during run(), as the profiler recorded
+    them (its first session of a process may record nothing)."""
+    import json
+    import tempfile
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    grids = []
+    for _ in range(2):
+        if not grids:
+            with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as prof:
+                run()
+                torch.cuda.synchronize()
+            with tempfile.NamedTemporaryFile(suffix=".json") as f:
+                prof.export_chrome_trace(f.name)
+                events = json.load(open(f.name))["traceEvents"]
+            grids = [e["args"]["grid"][0] for e in events if e.get("cat") == "kernel" and kernel in e["name"]]
+    return grids
+
+
+@pytest.mark.parametrize("rows,count", [(4, 256), (4, 12), (2, 40)])
+def test_the_launch_shape_reported_is_the_one_launched(rows, count):
+    """A full wave, and every smaller grid, half the kernel's own and those
+    around the shared-memory kernel's full wave (one segment of 128 columns a
+    CTA) among them: get_launch and info give the CTAs launched, never more
+    than were asked for, and a full wave no more than there are CTAs' worth of
+    work (a column at least to each)."""
+    st = (1.0, 0.3, 0.05, 1.0)
+    probs = [W.uniform(100 + 7 * k % 300, rows, st, dx=DX, sides=(O, O, P, P)) for k in range(count)]
+    fields = [W.initial_fields(p, seed=k, sigma=0.01) for k, p in enumerate(probs)]
+    segments = sum((p.nx + 127) // 128 for p in probs)
+    with lbm.Batch(probs, "fp32_cons") as b:
+        b.init(fields).set_launch(1, 0, 5)
+        full = b.get_launch()[1]
+        for want in sorted({1, 7, full // 2, min(segments, full), min(304, full), full - 1, full}):
+            b.set_launch(1, want, 5)
+            npt, grid, block = b.get_launch()
+            assert (npt, block) == (1, 5) and 1 <= grid <= want and b.info()[0] == grid
+            assert set(_launched(lambda: b.step(5), "k_strip")) == {grid}, want
+        with pytest.raises(lbm.LbmError) as ei:
+            b.set_launch(1, 10 ** 6, 5)
+        assert ei.value.status == lbm.LBM_E_INVAL and b.get_launch() == (npt, grid, block)
+        (npt, grid, block), _ = b.autotune(steps=5)
+        assert (npt, grid, block) == b.get_launch()
+        if block:
+            assert grid == b.info()[0] and set(_launched(lambda: b.step(block), "k_strip")) == {grid}
+    assert full <= sum(p.nx for p in probs)
