@@ -294,6 +294,20 @@ typedef struct lbm_launch {
 lbm_status lbm_set_launch(lbm_ctx* ctx, const lbm_launch* launch);
 lbm_status lbm_get_launch(const lbm_ctx* ctx, lbm_launch* launch);
 
+/* Several steps per launch on small grids (lbm_step): the CTAs of such a
+ * launch (0 if the grid takes a launch a step), the steps between their
+ * exchanges, and the launches queued so far by lbm_step and lbm_adjoint_step.
+ * Outputs may be NULL.
+ *
+ * lbm_plant_stall: failure injection for tests, on the host side.  While on is
+ * not zero, such launches leave out their last CTA, so the bounded waits of
+ * those next to it (lbm_batch_set_wait_limit) run out, all CTAs leave and
+ * LBM_E_TIMEOUT is reported; nothing faults or hangs.  lbm_init makes the
+ * context usable again.  LBM_E_STATE if the context has no launch whose CTAs
+ * exchange. */
+lbm_status lbm_resident_info(const lbm_ctx* ctx, int* ctas, int* depth, long long* launches);
+lbm_status lbm_plant_stall(lbm_ctx* ctx, int on);
+
 /* Time every available launch shape for `steps` steps each (CUDA events on
  * the context's stream, after one untimed step), keep the fastest, and
  * restore the state and step counter the context had before.  Writes the
@@ -433,7 +447,8 @@ lbm_status lbm_batch_autotune(lbm_batch* batch, int steps, lbm_batch_launch* bes
  * lbm_batch_init makes the batch usable again.
  *
  * lbm_batch_set_wait_limit: that bound in seconds, (0, 60], for every batch
- * of the current device (default 2 s); converted to SM cycles at the
+ * of the current device and for the launches of several steps of a small grid
+ * (lbm_step) there (default 2 s); converted to SM cycles at the
  * device's nominal clock.  LBM_E_INVAL outside the range.
  *
  * lbm_batch_plant_stall: failure injection for tests, on the host side.

@@ -464,7 +464,11 @@ cudaError_t step_resident(lbm_ctx* c, int n, const char* fin, char* seg, long lo
         A.sync = c->d_res;
         A.xch = c->d_xch;
         A.status = c->d_status;
-        return launch_resident<S, decltype(tm)::value>(c->res, model_of<S>(c), c->f64, grid_of<S>(c), A, c->stream);
+        const cudaError_t e =
+            launch_resident<S, decltype(tm)::value>(c->res, model_of<S>(c), c->f64, grid_of<S>(c), A, c->res_stall,
+                                                    c->stream);
+        if (e == cudaSuccess) ++c->res_launches;
+        return e;
     });
 }
 
@@ -1158,6 +1162,22 @@ lbm_status lbm_get_launch(const lbm_ctx* c, lbm_launch* l) {
     l->tx = c->cfg.tx;
     l->ring = c->cfg.ring;
     l->grid = c->cfg.grid;
+    return LBM_OK;
+}
+
+lbm_status lbm_resident_info(const lbm_ctx* c, int* ctas, int* depth, long long* launches) {
+    if (!c) return fail(nullptr, LBM_E_INVAL, "lbm_resident_info: NULL context");
+    if (ctas) *ctas = c->res_ok ? c->res.px * c->res.py : 0;
+    if (depth) *depth = c->res_ok ? c->res.depth : 0;
+    if (launches) *launches = c->res_launches;
+    return LBM_OK;
+}
+
+lbm_status lbm_plant_stall(lbm_ctx* c, int on) {
+    if (!c) return fail(nullptr, LBM_E_INVAL, "lbm_plant_stall: NULL context");
+    if (on && (!c->res_ok || c->res.cells == 0))
+        return fail(c, LBM_E_STATE, "lbm_plant_stall: no launch of this context exchanges between CTAs");
+    c->res_stall = on != 0;
     return LBM_OK;
 }
 

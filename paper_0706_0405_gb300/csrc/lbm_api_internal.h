@@ -56,6 +56,8 @@ struct lbm_ctx {
     bool res_ok = false;
     unsigned* d_res = nullptr;  // its tag counter and leave count
     ResWord* d_xch = nullptr;   // its exchange buffer (behind f[1], or behind the status words)
+    bool res_stall = false;     // lbm_plant_stall
+    long long res_launches = 0; // launches queued so far
     CUtensorMap tmap[2];  // FP32: tensor maps of the two level buffers (tile kernel)
     bool tmap_ok = false;
     // adjoint: checkpoints every ck_every steps from level ck_base

@@ -493,7 +493,8 @@ int batch_tile_owner(int t, int ntiles, int grid) {
 }
 
 cudaError_t batch_set_wait_cycles(long long cycles) {
-    const cudaError_t e = strip_set_wait_cycles(cycles);
+    cudaError_t e = strip_set_wait_cycles(cycles);
+    if (e == cudaSuccess) e = resident_set_wait_cycles(cycles);
     return e != cudaSuccess ? e : cudaMemcpyToSymbol(g_wait_cycles, &cycles, sizeof(cycles));
 }
 

@@ -98,13 +98,16 @@ struct ResRun {
     unsigned* sync;              // tag counter, count of CTAs that have left (both zero at first)
     unsigned* status;
 };
+// Bound of its polls, in SM cycles (default ~2 s).
+cudaError_t resident_set_wait_cycles(long long cycles);
 // False if the grid does not fit.
 template <typename S, int TM>
 bool resident_plan(int nx, int ny, ResPlan* plan);
-// M64: the constants of FP64 steps (unused otherwise).
+// M64: the constants of FP64 steps (unused otherwise).  stall: a launch whose
+// polls run out (lbm_plant_stall; more than one CTA).
 template <typename S, int TM>
 cudaError_t launch_resident(const ResPlan& R, const Model<S>& M, const Fp64Step& M64, const Grid<S>& G,
-                            const ResRun<S>& A, cudaStream_t st);
+                            const ResRun<S>& A, bool stall, cudaStream_t st);
 
 // f = f^eq(fields) on the interior (fields are ny x nx, storage type), and the
 // ghost layer for time level 0.

@@ -43,15 +43,17 @@
 //  * the last two steps also write their levels to the context's buffers,
 //    ghosts included, so that every call leaves what the one-step kernels
 //    would have left.
-// Polls are bounded: on give-up the CTA raises ST_TIMEOUT and leaves, and so
-// do the others, which watch that word while they poll.
+// Polls are bounded (lbm_batch_set_wait_limit): on give-up the CTA raises
+// ST_TIMEOUT and leaves, and so do the others, which watch that word while
+// they poll.
 #include "lbm_launch.h"
 
 namespace lbm {
 
 namespace {
-constexpr long long kPollCycles = 4000000000LL;  // ~2 s, then a poll gives up
-constexpr int kMaxDepth = 4;                     // steps between exchanges at most
+// SM cycles a poll lasts before it gives up, ~2 s at 2 GHz (resident_set_wait_cycles)
+__device__ long long g_poll_cycles = 4000000000LL;
+constexpr int kMaxDepth = 4;  // steps between exchanges at most
 
 __device__ __forceinline__ void st_word(ResWord* p, unsigned a, unsigned b, unsigned c, unsigned tag) {
     asm volatile(
@@ -235,7 +237,7 @@ __device__ __forceinline__ bool receive(const ResWord* src, unsigned tag, S* dst
         if ((spins & 63) == 63) {
             const long long t = clock64();
             if (t0 == 0) t0 = t;
-            if (t - t0 > kPollCycles || (*(volatile const unsigned*)status & ST_TIMEOUT)) return false;
+            if (t - t0 > g_poll_cycles || (*(volatile const unsigned*)status & ST_TIMEOUT)) return false;
         }
     }
 #pragma unroll
@@ -560,11 +562,15 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
     return true;
 }
 
+// A stalled launch leaves its last CTA out, which makes the halves of the
+// exchange buffer smaller by its cells.  The cells that the others then wait
+// for still lie in the buffer: behind their half, where there are tags of the
+// other parity, or of earlier launches.
 template <typename S, int TM>
 cudaError_t launch_resident(const ResPlan& R, const Model<S>& M, const Fp64Step& M64, const Grid<S>& G,
-                            const ResRun<S>& A, cudaStream_t st) {
+                            const ResRun<S>& A, bool stall, cudaStream_t st) {
     cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(R.px * R.py);
+    lc.gridDim = dim3(R.px * R.py - (stall ? 1 : 0));
     lc.blockDim = dim3(R.threads);
     lc.dynamicSmemBytes = R.smem;
     lc.stream = st;
@@ -579,10 +585,14 @@ cudaError_t launch_resident(const ResPlan& R, const Model<S>& M, const Fp64Step&
         return cudaLaunchKernelEx(&lc, kernel_of<S, TM>(), M64, G, R, A);
 }
 
+cudaError_t resident_set_wait_cycles(long long cycles) {
+    return cudaMemcpyToSymbol(g_poll_cycles, &cycles, sizeof(cycles));
+}
+
 #define LBM_RES_INST(S, TM)                                                                              \
     template bool resident_plan<S, TM>(int, int, ResPlan*);                                              \
     template cudaError_t launch_resident<S, TM>(const ResPlan&, const Model<S>&, const Fp64Step&,        \
-                                                const Grid<S>&, const ResRun<S>&, cudaStream_t);
+                                                const Grid<S>&, const ResRun<S>&, bool, cudaStream_t);
 LBM_RES_INST(double, T_PLAIN)
 LBM_RES_INST(float, T_INT32)
 LBM_RES_INST(float, T_INT64)

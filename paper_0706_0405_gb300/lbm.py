@@ -33,6 +33,7 @@ EXPORTS = ("lbm_create", "lbm_destroy", "lbm_last_error", "lbm_init", "lbm_step"
            "lbm_batch_step", "lbm_batch_sync", "lbm_batch_problem", "lbm_batch_info",
            "lbm_probe_rates", "lbm_vn_scan", "lbm_batch_set_launch", "lbm_batch_get_launch",
            "lbm_batch_autotune", "lbm_probe_tile_copy", "lbm_batch_set_wait_limit", "lbm_batch_plant_stall",
+           "lbm_resident_info", "lbm_plant_stall",
            "lbm_inject_alloc_failure", "lbm_level_bytes")
 LBM_FLAG_NONPHYSICAL, LBM_FLAG_TIMEOUT, LBM_FLAG_T_NONPOSITIVE = 1, 2, 4
 
@@ -127,6 +128,9 @@ def load():
         "lbm_probe_tile_copy": ([ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double)],
                                 ctypes.c_int),
         "lbm_batch_set_wait_limit": ([ctypes.c_double], ctypes.c_int),
+        "lbm_resident_info": ([ctx, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
+                               ctypes.POINTER(ctypes.c_longlong)], ctypes.c_int),
+        "lbm_plant_stall": ([ctx, ctypes.c_int], ctypes.c_int),
         "lbm_batch_plant_stall": ([_VP, ctypes.c_int], ctypes.c_int),
         "lbm_inject_alloc_failure": ([ctypes.c_longlong], ctypes.c_int),
         "lbm_batch_create": ([ctypes.c_int, ctypes.POINTER(lbm_problem), ctypes.c_int, _VP,
@@ -448,6 +452,17 @@ def lbm_batch_set_wait_limit(seconds: float) -> None:
 def lbm_inject_alloc_failure(after: int) -> None:
     """The library's device allocation after the next `after` ones fails (after < 0: off)."""
     load().lbm_inject_alloc_failure(int(after))
+
+
+def lbm_resident_info(ctx):
+    """(CTAs, steps between exchanges, launches so far) of the launches of several steps."""
+    n, d, l = ctypes.c_int(), ctypes.c_int(), ctypes.c_longlong()
+    _check(ctx, load().lbm_resident_info(ctx, ctypes.byref(n), ctypes.byref(d), ctypes.byref(l)))
+    return n.value, d.value, l.value
+
+
+def lbm_plant_stall(ctx, on: bool):
+    return _check(ctx, load().lbm_plant_stall(ctx, int(on)))
 
 
 def lbm_batch_plant_stall(b, cta: int):

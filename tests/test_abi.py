@@ -166,3 +166,9 @@ def test_batch_wait_limit_rejects_out_of_range(seconds):
 
 def test_batch_plant_stall_on_null_batch_fails_cleanly():
     assert lbm.load().lbm_batch_plant_stall(None, 0) == lbm.LBM_E_INVAL
+
+
+def test_small_grid_hooks_on_a_null_context_fail_cleanly():
+    lib = lbm.load()
+    assert lib.lbm_resident_info(None, None, None, None) == lbm.LBM_E_INVAL
+    assert lib.lbm_plant_stall(None, 0) == lbm.LBM_E_INVAL

@@ -172,3 +172,100 @@ def test_a_captured_call_of_several_steps_replays():
     with lbm.Lattice(p, "fp32_cons") as ref:
         assert torch.equal(ref.init(*fields).step(22).get_f(), got)
     lat.close()
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(nx, ny, prec) for nx, ny in RESIDENT[:-1]
+                                        for prec in ("fp32", "fp32_t64", "fp32_tdf", "fp32_cons")] +
+                         [(nx, ny, "fp64") for nx, ny in [(1, 1), (33, 4), (8, 4), (97, 5), (305, 2), (120, 80)]])
+def test_small_grids_take_one_launch_for_several_steps(nx, ny, prec):
+    """The grids above whose steps are compared do take that launch, for three
+    steps or more and with the default launch shape only."""
+    p, fields = _problem(nx, ny, INFLOW)
+    with lbm.Lattice(p, prec) as lat:
+        count = lambda: lbm.lbm_resident_info(lat.ctx)[2]
+        lat.init(*fields)
+        assert lbm.lbm_resident_info(lat.ctx)[0] > 0 and count() == 0
+        assert [lat.step(n) and count() for n in (1, 2, 3, 11)] == [0, 0, 1, 2]
+        lbm.lbm_record(lat.ctx, 5)
+        lat.step(12)  # five steps to each recorded level, two more
+        assert count() == 4
+        lbm.lbm_set_launch(lat.ctx, 0, 0, 0, 1)
+        lat.step(5)
+        assert count() == 4
+        lat.sync()
+
+
+def test_larger_grids_take_a_launch_a_step():
+    p, fields = _problem(*RESIDENT[-1], WALLS)
+    with lbm.Lattice(p, "fp32") as lat:
+        lat.init(*fields).step(5).sync()
+        assert lbm.lbm_resident_info(lat.ctx) == (0, 0, 0)
+        with pytest.raises(lbm.LbmError) as ei:
+            lbm.lbm_plant_stall(lat.ctx, True)
+        assert ei.value.status == lbm.LBM_E_STATE
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(2000, 4, "fp32_tdf"), (400, 100, "fp32_cons"), (400, 4, "fp64"),
+                                        (120, 80, "fp64"), (1240, 310, "fp32_t64")])
+def test_a_value_that_never_arrives_times_out_and_the_context_recovers(nx, ny, prec):
+    """Failure made on the host: the launches lack a CTA, so that those next
+    to it wait for values that nobody publishes.  Their bounded waits run out
+    (0.2 s here), all CTAs leave, LBM_E_TIMEOUT reaches the caller and stays
+    until lbm_init, after which the same context gives the bits of one that
+    never failed."""
+    import torch
+    p, fields = _problem(nx, ny, WALLS)
+    lbm.lbm_batch_set_wait_limit(0.2)
+    try:
+        with lbm.Lattice(p, prec) as lat, lbm.Lattice(p, prec) as ref:
+            for first in (3, 4, 7):  # the exchange buffer's halves in either order
+                lat.init(*fields).step(first)
+                lat.sync()
+                lbm.lbm_plant_stall(lat.ctx, True)
+                for n in (9, 4):  # the second launch finds the status already set
+                    lat.step(n)
+                    with pytest.raises(lbm.LbmError) as ei:
+                        lat.sync()
+                    assert ei.value.status == lbm.LBM_E_TIMEOUT
+                lbm.lbm_plant_stall(lat.ctx, False)
+            got = lat.init(*fields).step(25).get_f()
+            lat.sync()
+            assert torch.equal(ref.init(*fields).step(25).get_f(), got)
+    finally:
+        lbm.lbm_batch_set_wait_limit(2.0)
+
+
+def test_contexts_on_several_streams_at_once():
+    """Launches of several steps queued from one thread per context, each on a
+    stream of its own, beside other work on the device: the bits of each
+    context stepped alone."""
+    import threading
+    import torch
+    cases = [(2000, 4, "fp32_tdf"), (900, 300, "fp32_cons"), (400, 100, "fp32"), (400, 4, "fp64"),
+             (1024, 256, "fp32_t64"), (120, 80, "fp64")]
+    problems = [_problem(nx, ny, WALLS) for nx, ny, _ in cases]
+    want = []
+    for (p, fields), (_, _, prec) in zip(problems, cases):
+        with lbm.Lattice(p, prec) as lat:
+            want.append(lat.init(*fields).step(300).get_f())
+    got = [None] * len(cases)
+
+    def run(k):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            with lbm.Lattice(problems[k][0], cases[k][2]) as lat:
+                lat.init(*problems[k][1])
+                for _ in range(10):
+                    lat.step(30)
+                lat.sync()
+                got[k] = lat.get_f()
+
+    a = torch.ones((4096, 4096), device="cuda")
+    for _ in range(20):
+        a = a * 0.5 + 1.0
+    threads = [threading.Thread(target=run, args=(k,)) for k in range(len(cases))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for w, g in zip(want, got):
+        assert g is not None and torch.equal(w, g)
