@@ -455,8 +455,9 @@ lbm_status lbm_batch_autotune(lbm_batch* batch, int steps, lbm_batch_launch* bes
  * cta in [0, grid) adds to that CTA's neighbour list a counter that no CTA
  * ever advances, so its wait before its second step of the next launch runs
  * out (after the bound above) and the launch reports LBM_E_TIMEOUT; nothing
- * faults or hangs.  cta < 0 restores the lists.  LBM_E_STATE if the current
- * launch shape has no neighbour lists (temporal blocking, or lists too long);
+ * faults or hangs.  cta < 0 restores the lists.  Launch shapes without
+ * neighbour lists (temporal blocking, or lists too long) have their grid
+ * barriers miss an arrival instead, until lbm_batch_init or cta < 0.
  * LBM_E_INVAL for cta >= grid.  Synchronises the batch's stream. */
 lbm_status lbm_batch_set_wait_limit(double seconds);
 lbm_status lbm_batch_plant_stall(lbm_batch* batch, int cta);

@@ -565,16 +565,19 @@ lbm_status lbm_batch_plant_stall(lbm_batch* b, int cta) {
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess) e = batch_prepare_sync(b);
     if (e != cudaSuccess) return bfail(b, LBM_E_CUDA, std::string("lbm_batch_plant_stall: ") + cudaGetErrorString(e));
-    if (cta < 0) {  // back to the lists of the current grid
+    if (cta < 0) {  // back to the lists of the current grid, and to a barrier without arrivals
         b->nbr_grid = -1;
         e = batch_prepare_sync(b);
+        if (e == cudaSuccess) e = cudaMemset(b->d_bar, 0, 3 * sizeof(unsigned));
         batch_drop_graph(b);
         return e == cudaSuccess ? LBM_OK : bfail(b, LBM_E_CUDA, "lbm_batch_plant_stall: restoring the lists failed");
     }
-    if (b->block > 1 || !b->nbr_ok)
-        return bfail(b, LBM_E_STATE, "lbm_batch_plant_stall: the current launch shape has no neighbour lists");
     if (cta >= b->grid)
         return bfail(b, LBM_E_INVAL, "lbm_batch_plant_stall: cta must lie in [0, " + std::to_string(b->grid) + ")");
+    if (b->block > 1 || !b->nbr_ok) {  // grid barriers only: one arrival too few
+        e = cudaMemset(b->d_bar, 0xff, sizeof(unsigned));
+        return e == cudaSuccess ? LBM_OK : bfail(b, LBM_E_CUDA, "lbm_batch_plant_stall: setting the barrier failed");
+    }
     std::vector<int> lists;
     batch_neighbour_lists(b, b->grid, lists);
     int* row = lists.data() + (size_t)cta * kBatchMaxNbr;

@@ -120,7 +120,10 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
             if (threadIdx.x == 0) sRound = (int)(atomicAdd(ticket, 1u) - base);
             __syncthreads();
         }
-        for (int round = drawn ? sRound : (int)blockIdx.x; round < rounds;) {
+        // (unsigned: a launch that follows one that gave up may find the barrier's
+        // count in between, and a ticket drawn beside one that has been taken back
+        // to zero, which must not be a round)
+        for (int round = drawn ? sRound : (int)blockIdx.x; (unsigned)round < (unsigned)rounds;) {
             const StripWarp W = warps[(size_t)round * kStripWarps + w];
             const bool busy = W.prob >= 0;
             const BatchProb& P = probs[busy ? W.prob : 0];

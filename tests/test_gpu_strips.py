@@ -96,3 +96,38 @@ def test_the_launch_shape_reported_is_the_one_launched(rows, count):
         if block:
             assert grid == b.info()[0] and set(_launched(lambda: b.step(block), "k_strip")) == {grid}
     assert full <= sum(p.nx for p in probs)
+
+
+@pytest.mark.parametrize("rows,sides,grid,block", [(4, (O, O, P, P), 0, 7), (2, (O, O, P, P), 3, 3),
+                                                   (4, (O, O, P, P), 1, 5), (4, (O, O, R, R), 0, 5)])
+def test_a_barrier_that_misses_an_arrival_times_out_and_the_batch_recovers(rows, sides, grid, block):
+    """Failure made on the host: the grid barrier of a blocking launch
+    (columns in registers, rounds drawn by ticket or not; the last case in
+    shared memory) never completes.  Its bounded wait runs out (0.2 s here),
+    LBM_E_TIMEOUT reaches the caller, and after lbm_batch_init the same batch
+    gives each problem's own bits."""
+    probs = [W.uniform(nx, rows, (1.0, 0.3, 0.05, 1.0), dx=DX, sides=sides) for nx in WIDTHS]
+    fields = [W.initial_fields(p, seed=k, sigma=0.01) for k, p in enumerate(probs)]
+    lbm.lbm_batch_set_wait_limit(0.2)
+    try:
+        with lbm.Batch(probs, "fp32_cons") as b:
+            b.init(fields).set_launch(1, grid, block).step(block)
+            b.sync()
+            for restore in (False, True):
+                b.plant_stall(0)
+                for _ in range(2):  # the second launch finds the status already set
+                    b.step(2 * block)
+                    with pytest.raises(lbm.LbmError) as ei:
+                        b.sync()
+                    assert ei.value.status == lbm.LBM_E_TIMEOUT
+                if restore:
+                    b.plant_stall(-1)
+                b.init(fields).step(3 * block)
+                b.sync()
+                got = [b.get_f(k).cpu().numpy() for k in range(len(probs))]
+                for p, fl, g in zip(probs, fields, got):
+                    with lbm.Lattice(p, "fp32_cons") as lat:
+                        want = lat.init(*fl).step(3 * block).get_f().cpu().numpy()
+                    assert np.array_equal(g, want), p.nx
+    finally:
+        lbm.lbm_batch_set_wait_limit(2.0)
