@@ -260,7 +260,9 @@ lbm_status lbm_adjoint_seed(lbm_ctx* ctx, const void* qbar_rho, const void* qbar
  * checkpoints).  *dL_dtau (host, may be NULL) is incremented by the tau
  * derivative of these n steps, d out_i / d tau = -(dt / tau^2) (f^eq_i - f_i).
  * Afterwards the context's current level is k - n.  LBM_E_STATE without a
- * recording, LBM_E_INVAL if fewer than n steps are recorded. */
+ * recording, LBM_E_INVAL if fewer than n steps are recorded, LBM_E_TIMEOUT if a
+ * bounded wait gave up in these steps or before (abar is then not valid and
+ * *dL_dtau unchanged). */
 lbm_status lbm_adjoint_step(lbm_ctx* ctx, int n, void* abar, double* dL_dtau);
 
 /* Gradient with respect to the fields of an initial condition f = f^eq(q):

@@ -1077,9 +1077,11 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step: packing abar");
     if (!dev)
         LBM_CUDA(c, cudaMemcpyAsync(abar, c->d_astage, 9 * fb, cudaMemcpyDeviceToHost, c->stream), "copying abar out");
-    e = launch_sum(c->d_taup, np, c->h_tau, c->stream);
+    e = launch_sum(c->d_taup, np, c->h_tau, c->d_status, c->h_status, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint_step: summing the tau partials");
     LBM_CUDA(c, cudaStreamSynchronize(c->stream), "synchronising the stream");
+    if (*c->h_status & ST_TIMEOUT)
+        return fail(c, LBM_E_TIMEOUT, "lbm_adjoint_step: a bounded device wait gave up");
     if (dL_dtau) *dL_dtau += -(c->dt / (c->tau * c->tau)) * *c->h_tau;
     return LBM_OK;
 }

@@ -520,7 +520,8 @@ cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S
 }
 
 // Sum of n doubles by one CTA: strided partial sums, then a fixed tree.
-__global__ void __launch_bounds__(1024) k_sum(const double* __restrict__ v, int n, double* out) {
+__global__ void __launch_bounds__(1024) k_sum(const double* __restrict__ v, int n, double* out,
+                                              const unsigned* status, unsigned* out_status) {
     __shared__ double sh[32];
     double t = 0.0;
     for (int k = threadIdx.x; k < n; k += 1024) t += v[k];
@@ -532,12 +533,16 @@ __global__ void __launch_bounds__(1024) k_sum(const double* __restrict__ v, int 
         t = sh[threadIdx.x];
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) t += __shfl_down_sync(0xffffffffu, t, s);
-        if (threadIdx.x == 0) *out = t;
+        if (threadIdx.x == 0) {
+            *out = t;
+            *out_status = *status;
+        }
     }
 }
 
-cudaError_t launch_sum(const double* v, int n, double* out, cudaStream_t st) {
-    k_sum<<<1, 1024, 0, st>>>(v, n, out);
+cudaError_t launch_sum(const double* v, int n, double* out, const unsigned* status, unsigned* out_status,
+                       cudaStream_t st) {
+    k_sum<<<1, 1024, 0, st>>>(v, n, out, status, out_status);
     return cudaGetLastError();
 }
 

@@ -135,9 +135,10 @@ cudaError_t launch_conservation(const S* f, const Model<double>& M, const Grid<S
                                 unsigned* left, const unsigned* status, double* out, unsigned* out_status,
                                 cudaStream_t st);
 
-// out (page-locked host memory, valid once the stream has been synchronised)
-// = sum of v[0..n) in a fixed order.
-cudaError_t launch_sum(const double* v, int n, double* out, cudaStream_t st);
+// out = sum of v[0..n) in a fixed order, out_status = the health word `status`
+// (both page-locked host memory, valid once the stream has been synchronised).
+cudaError_t launch_sum(const double* v, int n, double* out, const unsigned* status, unsigned* out_status,
+                       cudaStream_t st);
 
 // Interior <-> dense 9 x ny x nx copies.
 template <typename S>

@@ -269,3 +269,35 @@ def test_contexts_on_several_streams_at_once():
         t.join()
     for w, g in zip(want, got):
         assert g is not None and torch.equal(w, g)
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(256, 8, "fp64"), (400, 100, "fp32_tdf")])
+def test_a_recomputation_that_gives_up_is_reported_by_the_adjoint(nx, ny, prec):
+    """The forward steps run through; the levels between the checkpoints are
+    recomputed by launches that lack a CTA.  lbm_adjoint_step returns
+    LBM_E_TIMEOUT and leaves the tau derivative alone; after lbm_init the same
+    context gives the gradient of one that never failed."""
+    import ctypes
+    import torch
+    p, fields = _problem(nx, ny, WALLS)
+
+    def gradient(lat, stall):
+        lat.init(*fields)
+        lbm.lbm_record(lat.ctx, 10)
+        lat.step(20).sync()
+        abar = torch.ones((9, ny, nx), dtype=lat.dtype, device="cuda")
+        dtau = ctypes.c_double(7.0)
+        if stall:
+            lbm.lbm_plant_stall(lat.ctx, True)
+        st = lbm.load().lbm_adjoint_step(lat.ctx, 20, ctypes.c_void_p(abar.data_ptr()), ctypes.byref(dtau))
+        lbm.load().lbm_plant_stall(lat.ctx, 0)
+        return st, dtau.value, abar
+
+    lbm.lbm_batch_set_wait_limit(0.2)
+    try:
+        with lbm.Lattice(p, prec) as lat, lbm.Lattice(p, prec) as ref:
+            assert gradient(lat, True)[:2] == (lbm.LBM_E_TIMEOUT, 7.0)
+            got, want = gradient(lat, False), gradient(ref, False)
+    finally:
+        lbm.lbm_batch_set_wait_limit(2.0)
+    assert got[0] == want[0] == lbm.LBM_OK and got[1] == want[1] != 7.0 and torch.equal(got[2], want[2])
