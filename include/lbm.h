@@ -36,7 +36,8 @@
  *    ABI.  lbm_last_error gives a message for the last failing call.
  *  - Health flags (sticky, cleared by lbm_init / lbm_set_f / lbm_load) record
  *    what the kernels saw in the levels they read: LBM_FLAG_NONPHYSICAL
- *    (rho <= 0 or a non-finite moment at some node) makes the next
+ *    (rho <= 0 or a non-finite moment at some node; in FP64 also a rho
+ *    outside [2^-1022, 2^1022) in a level that was stepped) makes the next
  *    synchronising call return LBM_E_NONPHYSICAL; LBM_FLAG_T_NONPOSITIVE
  *    (T <= 0 at some node) is informational only: the scheme passes through
  *    short episodes of T < 0 right behind strong shocks (e.g. the 1000:1 tube
