@@ -192,11 +192,11 @@ __device__ __forceinline__ void star_neighbours(const Grid<S>& G, int ix, int iy
 // nodes of the flattened grid per CTA: the FP64 adjoint is bound by the FP64
 // pipe (64 cycles a warp instruction on a quarter of an SM), so a small grid
 // wants its warps spread over all SMs (256 x 8, us a step: 20 with CTAs of
-// eight warps, 9.6 with one, 6.6 with k_adjoint_quad).  a: adjoint of level n + 1, abar: adjoint of
-// level n (interior of the padded layout; ghost cells are never read or
-// written).  taup[block] += sum over the block's nodes of the node tau terms
-// (per node in the storage precision, across nodes in FP64; the tau
-// derivative is -(dt / tau^2) times the total).
+// eight warps, 9.6 with one, 6.6 with k_adjoint_quad).  a: adjoint of level
+// n + 1, abar: adjoint of level n (interior of the padded layout; ghost cells
+// are never read or written).  taup[block] += sum over the block's nodes of the
+// node tau terms (per node in the storage precision, across nodes in FP64; the
+// tau derivative is -(dt / tau^2) times the total).
 template <typename S, int TM>
 __global__ void __launch_bounds__(32) k_adjoint(const S* __restrict__ f, const S* __restrict__ a,
                                                 S* __restrict__ abar, const AdjointModel<S> C,
@@ -247,7 +247,9 @@ __global__ void __launch_bounds__(32) k_adjoint(const S* __restrict__ f, const S
 // (lbm_resident.cu).  Alone, a warp spends 150 x 64 cycles on them; here each
 // spends about 80, pair sums and linear combinations formed by one warp each
 // and handed over in shared memory, the rest of the backward pass by all.  The
-// operations are those of adjoint_collision and adjoint_star.
+// operations are those of adjoint_collision and adjoint_star, but for the sum
+// of a_i f_i in the tau term, which is taken pair by pair: the tau derivative
+// has its own last bits.
 __global__ void __launch_bounds__(128) k_adjoint_quad(const double* __restrict__ f, const double* __restrict__ a,
                                                       double* __restrict__ abar, const Fp64Adjoint C,
                                                       const Grid<double> G, long long level,
@@ -562,7 +564,7 @@ __global__ void k_feq_vjp(const S* __restrict__ r, const S* __restrict__ ux, con
 // instructions in all (us a step of lbm_adjoint_step with every level
 // recorded, four warps / one: 256 x 8 8.8 / 12.9, 512 x 16 10.9 / 12.9, 160 x 100
 // 19.8 / 17.0).
-constexpr long long kQuadNodes = 64 * 152;
+constexpr int kQuadNodesPerSm = 64;
 
 template <typename S, int TM>
 cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const AdjointModel<S>& C, const Grid<S>& G,
@@ -578,7 +580,7 @@ cudaError_t launch_adjoint(const S* f, const S* a, S* abar, const AdjointModel<S
     lc.attrs = at;
     lc.numAttrs = 1;
     if constexpr (sizeof(S) == 8) {
-        if (n <= kQuadNodes) {
+        if (n <= (long long)kQuadNodesPerSm * device_sms()) {
             lc.blockDim = dim3(128);
             return cudaLaunchKernelEx(&lc, k_adjoint_quad, f, a, abar, C, G, level, taup);
         }

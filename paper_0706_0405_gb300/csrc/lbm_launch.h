@@ -50,6 +50,19 @@ inline int full_wave(int threads, size_t smem) {
     return v;
 }
 
+// SMs of the current device, cached in the same way.
+inline int device_sms() {
+    static std::atomic<int> cache[64];
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    const bool cached = dev >= 0 && dev < 64;
+    if (cached && (v = cache[dev].load(std::memory_order_relaxed)) > 0) return v;
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    if (v < 1) v = 1;
+    if (cached) cache[dev].store(v, std::memory_order_relaxed);
+    return v;
+}
+
 // Kernel variant and launch shape of the step (chosen by the host, see
 // lbm_tune in lbm.h).
 enum StepVariant : int { STEP_SIMPLE = 0, STEP_RING = 1, STEP_VEC = 2, STEP_TILE = 3 };
