@@ -197,9 +197,10 @@ lbm_status lbm_init(lbm_ctx* ctx, const void* rho, const void* ux, const void* u
  * Each step reads level k, writes level k + 1 into the other buffer and fills
  * that level's ghost layer for t = (k + 1) dt in the same kernel.  With the
  * default launch shape, small grids (FP32 modes: about 400 000 nodes, FP64:
- * 14 000) run n >= 3 steps in one cooperative launch that keeps the level in
- * shared memory and writes the last two levels to the buffers; the bits are
- * those of a launch a step. */
+ * 14 000) run n steps in one cooperative launch where n is large enough for
+ * that to be faster (4 to 17, lbm_resident_info); it keeps the level in shared
+ * memory and writes the last two levels to the buffers, and the bits are those
+ * of a launch a step. */
 lbm_status lbm_step(lbm_ctx* ctx, int n);
 
 /* Macroscopic fields of the current level (Eqs. e4, e5, e7): rho, ux, uy, T
@@ -299,8 +300,13 @@ lbm_status lbm_get_launch(const lbm_ctx* ctx, lbm_launch* launch);
 
 /* Several steps per launch on small grids (lbm_step): the CTAs of such a
  * launch (0 if the grid takes a launch a step), the steps between their
- * exchanges, and the launches queued so far by lbm_step and lbm_adjoint_step.
- * Outputs may be NULL.
+ * exchanges, the fewest steps of lbm_step and the fewest levels recomputed by
+ * lbm_adjoint_step that take one, where it becomes the faster way (INT_MAX:
+ * none), and the launches queued so far.  Outputs may be NULL.
+ *
+ * lbm_resident_set: take such launches from `steps` >= 3 steps or levels on
+ * (0: where they are the faster way, as at creation).  LBM_E_STATE if the grid
+ * takes a launch a step.
  *
  * lbm_plant_stall: failure injection for tests, on the host side.  While on is
  * not zero, such launches leave out their last CTA, so the bounded waits of
@@ -308,7 +314,9 @@ lbm_status lbm_get_launch(const lbm_ctx* ctx, lbm_launch* launch);
  * LBM_E_TIMEOUT is reported; nothing faults or hangs.  lbm_init makes the
  * context usable again.  LBM_E_STATE if the context has no launch whose CTAs
  * exchange. */
-lbm_status lbm_resident_info(const lbm_ctx* ctx, int* ctas, int* depth, long long* launches);
+lbm_status lbm_resident_info(const lbm_ctx* ctx, int* ctas, int* depth, int* steps, int* levels,
+                             long long* launches);
+lbm_status lbm_resident_set(lbm_ctx* ctx, int steps);
 lbm_status lbm_plant_stall(lbm_ctx* ctx, int on);
 
 /* Time every available launch shape for `steps` steps each (CUDA events on
@@ -318,7 +326,9 @@ lbm_status lbm_plant_stall(lbm_ctx* ctx, int on);
  * candidate to ms[0..n) if ms is not NULL (n = the number of candidates,
  * at most 8, stored in *n_candidates if not NULL).  Candidates, in order:
  * variant 0; for FP32 also (3), (2, 4), (2, 2), (1, 256, 4), (1, 256, 6),
- * (1, 128, 4). */
+ * (1, 128, 4).  The time is that of calls of `steps` steps: on a small grid the
+ * default shape runs them in one launch from a number of steps on
+ * (lbm_resident_info), so fewer say little about longer calls. */
 lbm_status lbm_autotune(lbm_ctx* ctx, int steps, lbm_launch* best, double* ms, int* n_candidates);
 
 /* FP64 conservation totals (out[0..3] = sum rho, sum rho ux, sum rho uy,

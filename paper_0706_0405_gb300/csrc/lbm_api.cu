@@ -421,15 +421,14 @@ bool plan_resident(lbm_ctx* c) {
     bool ok = false;
     dispatch(c, [&](auto tag, auto tm) {
         using S = decltype(tag);
-        ok = resident_plan<S, decltype(tm)::value>(c->nx, c->ny, &c->res);
+        constexpr int TM = decltype(tm)::value;
+        ok = resident_plan<S, TM>(c->nx, c->ny, &c->res);
+        c->res_steps = ok ? resident_min_steps<S, TM>(c->res, false) : 0;
+        c->res_levels = ok ? resident_min_steps<S, TM>(c->res, true) : 0;
         return cudaSuccess;
     });
     return ok;
 }
-
-// Fewest steps for which one launch of the resident kernel beats a launch a
-// step: it reads the level, exchanges n - 1 times and writes two levels.
-constexpr int kResidentMinSteps = 3;
 
 // The default launch shape: lbm_step and the adjoint's recomputation may run
 // several steps per launch.
@@ -737,7 +736,7 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
             if (left < m) m = (int)left;
         }
         cudaError_t e;
-        if (resident && m >= kResidentMinSteps) {
+        if (resident && m >= c->res_steps) {
             e = step_resident(c, m, static_cast<const char*>(c->f[c->cur]), nullptr, c->step);
             if (e == cudaErrorCooperativeLaunchTooLarge) {
                 // not all of the device's SMs are there for this context
@@ -1023,7 +1022,7 @@ lbm_status lbm_adjoint_step(lbm_ctx* c, int n, void* abar, double* dL_dtau) {
         LBM_CUDA(c, cudaMemcpyAsync(c->seg, c->ck[(size_t)k], lb, cudaMemcpyDeviceToDevice, c->stream),
                  "restoring a checkpoint");
         long long l0 = c0;
-        if (c->res_ok && default_launch(c) && L - 1 - c0 >= kResidentMinSteps) {
+        if (c->res_ok && default_launch(c) && L - 1 - c0 >= c->res_levels) {
             e = step_resident(c, (int)(L - 1 - c0), c->seg, c->seg, c0);
             if (e == cudaErrorCooperativeLaunchTooLarge) {
                 cudaGetLastError();
@@ -1167,11 +1166,30 @@ lbm_status lbm_get_launch(const lbm_ctx* c, lbm_launch* l) {
     return LBM_OK;
 }
 
-lbm_status lbm_resident_info(const lbm_ctx* c, int* ctas, int* depth, long long* launches) {
+lbm_status lbm_resident_info(const lbm_ctx* c, int* ctas, int* depth, int* steps, int* levels, long long* launches) {
     if (!c) return fail(nullptr, LBM_E_INVAL, "lbm_resident_info: NULL context");
     if (ctas) *ctas = c->res_ok ? c->res.px * c->res.py : 0;
     if (depth) *depth = c->res_ok ? c->res.depth : 0;
+    if (steps) *steps = c->res_ok ? c->res_steps : 0;
+    if (levels) *levels = c->res_ok ? c->res_levels : 0;
     if (launches) *launches = c->res_launches;
+    return LBM_OK;
+}
+
+lbm_status lbm_resident_set(lbm_ctx* c, int steps) {
+    if (!c) return fail(nullptr, LBM_E_INVAL, "lbm_resident_set: NULL context");
+    if (steps != 0 && steps < kResidentFewest)
+        return fail(c, LBM_E_INVAL, "lbm_resident_set: steps must be 0 or at least %d", kResidentFewest);
+    if (!c->res_ok) return fail(c, LBM_E_STATE, "lbm_resident_set: this context takes a launch a step");
+    c->res_steps = c->res_levels = steps;
+    if (steps == 0)
+        dispatch(c, [&](auto tag, auto tm) {
+            using S = decltype(tag);
+            constexpr int TM = decltype(tm)::value;
+            c->res_steps = resident_min_steps<S, TM>(c->res, false);
+            c->res_levels = resident_min_steps<S, TM>(c->res, true);
+            return cudaSuccess;
+        });
     return LBM_OK;
 }
 

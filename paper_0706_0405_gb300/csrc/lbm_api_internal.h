@@ -54,6 +54,8 @@ struct lbm_ctx {
     // several steps of a small grid per launch (lbm_resident.cu)
     ResPlan res{};
     bool res_ok = false;
+    int res_steps = 0;          // fewest steps of lbm_step that take such a launch
+    int res_levels = 0;         // fewest levels to recompute that do
     unsigned* d_res = nullptr;  // its tag counter and leave count
     ResWord* d_xch = nullptr;   // its exchange buffer (behind f[1], or behind the status words)
     bool res_stall = false;     // lbm_plant_stall

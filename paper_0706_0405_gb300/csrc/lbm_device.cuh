@@ -158,7 +158,6 @@ __device__ __forceinline__ float2 lanes(F2 a) {
 __device__ __forceinline__ float lane0(F2 a) { return lanes(a).x; }
 __device__ __forceinline__ float lane1(F2 a) { return lanes(a).y; }
 __device__ __forceinline__ float lane0(float a) { return a; }
-__device__ __forceinline__ double lane0(double a) { return a; }
 __device__ __forceinline__ F2 add2_(F2 a, F2 b) {
     F2 r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
@@ -396,43 +395,32 @@ __device__ __forceinline__ void conserve_increment(const MT& M, V (&d)[9]) {
     }
 }
 
-// The relaxation term of Eq. (SEC-VON-11) at a node, in the form update()
-// takes it.  FP32 (increment form): r_i = omega (f^eq_i - f_i), moment-exact
-// in the modes that ask for it.  FP64: r_i = omega f^eq_i.
+// The relaxation term of Eq. (SEC-VON-11) at a node, in the increment form
+// that update() takes: r_i = omega (f^eq_i - f_i), moment-exact in the modes
+// that ask for it.  (FP32; the FP64 node update is in lbm_fp64.cuh.)
 template <typename S, int TM, typename V = S, typename MT>
 __device__ __forceinline__ void relaxation(const MT& M, const V (&f)[9], V rho, V ux, V uy, V T,
                                            V (&r)[9]) {
     omega_equilibrium<S, V>(M, rho, ux, uy, T, r);
-    if constexpr (std::is_same<S, float>::value) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) r[i] = fma_(neg_(M.omega), f[i], r[i]);
-        conserve_increment<S, TM, V>(M, r);
-    }
+    for (int i = 0; i < 9; ++i) r[i] = fma_(neg_(M.omega), f[i], r[i]);
+    conserve_increment<S, TM, V>(M, r);
 }
 
 // Update of one population from its five-point star and the relaxation term
-// r (Eq. SEC-VON-11 with the folded weights of Model).  FP32: the paper's
+// r (Eq. SEC-VON-11 with the folded weights of Model), in FP32 the paper's
 // increment form, f' = c + (r + wi c + w1 e + w2 w + w3 n + w4 s): the
 // increment is small next to c, so its rounding errors are too, and a node
 // whose increment rounds away keeps its bits (a uniform state stays put
 // instead of drifting by the roundings of a full recomputation every step).
-// FP64: f' = w0 c + w1 e + w2 w + w3 n + w4 s + r.
 template <typename V, typename MT>
 __device__ __forceinline__ V update(const MT& M, int i, V r, V c, V e, V w, V n, V s) {
-    if constexpr (!std::is_same<V, double>::value) {
-        V acc = fma_(M.wi[i], c, r);
-        acc = fma_(M.w[i][1], e, acc);
-        acc = fma_(M.w[i][2], w, acc);
-        acc = fma_(M.w[i][3], n, acc);
-        acc = fma_(M.w[i][4], s, acc);
-        return add_(c, acc);
-    } else {
-        V acc = fma_(M.w[i][0], c, r);
-        acc = fma_(M.w[i][1], e, acc);
-        acc = fma_(M.w[i][2], w, acc);
-        acc = fma_(M.w[i][3], n, acc);
-        return fma_(M.w[i][4], s, acc);
-    }
+    V acc = fma_(M.wi[i], c, r);
+    acc = fma_(M.w[i][1], e, acc);
+    acc = fma_(M.w[i][2], w, acc);
+    acc = fma_(M.w[i][3], n, acc);
+    acc = fma_(M.w[i][4], s, acc);
+    return add_(c, acc);
 }
 
 // ---------------------------------------------------------- ghost layer
@@ -643,34 +631,28 @@ __device__ __forceinline__ unsigned pair_update(const Model<float>& M, const flo
 }
 
 // ------------------------------------------------------ one node per thread
-// Reads the node and its four star neighbours of all nine planes (kCoherent:
-// through L2 only, for data written earlier in the same kernel by other
-// CTAs), updates it, writes nine values and, at an edge, the next level's
-// ghost cells.  Returns the node's health bits.
-template <typename S, bool kCoherent>
-__device__ __forceinline__ S load_s(const S* p) {
-    return kCoherent ? __ldcg(p) : __ldg(p);
-}
-
-template <typename S, int TM, bool kCoherent>
-__device__ __forceinline__ unsigned node_step(const S* __restrict__ fin, S* __restrict__ fout, const Model<S>& M,
-                                              const Grid<S>& G, int ix, int iy, long long level) {
+// Reads the node and its four star neighbours of all nine planes, updates it,
+// writes nine values and, at an edge, the next level's ghost cells.  Returns
+// the node's health bits.
+template <int TM>
+__device__ __forceinline__ unsigned node_step(const float* __restrict__ fin, float* __restrict__ fout,
+                                              const Model<float>& M, const Grid<float>& G, int ix, int iy,
+                                              long long level) {
     const size_t pl = (size_t)G.plane;
     const size_t c = cell(G, ix, iy);
-    S f[9];
+    float f[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) f[i] = load_s<S, kCoherent>(fin + i * pl + c);
-    S rho, ux, uy, T;
-    moments<S, TM>(f, M, rho, ux, uy, T);
+    for (int i = 0; i < 9; ++i) f[i] = __ldg(fin + i * pl + c);
+    float rho, ux, uy, T;
+    moments<float, TM>(f, M, rho, ux, uy, T);
     const unsigned bits = health(rho, ux, uy, T);
-    S ofe[9];
-    relaxation<S, TM>(M, f, rho, ux, uy, T, ofe);
-    S o[9];
+    float ofe[9];
+    relaxation<float, TM>(M, f, rho, ux, uy, T, ofe);
+    float o[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        const S* p = fin + i * pl + c;
-        o[i] = update(M, i, ofe[i], f[i], load_s<S, kCoherent>(p + 1), load_s<S, kCoherent>(p - 1),
-                      load_s<S, kCoherent>(p + G.row), load_s<S, kCoherent>(p - G.row));
+        const float* p = fin + i * pl + c;
+        o[i] = update(M, i, ofe[i], f[i], __ldg(p + 1), __ldg(p - 1), __ldg(p + G.row), __ldg(p - G.row));
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) fout[i * pl + c] = o[i];
@@ -684,9 +666,7 @@ __device__ __forceinline__ unsigned node_step(const S* __restrict__ fin, S* __re
 // as V-wide vectors and the two x-neighbours at the ends as scalars; the
 // arithmetic per node is the explicitly rounded sequence of moments,
 // equilibrium and update, so every kernel built on it gives the same bits.
-// kCoherent: read through L2 only (data written earlier in the same kernel
-// by other CTAs); otherwise through the read-only path.  Returns the health
-// bits of the nodes inside the grid.
+// Returns the health bits of the nodes inside the grid.
 template <int V>
 struct VecT;
 template <>
@@ -698,10 +678,10 @@ struct VecT<4> {
     using type = float4;
 };
 
-template <int V, bool kCoherent>
+template <int V>
 __device__ __forceinline__ void load_vec(const float* p, float (&out)[V]) {
     using T = typename VecT<V>::type;
-    const T v = kCoherent ? __ldcg(reinterpret_cast<const T*>(p)) : __ldg(reinterpret_cast<const T*>(p));
+    const T v = __ldg(reinterpret_cast<const T*>(p));
     if constexpr (V == 2) {
         out[0] = v.x;
         out[1] = v.y;
@@ -729,12 +709,7 @@ __device__ __forceinline__ void store_vec(float* p, const float (&o)[V]) {
     *reinterpret_cast<T*>(p) = v;
 }
 
-template <bool kCoherent>
-__device__ __forceinline__ float load1(const float* p) {
-    return kCoherent ? __ldcg(p) : __ldg(p);
-}
-
-template <int V, int TM, bool kCoherent>
+template <int V, int TM>
 __device__ __forceinline__ unsigned vec_group(const float* __restrict__ fin, float* __restrict__ fout,
                                               const Model<float>& M, const Grid<float>& G, int ix0, int iy,
                                               long long level) {
@@ -745,7 +720,7 @@ __device__ __forceinline__ unsigned vec_group(const float* __restrict__ fin, flo
 
     float C[9][V];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) load_vec<V, kCoherent>(in + i * pl, C[i]);
+    for (int i = 0; i < 9; ++i) load_vec<V>(in + i * pl, C[i]);
 
     float acc[9][V];  // omega f^eq, the first term of the update
     unsigned bits = 0;
@@ -768,11 +743,11 @@ __device__ __forceinline__ unsigned vec_group(const float* __restrict__ fin, flo
     for (int i = 0; i < 9; ++i) {
         const float* p = in + i * pl;
         float Nn[V], Ss[V];
-        load_vec<V, kCoherent>(p + G.row, Nn);
-        load_vec<V, kCoherent>(p - G.row, Ss);
+        load_vec<V>(p + G.row, Nn);
+        load_vec<V>(p - G.row, Ss);
         float row[V + 2];
-        row[0] = load1<kCoherent>(p - 1);
-        row[V + 1] = load1<kCoherent>(p + V);
+        row[0] = __ldg(p - 1);
+        row[V + 1] = __ldg(p + V);
 #pragma unroll
         for (int k = 0; k < V; ++k) row[k + 1] = C[i][k];
         float o[V];

@@ -116,6 +116,12 @@ cudaError_t resident_set_wait_cycles(long long cycles);
 // False if the grid does not fit.
 template <typename S, int TM>
 bool resident_plan(int nx, int ny, ResPlan* plan);
+// Fewest steps for which one such launch is the faster way, with the last two
+// levels written or with all of them (INT_MAX: none).  At least
+// kResidentFewest, of which the kernel takes any number.
+constexpr int kResidentFewest = 3;
+template <typename S, int TM>
+int resident_min_steps(const ResPlan& R, bool all_levels);
 // M64: the constants of FP64 steps (unused otherwise).  stall: a launch whose
 // polls run out (lbm_plant_stall; more than one CTA).
 template <typename S, int TM>

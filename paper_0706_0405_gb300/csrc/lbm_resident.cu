@@ -46,6 +46,8 @@
 // Polls are bounded (lbm_batch_set_wait_limit): on give-up the CTA raises
 // ST_TIMEOUT and leaves, and so do the others, which watch that word while
 // they poll.
+#include <climits>
+
 #include "lbm_launch.h"
 
 namespace lbm {
@@ -562,6 +564,44 @@ bool resident_plan(int nx, int ny, ResPlan* best) {
     return true;
 }
 
+// A launch costs 10 to 40 us besides its steps, the more the larger the tiles
+// (their level read, the last two written), and a step in it saves what the
+// tile kernel's launch and drain take, 2 to 4 us, or with the FP64 sum and on
+// thin FP64 grids 2 to 5.  Where the two meet, in steps, and per node of a tile
+// the line above it taken here (us a call, launches of a step / one launch):
+// FP32_CONS 400 x 4 (12 nodes) 4, 400 x 100 (280) 6, 512 x 256 (900) 8, 900 x 300
+// (1950) 11 (n = 8: 53 / 61, 24: 159 / 119), 1240 x 310 (2574) 13 (n = 8: 62 /
+// 74, 24: 184 / 150); FP32_TDF 4, 6, 9, 15, 13; FP32_T64 4, 5, 5, 6, 10.  With
+// every level written a step also stores a level, as the tile kernel does, but
+// with nothing to hide it: recomputation of 23 levels and their adjoint, 400 x
+// 100 220 / 206, 512 x 128 (450) 239 / 235, 512 x 256 325 / 340, 900 x 300 414 /
+// 512 (FP32_T64 274 / 246, 296 / 286, 439 / 423, 598 / 634).  FP64, where a step
+// by launches takes 6.0 us: one group of 32 nodes a CTA 4 steps, two groups 5 to
+// 30 with their number of nodes (64: 5.8 us a step), three 10 on thin grids (4.9
+// to 5.2) and none on others (7.2); with every level written two groups win from
+// the start (a launch less on the host beside the adjoint's) and three lose.
+template <typename S, int TM>
+int resident_min_steps(const ResPlan& R, bool all_levels) {
+    const int nodes = R.bw * R.bh;
+    int n;
+    if (sizeof(S) == 8) {
+        const int groups = (nodes + 31) / 32;
+        if (all_levels)
+            n = groups <= 2 ? kResidentFewest : INT_MAX;
+        else if (groups == 1)
+            n = 4;
+        else if (R.py == 1)
+            n = groups == 2 ? 5 : 10;
+        else
+            n = groups == 2 ? 5 + (nodes - 32) * (nodes - 32) / 40 : INT_MAX;
+    } else if (TM == T_INT64) {
+        n = !all_levels ? 5 + nodes / 400 : nodes <= 950 ? 5 + nodes / 60 : INT_MAX;
+    } else {
+        n = !all_levels ? 6 + nodes / 220 : nodes <= 320 ? 7 + nodes / 50 : INT_MAX;
+    }
+    return n;
+}
+
 // A stalled launch leaves its last CTA out, which makes the halves of the
 // exchange buffer smaller by its cells.  The cells that the others then wait
 // for still lie in the buffer: behind their half, where there are tags of the
@@ -591,6 +631,7 @@ cudaError_t resident_set_wait_cycles(long long cycles) {
 
 #define LBM_RES_INST(S, TM)                                                                              \
     template bool resident_plan<S, TM>(int, int, ResPlan*);                                              \
+    template int resident_min_steps<S, TM>(const ResPlan&, bool);                                        \
     template cudaError_t launch_resident<S, TM>(const ResPlan&, const Model<S>&, const Fp64Step&,        \
                                                 const Grid<S>&, const ResRun<S>&, bool, cudaStream_t);
 LBM_RES_INST(double, T_PLAIN)

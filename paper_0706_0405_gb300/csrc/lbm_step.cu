@@ -7,7 +7,6 @@
 #include "lbm_launch.h"
 #include "lbm_ptx.cuh"
 
-
 namespace lbm {
 
 // Probes of an mbarrier before a wait gives up (each probe may suspend the
@@ -25,7 +24,7 @@ __global__ void __launch_bounds__(256) k_step_simple(const float* __restrict__ f
     const int ix = blockIdx.x * blockDim.x + threadIdx.x;
     const int iy = blockIdx.y * blockDim.y + threadIdx.y;
     if (ix >= G.nx || iy >= G.ny) return;
-    report(status, node_step<float, TM, false>(fin, fout, M, G, ix, iy, level));
+    report(status, node_step<TM>(fin, fout, M, G, ix, iy, level));
 }
 
 // ------------------------------------------------------------ FP64 kernel
@@ -106,7 +105,7 @@ __global__ void __launch_bounds__(256) k_step_vec(const float* __restrict__ fin,
     const int ix0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int iy = blockIdx.y * blockDim.y + threadIdx.y;
     if (ix0 >= G.nx || iy >= G.ny) return;
-    report(status, vec_group<V, TM, false>(fin, fout, M, G, ix0, iy, level));
+    report(status, vec_group<V, TM>(fin, fout, M, G, ix0, iy, level));
 }
 
 template <int V, int TM>

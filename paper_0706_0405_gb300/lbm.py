@@ -33,7 +33,7 @@ EXPORTS = ("lbm_create", "lbm_destroy", "lbm_last_error", "lbm_init", "lbm_step"
            "lbm_batch_step", "lbm_batch_sync", "lbm_batch_problem", "lbm_batch_info",
            "lbm_probe_rates", "lbm_vn_scan", "lbm_batch_set_launch", "lbm_batch_get_launch",
            "lbm_batch_autotune", "lbm_probe_tile_copy", "lbm_batch_set_wait_limit", "lbm_batch_plant_stall",
-           "lbm_resident_info", "lbm_plant_stall",
+           "lbm_resident_info", "lbm_resident_set", "lbm_plant_stall",
            "lbm_inject_alloc_failure", "lbm_level_bytes")
 LBM_FLAG_NONPHYSICAL, LBM_FLAG_TIMEOUT, LBM_FLAG_T_NONPOSITIVE = 1, 2, 4
 
@@ -128,8 +128,9 @@ def load():
         "lbm_probe_tile_copy": ([ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double)],
                                 ctypes.c_int),
         "lbm_batch_set_wait_limit": ([ctypes.c_double], ctypes.c_int),
-        "lbm_resident_info": ([ctx, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
-                               ctypes.POINTER(ctypes.c_longlong)], ctypes.c_int),
+        "lbm_resident_info": ([ctx] + [ctypes.POINTER(ctypes.c_int)] * 4 + [ctypes.POINTER(ctypes.c_longlong)],
+                              ctypes.c_int),
+        "lbm_resident_set": ([ctx, ctypes.c_int], ctypes.c_int),
         "lbm_plant_stall": ([ctx, ctypes.c_int], ctypes.c_int),
         "lbm_batch_plant_stall": ([_VP, ctypes.c_int], ctypes.c_int),
         "lbm_inject_alloc_failure": ([ctypes.c_longlong], ctypes.c_int),
@@ -455,10 +456,15 @@ def lbm_inject_alloc_failure(after: int) -> None:
 
 
 def lbm_resident_info(ctx):
-    """(CTAs, steps between exchanges, launches so far) of the launches of several steps."""
-    n, d, l = ctypes.c_int(), ctypes.c_int(), ctypes.c_longlong()
-    _check(ctx, load().lbm_resident_info(ctx, ctypes.byref(n), ctypes.byref(d), ctypes.byref(l)))
-    return n.value, d.value, l.value
+    """Of the launches of several steps: CTAs, steps between exchanges, fewest
+    steps, fewest recomputed levels, launches so far."""
+    v = [ctypes.c_int() for _ in range(4)] + [ctypes.c_longlong()]
+    _check(ctx, load().lbm_resident_info(ctx, *[ctypes.byref(x) for x in v]))
+    return tuple(x.value for x in v)
+
+
+def lbm_resident_set(ctx, steps: int):
+    return _check(ctx, load().lbm_resident_set(ctx, int(steps)))
 
 
 def lbm_plant_stall(ctx, on: bool):

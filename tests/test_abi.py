@@ -170,5 +170,6 @@ def test_batch_plant_stall_on_null_batch_fails_cleanly():
 
 def test_small_grid_hooks_on_a_null_context_fail_cleanly():
     lib = lbm.load()
-    assert lib.lbm_resident_info(None, None, None, None) == lbm.LBM_E_INVAL
+    assert lib.lbm_resident_info(None, None, None, None, None, None) == lbm.LBM_E_INVAL
+    assert lib.lbm_resident_set(None, 3) == lbm.LBM_E_INVAL
     assert lib.lbm_plant_stall(None, 0) == lbm.LBM_E_INVAL

@@ -178,31 +178,67 @@ def test_a_captured_call_of_several_steps_replays():
                                         for prec in ("fp32", "fp32_t64", "fp32_tdf", "fp32_cons")] +
                          [(nx, ny, "fp64") for nx, ny in [(1, 1), (33, 4), (8, 4), (97, 5), (305, 2), (120, 80)]])
 def test_small_grids_take_one_launch_for_several_steps(nx, ny, prec):
-    """The grids above whose steps are compared do take that launch, for three
-    steps or more and with the default launch shape only."""
+    """The grids above whose steps are compared do take that launch, from the
+    stated number of steps on and with the default launch shape only."""
     p, fields = _problem(nx, ny, INFLOW)
     with lbm.Lattice(p, prec) as lat:
-        count = lambda: lbm.lbm_resident_info(lat.ctx)[2]
+        count = lambda: lbm.lbm_resident_info(lat.ctx)[4]
         lat.init(*fields)
-        assert lbm.lbm_resident_info(lat.ctx)[0] > 0 and count() == 0
-        assert [lat.step(n) and count() for n in (1, 2, 3, 11)] == [0, 0, 1, 2]
-        lbm.lbm_record(lat.ctx, 5)
-        lat.step(12)  # five steps to each recorded level, two more
+        ctas, depth, steps, levels, n = lbm.lbm_resident_info(lat.ctx)
+        assert ctas > 0 and 1 <= depth <= 4 and 3 <= steps <= 30 and levels >= 3 and n == 0
+        assert [lat.step(n) and count() for n in (1, 2, steps - 1, steps, 2 * steps)] == [0, 0, 0, 1, 2]
+        lbm.lbm_record(lat.ctx, steps)
+        lat.step(2 * steps + steps - 1)  # as many to each recorded level, and the others
         assert count() == 4
+        lbm.lbm_resident_set(lat.ctx, 3)
+        assert [lat.init(*fields).step(n) and count() for n in (2, 3, 11)] == [4, 5, 6]
+        lbm.lbm_resident_set(lat.ctx, 0)
+        assert lbm.lbm_resident_info(lat.ctx)[2:4] == (steps, levels)
+        for bad in (-1, 1, 2):
+            with pytest.raises(lbm.LbmError) as ei:
+                lbm.lbm_resident_set(lat.ctx, bad)
+            assert ei.value.status == lbm.LBM_E_INVAL
         lbm.lbm_set_launch(lat.ctx, 0, 0, 0, 1)
-        lat.step(5)
-        assert count() == 4
+        lat.step(50)
+        assert count() == 6
         lat.sync()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp32_t64", "fp32_tdf", "fp32_cons", "fp64"])
+@pytest.mark.parametrize("sides", [PERIODIC, WALLS, INFLOW])
+@pytest.mark.parametrize("nx,ny", RESIDENT[:-1])
+def test_one_launch_from_three_steps_on_equals_a_launch_a_step(nx, ny, sides, prec):
+    """As above with that launch from the fewest steps on that the kernel
+    takes, also where a launch a step is the default for so few: for the
+    lengths around the steps between exchanges, and to recorded levels."""
+    import torch
+    p, fields = _problem(nx, ny, sides)
+    with lbm.Lattice(p, prec) as one, lbm.Lattice(p, prec) as many:
+        if lbm.lbm_resident_info(many.ctx)[0] == 0:
+            assert prec == "fp64" and nx * ny > 9000
+            return
+        lbm.lbm_resident_set(many.ctx, 3)
+        one.init(*fields), many.init(*fields)
+        for n in (3, 4, 5, 6, 20):
+            if n == 20:
+                lbm.lbm_record(many.ctx, 7)
+            for _ in range(n):
+                one.step(1)
+            many.step(n)
+            assert torch.equal(one.get_f(), many.get_f()), n
+        assert lbm.lbm_resident_info(many.ctx)[4] == 7 and lbm.lbm_resident_info(one.ctx)[4] == 0
+        assert one.health() == many.health()
 
 
 def test_larger_grids_take_a_launch_a_step():
     p, fields = _problem(*RESIDENT[-1], WALLS)
     with lbm.Lattice(p, "fp32") as lat:
         lat.init(*fields).step(5).sync()
-        assert lbm.lbm_resident_info(lat.ctx) == (0, 0, 0)
-        with pytest.raises(lbm.LbmError) as ei:
-            lbm.lbm_plant_stall(lat.ctx, True)
-        assert ei.value.status == lbm.LBM_E_STATE
+        assert lbm.lbm_resident_info(lat.ctx) == (0, 0, 0, 0, 0)
+        for call in (lambda: lbm.lbm_plant_stall(lat.ctx, True), lambda: lbm.lbm_resident_set(lat.ctx, 3)):
+            with pytest.raises(lbm.LbmError) as ei:
+                call()
+            assert ei.value.status == lbm.LBM_E_STATE
 
 
 @pytest.mark.parametrize("nx,ny,prec", [(2000, 4, "fp32_tdf"), (400, 100, "fp32_cons"), (400, 4, "fp64"),
@@ -218,6 +254,7 @@ def test_a_value_that_never_arrives_times_out_and_the_context_recovers(nx, ny, p
     lbm.lbm_batch_set_wait_limit(0.2)
     try:
         with lbm.Lattice(p, prec) as lat, lbm.Lattice(p, prec) as ref:
+            lbm.lbm_resident_set(lat.ctx, 3)
             for first in (3, 4, 7):  # the exchange buffer's halves in either order
                 lat.init(*fields).step(first)
                 lat.sync()
@@ -296,6 +333,7 @@ def test_a_recomputation_that_gives_up_is_reported_by_the_adjoint(nx, ny, prec):
     lbm.lbm_batch_set_wait_limit(0.2)
     try:
         with lbm.Lattice(p, prec) as lat, lbm.Lattice(p, prec) as ref:
+            lbm.lbm_resident_set(lat.ctx, 3), lbm.lbm_resident_set(ref.ctx, 3)
             assert gradient(lat, True)[:2] == (lbm.LBM_E_TIMEOUT, 7.0)
             got, want = gradient(lat, False), gradient(ref, False)
     finally:
