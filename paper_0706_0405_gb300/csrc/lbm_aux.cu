@@ -9,14 +9,51 @@ constexpr int kThreads = 256;
 
 inline unsigned blocks_for(long long n, int per) { return (unsigned)((n + per - 1) / per); }
 
-// Shape of the kernels that walk the grid row by row: CTAs of 64 x 4 threads,
-// each thread V consecutive columns of a row and every gridDim.y * 4-th row
-// from its own, so that no index is divided (a 64-bit division per element
-// had cost more than the copy: see launch_pack).
-constexpr int kRowX = 64, kRowY = 4;
-inline dim3 row_grid(long long columns, long long rows, int V) {
-    const long long gy = (rows + kRowY - 1) / kRowY;
-    return dim3(blocks_for(columns, kRowX * V), (unsigned)(gy < 32768 ? gy : 32768));
+// The kernels below give a thread V consecutive columns of a row, a run.
+// Where the rows' runs nearly fill CTAs of 64 x 4, a CTA takes such a patch, so
+// that no index is divided (a 64-bit division per element had cost more than
+// the copy: see launch_pack).  Other grids -- narrow, or a row of little more
+// than so many runs -- take the runs in the order of the rows, a thread's row
+// and column from one division, in 32 bits where that is enough (4 x 100000,
+// FP32: moments 23 us, initial levels 63; in patches 54 and 141), in CTAs of
+// one warp where there are few.
+constexpr int kRunX = 64;
+struct RunGrid {
+    dim3 grid;
+    int threads;
+    bool patch;
+};
+inline RunGrid run_grid(long long columns, long long rows, int V) {
+    const long long runs = (columns + V - 1) / V, padded = (runs + kRunX - 1) / kRunX * kRunX;
+    constexpr int kRunY = kThreads / kRunX;
+    const bool few = runs * rows <= 512LL * kThreads;
+    if ((few ? 2 * padded <= 3 * runs : 5 * padded <= 6 * runs) && rows >= kRunY &&
+        rows <= 65535LL * kRunY)
+        return {dim3((unsigned)(padded / kRunX), blocks_for(rows, kRunY)), kThreads, true};
+    const int threads = few ? 32 : kThreads;
+    return {dim3(blocks_for(runs * rows, threads)), threads, false};
+}
+template <int V, bool kPatch>
+__device__ __forceinline__ bool run_place(int columns, int rows, int& x, int& row) {
+    const unsigned runs = ((unsigned)columns + V - 1) / V;
+    if constexpr (kPatch) {
+        const unsigned k = blockIdx.x * kRunX + threadIdx.x % kRunX;
+        row = (int)(blockIdx.y * (kThreads / kRunX) + threadIdx.x / kRunX);
+        x = (int)k * V;
+        return k < runs && row < rows;
+    } else {
+        const unsigned long long total = (unsigned long long)runs * (unsigned)rows;
+        const unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (q >= total) return false;
+        if (total <= 0xffffffffull) {
+            row = (int)((unsigned)q / runs);
+            x = (int)((unsigned)q % runs) * V;
+        } else {
+            row = (int)(q / runs);
+            x = (int)(q % runs) * V;
+        }
+        return true;
+    }
 }
 
 inline bool aligned(const void* p, size_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
@@ -105,15 +142,13 @@ __device__ __forceinline__ void init_run(float* __restrict__ f, const float* __r
     }
 }
 
-template <int V>
+template <int V, bool kPatch>
 __global__ void __launch_bounds__(kThreads) k_init32(float* __restrict__ f, const float* __restrict__ rho,
                                                      const float* __restrict__ ux, const float* __restrict__ uy,
                                                      const float* __restrict__ T, const Model<float> M,
                                                      const Grid<float> G, bool wide) {
-    const int ix = (blockIdx.x * kRowX + threadIdx.x) * V;
-    if (ix >= G.nx) return;
-    for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY)
-        init_run<V>(f, rho, ux, uy, T, M, G, wide, ix, iy);
+    int ix, iy;
+    if (run_place<V, kPatch>(G.nx, G.ny, ix, iy)) init_run<V>(f, rho, ux, uy, T, M, G, wide, ix, iy);
 }
 
 // A batch's problems, one 64 x 4 tile of its tile list a CTA, the arrays'
@@ -136,39 +171,49 @@ __global__ void __launch_bounds__(128) k_init_batch(const __grid_constant__ Batc
 
 template <int V>
 void init32(float* f, const float* rho, const float* ux, const float* uy, const float* T, const Model<float>& M,
-            const Grid<float>& G, cudaStream_t st) {
-    const bool wide = G.nx % V == 0 && aligned(rho, 4 * V) && aligned(ux, 4 * V) && aligned(uy, 4 * V) &&
-                      aligned(T, 4 * V);
-    k_init32<V><<<row_grid(G.nx, G.ny, V), dim3(kRowX, kRowY), 0, st>>>(f, rho, ux, uy, T, M, G, wide);
+            const Grid<float>& G, bool wide, cudaStream_t st) {
+    const RunGrid R = run_grid(G.nx, G.ny, V);
+    (R.patch ? k_init32<V, true> : k_init32<V, false>)<<<R.grid, R.threads, 0, st>>>(f, rho, ux, uy, T, M, G, wide);
 }
 
-__global__ void __launch_bounds__(kThreads) k_init64(double* __restrict__ f, const double* __restrict__ rho,
-                                                     const double* __restrict__ ux, const double* __restrict__ uy,
-                                                     const double* __restrict__ T, const Model<double> M,
-                                                     const Grid<double> G) {
-    const int ix = blockIdx.x * kRowX + threadIdx.x;
-    if (ix >= G.nx) return;
-    for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
-        const size_t q = (size_t)iy * G.nx + ix;
-        double fe[9];
-        equilibrium(M, rho[q], ux[q], uy[q], T[q], fe);
-        const size_t c = cell(G, ix, iy);
+// One node a thread: FP64, and FP32 on large grids whose fields do not allow
+// 16-byte accesses (a run of four would be read value by value: 4095 x 1023 64
+// us, 47 here).
+template <typename S, bool kGhosts>
+__global__ void __launch_bounds__(kThreads) k_init(S* __restrict__ f, const S* __restrict__ rho,
+                                                   const S* __restrict__ ux, const S* __restrict__ uy,
+                                                   const S* __restrict__ T, const Model<S> M, const Grid<S> G) {
+    int ix, iy;
+    if (!run_place<1, false>(G.nx, G.ny, ix, iy)) return;
+    const size_t q = (size_t)iy * G.nx + ix;
+    S fe[9];
+    equilibrium(M, rho[q], ux[q], uy[q], T[q], fe);
+    const size_t c = cell(G, ix, iy);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i * (size_t)G.plane + c] = fe[i];
-        if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) write_ghosts(G, f, ix, iy, fe, 0);
-    }
+    for (int i = 0; i < 9; ++i) f[i * (size_t)G.plane + c] = fe[i];
+    if constexpr (!kGhosts) return;
+    if (ix == 0 || iy == 0 || ix == G.nx - 1 || iy == G.ny - 1) write_ghosts(G, f, ix, iy, fe, 0);
 }
 
 template <typename S>
 cudaError_t launch_init(S* f, const S* rho, const S* ux, const S* uy, const S* T,
                         const Model<S>& M, const Grid<S>& G, cudaStream_t st) {
     if constexpr (sizeof(S) == 4) {
-        if ((long long)G.nx * G.ny >= kInitWideNodes)
-            init32<4>(f, rho, ux, uy, T, M, G, st);
+        auto wide = [&](int V) {
+            return G.nx % V == 0 && aligned(rho, 4 * V) && aligned(ux, 4 * V) && aligned(uy, 4 * V) && aligned(T, 4 * V);
+        };
+        const bool large = (long long)G.nx * G.ny >= kInitWideNodes;
+        if (!large)
+            init32<2>(f, rho, ux, uy, T, M, G, wide(2), st);
+        else if (wide(4))
+            init32<4>(f, rho, ux, uy, T, M, G, true, st);
         else
-            init32<2>(f, rho, ux, uy, T, M, G, st);
+            k_init<S, true><<<blocks_for((long long)G.nx * G.ny, kThreads), kThreads, 0, st>>>(f, rho, ux, uy, T, M, G);
+    } else if ((long long)G.nx * G.ny >= kInitWideNodes) {
+        k_init<S, false><<<blocks_for((long long)G.nx * G.ny, 32), 32, 0, st>>>(f, rho, ux, uy, T, M, G);
+        return launch_fill_ghosts<S>(f, G, 0, st);
     } else {
-        k_init64<<<row_grid(G.nx, G.ny, 1), dim3(kRowX, kRowY), 0, st>>>(f, rho, ux, uy, T, M, G);
+        k_init<S, true><<<blocks_for((long long)G.nx * G.ny, 32), 32, 0, st>>>(f, rho, ux, uy, T, M, G);
     }
     return cudaGetLastError();
 }
@@ -217,55 +262,52 @@ cudaError_t launch_fill_ghosts(S* f, const Grid<S>& G, long long level, cudaStre
 // and 35.7 (total energy), as with one node a thread; 1024 x 256 with the
 // FP64 sum 10.0, one node a thread and its index divided 16.9.  Four nodes a
 // thread: 59.9 and 47.5 (too few warps for their registers).
-template <int TM>
-__global__ void __launch_bounds__(kThreads) k_moments32(const float* __restrict__ f, float* __restrict__ rho,
+// (CTAs an SM: the FP64 sum spills in the 48 registers of five)
+template <int TM, bool kPatch>
+__global__ void __launch_bounds__(kThreads, TM == T_INT64 ? 4 : TM != T_CONS ? 5 : kPatch ? 8 : 6) k_moments32(const float* __restrict__ f, float* __restrict__ rho,
                                                         float* __restrict__ ux, float* __restrict__ uy,
                                                         float* __restrict__ T, const Model<float> M,
                                                         const Grid<float> G, unsigned* status, bool wide) {
-    const int ix = (blockIdx.x * kRowX + threadIdx.x) * 2;
+    int ix, iy;
     unsigned bits = 0;
-    if (ix < G.nx) {
+    if (run_place<2, kPatch>(G.nx, G.ny, ix, iy)) {
         const int n = min(2, G.nx - ix);
         const size_t pl = (size_t)G.plane;
-        for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
-            const float* in = f + cell(G, ix, iy);  // 8-byte aligned
-            F2 v[9];
+        const float* in = f + cell(G, ix, iy);  // 8-byte aligned
+        F2 v[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) v[i] = load_run<2>(in + i * pl, n == 2, n).h[0];
-            Run<2> r, u, w, t;
-            moments<float, TM, F2>(v, M, r.h[0], u.h[0], w.h[0], t.h[0]);
-            // the second lane of a last odd node repeats the first
-            bits |= health(r.at(0), u.at(0), w.at(0), t.at(0)) | health(r.at(1), u.at(1), w.at(1), t.at(1));
-            const size_t q = (size_t)iy * G.nx + ix;
-            if (rho) store_run<2>(rho + q, r, wide, n);
-            if (ux) store_run<2>(ux + q, u, wide, n);
-            if (uy) store_run<2>(uy + q, w, wide, n);
-            if (T) store_run<2>(T + q, t, wide, n);
-        }
+        for (int i = 0; i < 9; ++i) v[i] = load_run<2>(in + i * pl, n == 2, n).h[0];
+        Run<2> r, u, w, t;
+        moments<float, TM, F2>(v, M, r.h[0], u.h[0], w.h[0], t.h[0]);
+        // the second lane of a last odd node repeats the first
+        bits |= health(r.at(0), u.at(0), w.at(0), t.at(0)) | health(r.at(1), u.at(1), w.at(1), t.at(1));
+        const size_t q = (size_t)iy * G.nx + ix;
+        if (rho) store_run<2>(rho + q, r, wide, n);
+        if (ux) store_run<2>(ux + q, u, wide, n);
+        if (uy) store_run<2>(uy + q, w, wide, n);
+        if (T) store_run<2>(T + q, t, wide, n);
     }
     report(status, bits);
 }
 
-__global__ void __launch_bounds__(kThreads) k_moments64(const double* __restrict__ f, double* __restrict__ rho,
+__global__ void __launch_bounds__(32) k_moments64(const double* __restrict__ f, double* __restrict__ rho,
                                                         double* __restrict__ ux, double* __restrict__ uy,
                                                         double* __restrict__ T, const Model<double> M,
                                                         const Grid<double> G, unsigned* status) {
-    const int ix = blockIdx.x * kRowX + threadIdx.x;
+    int ix, iy;
     unsigned bits = 0;
-    if (ix < G.nx) {
-        for (int iy = blockIdx.y * kRowY + threadIdx.y; iy < G.ny; iy += gridDim.y * kRowY) {
-            const size_t c = cell(G, ix, iy);
-            double v[9], r, u, w, t;
+    if (run_place<1, false>(G.nx, G.ny, ix, iy)) {
+        const size_t c = cell(G, ix, iy);
+        double v[9], r, u, w, t;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) v[i] = f[i * (size_t)G.plane + c];
-            moments<double, T_PLAIN>(v, M, r, u, w, t);
-            bits |= health(r, u, w, t);
-            const size_t q = (size_t)iy * G.nx + ix;
-            if (rho) rho[q] = r;
-            if (ux) ux[q] = u;
-            if (uy) uy[q] = w;
-            if (T) T[q] = t;
-        }
+        for (int i = 0; i < 9; ++i) v[i] = f[i * (size_t)G.plane + c];
+        moments<double, T_PLAIN>(v, M, r, u, w, t);
+        bits |= health(r, u, w, t);
+        const size_t q = (size_t)iy * G.nx + ix;
+        if (rho) rho[q] = r;
+        if (ux) ux[q] = u;
+        if (uy) uy[q] = w;
+        if (T) T[q] = t;
     }
     report(status, bits);
 }
@@ -273,12 +315,13 @@ __global__ void __launch_bounds__(kThreads) k_moments64(const double* __restrict
 template <typename S, int TM>
 cudaError_t launch_moments(const S* f, S* rho, S* ux, S* uy, S* T, const Model<S>& M,
                            const Grid<S>& G, unsigned* status, cudaStream_t st) {
-    const dim3 block(kRowX, kRowY);
     if constexpr (sizeof(S) == 4) {
         const bool wide = G.nx % 2 == 0 && aligned(rho, 8) && aligned(ux, 8) && aligned(uy, 8) && aligned(T, 8);
-        k_moments32<TM><<<row_grid(G.nx, G.ny, 2), block, 0, st>>>(f, rho, ux, uy, T, M, G, status, wide);
+        const RunGrid R = run_grid(G.nx, G.ny, 2);
+        (R.patch ? k_moments32<TM, true> : k_moments32<TM, false>)<<<R.grid, R.threads, 0, st>>>(
+            f, rho, ux, uy, T, M, G, status, wide);
     } else {
-        k_moments64<<<row_grid(G.nx, G.ny, 1), block, 0, st>>>(f, rho, ux, uy, T, M, G, status);
+        k_moments64<<<blocks_for((long long)G.nx * G.ny, 32), 32, 0, st>>>(f, rho, ux, uy, T, M, G, status);
     }
     return cudaGetLastError();
 }
@@ -298,10 +341,24 @@ cudaError_t launch_moments(const S* f, S* rho, S* ux, S* uy, S* T, const Model<S
 constexpr int kConsSeg = 512, kConsSeg64 = 128;
 constexpr int kConsBlocks = 608;  // 4 per SM
 
+// Grids of at most kConsNarrow columns: a unit is kConsSeg (FP64: kConsSeg64)
+// places, 2^cons_shift columns of several rows (a row alone would leave most
+// of a warp's lanes idle: 4 x 100000, us a call, FP32 274, FP64 216).
+constexpr int kConsNarrow = 64;
+__host__ __device__ inline int cons_shift(int nx) {
+    int s = 2;  // a run of four
+    while ((1 << s) < nx) ++s;
+    return s;
+}
+
 template <typename S>
 int conservation_partials(const Grid<S>& G) {
     const int seg = sizeof(S) == 4 ? kConsSeg : kConsSeg64;
-    const long long units = (long long)G.ny * ((G.nx + seg - 1) / seg);
+    long long units = (long long)G.ny * ((G.nx + seg - 1) / seg);
+    if (G.nx <= kConsNarrow) {
+        const int rows = seg >> cons_shift(G.nx);
+        units = ((long long)G.ny + rows - 1) / rows;
+    }
     return (int)(units < kConsBlocks ? units : kConsBlocks);
 }
 
@@ -406,7 +463,32 @@ __global__ void __launch_bounds__(kConsThreads32, 4)
         return f + (size_t)(row + 1) * (size_t)G.row + (size_t)pop * (size_t)G.plane + (PADX + x0);  // 16-byte aligned
     };
     Sum3<F2> a, b;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+    const bool narrow = G.nx <= kConsNarrow;
+    const int shift = cons_shift(G.nx), unit_rows = kConsSeg >> shift;
+    auto row_of = [&](long long r) {
+        return f + (size_t)(r + 1) * (size_t)G.row + (size_t)pop * (size_t)G.plane + PADX;
+    };
+    for (long long r0 = (long long)blockIdx.x * unit_rows; r0 < G.ny && narrow; r0 += (long long)gridDim.x * unit_rows) {
+        float4 v[kConsSeg / 128];
+#pragma unroll
+        for (int k = 0; k < kConsSeg / 128; ++k) {
+            const int q = k * 128 + lane * 4, x = q & ((1 << shift) - 1);
+            const long long r = r0 + (q >> shift);
+            v[k] = float4{0.0f, 0.0f, 0.0f, 0.0f};
+            if (r < G.ny && x < G.nx) {
+                v[k] = __ldg(reinterpret_cast<const float4*>(row_of(r) + x));  // within the row's padding
+                if (x + 1 >= G.nx) v[k].y = 0.0f;
+                if (x + 2 >= G.nx) v[k].z = 0.0f;
+                if (x + 3 >= G.nx) v[k].w = 0.0f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kConsSeg / 128; ++k) {
+            a.add(pair(v[k].x, v[k].y));
+            b.add(pair(v[k].z, v[k].w));
+        }
+    }
+    for (long long u = blockIdx.x; u < units && !narrow; u += gridDim.x) {
         int n;
         const float* p = run_of(u, n);
         float4 v[kConsSeg / 128];
@@ -442,7 +524,11 @@ __global__ void __launch_bounds__(kConsThreads32, 4)
     double part[3] = {(double)s.h, (double)s.l, (double)s.c};
     if (!__shfl_sync(0xffffffffu, (int)fine, 0)) {
         double acc = 0.0;
-        for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        for (long long r0 = (long long)blockIdx.x * unit_rows; r0 < G.ny && narrow;
+             r0 += (long long)gridDim.x * unit_rows)
+            for (long long r = r0; r < r0 + unit_rows && r < G.ny; ++r)
+                for (int x = lane; x < G.nx; x += 32) acc += (double)row_of(r)[x];
+        for (long long u = blockIdx.x; u < units && !narrow; u += gridDim.x) {
             int n;
             const float* p = run_of(u, n);
             for (int x = lane; x < n; x += 32) acc += (double)p[x];
@@ -478,22 +564,30 @@ __global__ void __launch_bounds__(kConsThreads64)
     const long long units = (long long)G.ny * segs;
     const size_t pl = (size_t)G.plane;
     double s0 = 0.0, s14 = 0.0, s58 = 0.0, ax = 0.0, ay = 0.0, ar = 0.0, am = 0.0;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+    auto node = [&](const double* p) {
+        double v[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) v[i] = __ldg(p + i * pl);
+        s0 += v[0];
+        s14 += (v[1] + v[3]) + (v[2] + v[4]);
+        s58 += (v[5] + v[7]) + (v[6] + v[8]);
+        ax += v[3] - v[1];
+        ay += v[4] - v[2];
+        ar += v[7] - v[5];
+        am += v[6] - v[8];
+    };
+    const bool narrow = G.nx <= kConsNarrow;
+    if (narrow) {
+        const int shift = cons_shift(G.nx), x = threadIdx.x & ((1 << shift) - 1), rows = kConsSeg64 >> shift;
+        for (long long r = (long long)blockIdx.x * rows + (threadIdx.x >> shift); r < G.ny;
+             r += (long long)gridDim.x * rows)
+            if (x < G.nx) node(f + cell(G, x, (int)r));
+    }
+    for (long long u = blockIdx.x; u < units && !narrow; u += gridDim.x) {
         const int row = (int)(u / segs), x0 = (int)(u % segs) * kConsSeg64;
         const int n = min(kConsSeg64, G.nx - x0);
         const double* p = f + cell(G, x0, row);
-        for (int x = threadIdx.x; x < n; x += kConsThreads64) {
-            double v[9];
-#pragma unroll
-            for (int i = 0; i < 9; ++i) v[i] = __ldg(p + i * pl + x);
-            s0 += v[0];
-            s14 += (v[1] + v[3]) + (v[2] + v[4]);
-            s58 += (v[5] + v[7]) + (v[6] + v[8]);
-            ax += v[3] - v[1];
-            ay += v[4] - v[2];
-            ar += v[7] - v[5];
-            am += v[6] - v[8];
-        }
+        for (int x = threadIdx.x; x < n; x += kConsThreads64) node(p + x);
     }
     double t[4] = {s0 + s14 + s58, M.c1 * ax + M.d * (ar + am), M.c1 * ay + M.d * (ar - am),
                    M.eta2 * s0 + M.c1s * s14 + M.c2s * s58};
@@ -550,24 +644,21 @@ cudaError_t launch_sum(const double* v, int n, double* out, const unsigned* stat
 // Interior of a level <-> dense 9 x ny x nx array (kUnpack: dense to level),
 // one population row at a time in the level's order ([row][population]), V
 // values per access: 16 bytes where the dense rows allow it, else one value.
-template <typename S, int V, bool kUnpack>
+template <typename S, int V, bool kUnpack, bool kPatch>
 __global__ void __launch_bounds__(kThreads) k_pack(S* __restrict__ f, S* __restrict__ dense, const Grid<S> G) {
     struct alignas(V * sizeof(S)) Vec {
         S v[V];
     };
-    const int x = (blockIdx.x * kRowX + threadIdx.x) * V;
-    if (x >= G.nx) return;
-    const int rows = 9 * G.ny;  // ny is at most 2^24
+    int x, r;
+    if (!run_place<V, kPatch>(G.nx, 9 * G.ny, x, r)) return;  // ny is at most 2^24
+    const int iy = r / 9, i = r - iy * 9;
     const long long n = (long long)G.nx * G.ny;
-    for (int r = blockIdx.y * kRowY + threadIdx.y; r < rows; r += gridDim.y * kRowY) {
-        const int iy = r / 9, i = r - iy * 9;
-        Vec* a = reinterpret_cast<Vec*>(f + (size_t)(iy + 1) * (size_t)G.row + (size_t)i * (size_t)G.plane + (PADX + x));
-        Vec* b = reinterpret_cast<Vec*>(dense + i * n + (long long)iy * G.nx + x);
-        if constexpr (kUnpack)
-            *a = *b;
-        else
-            *b = *a;
-    }
+    Vec* a = reinterpret_cast<Vec*>(f + (size_t)(iy + 1) * (size_t)G.row + (size_t)i * (size_t)G.plane + (PADX + x));
+    Vec* b = reinterpret_cast<Vec*>(dense + i * n + (long long)iy * G.nx + x);
+    if constexpr (kUnpack)
+        *a = *b;
+    else
+        *b = *a;
 }
 
 // 4096 x 1024 in FP32 (302 MB moved): 50 us, against 218 with one element a
@@ -575,11 +666,11 @@ __global__ void __launch_bounds__(kThreads) k_pack(S* __restrict__ f, S* __restr
 template <typename S, bool kUnpack>
 cudaError_t launch_copy(S* f, S* dense, const Grid<S>& G, cudaStream_t st) {
     constexpr int V = 16 / sizeof(S);
-    const dim3 block(kRowX, kRowY);
-    if (G.nx % V == 0 && aligned(dense, 16))
-        k_pack<S, V, kUnpack><<<row_grid(G.nx, 9LL * G.ny, V), block, 0, st>>>(f, dense, G);
-    else
-        k_pack<S, 1, kUnpack><<<row_grid(G.nx, 9LL * G.ny, 1), block, 0, st>>>(f, dense, G);
+    const bool wide = G.nx % V == 0 && aligned(dense, 16);
+    const RunGrid R = run_grid(G.nx, 9LL * G.ny, wide ? V : 1);
+    auto kern = wide ? (R.patch ? k_pack<S, V, kUnpack, true> : k_pack<S, V, kUnpack, false>)
+                     : (R.patch ? k_pack<S, 1, kUnpack, true> : k_pack<S, 1, kUnpack, false>);
+    kern<<<R.grid, R.threads, 0, st>>>(f, dense, G);
     return cudaGetLastError();
 }
 

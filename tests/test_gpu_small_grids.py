@@ -339,3 +339,52 @@ def test_a_recomputation_that_gives_up_is_reported_by_the_adjoint(nx, ny, prec):
     finally:
         lbm.lbm_batch_set_wait_limit(2.0)
     assert got[0] == want[0] == lbm.LBM_OK and got[1] == want[1] != 7.0 and torch.equal(got[2], want[2])
+
+
+# Narrow grids (units of several rows, runs in the order of the rows), widths on
+# either side of where rows are cut into patches, and large grids whose rows
+# allow 16-byte, 8-byte or single accesses
+READ_OUT = [(1, 130), (2, 257), (3, 1000), (4, 129), (5, 64), (7, 33), (16, 100), (17, 9), (63, 130), (64, 65),
+            (65, 40), (100, 5), (129, 900), (257, 5), (1, 40000), (3, 70001), (1024, 1025), (1030, 1031), (1027, 1029)]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_cons", "fp32_t64"])
+@pytest.mark.parametrize("nx,ny", READ_OUT)
+def test_read_out_of_narrow_and_large_grids(nx, ny, prec):
+    """Initial levels and moments are those of the same nodes in one row, on
+    and off 16-byte boundaries; the ghost cells of an initial level are those
+    that lbm_set_f makes (one step from either); totals to 1e-14 of the sum of
+    their terms' magnitudes, also where a sum is taken again in FP64."""
+    import torch
+    p, fields = _problem(nx, ny, WALLS)
+    row, _ = _problem(nx * ny, 1, WALLS)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    shifted = []
+    for a in fields:
+        buf = torch.empty(nx * ny + 1, dtype=dt, device="cuda")[1:]
+        buf.copy_(torch.as_tensor(a.reshape(-1)))
+        shifted.append(buf)
+    with lbm.Lattice(p, prec) as lat, lbm.Lattice(row.with_(tau=p.tau, dt=p.dt), prec) as line:
+        f = lat.init(*fields).get_f()
+        assert torch.equal(line.init(*[a.reshape(1, -1) for a in fields]).get_f().reshape(9, -1), f.reshape(9, -1))
+        for a, b in zip(lat.moments(), line.moments()):
+            assert torch.equal(a.reshape(-1), b.reshape(-1))
+        sums = lat.conservation()
+        after = lat.step(1).get_f()
+        lbm.lbm_init(lat.ctx, *shifted)
+        assert torch.equal(lat.get_f(), f)
+        assert torch.equal(lat.set_f(f).step(1).get_f(), after)
+        if prec != "fp64":
+            g = f.clone()
+            g[3, ny - 1, nx - 1] = 3e38
+            g[3, 0, 0] = 3e38
+            big = lat.set_f(g).conservation()[0]
+            want = g.double().sum(dtype=torch.float64).item()
+            assert np.isfinite(big) and abs(big - want) <= 1e-14 * want
+    v = f.double().cpu().numpy().reshape(9, -1)
+    vx, vy = oracle.velocities(p.c1, p.c2)
+    e = vx ** 2 + vy ** 2
+    e[0] = p.eta0 ** 2
+    for got, w in zip(sums, (np.ones(9), vx, vy, e)):
+        terms = (w[:, None] * v).astype(np.longdouble)
+        assert abs(got - float(terms.sum())) <= 1e-14 * float(np.abs(terms).sum())
