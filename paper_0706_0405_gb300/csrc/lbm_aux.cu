@@ -15,8 +15,8 @@ inline unsigned blocks_for(long long n, int per) { return (unsigned)((n + per - 
 // the copy: see launch_pack).  Other grids -- narrow, or a row of little more
 // than so many runs -- take the runs in the order of the rows, a thread's row
 // and column from one division, in 32 bits where that is enough (4 x 100000,
-// FP32: moments 23 us, initial levels 63; in patches 54 and 141), in CTAs of
-// one warp where there are few.
+// FP32: moments 23 us, initial levels 42, get_f 21; in patches 54, 141 and 67),
+// in CTAs of one warp where there are few.
 constexpr int kRunX = 64;
 struct RunGrid {
     dim3 grid;
@@ -178,7 +178,9 @@ void init32(float* f, const float* rho, const float* ux, const float* uy, const 
 
 // One node a thread: FP64, and FP32 on large grids whose fields do not allow
 // 16-byte accesses (a run of four would be read value by value: 4095 x 1023 64
-// us, 47 here).
+// us, 40 here).  FP64 takes the nodes in their order in one-warp CTAs, and on
+// large grids leaves the ghost cells to a kernel of their own: 4096 x 1024 320
+// us, in patches and with them 347.
 template <typename S, bool kGhosts>
 __global__ void __launch_bounds__(kThreads) k_init(S* __restrict__ f, const S* __restrict__ rho,
                                                    const S* __restrict__ ux, const S* __restrict__ uy,
@@ -343,7 +345,8 @@ constexpr int kConsBlocks = 608;  // 4 per SM
 
 // Grids of at most kConsNarrow columns: a unit is kConsSeg (FP64: kConsSeg64)
 // places, 2^cons_shift columns of several rows (a row alone would leave most
-// of a warp's lanes idle: 4 x 100000, us a call, FP32 274, FP64 216).
+// of a warp's lanes idle: 4 x 100000, us a call, FP32 44 against 274, FP64 46
+// against 216).
 constexpr int kConsNarrow = 64;
 __host__ __device__ inline int cons_shift(int nx) {
     int s = 2;  // a run of four
