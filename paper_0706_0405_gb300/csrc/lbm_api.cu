@@ -912,18 +912,19 @@ lbm_status lbm_adjoint_seed(lbm_ctx* c, const void* qr, const void* qx, const vo
     const size_t fb = nodes(c) * c->esize;
     const void* in[4] = {qr, qx, qy, qT};
     const void* d[4];
-    for (const void* p : {in[0], in[1], in[2], in[3], (const void*)abar})
-        if (p && !is_device_ptr(p) && (s = ensure_astage(c, 13 * fb)) != LBM_OK) return s;
+    // (the staging buffer is made by the first host argument)
     for (int k = 0; k < 4; ++k) {
         if (!in[k] || is_device_ptr(in[k])) {
             d[k] = in[k];
         } else {
+            if ((s = ensure_astage(c, 13 * fb)) != LBM_OK) return s;
             char* dst = static_cast<char*>(c->d_astage) + (9 + k) * fb;
             LBM_CUDA(c, cudaMemcpyAsync(dst, in[k], fb, cudaMemcpyHostToDevice, c->stream), "copying host qbar");
             d[k] = dst;
         }
     }
     const bool dev_out = is_device_ptr(abar);
+    if (!dev_out && (s = ensure_astage(c, 13 * fb)) != LBM_OK) return s;
     void* out = dev_out ? abar : c->d_astage;
     cudaError_t e = dispatch(c, [&](auto tag, auto tm) {
         using S = decltype(tag);
@@ -1092,10 +1093,6 @@ lbm_status lbm_feq_vjp(lbm_ctx* c, const void* rho, const void* ux, const void* 
     if (!rho || !ux || !uy || !T || !abar) return fail(c, LBM_E_INVAL, "lbm_feq_vjp: NULL input");
     const size_t fb = nodes(c) * c->esize;
     const void* in[5] = {rho, ux, uy, T, abar};
-    for (const void* p : {in[0], in[1], in[2], in[3], in[4], (const void*)grho, (const void*)gux, (const void*)guy,
-                          (const void*)gT})
-        if (p && !is_device_ptr(p) && (s = ensure_astage(c, 17 * fb)) != LBM_OK) return s;
-    char* st = static_cast<char*>(c->d_astage);
     const size_t sz[5] = {fb, fb, fb, fb, 9 * fb};
     const size_t off[5] = {0, fb, 2 * fb, 3 * fb, 4 * fb};
     const void* d[5];
@@ -1103,8 +1100,10 @@ lbm_status lbm_feq_vjp(lbm_ctx* c, const void* rho, const void* ux, const void* 
         if (is_device_ptr(in[k])) {
             d[k] = in[k];
         } else {
-            LBM_CUDA(c, cudaMemcpyAsync(st + off[k], in[k], sz[k], cudaMemcpyHostToDevice, c->stream), "copying inputs");
-            d[k] = st + off[k];
+            if ((s = ensure_astage(c, 17 * fb)) != LBM_OK) return s;
+            char* dst = static_cast<char*>(c->d_astage) + off[k];
+            LBM_CUDA(c, cudaMemcpyAsync(dst, in[k], sz[k], cudaMemcpyHostToDevice, c->stream), "copying inputs");
+            d[k] = dst;
         }
     }
     void* outs[4] = {grho, gux, guy, gT};
@@ -1112,8 +1111,9 @@ lbm_status lbm_feq_vjp(lbm_ctx* c, const void* rho, const void* ux, const void* 
     bool host_any = false;
     for (int k = 0; k < 4; ++k) {
         const bool h = outs[k] && !is_device_ptr(outs[k]);
+        if (h && (s = ensure_astage(c, 17 * fb)) != LBM_OK) return s;
         host_any |= h;
-        dout[k] = !outs[k] ? nullptr : (h ? static_cast<void*>(st + (13 + k) * fb) : outs[k]);
+        dout[k] = h ? static_cast<char*>(c->d_astage) + (13 + k) * fb : outs[k];
     }
     cudaError_t e = dispatch(c, [&](auto tag, auto) {
         using S = decltype(tag);
