@@ -30,7 +30,7 @@ inline RunGrid run_grid(long long columns, long long rows, int V) {
     if ((few ? 2 * padded <= 3 * runs : 5 * padded <= 6 * runs) && rows >= kRunY &&
         rows <= 65535LL * kRunY)
         return {dim3((unsigned)(padded / kRunX), blocks_for(rows, kRunY)), kThreads, true};
-    const int threads = few ? 32 : kThreads;
+    const int threads = runs * rows <= 16384 ? 32 : kThreads;
     return {dim3(blocks_for(runs * rows, threads)), threads, false};
 }
 template <int V, bool kPatch>
