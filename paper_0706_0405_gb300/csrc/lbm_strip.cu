@@ -13,7 +13,9 @@
 // different operands takes three cycles on a quarter of an SM, two with one
 // that the instruction before used too (measured), so that two, three and four
 // warps to a scheduler take 24.6, 22.0 and 21.1 us a step on 256 tubes, and a
-// fifth, whose 96 registers a thread spill, 24.6.  Four CTAs of four warps
+// fifth, with 96 registers a thread, 24.6.  In the 128 registers of four, the
+// kernel of four rows spills 44 bytes a thread in the double-float mode, 20 in
+// the total-energy mode and 232 with the FP64 sum.  Four CTAs of four warps
 // to an SM, so that some load or store their columns while others compute: two
 // of eight and one of sixteen take 3 and 5 % longer.  Against the tile kernel,
 // us a step: 256 Riemann tubes 21.1 / 24.9 (total-energy mode 17.1 / 22.8), 64
@@ -105,7 +107,7 @@ __global__ void __launch_bounds__(kStripThreads, 16 / kStripWarps)
     const long long level0 = *(volatile long long*)level_ptr;
     unsigned bits = 0;
     // More rounds than CTAs: each CTA draws its next round while it works on
-    // one (an SM does not share its issue slots evenly between its two CTAs).
+    // one (an SM does not share its issue slots evenly between its CTAs).
     // Every CTA draws until it gets one past the last, rounds + gridDim.x
     // tickets a pass in all.
     const bool drawn = rounds > (int)gridDim.x;
