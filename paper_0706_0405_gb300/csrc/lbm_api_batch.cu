@@ -568,14 +568,14 @@ lbm_status lbm_batch_plant_stall(lbm_batch* b, int cta) {
     if (cta < 0) {  // back to the lists of the current grid, and to a barrier without arrivals
         b->nbr_grid = -1;
         e = batch_prepare_sync(b);
-        if (e == cudaSuccess) e = cudaMemset(b->d_bar, 0, 3 * sizeof(unsigned));
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, 3 * sizeof(unsigned), b->stream);
         batch_drop_graph(b);
         return e == cudaSuccess ? LBM_OK : bfail(b, LBM_E_CUDA, "lbm_batch_plant_stall: restoring the lists failed");
     }
     if (cta >= b->grid)
         return bfail(b, LBM_E_INVAL, "lbm_batch_plant_stall: cta must lie in [0, " + std::to_string(b->grid) + ")");
     if (b->block > 1 || !b->nbr_ok) {  // grid barriers only: one arrival too few
-        e = cudaMemset(b->d_bar, 0xff, sizeof(unsigned));
+        e = cudaMemsetAsync(b->d_bar, 0xff, sizeof(unsigned), b->stream);
         return e == cudaSuccess ? LBM_OK : bfail(b, LBM_E_CUDA, "lbm_batch_plant_stall: setting the barrier failed");
     }
     std::vector<int> lists;
